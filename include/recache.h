@@ -325,8 +325,8 @@ RECACHE_API recache_status recache_attend_decode(recache_ctx* ctx,
  *   route_rows: number of entries of route_idx (an item whose route_cu range does
  *   not lie inside it is reported as RECACHE_DEV_OVERFLOW and read as an empty route);
  *   pool_tokens > 0;
- *   max_res_pages: upper bound of ceil(route length / page_tokens), used to size
- *   the split plan and the workspace (recache_decode_workspace_bytes).
+ *   max_res_pages: upper bound of ceil(route length / page_tokens), as given to
+ *   recache_decode_workspace_bytes.
  * bf16 contexts with head_dim 128 and 64-token pages only.
  */
 RECACHE_API recache_status recache_attend_decode_gather(recache_ctx* ctx,
@@ -372,9 +372,9 @@ RECACHE_API recache_status recache_build_routes(const double* s_layers, int32_t 
  * Limits and rules
  *  - bf16 contexts with head_dim 128 and 64-token pages only (RECACHE_EUNSUPPORTED
  *    otherwise); the kernel timer must be off (it creates event objects).
- *  - batch * n_kv_heads * splits * heads-per-group * 520 bytes must fit in 4 MiB
- *    (e.g. batch 64 with 8 KV groups of 4 heads uses 2.1 MiB); beyond that the
- *    call returns RECACHE_ENOMEM with a message and launches nothing.
+ *  - batch * n_q_heads * 520 bytes must fit in 4 MiB (e.g. batch 64 with 32 query
+ *    heads: 1.0 MiB); beyond that the call returns RECACHE_ENOMEM with a message
+ *    and launches nothing.
  *  - The first call on a device looks up the scratch array's device address
  *    (once per device, with that device current).  Make that first call outside
  *    any stream capture.

@@ -365,7 +365,6 @@ recache_status recache_attend_decode(recache_ctx* ctx, const void* q, const int3
   RC_CUDA(cudaSetDevice(ctx->device), "decode: set device");
   DecodeArgs a{q, q_pos, batch, k_new, v_new, k_pages, v_pages, n_pages, res_page_table, max_res_pages, res_len,
                hist_page_table, max_hist_pages, hist_len, out_o, out_dtype, workspace, workspace_bytes};
-  if (k_new) RC_CUDA(rc_launch_decode_append(ctx, a, st), "decode: append launch");
   RC_CUDA(rc_launch_decode(ctx, a, st), "decode: attention launch");
   return RECACHE_OK;
 }
@@ -399,7 +398,6 @@ recache_status recache_attend_decode_gather(recache_ctx* ctx, const void* q, con
                hist_page_table, max_hist_pages, hist_len, out_o, out_dtype, workspace, workspace_bytes};
   a.k_cache = k_cache; a.v_cache = v_cache; a.pool_tokens = pool_tokens; a.route_idx = route_idx; a.route_cu = route_cu;
   a.route_rows = route_rows;
-  if (k_new) RC_CUDA(rc_launch_decode_append(ctx, a, st), "decode_gather: append launch");
   RC_CUDA(rc_launch_decode_split(ctx, a, st), "decode_gather: attention launch");
   return RECACHE_OK;
 }

@@ -63,6 +63,32 @@ inline void rc_fork_point(const recache_ctx* ctx, cudaStream_t st) {
   ctx->forked = ctx->side && (!ctx->timer_on || ctx->timer_attn_only) && cudaEventRecord(ctx->ev_fork, st) == cudaSuccess;
 }
 
+// ---- overlapped launches (programmatic dependent launch) ----
+// A kernel launched this way may come up while the kernel before it in the stream still runs: what
+// needs no memory (barriers, tensor memory, descriptor prefetch) overlaps that kernel's tail, and
+// rc_grid_wait() then waits until it has ended and its writes are visible.  Every block of every such
+// kernel executes rc_grid_wait() before it reads or writes global memory, also one that has nothing
+// to do: the end of a kernel then implies the end of all before it.
+__device__ __forceinline__ void rc_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next kernel of the stream come up once every block has said so (or ended).
+__device__ __forceinline__ void rc_grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline cudaError_t rc_launch_overlapped(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A&&... args) {
+  // (the opt-in to more than 48 KB of shared memory is per kernel and device: a few hundred nanoseconds)
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cfg.attrs = &at; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // First device-side error wins.
 __device__ __forceinline__ void rc_set_status(int32_t* status, int32_t code) {
   atomicCAS(status, 0, code);

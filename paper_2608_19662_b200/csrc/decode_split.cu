@@ -1,11 +1,16 @@
 // Routed split-KV decode for bf16, head_dim 128, 64-token pages: memory-bound.
 //
-// Persistent kernel, one CTA per SM.  A work unit is (item = sequence x KV group,
-// split) = a contiguous range of the item's logical pages (resource pages first,
-// then history pages).  Units are dealt round-robin to the CTAs.  Inside a CTA
-//   warp 3     : TMA producer.  Walks its units' pages in order and keeps a ring
+// Persistent kernel, one CTA per SM.  The pages of all items (item = sequence x KV group; its
+// resource pages first, then its history pages) form one list, and CTA c of n takes pages
+// T c / n .. T (c+1) / n - 1 of the T there are, across item boundaries: every CTA streams the same
+// number of bytes whatever the lengths are.  (The list is never stored: each CTA sums the items'
+// page counts itself, 512 items in about half a microsecond.  A fixed number of splits per item
+// instead made the launch as long as the longest histories' units: 16 sequences with 300 .. 4000
+// history rows took 70 us for 203 MB that way and take 46 us now; 64 equal ones 128 us and 116 us
+// for 727 MB, 6.3 TB/s.)  Inside a CTA
+//   warp 3     : TMA producer.  Walks the CTA's pages in order and keeps a ring
 //                of NSTAGE (K page + V page) buffers full; it runs ahead across
-//                unit boundaries, so the HBM stream never drains.
+//                item boundaries, so the HBM stream never drains.
 //   warps 0-2  : consumers.  The page at ring position n belongs to warp n % 3
 //                and stage n % 6, so a stage is always consumed by the same warp
 //                and that warp sees every phase of its stages' barriers in
@@ -15,9 +20,13 @@
 //                Scores: m16n8k16 over ldmatrix fragments of the swizzled K page;
 //                online softmax in registers (quad shuffles); O += P V with
 //                transposed ldmatrix fragments of the V page.
-// The consumer warps' partial (max, sum, O) are merged through shared memory; with
-// more than one split the unit's partial goes to the workspace and a second
-// small kernel merges the splits.
+// The current token's key and value (k_new / v_new) are appended by the warp that consumes the
+// item's last history page: into the page in HBM, and into the copy in shared memory, which was
+// loaded before the row existed.
+// The consumer warps' partial (max, sum, O) are merged through shared memory.  An item that lies
+// inside one CTA's range is written out there; the parts of one that spans several go to the
+// workspace (at most two per CTA: one for an item that began in an earlier CTA, one for an item
+// that goes on in a later one) and a second small kernel merges them.
 // Every K/V byte crosses HBM once; the roofline is bytes / HBM bandwidth.
 #include <cuda.h>
 
@@ -36,34 +45,33 @@ constexpr int STAGE_BYTES = 2 * PAGE_BYTES;
 // Gather variant: the resource rows of a chunk come straight from the cache with 16-byte cp.async
 // copies (half a warp per 256-byte row) written at the swizzled positions a TMA page load would use,
 // so the consumers see one layout.  Four producer warps share a chunk (16 rows each): one warp alone
-// cannot issue the 2048 copies of a chunk fast enough.  A full barrier then takes 128 arrivals: every
-// producer lane's copies (gathered chunk), or the expect-tx arrival plus 127 plain ones (TMA page).
+// cannot issue the 2048 copies of a chunk fast enough.  (TMA's four-row gather, 64 instructions a
+// chunk from one warp, is slower still: 89 us against 46 us for 16 sequences with 203 MB to read.)  A full barrier then
+// takes 128 arrivals: every producer lane's copies (gathered chunk), or the expect-tx arrival plus 127
+// plain ones (TMA page).
 constexpr int NCW = 3;                 // consumer warps; NSTAGE % NCW == 0
+constexpr int NPW_GATHER = 4;          // producer warps of the gather variant (the paged variant has one)
 static_assert(NSTAGE % NCW == 0, "a stage must always be consumed by the same warp");
-constexpr int NPW_GATHER = 4;           // producer warps of the gather variant (the paged variant has one)
-constexpr int NTHREADS = (NCW + 1) * 32;
-constexpr int NTHREADS_GATHER = (NCW + NPW_GATHER) * 32;
-constexpr int SM_STAGES = 0;
-template <bool GATHER> struct Lay {
-  static constexpr int STAGE = STAGE_BYTES;
-  static constexpr int VOFF = PAGE_BYTES;                               // V half inside a stage
-  static constexpr int BAR = NSTAGE * STAGE;                            // full[NSTAGE], empty[NSTAGE]
-  static constexpr int Q = BAR + 2 * NSTAGE * 8 + 32;                   // per-warp rotated q: NCW x 8 x 128 bf16
-  static constexpr int MERGE = Q + NCW * 8 * D * 2;                     // NCW x 8 x (2 + 128) floats
-  static constexpr int MISC = MERGE + NCW * 8 * 130 * 4;
-  static constexpr int TOTAL = MISC + 64;
-  static constexpr int ALLOC = TOTAL + 1024;
-};
-static_assert(Lay<true>::ALLOC <= 232448, "shared memory");
+template <bool GATHER> constexpr int THREADS = (NCW + (GATHER ? NPW_GATHER : 1)) * 32;
+constexpr int SM_BAR = NSTAGE * STAGE_BYTES;                          // full[NSTAGE], empty[NSTAGE]
+constexpr int SM_Q = SM_BAR + 2 * NSTAGE * 8 + 32;                    // per-warp rotated q: NCW x 8 x 128 bf16
+constexpr int SM_MERGE = SM_Q + NCW * 8 * D * 2;                      // NCW x 8 x (2 + 128) floats
+constexpr int SM_MISC = SM_MERGE + NCW * 8 * 130 * 4;                 // abort flag, the CTA's page range, scan sums
+constexpr int SM_TOTAL = SM_MISC + 64;
+constexpr int SM_ALLOC = SM_TOTAL + 1024;
+static_assert(SM_ALLOC <= 232448, "shared memory");
 constexpr uint32_t WAIT_PROBES = 1u << 21;   // ~2.8 s
 
 struct DecParams {
   const __nv_bfloat16* q; const int32_t* q_pos;
+  const __nv_bfloat16* k_new; const __nv_bfloat16* v_new;   // current token's key / value, or null
+  __nv_bfloat16* k_pages; __nv_bfloat16* v_pages;
   const int32_t* res_pt; int max_res_pages; const int32_t* res_len;
   const int32_t* hist_pt; int max_hist_pages; const int32_t* hist_len;
-  int n_items, n_splits, G, Hq, s;
+  int n_items, G, Hq, s;
   int64_t n_pages;
-  void* out; float* part_o; float* part_ml;      // partials: [unit][s][128], [unit][s][2]
+  // partials: [slot][s][128], [slot][s][2]; part_cta[item] = first and last CTA of the item
+  void* out; float* part_o; float* part_ml; int2* part_cta;
   const float* cos_tab; const float* sin_tab; int max_pos;
   float scale_log2;
   int32_t* status;
@@ -120,79 +128,117 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
 }
 __device__ __forceinline__ void bar_consumers() { asm volatile("bar.sync 1, %0;" ::"n"(NCW * 32) : "memory"); }
 
-// Pages of item `it` and the range split `sp` owns.
-struct UnitPages { int n_res_pages, n_hist_pages, p0, p1, res_len, hist_len; };
+// Pages of item `it`.  An item without a readable row still counts one page, so that its (zero)
+// output is written by somebody.
+struct ItemPages { int n_res, n_hist, total, res_len, hist_len, r0; };
 template <bool GATHER>
-__device__ __forceinline__ UnitPages unit_pages(const DecParams& p, int it, int sp) {
-  UnitPages u;
+__device__ __forceinline__ ItemPages item_pages(const DecParams& p, int it) {
+  ItemPages u;
+  u.r0 = 0;
   if (GATHER) {
     // the item's slice of the index list must lie inside it; otherwise the route is treated as empty
     const int r0 = p.route_cu[it], r1 = p.route_cu[it + 1];
     const bool ok = r0 >= 0 && r1 >= r0 && (int64_t)r1 <= p.route_rows;
     if (!ok) rc_set_status(p.status, RECACHE_DEV_OVERFLOW);
+    u.r0 = ok ? r0 : 0;
     u.res_len = ok ? r1 - r0 : 0;
   } else {
     u.res_len = max(p.res_len[it], 0);
   }
   u.hist_len = max(p.hist_len[it], 0);
-  u.n_res_pages = GATHER ? (u.res_len + PT - 1) / PT : min((u.res_len + PT - 1) / PT, p.max_res_pages);
-  u.n_hist_pages = min((u.hist_len + PT - 1) / PT, p.max_hist_pages);
-  const int total = u.n_res_pages + u.n_hist_pages;
-  u.p0 = (int)((int64_t)total * sp / p.n_splits);
-  u.p1 = (int)((int64_t)total * (sp + 1) / p.n_splits);
+  u.n_res = GATHER ? (u.res_len + PT - 1) / PT : min((u.res_len + PT - 1) / PT, p.max_res_pages);
+  u.n_hist = min((u.hist_len + PT - 1) / PT, p.max_hist_pages);
+  u.total = max(u.n_res + u.n_hist, 1);
   return u;
 }
+// CTA of n whose range of the T pages holds page x
+__device__ __forceinline__ int cta_of_page(int64_t x, int64_t T, int n) { return (int)(((x + 1) * n - 1) / T); }
 
 template <typename TO, bool GATHER>
-__global__ void __launch_bounds__(GATHER ? NTHREADS_GATHER : NTHREADS, 1) decode_split_kernel(const __grid_constant__ CUtensorMap tm_k,
+__global__ void __launch_bounds__(THREADS<GATHER>, 1) decode_split_kernel(const __grid_constant__ CUtensorMap tm_k,
                                                                    const __grid_constant__ CUtensorMap tm_v,
                                                                    const DecParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t sm = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* sm_gen = smem_raw + (sm - smem_u32(smem_raw));
-  using L = Lay<GATHER>;
-  constexpr int SM_BAR = L::BAR, SM_Q = L::Q, SM_MERGE = L::MERGE, SM_MISC = L::MISC, STAGE = L::STAGE, VOFF = L::VOFF;
   const uint32_t bars = sm + SM_BAR;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sm_gen + SM_MISC);
+  volatile int* range_sm = reinterpret_cast<volatile int*>(sm_gen + SM_MISC + 8);    // first item, pages of it before the range
+  volatile int* sums_sm = reinterpret_cast<volatile int*>(sm_gen + SM_MISC + 32);    // per-warp page sums
   auto full = [&](int i) { return bars + 8u * (uint32_t)i; };
   auto empty = [&](int i) { return bars + 8u * (uint32_t)(NSTAGE + i); };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_units = p.n_items * p.n_splits;
 
   if (threadIdx.x == 0) {
     *abort_flag = 0;
     for (int i = 0; i < NSTAGE; ++i) { mbar_init(full(i), GATHER ? 32 * NPW_GATHER : 1); mbar_init(empty(i), 1); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  rc_grid_wait();
+  rc_grid_launch_next();   // (the merge waits for this grid's end; it only comes up early)
+
+  // ---- this CTA's share of the page list: every thread sums a run of items, then one block scan ----
+  constexpr int NTHREADS = THREADS<GATHER>;
+  const int per = (p.n_items + NTHREADS - 1) / NTHREADS;
+  const int i0 = min(p.n_items, (int)threadIdx.x * per), i1 = min(p.n_items, i0 + per);
+  int sum = 0;
+#pragma unroll 4
+  for (int i = i0; i < i1; ++i) sum += item_pages<GATHER>(p, i).total;
+  int incl = sum;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += v;
+  }
+  if (lane == 31) sums_sm[warp] = incl;
   __syncthreads();
+  int before = 0, T = 0;
+#pragma unroll
+  for (int w = 0; w < NTHREADS / 32; ++w) { if (w < warp) before += sums_sm[w]; T += sums_sm[w]; }
+  const int n_cta = min((int)gridDim.x, T);          // every one of them has a page
+  if ((int)blockIdx.x >= n_cta) return;
+  const int lo = (int)((int64_t)T * blockIdx.x / n_cta), hi = (int)((int64_t)T * (blockIdx.x + 1) / n_cta);
+  before += incl - sum;
+  if (lo >= before && lo < before + sum) {
+    int i = i0, acc = before;
+    for (;; ++i) {
+      const int m = item_pages<GATHER>(p, i).total;
+      if (lo < acc + m) break;
+      acc += m;
+    }
+    range_sm[0] = i; range_sm[1] = lo - acc;
+  }
+  __syncthreads();
+  const int first_item = range_sm[0], first_off = range_sm[1];
 
   if (warp >= NCW) {
     // ===================== producer(s) =====================
     const int pw = warp - NCW;                         // producer warp index (0 in the paged variant)
-    int64_t idx_next = 0;                              // gather variant: row index prefetched for the next chunk
     uint32_t n = 0;   // pages issued so far (ring position)
-    for (int unit = blockIdx.x; unit < n_units; unit += gridDim.x) {
-      const int it = unit / p.n_splits, sp = unit % p.n_splits;
-      const UnitPages u = unit_pages<GATHER>(p, it, sp);
-      for (int lp = u.p0; lp < u.p1; ++lp, ++n) {
+    int it = first_item, off = first_off;
+    for (int pos = lo; pos < hi; ++it) {
+      const ItemPages u = item_pages<GATHER>(p, it);
+      const int p0 = off, p1 = min(u.total, off + hi - pos);
+      off = 0; pos += p1 - p0;
+      // gather variant: cache row of chunk row pw * 16 + lane % 16, fetched one chunk ahead inside an item
+      constexpr int RPW = PT / NPW_GATHER;             // rows of a chunk per producer warp (16)
+      auto load_idx = [&](int chunk) {
+        const int r = chunk * PT + pw * RPW + (lane & (RPW - 1));
+        return r < u.res_len ? p.route_idx[u.r0 + r] : 0;
+      };
+      int idx_next = GATHER && p0 < u.n_res ? load_idx(p0) : 0;
+      const int64_t group_off = (int64_t)(it % p.G) * p.pool_tokens * D;
+      for (int lp = p0; lp < p1; ++lp, ++n) {
         const int st = n % NSTAGE;
-        const uint32_t dst = sm + SM_STAGES + st * STAGE;
-        if (GATHER && lp < u.n_res_pages) {
+        const uint32_t dst = sm + st * STAGE_BYTES;
+        if (GATHER && lp < u.n_res) {
           // 64 route rows straight from the cache: half a warp copies one 256-byte row, 16 bytes per lane
-          const int g = it % p.G;
-          const int r0 = p.route_cu[it] + lp * PT;
           const int valid = min(PT, u.res_len - lp * PT);
-          constexpr int RPW = PT / NPW_GATHER;                 // rows per producer warp (16)
-          // cache row of chunk row pw * 16 + lane (lanes 0..15): fetched one chunk ahead inside a unit
-          auto load_idx = [&](int chunk) -> int64_t {
-            const int rr = chunk * PT + pw * RPW + lane;
-            return (lane < RPW && rr < u.res_len) ? (int64_t)p.route_idx[p.route_cu[it] + rr] : 0;
-          };
-          int64_t idx_l = (lp == u.p0) ? load_idx(lp) : idx_next;
-          if (lp + 1 < u.p1 && lp + 1 < u.n_res_pages) idx_next = load_idx(lp + 1);
+          int idx_l = idx_next;
+          if (lp + 1 < p1 && lp + 1 < u.n_res) idx_next = load_idx(lp + 1);
           if (idx_l < 0 || idx_l >= p.pool_tokens) {
             rc_set_status(p.status, RECACHE_DEV_BAD_SLOT);
-            idx_l = min(max(idx_l, (int64_t)0), p.pool_tokens - 1);
+            idx_l = (int)min(max((int64_t)idx_l, (int64_t)0), p.pool_tokens - 1);
           }
           if (lane == 0) mbar_wait(empty(st), ((n / NSTAGE) & 1u) ^ 1u, abort_flag, p.status);
           __syncwarp();
@@ -201,26 +247,26 @@ __global__ void __launch_bounds__(GATHER ? NTHREADS_GATHER : NTHREADS, 1) decode
           for (int rr = 0; rr < RPW; rr += 2) {
             const int lrow = rr + (lane >> 4);
             const int row = pw * RPW + lrow;
-            const int64_t idx = __shfl_sync(0xffffffffu, idx_l, lrow);
+            const int idx = __shfl_sync(0xffffffffu, idx_l, lrow);
             if (row < valid) {
-              const int64_t off = ((int64_t)g * p.pool_tokens + idx) * D + c * 8;
+              const int64_t src = group_off + (int64_t)idx * D + c * 8;
               const uint32_t d0 = dst + (c >> 3) * BOX_BYTES + row * 128 + (((c & 7) ^ (row & 7)) << 4);
-              cp_async16(d0, p.k_cache + off);
-              cp_async16(d0 + VOFF, p.v_cache + off);
+              cp_async16(d0, p.k_cache + src);
+              cp_async16(d0 + PAGE_BYTES, p.v_cache + src);
             }
           }
           cp_async_arrive(full(st));
         } else {
           if (lane == 0 && pw == 0) {
-            int pg = (!GATHER && lp < u.n_res_pages) ? p.res_pt[(int64_t)it * p.max_res_pages + lp]
-                                                     : p.hist_pt[(int64_t)it * p.max_hist_pages + (lp - u.n_res_pages)];
+            int pg = (!GATHER && lp < u.n_res) ? p.res_pt[(int64_t)it * p.max_res_pages + lp]
+                                               : p.hist_pt[(int64_t)it * p.max_hist_pages + (lp - u.n_res)];
             if (pg < 0 || pg >= p.n_pages) { rc_set_status(p.status, RECACHE_DEV_BAD_PAGE); pg = 0; }
             mbar_wait(empty(st), ((n / NSTAGE) & 1u) ^ 1u, abort_flag, p.status);
             mbar_expect_tx(full(st), STAGE_BYTES);
             tma_load_2d(dst, &tm_k, full(st), 0, pg * PT);
             tma_load_2d(dst + BOX_BYTES, &tm_k, full(st), 64, pg * PT);
-            tma_load_2d(dst + VOFF, &tm_v, full(st), 0, pg * PT);
-            tma_load_2d(dst + VOFF + BOX_BYTES, &tm_v, full(st), 64, pg * PT);
+            tma_load_2d(dst + PAGE_BYTES, &tm_v, full(st), 0, pg * PT);
+            tma_load_2d(dst + PAGE_BYTES + BOX_BYTES, &tm_v, full(st), 64, pg * PT);
           }
           if (GATHER) {           // the other 127 of the 128 arrivals a full barrier takes in this variant
             if (lane == 0 && pw != 0) mbar_wait(empty(st), ((n / NSTAGE) & 1u) ^ 1u, abort_flag, p.status);
@@ -235,34 +281,46 @@ __global__ void __launch_bounds__(GATHER ? NTHREADS_GATHER : NTHREADS, 1) decode
     // ===================== consumers =====================
     const int gq = lane >> 2, tq = lane & 3;           // fragment row (query head) and column pair
     const int s = p.s;
-    uint32_t n_base = 0;                                // ring position of the unit's first page
+    uint32_t n_base = 0;                                // ring position of the item's first page here
     __nv_bfloat16* q_sm = reinterpret_cast<__nv_bfloat16*>(sm_gen + SM_Q) + warp * 8 * D;
     float* mrg = reinterpret_cast<float*>(sm_gen + SM_MERGE);
-    for (int unit = blockIdx.x; unit < n_units; unit += gridDim.x) {
-      const int it = unit / p.n_splits, sp = unit % p.n_splits;
+    int it = first_item, off = first_off;
+    for (int pos = lo; pos < hi; ++it) {
       const int b = it / p.G, g = it % p.G;
-      const UnitPages u = unit_pages<GATHER>(p, it, sp);
-      if (sp == 0 && lane == 0 && warp == 0) {
+      const ItemPages u = item_pages<GATHER>(p, it);
+      const int p0 = off, p1 = min(u.total, off + hi - pos);
+      const int start = pos - p0;                       // the item's first page in the list
+      off = 0; pos += p1 - p0;
+      const bool whole = p0 == 0 && p1 == u.total;
+      if (p0 == 0 && lane == 0 && warp == 0) {
+        p.part_cta[it] = make_int2(blockIdx.x, whole ? (int)blockIdx.x : cta_of_page(start + u.total - 1, T, n_cta));
         if (u.hist_len < 1 || (!GATHER && (u.res_len + PT - 1) / PT > p.max_res_pages) ||
             (u.hist_len + PT - 1) / PT > p.max_hist_pages)
           rc_set_status(p.status, RECACHE_DEV_BAD_PAGE);
       }
+      const int pos_q = p.q_pos[b];
+      const bool pos_ok = pos_q >= 0 && pos_q < p.max_pos;
+      const int64_t tab = (int64_t)min(max(pos_q, 0), p.max_pos - 1) * 64;   // cos / sin row
+      if (!pos_ok) rc_set_status(p.status, RECACHE_DEV_BAD_POS);
       // ---- rotated query heads of the group -> A fragments (rows >= s are zero) ----
       {
-        int pos = p.q_pos[b];
-        if (pos < 0 || pos >= p.max_pos) { rc_set_status(p.status, RECACHE_DEV_BAD_POS); pos = min(max(pos, 0), p.max_pos - 1); }
         const __nv_bfloat16* qg = p.q + ((int64_t)b * p.Hq + g * s) * D;
-        for (int e = lane; e < 8 * 64; e += 32) {
-          const int h = e >> 6, i = e & 63;
-          float olo = 0.f, ohi = 0.f;
+        // lane -> the rotation pairs 2 lane, 2 lane + 1 of every head
+        const float2 c = *reinterpret_cast<const float2*>(p.cos_tab + tab + 2 * lane);
+        const float2 sn = *reinterpret_cast<const float2*>(p.sin_tab + tab + 2 * lane);
+#pragma unroll
+        for (int h = 0; h < 8; ++h) {
+          uint32_t wl = 0, wh = 0;
           if (h < s) {
-            const float lo = __bfloat162float(qg[h * D + i]), hi = __bfloat162float(qg[h * D + i + 64]);
-            const float c = p.cos_tab[(int64_t)pos * 64 + i], sn = p.sin_tab[(int64_t)pos * 64 + i];
-            olo = __fmaf_rn(lo, c, -__fmul_rn(hi, sn));
-            ohi = __fmaf_rn(hi, c, __fmul_rn(lo, sn));
+            wl = *reinterpret_cast<const uint32_t*>(qg + h * D + 2 * lane);
+            wh = *reinterpret_cast<const uint32_t*>(qg + h * D + 64 + 2 * lane);
           }
-          q_sm[h * D + i] = __float2bfloat16_rn(olo);
-          q_sm[h * D + i + 64] = __float2bfloat16_rn(ohi);
+          const float l0 = __uint_as_float(wl << 16), l1 = __uint_as_float(wl & 0xffff0000u);
+          const float h0 = __uint_as_float(wh << 16), h1 = __uint_as_float(wh & 0xffff0000u);
+          *reinterpret_cast<uint32_t*>(q_sm + h * D + 2 * lane) =
+              pack2(__fmaf_rn(l0, c.x, -__fmul_rn(h0, sn.x)), __fmaf_rn(l1, c.y, -__fmul_rn(h1, sn.y)));
+          *reinterpret_cast<uint32_t*>(q_sm + h * D + 64 + 2 * lane) =
+              pack2(__fmaf_rn(h0, c.x, __fmul_rn(l0, sn.x)), __fmaf_rn(h1, c.y, __fmul_rn(l1, sn.y)));
         }
         __syncwarp();
       }
@@ -279,25 +337,54 @@ __global__ void __launch_bounds__(GATHER ? NTHREADS_GATHER : NTHREADS, 1) decode
       for (int nt = 0; nt < 16; ++nt) { o[nt][0] = o[nt][1] = o[nt][2] = o[nt][3] = 0.f; }
       float m_run = -INFINITY, l_run = 0.f;      // row gq (replicated over the quad), log2 domain
 
-      // first page of the unit whose ring position belongs to this warp
+      // first page of the range whose ring position belongs to this warp
       const int first = (int)(((uint32_t)warp + NCW - n_base % NCW) % NCW);
-      for (int lp = u.p0 + first; lp < u.p1; lp += NCW) {
-        const uint32_t n = n_base + (uint32_t)(lp - u.p0);
+      for (int lp = p0 + first; lp < p1; lp += NCW) {
+        const uint32_t n = n_base + (uint32_t)(lp - p0);
         const int st = n % NSTAGE;
         // tokens of this page that exist
         int valid = PT;
-        if (lp < u.n_res_pages) valid = min(PT, u.res_len - lp * PT);
-        else valid = min(PT, u.hist_len - (lp - u.n_res_pages) * PT);
+        if (lp < u.n_res) valid = min(PT, u.res_len - lp * PT);
+        else valid = min(PT, u.hist_len - (lp - u.n_res) * PT);
         mbar_wait(full(st), (n / NSTAGE) & 1u, abort_flag, p.status);
-        const uint32_t kb = sm + SM_STAGES + st * STAGE, vb = kb + VOFF;
+        const uint32_t kb = sm + st * STAGE_BYTES, vb = kb + PAGE_BYTES;
+        const int hn = u.hist_len - 1;                   // the current token's history row
+        const bool appends = p.k_new && hn >= 0 && pos_ok && lp >= u.n_res && hn / PT == lp - u.n_res;
         if (valid < PT) {
           // slots past the end of the part were never written: clear their values (0 * NaN would poison O)
-          uint8_t* vg = sm_gen + SM_STAGES + st * STAGE + VOFF;
+          uint8_t* vg = sm_gen + st * STAGE_BYTES + PAGE_BYTES;
           const int v0 = max(valid, 0);
           for (int e = lane; e < (PT - v0) * 16; e += 32) {
             const int r = v0 + (e >> 4), c = e & 15;
             *reinterpret_cast<uint4*>(vg + (c >> 3) * BOX_BYTES + r * 128 + (c & 7) * 16) = make_uint4(0, 0, 0, 0);
           }
+        }
+        if (appends) {
+          const int pg = p.hist_pt[(int64_t)it * p.max_hist_pages + hn / PT], r = hn % PT;
+          const __nv_bfloat16* ks = p.k_new + (int64_t)it * D;
+          const __nv_bfloat16* vs = p.v_new + (int64_t)it * D;
+          if (pg >= 0 && pg < p.n_pages) {
+            uint8_t* kg = sm_gen + st * STAGE_BYTES + r * 128;
+            const int64_t row = ((int64_t)pg * PT + r) * D;
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {                // element i of the low half, i + 64 of the high half (next box)
+              const int i = lane + 32 * x;
+              const float l = __bfloat162float(ks[i]), h = __bfloat162float(ks[i + 64]);
+              const float c = p.cos_tab[tab + i], sn = p.sin_tab[tab + i];
+              const __nv_bfloat16 kl = __float2bfloat16_rn(__fmaf_rn(l, c, -__fmul_rn(h, sn)));
+              const __nv_bfloat16 kh = __float2bfloat16_rn(__fmaf_rn(h, c, __fmul_rn(l, sn)));
+              const __nv_bfloat16 vl = vs[i], vh = vs[i + 64];
+              uint8_t* e = kg + (((i >> 3) ^ (r & 7)) << 4) + (i & 7) * 2;
+              *reinterpret_cast<__nv_bfloat16*>(e) = kl;
+              *reinterpret_cast<__nv_bfloat16*>(e + BOX_BYTES) = kh;
+              *reinterpret_cast<__nv_bfloat16*>(e + PAGE_BYTES) = vl;
+              *reinterpret_cast<__nv_bfloat16*>(e + PAGE_BYTES + BOX_BYTES) = vh;
+              p.k_pages[row + i] = kl; p.k_pages[row + i + 64] = kh;
+              p.v_pages[row + i] = vl; p.v_pages[row + i + 64] = vh;
+            }
+          }
+        }
+        if (valid < PT || appends) {
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // a later TMA load overwrites these bytes
           __syncwarp();
         }
@@ -362,7 +449,7 @@ __global__ void __launch_bounds__(GATHER ? NTHREADS_GATHER : NTHREADS, 1) decode
         __syncwarp();
         if (lane == 0) mbar_arrive(empty(st));
       }
-      n_base += (uint32_t)(u.p1 - u.p0);
+      n_base += (uint32_t)(p1 - p0);
 
       // ---- merge the consumer warps' partials (rows gq < s) ----
       if (gq < s) {
@@ -390,7 +477,7 @@ __global__ void __launch_bounds__(GATHER ? NTHREADS_GATHER : NTHREADS, 1) decode
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[c] += ow[c] * f;
           }
-          if (p.n_splits == 1) {
+          if (whole) {
             const float inv = Lsum > 0.f ? 1.f / Lsum : 0.f;
             TO* orow = reinterpret_cast<TO*>(p.out) + ((int64_t)b * p.Hq + g * s + h) * D + (t & 31) * 4;
             if constexpr (sizeof(TO) == 4) {
@@ -399,9 +486,9 @@ __global__ void __launch_bounds__(GATHER ? NTHREADS_GATHER : NTHREADS, 1) decode
               *reinterpret_cast<uint2*>(orow) = make_uint2(pack2(acc[0] * inv, acc[1] * inv), pack2(acc[2] * inv, acc[3] * inv));
             }
           } else {
-            float* po = p.part_o + ((int64_t)unit * s + h) * D + (t & 31) * 4;
-            *reinterpret_cast<float4*>(po) = make_float4(acc[0], acc[1], acc[2], acc[3]);
-            if ((t & 31) == 0) { p.part_ml[((int64_t)unit * s + h) * 2] = M; p.part_ml[((int64_t)unit * s + h) * 2 + 1] = Lsum; }
+            const int row = (2 * (int)blockIdx.x + (p0 == 0 ? 1 : 0)) * s + h;     // the CTA's slot for this part
+            *reinterpret_cast<float4*>(p.part_o + (int64_t)row * D + (t & 31) * 4) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+            if ((t & 31) == 0) *reinterpret_cast<float2*>(p.part_ml + row * 2) = make_float2(M, Lsum);
           }
         }
       }
@@ -411,28 +498,54 @@ __global__ void __launch_bounds__(GATHER ? NTHREADS_GATHER : NTHREADS, 1) decode
   if (*abort_flag) rc_timeout_drain();   // a wait ran out: let the loads in flight land before the CTA ends
 }
 
-// Combines the splits of every (sequence, head): one warp per output row (32 lanes x 4 dims), eight
-// rows per CTA.
-constexpr int MERGE_ROWS = 8;
+// Combines the parts of the items that span several CTAs: one warp per output row (32 lanes x 4
+// dims), MERGE_ROWS rows per CTA.  The parts of item it lie in slot 2a + 1 of its first CTA a and
+// slots 2c of the later ones up to b.  Lanes read 32 (max, sum) pairs at a time, and the rows of O
+// behind them eight at a time, so that the few microseconds are not one chain of loads.
+constexpr int MERGE_ROWS = 4;
 template <typename TO>
 __global__ void __launch_bounds__(32 * MERGE_ROWS) decode_merge_kernel(const float* __restrict__ part_o,
                                                                        const float* __restrict__ part_ml,
-                                                                       TO* __restrict__ out, int n_rows, int n_splits, int G, int Hq, int s) {
+                                                                       const int2* __restrict__ part_cta,
+                                                                       TO* __restrict__ out, int n_rows, int G, int Hq, int s) {
+  rc_grid_wait();
+  rc_grid_launch_next();
   const int row = blockIdx.x * MERGE_ROWS + (threadIdx.x >> 5);   // b * Hq + head
   if (row >= n_rows) return;
   const int b = row / Hq, head = row % Hq, g = head / s, h = head % s;
-  const int it = b * G + g;
   const int t = threadIdx.x & 31;
-  float M = -INFINITY;
-  for (int sp = 0; sp < n_splits; ++sp) M = fmaxf(M, part_ml[((int64_t)(it * n_splits + sp) * s + h) * 2]);
-  float L = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int sp = 0; sp < n_splits; ++sp) {
-    const int64_t u = ((int64_t)(it * n_splits + sp) * s + h);
-    const float mw = part_ml[u * 2];
-    const float f = mw == -INFINITY ? 0.f : ex2(mw - M);
-    L += part_ml[u * 2 + 1] * f;
-    const float4 v = *reinterpret_cast<const float4*>(part_o + u * D + t * 4);
-    acc[0] += v.x * f; acc[1] += v.y * f; acc[2] += v.z * f; acc[3] += v.w * f;
+  const int2 ab = part_cta[b * G + g];
+  if (ab.x == ab.y) return;                                        // written by the CTA that had all of it
+  const int n = ab.y - ab.x + 1;
+  auto slot_row = [&](int i) { return (i == 0 ? 2 * ab.x + 1 : 2 * (ab.x + i)) * s + h; };
+  float M = -INFINITY, L = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int i0 = 0; i0 < n; i0 += 32) {
+    float2 ml = make_float2(-INFINITY, 0.f);
+    if (i0 + t < n) ml = *reinterpret_cast<const float2*>(part_ml + slot_row(i0 + t) * 2);
+    float m_new = fmaxf(M, ml.x);
+#pragma unroll
+    for (int off = 16; off; off >>= 1) m_new = fmaxf(m_new, __shfl_xor_sync(0xffffffffu, m_new, off));
+    const float m_use = m_new == -INFINITY ? 0.f : m_new;
+    const float corr = ex2(M - m_use), f = ex2(ml.x - m_use);      // 0 where nothing was seen yet / in that part
+    M = m_new;
+    float l = ml.y * f;
+#pragma unroll
+    for (int off = 16; off; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+    L = L * corr + l;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[c] *= corr;
+    const int cnt = min(32, n - i0);
+    for (int j0 = 0; j0 < cnt; j0 += 8) {
+      float4 v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (j0 + j < cnt) v[j] = *reinterpret_cast<const float4*>(part_o + (int64_t)slot_row(i0 + j0 + j) * D + t * 4);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float fj = __shfl_sync(0xffffffffu, f, (j0 + j) & 31);
+        if (j0 + j < cnt) { acc[0] += v[j].x * fj; acc[1] += v[j].y * fj; acc[2] += v[j].z * fj; acc[3] += v[j].w * fj; }
+      }
+    }
   }
   const float inv = L > 0.f ? 1.f / L : 0.f;
   TO* orow = out + (int64_t)row * D + t * 4;
@@ -479,73 +592,57 @@ bool rc_decode_split_supported(const recache_ctx* ctx) {
   return ctx->desc.dtype == RECACHE_BF16 && ctx->desc.head_dim == 128 && ctx->desc.page_tokens == PT && s <= 8;
 }
 
-// Splits per item: the smallest count that fills the persistent grid evenly
-// (units / SMs close to an integer from below) while a split keeps >= 4 pages.
-int rc_decode_n_splits(const recache_ctx* ctx, int batch, int max_res_pages, int max_hist_pages) {
-  const int items = batch * ctx->desc.n_kv_heads, sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
-  const int pages = max_res_pages + max_hist_pages;
-  int best = 1; double best_eff = 0.0;
-  for (int ns = 1; ns <= 16; ++ns) {
-    if (ns > 1 && pages / ns < 4) break;
-    const int units = items * ns;
-    const double eff = (double)units / ((double)((units + sms - 1) / sms) * sms);
-    if (eff > best_eff + 0.02) { best_eff = eff; best = ns; }
-  }
-  return best;
-}
+static int grid_ctas(const recache_ctx* ctx) { return ctx->sm_count > 0 ? ctx->sm_count : 148; }
 
 int64_t rc_decode_split_workspace_bytes(const recache_ctx* ctx, int batch, int max_res_pages, int max_hist_pages) {
-  const int ns = rc_decode_n_splits(ctx, batch, max_res_pages, max_hist_pages);
   const int s = ctx->desc.n_q_heads / ctx->desc.n_kv_heads;
-  const int64_t units = (int64_t)batch * ctx->desc.n_kv_heads * ns;
-  return align256(units * s * D * 4) + align256(units * s * 2 * 4);
+  const int64_t slots = 2 * (int64_t)grid_ctas(ctx);
+  return align256(slots * s * D * 4) + align256(slots * s * 2 * 4) + align256((int64_t)batch * ctx->desc.n_kv_heads * 8);
 }
 
 cudaError_t rc_launch_decode_split(const recache_ctx* ctx, const DecodeArgs& a, cudaStream_t st) {
   const int G = ctx->desc.n_kv_heads, Hq = ctx->desc.n_q_heads, s = Hq / G;
-  const int ns = rc_decode_n_splits(ctx, a.batch, a.max_res_pages, a.max_hist_pages);
-  const int64_t units = (int64_t)a.batch * G * ns;
   if ((uint64_t)a.n_pages * PT > 0x7fffffffull) return cudaErrorInvalidValue;   // TMA coordinates are 32-bit row indices
+  const bool f32 = a.out_dtype == RECACHE_F32, gather = a.route_idx != nullptr;
   CUtensorMap tk, tv;
   if (!map_pages(&tk, a.k_pages, (uint64_t)a.n_pages) || !map_pages(&tv, a.v_pages, (uint64_t)a.n_pages))
     return cudaErrorInvalidValue;
+  const int64_t slots = 2 * (int64_t)grid_ctas(ctx);
   DecParams p;
   p.q = (const __nv_bfloat16*)a.q; p.q_pos = a.q_pos;
+  p.k_new = (const __nv_bfloat16*)a.k_new; p.v_new = (const __nv_bfloat16*)a.v_new;
+  p.k_pages = (__nv_bfloat16*)a.k_pages; p.v_pages = (__nv_bfloat16*)a.v_pages;
   p.res_pt = a.res_pt; p.max_res_pages = a.max_res_pages; p.res_len = a.res_len;
   p.hist_pt = a.hist_pt; p.max_hist_pages = a.max_hist_pages; p.hist_len = a.hist_len;
-  p.n_items = a.batch * G; p.n_splits = ns; p.G = G; p.Hq = Hq; p.s = s; p.n_pages = a.n_pages;
+  p.n_items = a.batch * G; p.G = G; p.Hq = Hq; p.s = s; p.n_pages = a.n_pages;
   p.out = a.o;
-  p.part_o = (float*)a.workspace;
-  p.part_ml = (float*)((uint8_t*)a.workspace + align256(units * s * D * 4));
+  uint8_t* ws = (uint8_t*)a.workspace;
+  p.part_o = (float*)ws; ws += align256(slots * s * D * 4);
+  p.part_ml = (float*)ws; ws += align256(slots * s * 2 * 4);
+  p.part_cta = (int2*)ws;
   p.cos_tab = ctx->cos_tab; p.sin_tab = ctx->sin_tab; p.max_pos = ctx->desc.max_pos;
   p.scale_log2 = (float)(1.4426950408889634 / sqrt((double)D));
   p.status = ctx->status;
   p.k_cache = (const __nv_bfloat16*)a.k_cache; p.v_cache = (const __nv_bfloat16*)a.v_cache;
   p.pool_tokens = a.pool_tokens; p.route_idx = a.route_idx; p.route_cu = a.route_cu; p.route_rows = a.route_rows;
-  const int sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
-  const unsigned grid = (unsigned)(units < sms ? units : sms);
-  const bool f32 = a.out_dtype == RECACHE_F32, gather = a.route_idx != nullptr;
+  // no more CTAs than pages there can be; the paged kernel's lengths live on the device, the tables' widths here
+  const int64_t most = (int64_t)p.n_items * (a.max_res_pages + (int64_t)a.max_hist_pages);
+  const unsigned grid = (unsigned)(gather || most > grid_ctas(ctx) ? grid_ctas(ctx) : (most > 0 ? most : 1));
+  cudaError_t e;
   {
     RcLaunchScope scope(ctx, RC_K_DECODE_ATTN, st);
-    auto launch = [&](auto kernel, int smem) {
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      kernel<<<grid, gather ? NTHREADS_GATHER : NTHREADS, smem, st>>>(tk, tv, p);
-    };
-    if (gather) {
-      if (f32) launch(decode_split_kernel<float, true>, Lay<true>::ALLOC);
-      else launch(decode_split_kernel<__nv_bfloat16, true>, Lay<true>::ALLOC);
-    } else {
-      if (f32) launch(decode_split_kernel<float, false>, Lay<false>::ALLOC);
-      else launch(decode_split_kernel<__nv_bfloat16, false>, Lay<false>::ALLOC);
-    }
+    auto launch = [&](auto kernel) { return rc_launch_overlapped(kernel, grid, gather ? THREADS<true> : THREADS<false>, SM_ALLOC, st, tk, tv, p); };
+    if (gather) e = f32 ? launch(decode_split_kernel<float, true>) : launch(decode_split_kernel<__nv_bfloat16, true>);
+    else e = f32 ? launch(decode_split_kernel<float, false>) : launch(decode_split_kernel<__nv_bfloat16, false>);
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || ns == 1) return e;
+  if (e != cudaSuccess) return e;
   RcLaunchScope scope(ctx, RC_K_DECODE_MERGE, st);
   const int n_rows = a.batch * Hq, blocks = (n_rows + MERGE_ROWS - 1) / MERGE_ROWS;
-  if (f32) decode_merge_kernel<float><<<blocks, 32 * MERGE_ROWS, 0, st>>>(p.part_o, p.part_ml, (float*)a.o, n_rows, ns, G, Hq, s);
-  else decode_merge_kernel<__nv_bfloat16><<<blocks, 32 * MERGE_ROWS, 0, st>>>(p.part_o, p.part_ml, (__nv_bfloat16*)a.o, n_rows, ns, G, Hq, s);
-  return cudaGetLastError();
+  if (f32)
+    return rc_launch_overlapped(decode_merge_kernel<float>, blocks, 32 * MERGE_ROWS, 0, st, (const float*)p.part_o, (const float*)p.part_ml,
+                                (const int2*)p.part_cta, (float*)a.o, n_rows, G, Hq, s);
+  return rc_launch_overlapped(decode_merge_kernel<__nv_bfloat16>, blocks, 32 * MERGE_ROWS, 0, st, (const float*)p.part_o,
+                              (const float*)p.part_ml, (const int2*)p.part_cta, (__nv_bfloat16*)a.o, n_rows, G, Hq, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -593,9 +690,10 @@ extern "C" RECACHE_API recache_status recache_attend_decode_noalloc(
     return fail(RECACHE_EUNSUPPORTED, "decode_noalloc: needs a bf16 context with head_dim 128 and 64-token pages");
   if (ctx->timer_on)
     return fail(RECACHE_EINVAL, "decode_noalloc: the kernel timer creates event objects; disable it first");
+  // the contract's bound is one unsplit partial per (sequence, query head); what a call really needs is below it
   const int64_t need = rc_decode_split_workspace_bytes(ctx, batch, max_res_pages, max_hist_pages);
-  if (need > NOALLOC_SCRATCH_BYTES)
-    return fail(RECACHE_ENOMEM, "decode_noalloc: batch x groups x splits exceeds the 4 MiB built-in scratch; "
+  if (need > NOALLOC_SCRATCH_BYTES || (int64_t)batch * ctx->desc.n_q_heads * (D + 2) * 4 > NOALLOC_SCRATCH_BYTES)
+    return fail(RECACHE_ENOMEM, "decode_noalloc: batch x query heads x 520 bytes exceeds the 4 MiB built-in scratch; "
                                 "use recache_attend_decode with a caller workspace");
   if (ctx->device < 0 || ctx->device >= NOALLOC_MAX_DEVICES)
     return fail(RECACHE_EUNSUPPORTED, "decode_noalloc: device index out of range");
@@ -614,9 +712,7 @@ extern "C" RECACHE_API recache_status recache_attend_decode_noalloc(
   cudaStream_t st = (cudaStream_t)stream;
   DecodeArgs a{q, q_pos, batch, k_new, v_new, k_pages, v_pages, n_pages, res_page_table, max_res_pages, res_len,
                hist_page_table, max_hist_pages, hist_len, out_o, out_dtype, scratch, NOALLOC_SCRATCH_BYTES};
-  cudaError_t e = cudaSuccess;
-  if (k_new) e = rc_launch_decode_append(ctx, a, st);
-  if (e == cudaSuccess) e = rc_launch_decode_split(ctx, a, st);
+  const cudaError_t e = rc_launch_decode_split(ctx, a, st);
   if (e != cudaSuccess) {
     ctx->err = std::string("decode_noalloc: launch: ") + cudaGetErrorString(e);
     return RECACHE_ECUDA;

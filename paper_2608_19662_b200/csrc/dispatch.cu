@@ -42,6 +42,10 @@ cudaError_t rc_launch_prefill_attn(const recache_ctx* ctx, const PrefillArgs& a,
 }
 
 cudaError_t rc_launch_decode(const recache_ctx* ctx, const DecodeArgs& a, cudaStream_t st) {
-  if (rc_decode_split_supported(ctx)) return rc_launch_decode_split(ctx, a, st);
+  if (rc_decode_split_supported(ctx)) return rc_launch_decode_split(ctx, a, st);   // appends k_new / v_new itself
+  if (a.k_new) {
+    const cudaError_t e = rc_launch_decode_append(ctx, a, st);
+    if (e != cudaSuccess) return e;
+  }
   return rc_launch_decode_rows(ctx, a, st);
 }
