@@ -123,9 +123,8 @@ RECACHE_API recache_status recache_selftest_wait_timeout(recache_ctx* ctx, int32
  *   recache_kernel_name(id)     static string, id in [0, K)
  *   recache_kernel_timer(ctx,e) 0 = off, 1 = every launch, 2 = the two attention launches only (light
  *       enough to leave on inside a timed region); clears counters and pending events.
- *       With 0 or 2 the small set-up kernel of the tensor-core attention runs on a
- *       second stream of the context beside the call's first kernel (forked from and
- *       joined to the caller's stream by events); with 1 everything stays on one stream.
+ *       With 0 or 2 a kernel's set-up overlaps the end of the kernel before it; the
+ *       events of 1 keep the kernels apart.
  *   recache_kernel_times(ctx, ms_total[K], launches[K])  waits for the recorded
  *       events, returns per-kernel summed device time in ms (0 when the timer
  *       was off) and launch counts since the last clear, then clears both.

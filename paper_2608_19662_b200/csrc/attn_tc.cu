@@ -34,12 +34,12 @@
 // bit-identical outputs whatever else is in the launch.
 #include <cuda.h>
 
-#include "common.cuh"
+#include "tile_plan.cuh"
 
 namespace {
 
 constexpr int D = 128;
-constexpr int TILE_N = 128;
+constexpr int TILE_N = RC_TILE_N;
 constexpr int NSTAGE = 2;
 constexpr int BOX_BYTES = 16384;   // [128 rows][64 bf16], 128-byte swizzle
 constexpr int TILE_BYTES = 32768;  // two boxes: head_dim halves
@@ -66,49 +66,15 @@ static_assert(B_COUNT <= 32, "barrier area");
 
 constexpr uint32_t COL_S = 0, COL_O = 256;           // + 128 * tile
 
-constexpr int SORT_MAX = 4096;                      // work items up to which the plan sorts a prefill by weight (encode: a quarter)
-
 constexpr uint32_t WAIT_PROBES = 1u << 21;           // ~2.8 s of suspended probes: a wait this long is a bug, not load
 
-struct TcParams {
-  const int2* items; int32_t* header;   // header[0] = number of items, header[1] = work counter, header[2] = order[] is valid
-  const int32_t* order;                 // work indices, heaviest first (launches of at most SORT_MAX work items)
+struct TcParams : RcPlan {
   // gather mode: route row n of group g is row route_idx[n] of gather_k / gather_v ([G][pool_tokens][128] bf16)
   const uint8_t* gather_k; const uint8_t* gather_v; const int32_t* route_idx; int64_t pool_tokens;
-  const int32_t* cu; const int32_t* pos0; const int32_t* slot; const int32_t* route_cu; const int32_t* hist;
-  int n_seq, G, Hq, s;
-  int prefix_len;   // > 0: every sequence sees rows g*prefix_len .. of the "route" tensors (shared prefix)
-  int64_t self_rows;
-  int64_t route_rows;   // rows of the packed route tensors / entries of route_idx
   void* out;
   const float* cos_tab; const float* sin_tab; int max_pos;
   float scale_log2;
-  int32_t* status;
 };
-
-// Optional in-kernel timeline (build with -DRC_TRACE; never part of the shipped library): CTA 0
-// stamps %clock64 at the hand-overs of its first TR_ITEMS work items, one row of 16 stamps per
-// (role, item).  Without the flag the macro is empty.
-#ifdef RC_TRACE
-constexpr int TR_ITEMS = 192, TR_ROLES = 5;   // roles: softmax A, softmax B, MMA, epilogue, producer
-__device__ long long g_trace[TR_ROLES * TR_ITEMS * 16];
-#ifndef RC_TRACE_ROLES
-#define RC_TRACE_ROLES 31   // bit per role: stamping the 32-register roles disturbs them most
-#endif
-#define TR(role, item, k) do { if (((RC_TRACE_ROLES >> (role)) & 1) && blockIdx.x == 0 && (item) < (uint32_t)TR_ITEMS) g_trace[((role) * TR_ITEMS + (item)) * 16 + (k)] = clock64(); } while (0)
-#define TRV(role, item, k, v) do { if (((RC_TRACE_ROLES >> (role)) & 1) && blockIdx.x == 0 && (item) < (uint32_t)TR_ITEMS) g_trace[((role) * TR_ITEMS + (item)) * 16 + (k)] = (v); } while (0)
-#else
-#define TR(role, item, k) do {} while (0)
-#define TRV(role, item, k, v) do {} while (0)
-#endif
-// A second, non-intrusive form (-DRC_OBSERVE): the otherwise idle warp 11 of CTA 0 polls the CTA's
-// barriers with test_wait and logs (clock, barrier) whenever one completes a phase, so the timeline
-// of the hand-overs is seen without a single extra instruction in the working roles.
-#ifdef RC_OBSERVE
-constexpr int OBS_PER = 2048;                 // events per barrier
-__device__ long long g_observe[32 * OBS_PER];   // row 31, entry 0: start time
-__device__ int g_observe_n[32];
-#endif
 
 // ------------------------------------------------------------------ PTX --
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -262,188 +228,9 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&p);
 }
 
-// One work item as published by the scheduler warp (16 ints in shared memory).
-struct Item {
-  int n_tiles;      // -1: no more work
-  int g, seq0, L, tok0, kv_end, pos0, rA0, lenA, nA, b_valid;
-  int H;            // rows that precede the sequence's own tokens in the self part (earlier turns), all visible
-  int64_t base;
-};
+using Item = RcItem;
 enum { IT_NTILES = 0, IT_G, IT_SEQ0, IT_L, IT_TOK0, IT_KVEND, IT_POS0, IT_RA0, IT_LENA, IT_NA, IT_BVALID, IT_BASE_LO,
        IT_BASE_HI, IT_H, IT_WORDS = 16 };
-
-// Work index w -> item; false when the caller's index arrays are inconsistent
-// (flagged in the status word; the scheduler skips the item).
-__device__ __forceinline__ bool load_item(const TcParams& p, int w, Item& it) {
-  const int2 e = p.items[w / p.G];
-  it.g = w % p.G;
-  const int b = e.x;
-  const int TQ = 128 / p.s;
-  it.seq0 = p.cu[b];
-  it.L = p.cu[b + 1] - it.seq0;
-  it.tok0 = e.y * 2 * TQ;
-  it.b_valid = it.tok0 + TQ < it.L;
-  it.H = p.hist ? p.hist[b] : 0;
-  it.kv_end = it.H + min(it.L, it.tok0 + 2 * TQ);   // self rows the pair can see: the history, then its causal range
-  it.base = p.slot ? (int64_t)p.slot[b] : (int64_t)it.seq0;
-  it.pos0 = p.pos0 ? p.pos0[b] : 0;
-  it.rA0 = 0; it.lenA = 0;
-  bool route_ok = true;
-  if (p.route_cu) {
-    it.rA0 = p.route_cu[b * p.G + it.g]; it.lenA = p.route_cu[b * p.G + it.g + 1] - it.rA0;
-    route_ok = (int64_t)it.rA0 + it.lenA <= p.route_rows;   // e.g. after a compaction that overflowed its capacity
-  }
-  else if (p.prefix_len > 0) { it.rA0 = it.g * p.prefix_len; it.lenA = p.prefix_len; }
-  it.nA = (it.lenA + TILE_N - 1) / TILE_N;
-  it.n_tiles = it.nA + (it.kv_end + TILE_N - 1) / TILE_N;
-  const bool ok = it.L > 0 && it.tok0 < it.L && it.lenA >= 0 && it.rA0 >= 0 && it.base >= 0 && it.H >= 0 &&
-                  it.base + it.H + it.L <= p.self_rows && it.seq0 >= 0 && route_ok;
-  if (!ok) rc_set_status(p.status, route_ok ? RECACHE_DEV_BAD_SLOT : RECACHE_DEV_OVERFLOW);
-  return ok;
-}
-
-// ------------------------------------------------------------- work list --
-// Items = (sequence, tile-pair index): sequence by sequence, the longest sequences
-// first, and inside a sequence the last (heaviest) tile pair first, so that the
-// launch ends on the light items of short sequences.  With the KV group as the
-// fastest index of the flattened work list, the CTAs that run at the same time
-// share one sequence's K/V, which then stays in L2 instead of being streamed
-// from HBM once per tile pair.  One CTA.  (Sequences of equal length land in an
-// order that may differ between launches; no result depends on it.)
-__global__ void __launch_bounds__(1024) tile_plan_kernel(const TcParams p, int tok_per_cta, int n_levels,
-                                                         int2* __restrict__ items, int32_t* __restrict__ level_off,
-                                                         int32_t* __restrict__ order, int max_items) {
-  __shared__ int warp_sum[32];
-  __shared__ int hist[1025];
-  const int n_seq = p.n_seq;
-  const int32_t* cu = p.cu;
-  // each thread owns a contiguous chunk of sequences: local sums, block scan of the chunk sums, then the items
-  const int per = (n_seq + blockDim.x - 1) / blockDim.x;
-  const int b0 = min(n_seq, (int)threadIdx.x * per), b1 = min(n_seq, b0 + per);
-  int sum = 0;
-  for (int b = b0; b < b1; ++b) {
-    const int len = cu[b + 1] - cu[b];
-    if (len < 0) rc_set_status(p.status, RECACHE_DEV_BAD_SEQLENS);
-    int nt = len > 0 ? (len + tok_per_cta - 1) / tok_per_cta : 0;
-    if (nt > n_levels) { rc_set_status(p.status, RECACHE_DEV_BAD_SEQLENS); nt = n_levels; }   // longer than the max_len given
-    sum += nt;
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int incl = sum;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, incl, off);
-    if (lane >= off) incl += v;
-  }
-  if (lane == 31) warp_sum[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    int w = warp_sum[lane], wi = w;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, wi, off);
-      if (lane >= off) wi += v;
-    }
-    warp_sum[lane] = wi - w;   // exclusive
-    if (lane == 31) {
-      p.header[0] = wi < max_items ? wi : max_items;
-      p.header[1] = 0;         // dynamic work counter of the attention kernel
-    }
-  }
-  __syncthreads();
-  // (an encode launch shares K/V between the items of a sequence only: beyond a thousand items the
-  // sequence-major order, which keeps a sequence's K/V in L2, is worth more than the balance)
-  const int n_work = p.header[0] * p.G;
-  const bool sorted = n_work <= (p.route_cu ? SORT_MAX : SORT_MAX / 4);
-  if (sorted) {
-    // few work items: they are sorted one by one below, so the sequences keep their order here
-    int k = warp_sum[warp] + incl - sum;
-    for (int b = b0; b < b1; ++b) {
-      const int len = cu[b + 1] - cu[b];
-      int nt = len > 0 ? (len + tok_per_cta - 1) / tok_per_cta : 0;
-      if (nt > n_levels) nt = n_levels;
-      level_off[b] = k;
-      for (int l = nt - 1; l >= 0; --l, ++k)
-        if (k < max_items) items[k] = make_int2(b, l);
-    }
-  } else {
-    // counting sort of the sequences by their number of tile pairs, longest first: hist[bin] = items of
-    // that bin, then (scanned from the top bin down) the first item index of the bin
-    for (int i = threadIdx.x; i < 1025; i += blockDim.x) hist[i] = 0;
-    __syncthreads();
-    for (int b = b0; b < b1; ++b) {
-      const int len = cu[b + 1] - cu[b];
-      int nt = len > 0 ? (len + tok_per_cta - 1) / tok_per_cta : 0;
-      if (nt > n_levels) nt = n_levels;
-      if (nt > 0) atomicAdd(&hist[min(nt, 1024)], nt);
-    }
-    __syncthreads();
-    if (warp == 0) {
-      int carry = 0;
-      for (int c0 = 1024; c0 >= 0; c0 -= 32) {      // lane 0 takes the highest bin of the chunk
-        const int bin_i = c0 - lane;
-        const int v = bin_i >= 0 ? hist[bin_i] : 0;
-        int vi = v;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-          const int u = __shfl_up_sync(0xffffffffu, vi, off);
-          if (lane >= off) vi += u;
-        }
-        if (bin_i >= 0) hist[bin_i] = carry + vi - v;
-        carry += __shfl_sync(0xffffffffu, vi, 31);
-      }
-    }
-    __syncthreads();
-    for (int b = b0; b < b1; ++b) {
-      const int len = cu[b + 1] - cu[b];
-      int nt = len > 0 ? (len + tok_per_cta - 1) / tok_per_cta : 0;
-      if (nt > n_levels) nt = n_levels;
-      if (nt == 0) continue;
-      int k = atomicAdd(&hist[min(nt, 1024)], nt);
-      level_off[b] = k;
-      for (int l = nt - 1; l >= 0; --l, ++k)
-        if (k < max_items) items[k] = make_int2(b, l);
-    }
-  }
-  // Few work items (a prefill of a handful of requests): one CTA gets one or two of them, so their
-  // order decides the tail.  Sort them by weight (K/V tiles), heaviest first, with a counting sort.
-  __syncthreads();
-  if (threadIdx.x == 0) p.header[2] = sorted ? 1 : 0;
-  if (!sorted) return;
-  for (int i = threadIdx.x; i < 1025; i += blockDim.x) hist[i] = 0;
-  __syncthreads();
-  int bin[SORT_MAX / 1024];
-#pragma unroll
-  for (int j = 0; j < SORT_MAX / 1024; ++j) {
-    const int w = threadIdx.x + j * 1024;
-    bin[j] = -1;
-    if (w < n_work) {
-      Item it;
-      const bool ok = load_item(p, w, it);
-      bin[j] = 1024 - (ok ? min(it.n_tiles, 1024) : 0);   // heaviest first
-      atomicAdd(&hist[bin[j]], 1);
-    }
-  }
-  __syncthreads();
-  if (warp == 0) {   // exclusive scan of the 1025 bins
-    int carry = 0;
-    for (int c0 = 0; c0 < 1025; c0 += 32) {
-      const int v = c0 + lane < 1025 ? hist[c0 + lane] : 0;
-      int vi = v;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, vi, off);
-        if (lane >= off) vi += u;
-      }
-      if (c0 + lane < 1025) hist[c0 + lane] = carry + vi - v;
-      carry += __shfl_sync(0xffffffffu, vi, 31);
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int j = 0; j < SORT_MAX / 1024; ++j)
-    if (bin[j] >= 0) order[atomicAdd(&hist[bin[j]], 1)] = threadIdx.x + j * 1024;
-}
 
 // ---------------------------------------------------------------- kernel --
 // Persistent: a scheduler warp draws work indices from a global counter (the
@@ -460,8 +247,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
                                                               const __grid_constant__ CUtensorMap tm_vr,
                                                               const TcParams p) {
   extern __shared__ uint8_t smem_raw[];
-  const int total = p.header[0] * p.G;
-  if ((int)blockIdx.x >= total) return;
   const int s = p.s, TQ = 128 / s;
 
   const uint32_t sm = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -502,6 +287,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  // (everything above touches no global memory: it overlaps the end of the kernel before)
+  rc_grid_wait();
+  rc_grid_launch_next();
 
   // Item n of this CTA lives in ring slot n & 1; every consumer copies it to
   // registers and then releases the slot.
@@ -574,7 +362,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
         kv_n += (uint32_t)it.n_tiles;
       }
       fetch_item(item_n + 1, nx, true);
-      if (row == 0) { TR(3, item_n, 0); TRV(3, item_n, 15, it.n_tiles * 2 + it.b_valid); }
       // The stores below and the rotation of the next item's Q go through the same load/store
       // path, and the rotation is the urgent one: a tile's O is written back once the same tile's
       // next Q has been rotated.  (O is not needed back before the next item's first P V, a whole
@@ -589,12 +376,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
       for (int x = 0; x < 2; ++x) {
         if (nx.n_tiles > 0 && (x == 0 || (it.b_valid && nx.b_valid)))
           mbar_wait(bar(B_QREADY + x), (item_n + 1u) & 1u, abort_flag, p.status);
-        if (row == 0) TR(3, item_n, 1 + 5 * x);
         if (x == 1 && !it.b_valid) continue;
         mbar_wait(bar(B_LREADY + x), done[x] & 1u, abort_flag, p.status);
-        if (row == 0) TR(3, item_n, 2 + 5 * x);
         mbar_wait(bar(B_ODONE + x), done[x] & 1u, abort_flag, p.status);
-        if (row == 0) TR(3, item_n, 3 + 5 * x);
         ++done[x];
         tc_fence_after();
         const float inv = inv_l[x * 128 + row];
@@ -632,41 +416,15 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
         // the next item's first P V overwrites O, its softmax overwrites 1 / l: both wait for this
         tc_fence_before();
         mbar_arrive(bar(B_ODRAIN + x));
-        if (row == 0) TR(3, item_n, 4 + 5 * x);
       }
       it = nx;
     }
   } else if (warp >= 8) {
   asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_AUX));
-#ifdef RC_OBSERVE
-  if (warp == 11 && blockIdx.x == 0) {
-    // lane b watches barrier b (lanes past the last barrier watch barrier 0 and log nothing)
-    const bool logs = lane < B_COUNT;
-    const uint32_t my = bar(logs ? lane : 0);
-    uint32_t par = 0;
-    int n = 0;
-    const long long start = clock64();
-    if (lane == 0) g_observe[OBS_PER * 31] = start;
-    uint32_t last = (uint32_t)start;
-    for (uint32_t iter = 0;; ++iter) {
-      uint32_t ok, now;
-      asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%2], %3;\n\tselp.u32 %0, 1, 0, p;\n\tmov.u32 %1, %%clock;\n\t}"
-                   : "=r"(ok), "=r"(now) : "r"(my), "r"(par) : "memory");
-      if (ok) {
-        par ^= 1u; last = now;
-        if (logs && n < OBS_PER) g_observe[lane * OBS_PER + n++] = start + (long long)(uint32_t)(now - (uint32_t)start);
-      }
-      if ((iter & 63u) == 63u) {
-        const uint32_t newest = __reduce_max_sync(0xffffffffu, last - (uint32_t)start);
-        if ((now - (uint32_t)start) - newest > 60000u) break;
-      }
-    }
-    if (logs) g_observe_n[lane] = n;
-  }
-#endif
   if (warp == 10) {
     // ===================== scheduler =====================
     if (lane == 0) {
+      const int total = p.header[0] * p.G;   // (a CTA without work publishes "no more work" at once)
       bool first = true;
       for (uint32_t n = 0;; ++n) {
         const int sl = n & 1u;
@@ -676,7 +434,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
           const int w = first ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(p.header + 1, 1);
           first = false;
           if (w >= total || *abort_flag) { it.n_tiles = -1; break; }
-          if (load_item(p, p.header[2] ? p.order[w] : w, it)) break;
+          if (rc_load_item(p, p.header[2] ? p.order[w] : w, it)) break;
         }
         volatile int* r = item_ring + sl * IT_WORDS;
         r[IT_NTILES] = it.n_tiles;
@@ -700,9 +458,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
         fetch_item(item_n, it, true);
         if (it.n_tiles < 0) break;
         // Q tiles: free once the previous item's last S = Q K^T has completed
-        TR(4, item_n, 0);
         mbar_wait(bar(B_QEMPTY), (item_n & 1u) ^ 1u, abort_flag, p.status);
-        TR(4, item_n, 1);
         uint32_t rot_bytes = 0;
         const int pos_start = it.pos0 + it.tok0;
         if (ROT_SMEM) {
@@ -727,7 +483,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
           // (gather mode: a route tile is filled by the epilogue warps; every stage barrier expects
           // their 128 arrivals plus one from here, whoever brings the data)
           mbar_wait(bar(B_KEMPTY + st), ph ^ 1u, abort_flag, p.status);
-          if (i == 0) TR(4, item_n, 2);
           if (GATHER && route) {
             mbar_arrive(bar(B_KFULL + st));
           } else {
@@ -743,8 +498,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
             for (int kc = 0; kc < 2; ++kc)
               tma_load_2d(sm + SM_V + st * TILE_BYTES + kc * BOX_BYTES, route ? &tm_vr : &tm_vs, bar(B_VFULL + st), kc * 64, row);
           }
-          if (i == 0) TR(4, item_n, 3);
-          if (i == it.n_tiles - 1) TR(4, item_n, 4);
         }
       }
     }
@@ -790,21 +543,16 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
       if (it.n_tiles < 0) break;
       const int n_tiles = it.n_tiles, nA = it.nA, lenA = it.lenA, L = it.H + it.L, kv_end = it.kv_end;
       const bool b_valid = it.b_valid != 0;
-      if (issuer) TR(2, item_n, 0);
       // each query tile starts as soon as its own half of Q has been rotated
       mbar_wait(bar(B_QREADY + 0), item_n & 1u, abort_flag, p.status);
-      if (issuer) TR(2, item_n, 1);
       mbar_wait(bar(B_KFULL + kv_n % NSTAGE), (kv_n / NSTAGE) & 1u, abort_flag, p.status);
-      if (issuer) TR(2, item_n, 2);
       if (GATHER) fence_async_smem();   // the tile may have been written by cp.async (generic proxy)
       tc_fence_after();
       const int st0 = kv_n % NSTAGE;
       if (issuer) { issue_qk(0, st0); tc_commit(bar(B_SFULL + 0)); }
       // (waited for even when the second tile is empty: its warps still rewrite that half of Q,
       // and the Q-empty commit below lets the next load overwrite it)
-      if (issuer) TR(2, item_n, 3);
       mbar_wait(bar(B_QREADY + 1), item_n & 1u, abort_flag, p.status);
-      if (issuer) TR(2, item_n, 4);
       tc_fence_after();
       if (issuer) {
         if (b_valid) { issue_qk(1, st0); tc_commit(bar(B_SFULL + 1)); }
@@ -820,7 +568,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
         const int vis_rows = i < nA ? seg_rows : kv_end - (i - nA) * TILE_N;
         const int ksteps = (min(vis_rows, TILE_N) + 15) >> 4;
         mbar_wait(bar(B_VFULL + st), ph, abort_flag, p.status);
-        if (issuer && i == 0) TR(2, item_n, 5);
         if (GATHER) fence_async_smem();
         if (seg_rows < ksteps * 16) {
           // rows past the segment hold whatever follows it in memory: zero them, 0 * NaN would poison O
@@ -838,9 +585,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
         const bool more = i + 1 < n_tiles;
         // P of keys 0..63 arrives first: half of P V runs while the softmax finishes the other half
         mbar_wait(bar(B_PHALF + 0), cnt[0] & 1u, abort_flag, p.status);
-        if (issuer && i == 0) TR(2, item_n, 6);
         if (i == 0 && items_x[0] > 0) mbar_wait(bar(B_ODRAIN + 0), (items_x[0] - 1u) & 1u, abort_flag, p.status);
-        if (issuer && i == 0) TR(2, item_n, 7);
         tc_fence_after();
         if (issuer) issue_pv(0, st, 0, min(ksteps, 4), i == 0);
         mbar_wait(bar(B_PREADY + 0), cnt[0]++ & 1u, abort_flag, p.status);
@@ -853,11 +598,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
           if (issuer) { issue_qk(0, st1); tc_commit(bar(B_SFULL + 0)); }
         }
         if (b_valid) {
-          if (issuer && i == 0) TR(2, item_n, 8);
           mbar_wait(bar(B_PHALF + 1), cnt[1] & 1u, abort_flag, p.status);
-          if (issuer && i == 0) TR(2, item_n, 9);
           if (i == 0 && items_x[1] > 0) mbar_wait(bar(B_ODRAIN + 1), (items_x[1] - 1u) & 1u, abort_flag, p.status);
-          if (issuer && i == 0) TR(2, item_n, 10);
           tc_fence_after();
           if (issuer) issue_pv(1, st, 0, min(ksteps, 4), i == 0);
           mbar_wait(bar(B_PREADY + 1), cnt[1]++ & 1u, abort_flag, p.status);
@@ -873,10 +615,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
           }
         }
         __syncwarp();
-        if (issuer && i == 0) TR(2, item_n, 11);
-        if (issuer && i == n_tiles - 2) TR(2, item_n, 12);
       }
-      if (issuer) { TR(2, item_n, 13); TRV(2, item_n, 15, n_tiles * 2 + (b_valid ? 1 : 0)); }
       kv_n += (uint32_t)n_tiles;
       ++items_x[0];
       if (b_valid) ++items_x[1];
@@ -899,9 +638,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
     // time and goes through the token's s heads, so that cos / sin are read once per token, not
     // once per row; the 8 lanes of a token cover whole 128-byte rows of Q.
     auto rotate_q = [&](const Item& it, uint32_t n_item) {
-      if (row == 0) TR(x, n_item, 0);
       mbar_wait(bar(B_QFULL), n_item & 1u, abort_flag, p.status);
-      if (row == 0) TR(x, n_item, 1);
       uint8_t* qt = sm_gen + SM_Q + x * TILE_BYTES;
       for (int u = row; u < TQ * 8; u += 128) {
         const int tok = u >> 3, c = u & 7;
@@ -952,7 +689,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
       }
       fence_async_smem();
       mbar_arrive(bar(B_QREADY + x));
-      if (row == 0) TR(x, n_item, 2);
     };
 
     Item it, nx;
@@ -968,9 +704,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
       if (active) {
         for (int i = 0; i < n_tiles; ++i, ++cnt) {
           mbar_wait(bar(B_SFULL + x), cnt & 1u, abort_flag, p.status);
-          if (row == 0 && i == 0) TR(x, item_n, 3);
-          if (row == 0 && i == 1) TR(x, item_n, 5);
-          if (row == 0 && i == n_tiles - 1) TR(x, item_n, 6);
           tc_fence_after();
           if (releaser) {
             // S of tile i is complete: so is every earlier MMA, i.e. the last reader of K tile i
@@ -1040,14 +773,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
           tmem_wait_st();
           tc_fence_before();
           mbar_arrive(bar(B_PREADY + x));
-          if (row == 0 && i == 0) TR(x, item_n, 4);
-          if (row == 0 && i == n_tiles - 1) TR(x, item_n, 7);
         }
       }
       // ---- hand the finished tile to the epilogue warps (they wait for its last P V themselves) ----
       if (active) {
         if (done_n > 0) mbar_wait(bar(B_ODRAIN + x), (done_n - 1u) & 1u, abort_flag, p.status);   // 1 / l of the item before was read
-        if (row == 0) TR(x, item_n, 8);
         reinterpret_cast<float*>(sm_gen + SM_INVL)[x * 128 + row] = 1.f / l_sum;
         mbar_arrive(bar(B_LREADY + x));
         ++done_n;
@@ -1055,7 +785,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
       kv_n += (uint32_t)n_tiles;
       // ---- next item's Q (its load was issued a tile ago) ----
       fetch_item(item_n + 1, nx, true);
-      if (row == 0) { TR(x, item_n, 9); TRV(x, item_n, 15, n_tiles * 2 + it.b_valid); }
       if (nx.n_tiles > 0) rotate_q(nx, item_n + 1);
       it = nx; ++item_n;
     }
@@ -1117,20 +846,6 @@ int64_t align256(int64_t x) { return (x + 255) & ~(int64_t)255; }
 
 }  // namespace
 
-#ifdef RC_OBSERVE
-extern "C" __attribute__((visibility("default"))) int recache_debug_observe(long long* host, int* counts) {
-  if (cudaMemcpyFromSymbol(counts, g_observe_n, sizeof(int) * 32) != cudaSuccess) return -1;
-  return cudaMemcpyFromSymbol(host, g_observe, sizeof(long long) * 32 * OBS_PER) == cudaSuccess ? 32 * OBS_PER : -1;
-}
-#endif
-#ifdef RC_TRACE
-extern "C" __attribute__((visibility("default"))) int recache_debug_trace(long long* host, int n) {
-  const int m = TR_ROLES * TR_ITEMS * 16;
-  if (n < m) return -m;
-  return cudaMemcpyFromSymbol(host, g_trace, sizeof(long long) * m) == cudaSuccess ? m : -1;
-}
-#endif
-
 bool rc_tc_supported(const recache_ctx* ctx) {
   const int s = ctx->desc.n_q_heads / ctx->desc.n_kv_heads;
   return ctx->desc.dtype == RECACHE_BF16 && ctx->desc.head_dim == 128 && (s == 2 || s == 4 || s == 8);
@@ -1146,19 +861,14 @@ static int tc_levels(const recache_ctx* ctx, int max_len) {
 }
 
 int64_t rc_tc_workspace_bytes(const recache_ctx* ctx, int n_seq, int total, int max_len) {
-  return 256 + align256(tc_max_items(ctx, n_seq, total) * 8) + align256((int64_t)(n_seq + 1) * 4) + align256(SORT_MAX * 4);
+  return 256 + align256(tc_max_items(ctx, n_seq, total) * 8) + align256(2 * RC_SORT_MAX * 4);
 }
 
-cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const TcAttnArgs& a, cudaStream_t st) {
+cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope, const TcAttnArgs& a, cudaStream_t st) {
   const int G = ctx->desc.n_kv_heads, Hq = ctx->desc.n_q_heads, s = Hq / G;
   if (a.total == 0 || a.n_seq == 0) return cudaSuccess;
   const int64_t max_items = tc_max_items(ctx, a.n_seq, a.total);
-  const int n_levels = tc_levels(ctx, a.max_len);
   uint8_t* ws = (uint8_t*)a.workspace;
-  int32_t* header = (int32_t*)ws;
-  int2* items = (int2*)(ws + 256);
-  int32_t* level_off = (int32_t*)(ws + 256 + align256(max_items * 8));
-  int32_t* order = (int32_t*)(ws + 256 + align256(max_items * 8) + align256((int64_t)(a.n_seq + 1) * 4));
 
   CUtensorMap tq, tks, tvs, tkr, tvr;
   const uint64_t self_total = (uint64_t)G * (uint64_t)a.self_rows;
@@ -1173,46 +883,29 @@ cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const TcAttnArgs& a, cudaS
     return cudaErrorInvalidValue;
 
   TcParams p;
-  p.items = items; p.header = header; p.cu = a.cu; p.pos0 = a.pos0; p.slot = a.slot; p.route_cu = a.route_cu;
-  p.n_seq = a.n_seq; p.G = G; p.Hq = Hq; p.s = s; p.self_rows = a.self_rows; p.route_rows = a.route_rows; p.out = a.o;
+  p.header = (int32_t*)ws; p.items = (int2*)(ws + 256); p.order = (int32_t*)(ws + 256 + align256(max_items * 8));
+  p.cu = a.cu; p.pos0 = a.pos0; p.slot = a.slot; p.route_cu = a.route_cu; p.hist = a.hist;
+  p.n_seq = a.n_seq; p.G = G; p.Hq = Hq; p.s = s; p.self_rows = a.self_rows; p.route_rows = a.route_rows;
   p.prefix_len = a.route_cu ? 0 : a.prefix_len;
-  p.hist = a.hist;
+  p.n_levels = tc_levels(ctx, a.max_len); p.max_items = (int)max_items;
+  p.status = ctx->status;
+  p.out = a.o;
   p.cos_tab = ctx->cos_tab; p.sin_tab = ctx->sin_tab; p.max_pos = ctx->desc.max_pos;
   p.scale_log2 = (float)(1.4426950408889634 / sqrt((double)ctx->desc.head_dim));
-  p.status = ctx->status;
-  p.order = order;
   const bool gather = a.route_idx != nullptr;
   p.gather_k = (const uint8_t*)a.k_cache; p.gather_v = (const uint8_t*)a.v_cache; p.route_idx = a.route_idx;
   p.pool_tokens = a.pool_tokens;
-  {
-    // The work list only depends on the index arrays: when the caller marked a fork point before the
-    // rotate-and-store pass, it is built on the side stream beside that pass.
-    const bool fork = ctx->forked && cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0) == cudaSuccess;
-    ctx->forked = false;
-    cudaStream_t ps = fork ? ctx->side : st;
-    {
-      RcLaunchScope scope(ctx, RC_K_TILE_PLAN, ps);
-      tile_plan_kernel<<<1, 1024, 0, ps>>>(p, tc_tok_per_cta(ctx), n_levels, items, level_off, order, (int)max_items);
-    }
-    if (fork && (cudaEventRecord(ctx->ev_join, ctx->side) != cudaSuccess ||
-                 cudaStreamWaitEvent(st, ctx->ev_join, 0) != cudaSuccess))
-      return cudaErrorUnknown;
-  }
+  const cudaError_t e = rc_launch_rope_store(ctx, rope, &p, st);   // builds the work list on the side
+  if (e != cudaSuccess) return e;
   const int sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
   const unsigned grid = (unsigned)(max_items * G < sms ? max_items * G : sms);
   RcLaunchScope scope(ctx, a.route_cu ? RC_K_PREFILL_ATTN : RC_K_ENCODE_ATTN, st);
-  auto launch = [&](auto kernel) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_ALLOC);
-    kernel<<<grid, NTHREADS, SM_ALLOC, st>>>(tq, tks, tvs, tkr, tvr, p);
-  };
+  auto launch = [&](auto kernel) { return rc_launch_overlapped(kernel, grid, NTHREADS, SM_ALLOC, st, tq, tks, tvs, tkr, tvr, p); };
   const bool f32 = a.out_dtype == RECACHE_F32, rot = s >= 4;   // 2 * 128 / s <= 64 positions fit the staging area
   if (gather) {
-    if (f32) { if (rot) launch(attn_tc_kernel<float, true, true>); else launch(attn_tc_kernel<float, false, true>); }
-    else { if (rot) launch(attn_tc_kernel<__nv_bfloat16, true, true>); else launch(attn_tc_kernel<__nv_bfloat16, false, true>); }
-  } else {
-    if (f32) { if (rot) launch(attn_tc_kernel<float, true, false>); else launch(attn_tc_kernel<float, false, false>); }
-    else { if (rot) launch(attn_tc_kernel<__nv_bfloat16, true, false>); else launch(attn_tc_kernel<__nv_bfloat16, false, false>); }
+    if (f32) return rot ? launch(attn_tc_kernel<float, true, true>) : launch(attn_tc_kernel<float, false, true>);
+    return rot ? launch(attn_tc_kernel<__nv_bfloat16, true, true>) : launch(attn_tc_kernel<__nv_bfloat16, false, true>);
   }
-  return cudaGetLastError();
+  if (f32) return rot ? launch(attn_tc_kernel<float, true, false>) : launch(attn_tc_kernel<float, false, false>);
+  return rot ? launch(attn_tc_kernel<__nv_bfloat16, true, false>) : launch(attn_tc_kernel<__nv_bfloat16, false, false>);
 }
-

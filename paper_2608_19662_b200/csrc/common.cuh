@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "recache.h"
@@ -25,12 +26,6 @@ struct recache_ctx {
   int32_t* status;    // device status word
   int sm_count;
   std::string err;
-  // A second stream for small set-up kernels that do not depend on the call's first kernel (the work
-  // list of the tensor-core attention beside the rotate-and-store pass): forked from and joined to
-  // the caller's stream with the two events, so the caller sees one stream's ordering.
-  cudaStream_t side = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-  mutable bool forked = false;   // ev_fork was recorded for the call in progress
   // launch accounting (host side only)
   mutable bool timer_on = false;
   mutable bool timer_attn_only = false;   // bracket the two attention launches only
@@ -56,13 +51,6 @@ struct RcLaunchScope {
   ~RcLaunchScope() { if (stop) cudaEventRecord(stop, st); }
 };
 
-// Marks the point of the caller's stream that the side stream may start from (everything enqueued
-// before the call): record it before the call's first kernel.
-// (Not while the timer brackets every kernel: its event pairs are meant for kernels that run alone.)
-inline void rc_fork_point(const recache_ctx* ctx, cudaStream_t st) {
-  ctx->forked = ctx->side && (!ctx->timer_on || ctx->timer_attn_only) && cudaEventRecord(ctx->ev_fork, st) == cudaSuccess;
-}
-
 // ---- overlapped launches (programmatic dependent launch) ----
 // A kernel launched this way may come up while the kernel before it in the stream still runs: what
 // needs no memory (barriers, tensor memory, descriptor prefetch) overlaps that kernel's tail, and
@@ -74,7 +62,7 @@ __device__ __forceinline__ void rc_grid_wait() { asm volatile("griddepcontrol.wa
 __device__ __forceinline__ void rc_grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... P, typename... A>
-inline cudaError_t rc_launch_overlapped(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A&&... args) {
+inline cudaError_t rc_launch(bool overlapped, void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A&&... args) {
   // (the opt-in to more than 48 KB of shared memory is per kernel and device: a few hundred nanoseconds)
   if (smem > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -82,11 +70,15 @@ inline cudaError_t rc_launch_overlapped(void (*kernel)(P...), dim3 grid, unsigne
   }
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
+  at.val.programmaticStreamSerializationAllowed = overlapped ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
   cfg.attrs = &at; cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t rc_launch_overlapped(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A&&... args) {
+  return rc_launch(true, kernel, grid, threads, smem, st, std::forward<A>(args)...);
 }
 
 // First device-side error wins.
@@ -178,7 +170,8 @@ struct RopeStoreArgs {
   int mode;
   const int32_t* hist = nullptr;      // mode 2: rows already in each sequence's region; new rows follow them
 };
-cudaError_t rc_launch_rope_store(const recache_ctx* ctx, const RopeStoreArgs& a, cudaStream_t st);
+struct RcPlan;   // work list of the tensor-core attention (tile_plan.cuh), built beside the copies when given
+cudaError_t rc_launch_rope_store(const recache_ctx* ctx, const RopeStoreArgs& a, const RcPlan* plan, cudaStream_t st);
 
 // Generic row-per-warp attention (exact fp32 arithmetic; the fp32 path and the
 // small-shape path of bf16).
@@ -252,8 +245,9 @@ struct PrefillArgs {
 int64_t rc_encode_workspace_bytes(const recache_ctx* ctx, int n_res, int total, int max_len);
 int64_t rc_prefill_workspace_bytes(const recache_ctx* ctx, int n_req, int total_q, int max_q);
 int64_t rc_decode_workspace_bytes(const recache_ctx* ctx, int batch, int max_res_pages, int max_hist_pages);
-cudaError_t rc_launch_encode_attn(const recache_ctx* ctx, const EncodeArgs& a, cudaStream_t st);
-cudaError_t rc_launch_prefill_attn(const recache_ctx* ctx, const PrefillArgs& a, cudaStream_t st);
+// (rotate-and-store of the call's keys and values, then the attention)
+cudaError_t rc_launch_encode(const recache_ctx* ctx, const RopeStoreArgs& rope, const EncodeArgs& a, cudaStream_t st);
+cudaError_t rc_launch_prefill(const recache_ctx* ctx, const RopeStoreArgs& rope, const PrefillArgs& a, cudaStream_t st);
 cudaError_t rc_launch_decode(const recache_ctx* ctx, const DecodeArgs& a, cudaStream_t st);
 
 // ---- bf16 tensor-core attention (tcgen05 / TMEM / TMA) ----
@@ -273,7 +267,7 @@ struct TcAttnArgs {
 };
 bool rc_tc_supported(const recache_ctx* ctx);
 int64_t rc_tc_workspace_bytes(const recache_ctx* ctx, int n_seq, int total, int max_len);
-cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const TcAttnArgs& a, cudaStream_t st);
+cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope, const TcAttnArgs& a, cudaStream_t st);
 
 // ---- self-test of the bounded barrier wait (report: 2 ints on the device) ----
 cudaError_t rc_launch_wait_selftest(const recache_ctx* ctx, int32_t* report, cudaStream_t st);

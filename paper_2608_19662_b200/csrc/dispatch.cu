@@ -15,26 +15,30 @@ int64_t rc_decode_workspace_bytes(const recache_ctx* ctx, int batch, int max_res
   return rc_decode_split_supported(ctx) ? rc_decode_split_workspace_bytes(ctx, batch, max_res_pages, max_hist_pages) : 0;
 }
 
-cudaError_t rc_launch_encode_attn(const recache_ctx* ctx, const EncodeArgs& a, cudaStream_t st) {
+cudaError_t rc_launch_encode(const recache_ctx* ctx, const RopeStoreArgs& rope, const EncodeArgs& a, cudaStream_t st) {
   if (rc_tc_supported(ctx)) {
     TcAttnArgs t{a.q, a.o, a.out_dtype, a.cu, a.n_res, a.total, a.max_len, a.pos_offset, a.slot, a.k_cache, a.v_cache,
                  a.pool_tokens, a.k_prefix, a.v_prefix, nullptr, (int64_t)ctx->desc.n_kv_heads * a.prefix_len,
                  a.workspace, a.prefix_len};
-    return rc_launch_attn_tc(ctx, t, st);
+    return rc_launch_attn_tc(ctx, rope, t, st);
   }
+  const cudaError_t e = rc_launch_rope_store(ctx, rope, nullptr, st);
+  if (e != cudaSuccess) return e;
   AttnRowsArgs r{a.q, a.o, a.out_dtype, a.cu, a.n_res, a.total, a.pos_offset, a.slot, a.k_cache, a.v_cache,
                  a.pool_tokens, a.k_prefix, a.v_prefix, nullptr, a.prefix_len};
   r.route_rows = (int64_t)ctx->desc.n_kv_heads * a.prefix_len;
   return rc_launch_attn_rows(ctx, r, st);
 }
 
-cudaError_t rc_launch_prefill_attn(const recache_ctx* ctx, const PrefillArgs& a, cudaStream_t st) {
+cudaError_t rc_launch_prefill(const recache_ctx* ctx, const RopeStoreArgs& rope, const PrefillArgs& a, cudaStream_t st) {
   if (rc_tc_supported(ctx)) {
     TcAttnArgs t{a.q, a.o, a.out_dtype, a.cu_q, a.n_req, a.total_q, a.max_q, a.pos0, a.conv_slot, a.k_conv, a.v_conv,
                  a.conv_rows, a.k_route, a.v_route, a.route_cu, a.route_rows, a.workspace, 0, a.hist};
     t.k_cache = a.k_cache; t.v_cache = a.v_cache; t.pool_tokens = a.pool_tokens; t.route_idx = a.route_idx;
-    return rc_launch_attn_tc(ctx, t, st);
+    return rc_launch_attn_tc(ctx, rope, t, st);
   }
+  const cudaError_t e = rc_launch_rope_store(ctx, rope, nullptr, st);
+  if (e != cudaSuccess) return e;
   AttnRowsArgs r{a.q, a.o, a.out_dtype, a.cu_q, a.n_req, a.total_q, a.pos0, a.conv_slot, a.k_conv, a.v_conv,
                  a.conv_rows, a.k_route, a.v_route, a.route_cu, 0, a.hist};
   r.route_rows = a.route_rows;

@@ -6,7 +6,7 @@
 // every resource).  Prefill: token t of request b has position
 // pos0[b] + (t - cu[b]) and goes to row t of the conversation KV.
 // Memory-bound: reads k, v once, writes both once; 16-byte accesses.
-#include "common.cuh"
+#include "tile_plan.cuh"
 
 namespace {
 
@@ -46,17 +46,25 @@ template <> __device__ __forceinline__ uint4 pack16<__nv_bfloat16>(const float* 
 // One thread handles one 16-byte chunk of the low half of a key row together
 // with the matching chunk of the high half (the rotation pairs i with i + d/2),
 // and the two matching chunks of the value row.
-template <typename T>
+// With PLAN, block 0 builds the attention's work list instead (a launch of its own would cost more
+// than the list: it only reads the call's index arrays, so it hides behind the copies).
+template <typename T, bool PLAN>
 __global__ void __launch_bounds__(256) rope_store_kernel(
     const T* __restrict__ k, const T* __restrict__ v, T* __restrict__ k_dst, T* __restrict__ v_dst,
     const int32_t* __restrict__ cu, int n_seq, int total, const int32_t* __restrict__ slot,
     const int32_t* __restrict__ pos0, const int32_t* __restrict__ hist, int64_t dst_rows, int mode, int G, int d,
     const float* __restrict__ cos_tab, const float* __restrict__ sin_tab, int max_pos,
-    int32_t* status) {
+    int32_t* status, const __grid_constant__ RcPlan plan, bool overlapped) {
+  rc_grid_wait();
+  if (overlapped) rc_grid_launch_next();
+  if constexpr (PLAN) {
+    __shared__ RcPlanSmem sh;
+    if (blockIdx.x == 0) { rc_build_plan(plan, sh); return; }
+  }
   constexpr int N = Vec16<T>::N;
   const int half = d / 2;
   const int chunks = half / N;                  // 16-byte chunks per half row
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t gid = (int64_t)(blockIdx.x - (PLAN ? 1 : 0)) * blockDim.x + threadIdx.x;
   const int64_t n_work = (int64_t)total * G * chunks;
   if (gid >= n_work) return;
   const int c = (int)(gid % chunks);
@@ -103,24 +111,27 @@ __global__ void __launch_bounds__(256) rope_store_kernel(
 
 }  // namespace
 
-cudaError_t rc_launch_rope_store(const recache_ctx* ctx, const RopeStoreArgs& a, cudaStream_t st) {
+cudaError_t rc_launch_rope_store(const recache_ctx* ctx, const RopeStoreArgs& a, const RcPlan* plan, cudaStream_t st) {
   const int d = ctx->desc.head_dim, G = ctx->desc.n_kv_heads;
   if (a.total == 0) return cudaSuccess;
   const bool bf = ctx->desc.dtype == RECACHE_BF16;
   const int chunks = (d / 2) / (bf ? 8 : 4);
   const int64_t n_work = (int64_t)a.total * G * chunks;
   const int threads = 256;
-  const unsigned blocks = (unsigned)((n_work + threads - 1) / threads);
+  const unsigned blocks = (unsigned)((n_work + threads - 1) / threads) + (plan ? 1 : 0);
+  // Overlapping its neighbours pays where the launch is a single wave (encoding one resource of 500
+  // tokens: 21 against 23 us).  A larger one would hold the SMs that the kernel before leaves early, and
+  // hand its own to the kernel after one by one: encoding 43k tokens 535 us with the overlap, 526 without,
+  // 95k tokens 1635 and 1590.
+  const bool overlapped = blocks <= 8u * (unsigned)(ctx->sm_count > 0 ? ctx->sm_count : 148);
   RcLaunchScope scope(ctx, RC_K_ROPE_STORE, st);
-  if (bf)
-    rope_store_kernel<__nv_bfloat16><<<blocks, threads, 0, st>>>(
-        (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, (__nv_bfloat16*)a.k_dst, (__nv_bfloat16*)a.v_dst,
-        a.cu, a.n_seq, a.total, a.slot, a.pos0, a.hist, a.dst_rows, a.mode, G, d, ctx->cos_tab, ctx->sin_tab,
-        ctx->desc.max_pos, ctx->status);
-  else
-    rope_store_kernel<float><<<blocks, threads, 0, st>>>(
-        (const float*)a.k, (const float*)a.v, (float*)a.k_dst, (float*)a.v_dst,
-        a.cu, a.n_seq, a.total, a.slot, a.pos0, a.hist, a.dst_rows, a.mode, G, d, ctx->cos_tab, ctx->sin_tab,
-        ctx->desc.max_pos, ctx->status);
-  return cudaGetLastError();
+  const RcPlan none = {};
+  auto launch = [&](auto kernel, auto type) {
+    using T = decltype(type);
+    return rc_launch(overlapped, kernel, blocks, threads, 0, st, (const T*)a.k, (const T*)a.v, (T*)a.k_dst, (T*)a.v_dst, a.cu, a.n_seq, a.total, a.slot, a.pos0,
+                                a.hist, a.dst_rows, a.mode, G, d, (const float*)ctx->cos_tab, (const float*)ctx->sin_tab, ctx->desc.max_pos,
+                                ctx->status, plan ? *plan : none, overlapped);
+  };
+  if (!bf) return launch(rope_store_kernel<float, false>, float());
+  return plan ? launch(rope_store_kernel<__nv_bfloat16, true>, __nv_bfloat16()) : launch(rope_store_kernel<__nv_bfloat16, false>, __nv_bfloat16());
 }

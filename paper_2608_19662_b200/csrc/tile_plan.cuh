@@ -1,0 +1,154 @@
+// Work list of the tensor-core attention.  Built by one block of the rotate-and-store kernel that
+// precedes the attention launch (it only depends on the call's index arrays), read by the attention
+// kernel's scheduler warps.  As a launch of its own, on a side stream between two events, it took 6-9 us
+// of the smallest calls (encoding one resource of 500 tokens: 26.6 us with it, 20.6 us now).
+#pragma once
+#include "common.cuh"
+
+constexpr int RC_TILE_N = 128;       // keys of a K/V tile
+constexpr int RC_SORT_MAX = 4096;    // work items up to which the plan sorts a prefill by weight (encode: a quarter)
+constexpr int RC_PLAN_BINS = 1024;   // weights (K/V tiles, tile pairs) are told apart up to this
+
+struct RcPlan {
+  int2* items; int32_t* header;   // header[0] = number of items, header[1] = work counter, header[2] = order[] is valid
+  int32_t* order;                 // work indices, heaviest first (launches of at most RC_SORT_MAX work items); bins behind them
+  const int32_t* cu; const int32_t* pos0; const int32_t* slot; const int32_t* route_cu; const int32_t* hist;
+  int n_seq, G, Hq, s;
+  int prefix_len;   // > 0: every sequence sees rows g*prefix_len .. of the "route" tensors (shared prefix)
+  int64_t self_rows;
+  int64_t route_rows;   // rows of the packed route tensors / entries of route_idx
+  int n_levels, max_items;   // tile pairs of the longest sequence, capacity of items[]
+  int32_t* status;
+};
+
+// One work item as published by the scheduler warp (16 ints in shared memory).
+struct RcItem {
+  int n_tiles;      // -1: no more work
+  int g, seq0, L, tok0, kv_end, pos0, rA0, lenA, nA, b_valid;
+  int H;            // rows that precede the sequence's own tokens in the self part (earlier turns), all visible
+  int64_t base;
+};
+
+// Work index w -> item; false when the caller's index arrays are inconsistent
+// (flagged in the status word; the scheduler skips the item).
+__device__ __forceinline__ bool rc_load_item(const RcPlan& p, int w, RcItem& it) {
+  const int2 e = p.items[w / p.G];
+  it.g = w % p.G;
+  const int b = e.x;
+  const int TQ = 128 / p.s;
+  it.seq0 = p.cu[b];
+  it.L = p.cu[b + 1] - it.seq0;
+  it.tok0 = e.y * 2 * TQ;
+  it.b_valid = it.tok0 + TQ < it.L;
+  it.H = p.hist ? p.hist[b] : 0;
+  it.kv_end = it.H + min(it.L, it.tok0 + 2 * TQ);   // self rows the pair can see: the history, then its causal range
+  it.base = p.slot ? (int64_t)p.slot[b] : (int64_t)it.seq0;
+  it.pos0 = p.pos0 ? p.pos0[b] : 0;
+  it.rA0 = 0; it.lenA = 0;
+  bool route_ok = true;
+  if (p.route_cu) {
+    it.rA0 = p.route_cu[b * p.G + it.g]; it.lenA = p.route_cu[b * p.G + it.g + 1] - it.rA0;
+    route_ok = (int64_t)it.rA0 + it.lenA <= p.route_rows;   // e.g. after a compaction that overflowed its capacity
+  }
+  else if (p.prefix_len > 0) { it.rA0 = it.g * p.prefix_len; it.lenA = p.prefix_len; }
+  it.nA = (it.lenA + RC_TILE_N - 1) / RC_TILE_N;
+  it.n_tiles = it.nA + (it.kv_end + RC_TILE_N - 1) / RC_TILE_N;
+  const bool ok = it.L > 0 && it.tok0 < it.L && it.lenA >= 0 && it.rA0 >= 0 && it.base >= 0 && it.H >= 0 &&
+                  it.base + it.H + it.L <= p.self_rows && it.seq0 >= 0 && route_ok;
+  if (!ok) rc_set_status(p.status, route_ok ? RECACHE_DEV_BAD_SLOT : RECACHE_DEV_OVERFLOW);
+  return ok;
+}
+
+struct RcPlanSmem { int hist[RC_PLAN_BINS + 1]; int warp_sum[33]; };
+
+// Exclusive block scan of one int per thread; *total gets the sum (same pattern of calls in every thread).
+__device__ __forceinline__ int rc_plan_scan(int v, RcPlanSmem& sh, int* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int incl = v;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += u;
+  }
+  __syncthreads();
+  if (lane == 31) sh.warp_sum[warp] = incl;
+  __syncthreads();
+  int before = 0, all = 0;
+  for (int w = 0; w < nw; ++w) { const int x = sh.warp_sum[w]; if (w < warp) before += x; all += x; }
+  *total = all;
+  return before + incl - v;
+}
+// Turns the bin counts into the first index of each bin, bin 0 first; all threads of the block.
+__device__ __forceinline__ void rc_plan_scan_bins(RcPlanSmem& sh) {
+  const int per = (RC_PLAN_BINS + 1 + blockDim.x - 1) / blockDim.x;
+  const int i0 = min(RC_PLAN_BINS + 1, (int)threadIdx.x * per), i1 = min(RC_PLAN_BINS + 1, i0 + per);
+  int sum = 0, total;
+  for (int i = i0; i < i1; ++i) sum += sh.hist[i];
+  int at = rc_plan_scan(sum, sh, &total);
+  for (int i = i0; i < i1; ++i) { const int c = sh.hist[i]; sh.hist[i] = at; at += c; }
+  __syncthreads();
+}
+
+// Items = (sequence, tile-pair index): sequence by sequence, the longest sequences
+// first, and inside a sequence the last (heaviest) tile pair first, so that the
+// launch ends on the light items of short sequences.  With the KV group as the
+// fastest index of the flattened work list, the CTAs that run at the same time
+// share one sequence's K/V, which then stays in L2 instead of being streamed
+// from HBM once per tile pair.  One block.  (Sequences of equal length land in an
+// order that may differ between launches; no result depends on it.)
+__device__ __forceinline__ void rc_build_plan(const RcPlan& p, RcPlanSmem& sh) {
+  const int tid = threadIdx.x, n_thr = blockDim.x, n_seq = p.n_seq, tok_per_item = 2 * 128 / p.s;
+  const int32_t* cu = p.cu;
+  auto n_pairs = [&](int b) {
+    const int len = cu[b + 1] - cu[b];
+    return min(len > 0 ? (len + tok_per_item - 1) / tok_per_item : 0, p.n_levels);
+  };
+  // each thread owns a contiguous chunk of sequences: local sums, block scan of the chunk sums, then the items
+  const int per = (n_seq + n_thr - 1) / n_thr;
+  const int b0 = min(n_seq, tid * per), b1 = min(n_seq, b0 + per);
+  int sum = 0, total;
+  for (int b = b0; b < b1; ++b) {
+    const int len = cu[b + 1] - cu[b];
+    if (len < 0 || (len + tok_per_item - 1) / tok_per_item > p.n_levels)   // not monotone, or longer than the max_len given
+      rc_set_status(p.status, RECACHE_DEV_BAD_SEQLENS);
+    sum += n_pairs(b);
+  }
+  for (int i = tid; i <= RC_PLAN_BINS; i += n_thr) sh.hist[i] = 0;
+  int k = rc_plan_scan(sum, sh, &total);
+  const int n_items = min(total, p.max_items), n_work = n_items * p.G;
+  // (an encode launch shares K/V between the items of a sequence only: beyond a thousand items the
+  // sequence-major order, which keeps a sequence's K/V in L2, is worth more than the balance)
+  const bool sorted = n_work <= (p.route_cu ? RC_SORT_MAX : RC_SORT_MAX / 4);
+  if (tid == 0) { p.header[0] = n_items; p.header[1] = 0; p.header[2] = sorted ? 1 : 0; }
+  if (!sorted) {
+    // counting sort of the sequences by their number of tile pairs, longest first: hist[bin] = items of
+    // that bin, then the first item index of the bin
+    for (int b = b0; b < b1; ++b) {
+      const int nt = n_pairs(b);
+      if (nt > 0) atomicAdd(&sh.hist[RC_PLAN_BINS - min(nt, RC_PLAN_BINS)], nt);
+    }
+    __syncthreads();
+    rc_plan_scan_bins(sh);
+  }
+  for (int b = b0; b < b1; ++b) {
+    const int nt = n_pairs(b);
+    if (nt == 0) continue;
+    if (!sorted) k = atomicAdd(&sh.hist[RC_PLAN_BINS - min(nt, RC_PLAN_BINS)], nt);
+    for (int l = nt - 1; l >= 0; --l, ++k)
+      if (k < p.max_items) p.items[k] = make_int2(b, l);
+  }
+  if (!sorted) return;
+  // Few work items (a prefill of a handful of requests): one CTA gets one or two of them, so their
+  // order decides the tail.  Sort them by weight (K/V tiles), heaviest first, with a counting sort.
+  __syncthreads();
+  for (int w = tid; w < n_work; w += n_thr) {
+    RcItem it;
+    const bool ok = rc_load_item(p, w, it);
+    const int bin = RC_PLAN_BINS - (ok ? min(it.n_tiles, RC_PLAN_BINS) : 0);
+    p.order[RC_SORT_MAX + w] = bin;
+    atomicAdd(&sh.hist[bin], 1);
+  }
+  __syncthreads();
+  rc_plan_scan_bins(sh);
+  for (int w = tid; w < n_work; w += n_thr) p.order[atomicAdd(&sh.hist[p.order[RC_SORT_MAX + w]], 1)] = w;
+}
