@@ -1,7 +1,18 @@
-// Row-per-warp attention in exact fp32 arithmetic (no tensor cores, accurate
-// expf): the fp32 path of encode and prefill.  One warp owns one (token, head)
-// output row, walks its keys 32 at a time with an online softmax (warp-shuffle
-// max / sum) and accumulates d / 32 output columns per lane.
+// Attention in exact fp32 arithmetic (no tensor cores, accurate expf): the fp32
+// path of encode and prefill, and the bf16 shapes that the tensor-core kernel
+// does not cover.
+//
+// One CTA owns a block of up to 8 query rows (8 / s consecutive tokens of a
+// sequence x the s query heads of a group).  Its eight warps deal the keys out
+// in tiles of 32 (tile t belongs to warp t % 8) and each runs an online softmax
+// of its own over all of them; the partial (max, sum, O) are merged through
+// shared memory at the end, so nothing synchronises in between.  For the scores
+// a lane owns a key and keeps a sum per row, with the queries broadcast from shared
+// memory (four FMA to a load); for P V a lane owns d / 32 columns and the
+// probabilities are broadcast.  Bound by FMA issue and, at the few hundred rows
+// of the calls made in earnest, by the length of one warp's chain: a warp per
+// row, with each key row read once for every query row, took 69 us for 1,250
+// tokens of six resources (4 / 2 heads of 64), ROWS_NOW us now.
 //
 // Key set of a row (token t of sequence b at local index j, head h, group g):
 //   route part : rows route_cu[b*G+g] .. route_cu[b*G+g+1]-1 of k_route/v_route,
@@ -10,83 +21,121 @@
 //                base = slot[b] for encoding (cache rows of the resource),
 //                cu[b] for prefill (rotated conversation keys).
 // The query is rotated on load at position pos0[b] + j (0 + j for encoding).
+// Blocks and tiles are aligned to the sequence, never to the batch: results do
+// not depend on what else is in the launch.
 #include "common.cuh"
 
 namespace {
 
-template <typename T>
-__device__ __forceinline__ float dot_row(const T* __restrict__ krow, const float* __restrict__ qs, int d);
+constexpr int WARPS = 8, ROWS = 8, KT = 32, VB = 8;    // VB: value rows loaded at a time
 
-template <>
-__device__ __forceinline__ float dot_row<float>(const float* __restrict__ krow, const float* __restrict__ qs, int d) {
-  float acc = 0.f;
-  for (int i = 0; i < d; i += 4) {
-    const float4 kv = *reinterpret_cast<const float4*>(krow + i);
-    acc = fmaf(kv.x, qs[i], acc); acc = fmaf(kv.y, qs[i + 1], acc);
-    acc = fmaf(kv.z, qs[i + 2], acc); acc = fmaf(kv.w, qs[i + 3], acc);
-  }
-  return acc;
+// N consecutive elements as floats, N * sizeof(T) a multiple of 4
+template <typename T, int N> __device__ __forceinline__ void load_f(const T* p, float* f);
+template <> __device__ __forceinline__ void load_f<float, 2>(const float* p, float* f) {
+  const float2 v = *reinterpret_cast<const float2*>(p);
+  f[0] = v.x; f[1] = v.y;
 }
-template <>
-__device__ __forceinline__ float dot_row<__nv_bfloat16>(const __nv_bfloat16* __restrict__ krow,
-                                                        const float* __restrict__ qs, int d) {
-  float acc = 0.f;
-  for (int i = 0; i < d; i += 8) {
-    const uint4 u = *reinterpret_cast<const uint4*>(krow + i);
-    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+template <> __device__ __forceinline__ void load_f<float, 4>(const float* p, float* f) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  f[0] = v.x; f[1] = v.y; f[2] = v.z; f[3] = v.w;
+}
+template <> __device__ __forceinline__ void load_f<float, 8>(const float* p, float* f) {
+  load_f<float, 4>(p, f); load_f<float, 4>(p + 4, f + 4);
+}
+template <> __device__ __forceinline__ void load_f<__nv_bfloat16, 2>(const __nv_bfloat16* p, float* f) {
+  const uint32_t w = *reinterpret_cast<const uint32_t*>(p);
+  f[0] = __uint_as_float(w << 16); f[1] = __uint_as_float(w & 0xffff0000u);
+}
+template <> __device__ __forceinline__ void load_f<__nv_bfloat16, 4>(const __nv_bfloat16* p, float* f) {
+  load_f<__nv_bfloat16, 2>(p, f); load_f<__nv_bfloat16, 2>(p + 2, f + 2);
+}
+template <> __device__ __forceinline__ void load_f<__nv_bfloat16, 8>(const __nv_bfloat16* p, float* f) {
+  const uint4 v = *reinterpret_cast<const uint4*>(p);
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      acc = fmaf(__uint_as_float(w[c] << 16), qs[i + 2 * c], acc);
-      acc = fmaf(__uint_as_float(w[c] & 0xffff0000u), qs[i + 2 * c + 1], acc);
-    }
-  }
-  return acc;
+  for (int i = 0; i < 4; ++i) { f[2 * i] = __uint_as_float(w[i] << 16); f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u); }
 }
 
-constexpr int WARPS = 4;
+template <int D> struct Smem {
+  float q[ROWS][D];
+  union {
+    float p[WARPS][KT][ROWS];                            // probabilities, key-major
+    float part[WARPS][ROWS][D];                          // partial O
+  };
+  float m[WARPS][ROWS], l[WARPS][ROWS];
+};
 
 template <typename T, typename TO, int D>
-__global__ void __launch_bounds__(WARPS * 32) attn_rows_kernel(
+__global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
     const T* __restrict__ q, TO* __restrict__ o, const int32_t* __restrict__ cu, int n_seq, int total,
     const int32_t* __restrict__ pos0, const int32_t* __restrict__ slot,
     const T* __restrict__ k_self, const T* __restrict__ v_self, int64_t self_rows,
     const T* __restrict__ k_route, const T* __restrict__ v_route, const int32_t* __restrict__ route_cu,
     int prefix_len, const int32_t* __restrict__ hist, int64_t route_rows, int Hq, int G, const float* __restrict__ cos_tab, const float* __restrict__ sin_tab, int max_pos,
     float scale, int32_t* status) {
-  __shared__ float q_s[WARPS][D];
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  Smem<D>& sh = *reinterpret_cast<Smem<D>*>(smem_raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t row = (int64_t)blockIdx.x * WARPS + warp;
-  if (row >= (int64_t)total * Hq) return;
-  const int t = (int)(row / Hq), h = (int)(row % Hq);
-  const int g = h / (Hq / G);
-  const int b = rc_find_segment(cu, n_seq, t);
-  const int j = t - cu[b];
-  if (t >= cu[n_seq] || j < 0) { if (lane == 0) rc_set_status(status, RECACHE_DEV_BAD_SEQLENS); return; }
-  const int pos = (pos0 ? pos0[b] : 0) + j;
-  const int64_t base = slot ? (int64_t)slot[b] : (int64_t)cu[b];
-  const int H = hist ? hist[b] : 0;      // earlier-turn rows at the start of the self part, all visible
-  if (pos < 0 || pos >= max_pos) { if (lane == 0) rc_set_status(status, RECACHE_DEV_BAD_POS); return; }
-  if (base < 0 || H < 0 || base + H + j >= self_rows) { if (lane == 0) rc_set_status(status, RECACHE_DEV_BAD_SLOT); return; }
+  const int s = Hq / G, TQ = ROWS / s, g = blockIdx.y;
+  rc_grid_wait();
+  rc_grid_launch_next();
 
-  // rotate the query row into shared memory
-  constexpr int HALF = D / 2;
-  const T* qrow = q + ((int64_t)t * Hq + h) * D;
-  for (int i = lane; i < HALF; i += 32) {
-    const float lo = rc_to_float<T>(qrow[i]), hi = rc_to_float<T>(qrow[i + HALF]);
-    const float c = cos_tab[(int64_t)pos * HALF + i], s = sin_tab[(int64_t)pos * HALF + i];
-    // the rotated query is a tensor of the storage dtype, like the cached keys
-    q_s[warp][i] = rc_to_float<T>(rc_from_float<T>(__fmaf_rn(lo, c, -__fmul_rn(hi, s))));
-    q_s[warp][i + HALF] = rc_to_float<T>(rc_from_float<T>(__fmaf_rn(hi, c, __fmul_rn(lo, s))));
+  // Block index -> (sequence, block of it).  Sequence b's blocks start at cu[b] / TQ + b, which leaves
+  // every sequence at least the ceil(len / TQ) it needs.
+  const int x = blockIdx.x;
+  int lo = 0, hi = n_seq;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (cu[mid] / TQ + mid <= x) lo = mid; else hi = mid;
   }
-  __syncwarp();
+  const int b = lo, seq0 = cu[b], L = cu[b + 1] - seq0;
+  if (x == 0 && g == 0 && threadIdx.x == 0 && cu[n_seq] < total) rc_set_status(status, RECACHE_DEV_BAD_SEQLENS);
+  const int tok0 = (x - (seq0 / TQ + b)) * TQ;           // first token of the block, local
+  if (seq0 < 0 || L < 0 || seq0 + L > total) { if (threadIdx.x == 0) rc_set_status(status, RECACHE_DEV_BAD_SEQLENS); return; }
+  if (tok0 < 0 || tok0 >= L) return;
+  const int64_t base = slot ? (int64_t)slot[b] : (int64_t)seq0;
+  const int H = hist ? hist[b] : 0;      // earlier-turn rows at the start of the self part, all visible
+  const int p0 = pos0 ? pos0[b] : 0;
+  // tokens that can be computed: inside the sequence, the rotary table and the cache
+  int n_tok = min(TQ, L - tok0);
+  if (base < 0 || H < 0 || base + H + tok0 + n_tok > self_rows) {
+    if (threadIdx.x == 0) rc_set_status(status, RECACHE_DEV_BAD_SLOT);
+    n_tok = base < 0 || H < 0 ? 0 : (int)min((int64_t)n_tok, max((int64_t)0, self_rows - base - H - tok0));
+  }
+  if (p0 + tok0 < 0 || p0 + tok0 + n_tok > max_pos) {
+    if (threadIdx.x == 0) rc_set_status(status, RECACHE_DEV_BAD_POS);
+    n_tok = p0 + tok0 < 0 ? 0 : min(n_tok, max(0, max_pos - p0 - tok0));
+  }
+  if (n_tok <= 0) return;
+  const int n_rows = n_tok * s;                          // row r = (token tok0 + r / s, head g * s + r % s)
 
-  constexpr int CPL = D / 32;   // output columns per lane
-  float acc[CPL];
+  // ---- rotated query rows, rounded to the storage dtype like the cached keys ----
+  constexpr int HALF = D / 2;
+  for (int e = threadIdx.x; e < ROWS * HALF; e += WARPS * 32) {
+    const int r = e / HALF, i = e % HALF;
+    float ol = 0.f, oh = 0.f;
+    if (r < n_rows) {
+      const T* qrow = q + ((int64_t)(seq0 + tok0 + r / s) * Hq + g * s + r % s) * D;
+      const int64_t at = (int64_t)(p0 + tok0 + r / s) * HALF + i;
+      const float l = rc_to_float<T>(qrow[i]), h = rc_to_float<T>(qrow[i + HALF]), c = cos_tab[at], sn = sin_tab[at];
+      ol = rc_to_float<T>(rc_from_float<T>(__fmaf_rn(l, c, -__fmul_rn(h, sn))));
+      oh = rc_to_float<T>(rc_from_float<T>(__fmaf_rn(h, c, __fmul_rn(l, sn))));
+    }
+    sh.q[r][i] = ol; sh.q[r][i + HALF] = oh;
+  }
+  __syncthreads();
+
+  constexpr int CPL = D / 32;   // output columns per lane: CPL * lane ..
+  float acc[ROWS][CPL], m[ROWS], l[ROWS];                // l: this lane's keys only
 #pragma unroll
-  for (int c = 0; c < CPL; ++c) acc[c] = 0.f;
-  float m = -INFINITY, l = 0.f;
+  for (int r = 0; r < ROWS; ++r) {
+    m[r] = -INFINITY; l[r] = 0.f;
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) acc[r][c] = 0.f;
+  }
+  float (*ps)[ROWS] = sh.p[warp];
 
-  // two key segments: route rows (all visible), then the causal self rows
+  int t = 0;                                             // key tiles so far
   for (int seg = 0; seg < 2; ++seg) {
     const T* kb; const T* vb; int n;
     if (seg == 0) {
@@ -97,62 +146,134 @@ __global__ void __launch_bounds__(WARPS * 32) attn_rows_kernel(
       // a range outside the route tensors (e.g. after a compaction that overflowed its capacity)
       // is reported and read as an empty route
       if (r0 < 0 || r1 < r0 || (int64_t)r1 > route_rows) {
-        if (lane == 0) rc_set_status(status, RECACHE_DEV_OVERFLOW);
+        if (threadIdx.x == 0) rc_set_status(status, RECACHE_DEV_OVERFLOW);
         continue;
       }
       kb = k_route + (int64_t)r0 * D; vb = v_route + (int64_t)r0 * D; n = r1 - r0;
     } else {
       kb = k_self + ((int64_t)g * self_rows + base) * D;
       vb = v_self + ((int64_t)g * self_rows + base) * D;
-      n = H + j + 1;
+      n = H + tok0 + n_tok;
     }
-    for (int k0 = 0; k0 < n; k0 += 32) {
-      const int kk = k0 + lane;
-      float s = -INFINITY;
-      if (kk < n) s = dot_row<T>(kb + (int64_t)kk * D, q_s[warp], D) * scale;
-      float mx = s;
+    for (int k0 = 0; k0 < n; k0 += KT, ++t) {
+      if (t % WARPS != warp) continue;
+      const int kk = k0 + lane, cnt = min(KT, n - k0);
+      // ---- scores of key kk with every row ----
+      float sc[ROWS];
 #pragma unroll
-      for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-      const float m_new = fmaxf(m, mx);
-      const float corr = (m == -INFINITY) ? 0.f : expf(m - m_new);
-      const float p = (kk < n) ? expf(s - m_new) : 0.f;
-      float ps = p;
+      for (int r = 0; r < ROWS; ++r) sc[r] = 0.f;
+      const T* krow = kb + (int64_t)min(kk, n - 1) * D;
+#pragma unroll 4
+      for (int i = 0; i < D; i += 8) {
+        float kv[8];
+        load_f<T, 8>(krow + i, kv);
 #pragma unroll
-      for (int off = 16; off; off >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, off);
-      l = l * corr + ps;
-      m = m_new;
-#pragma unroll
-      for (int c = 0; c < CPL; ++c) acc[c] *= corr;
-      const int cnt = min(32, n - k0);
-      for (int jj = 0; jj < cnt; ++jj) {
-        const float pj = __shfl_sync(0xffffffffu, p, jj);
-        const T* vrow = vb + (int64_t)(k0 + jj) * D;
-#pragma unroll
-        for (int c = 0; c < CPL; ++c) acc[c] = fmaf(pj, rc_to_float<T>(vrow[lane + 32 * c]), acc[c]);
+        for (int r = 0; r < ROWS; ++r) {
+          const float4 a = *reinterpret_cast<const float4*>(&sh.q[r][i]), c = *reinterpret_cast<const float4*>(&sh.q[r][i + 4]);
+          sc[r] = fmaf(kv[0], a.x, sc[r]); sc[r] = fmaf(kv[1], a.y, sc[r]); sc[r] = fmaf(kv[2], a.z, sc[r]); sc[r] = fmaf(kv[3], a.w, sc[r]);
+          sc[r] = fmaf(kv[4], c.x, sc[r]); sc[r] = fmaf(kv[5], c.y, sc[r]); sc[r] = fmaf(kv[6], c.z, sc[r]); sc[r] = fmaf(kv[7], c.w, sc[r]);
+        }
       }
+      // the first value rows are on their way while the softmax runs
+      const T* vp = vb + (int64_t)k0 * D + CPL * lane;
+      float vn[VB][CPL];
+      auto load_v = [&](int j0) {
+#pragma unroll
+        for (int j = 0; j < VB; ++j) load_f<T, CPL>(vp + (int64_t)min(j0 + j, cnt - 1) * D, vn[j]);   // (past the end: a repeat, with p = 0)
+      };
+      load_v(0);
+      // ---- online softmax, row by row (a key past the row's own token, or past the end, counts as -inf) ----
+      int tok = 0, head = 0;                             // of row r
+#pragma unroll
+      for (int r = 0; r < ROWS; ++r) {
+        const int lim = seg == 0 ? n : H + tok0 + tok + 1;
+        if (++head == s) { head = 0; ++tok; }
+        const float v = kk < lim && kk < n ? sc[r] * scale : -INFINITY;
+        float mx = v;
+#pragma unroll
+        for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+        const float m_new = fmaxf(m[r], mx);
+        const float pr = v == -INFINITY ? 0.f : expf(v - m_new);
+        if (m_new != m[r]) {                             // (uniform over the warp)
+          const float f = m[r] == -INFINITY ? 0.f : expf(m[r] - m_new);
+          l[r] *= f;
+#pragma unroll
+          for (int c = 0; c < CPL; ++c) acc[r][c] *= f;
+          m[r] = m_new;
+        }
+        l[r] += pr;
+        ps[lane][r] = pr;
+      }
+      __syncwarp();
+      // ---- O += P V ----
+#pragma unroll
+      for (int j0 = 0; j0 < KT; j0 += VB) {
+        if (j0 >= cnt) break;
+        float v[VB][CPL];
+#pragma unroll
+        for (int j = 0; j < VB; ++j)
+#pragma unroll
+          for (int c = 0; c < CPL; ++c) v[j][c] = vn[j][c];
+        if (j0 + VB < cnt) load_v(j0 + VB);
+#pragma unroll
+        for (int j = 0; j < VB; ++j) {
+#pragma unroll
+          for (int r = 0; r < ROWS; r += 4) {
+            const float4 pr = *reinterpret_cast<const float4*>(&ps[j0 + j][r]);
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) {
+              acc[r][c] = fmaf(pr.x, v[j][c], acc[r][c]); acc[r + 1][c] = fmaf(pr.y, v[j][c], acc[r + 1][c]);
+              acc[r + 2][c] = fmaf(pr.z, v[j][c], acc[r + 2][c]); acc[r + 3][c] = fmaf(pr.w, v[j][c], acc[r + 3][c]);
+            }
+          }
+        }
+      }
+      __syncwarp();
     }
   }
-  const float inv = 1.f / l;   // the self part always holds the token itself
-  TO* orow = o + ((int64_t)t * Hq + h) * D;
+
+  // ---- merge the warps' partial results ----
 #pragma unroll
-  for (int c = 0; c < CPL; ++c) orow[lane + 32 * c] = rc_from_float<TO>(acc[c] * inv);
+  for (int r = 0; r < ROWS; ++r) {
+#pragma unroll
+    for (int off = 16; off; off >>= 1) l[r] += __shfl_xor_sync(0xffffffffu, l[r], off);
+    if (lane == 0) { sh.m[warp][r] = m[r]; sh.l[warp][r] = l[r]; }
+  }
+  __syncthreads();                                       // the probabilities make room for the partial O
+#pragma unroll
+  for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) sh.part[warp][r][CPL * lane + c] = acc[r][c];
+  __syncthreads();
+  for (int e = threadIdx.x; e < n_rows * D; e += WARPS * 32) {
+    const int r = e / D, i = e % D;
+    float M = -INFINITY, sum = 0.f, v = 0.f;
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w) M = fmaxf(M, sh.m[w][r]);
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w) {
+      const float f = sh.m[w][r] == -INFINITY ? 0.f : expf(sh.m[w][r] - M);
+      sum = fmaf(sh.l[w][r], f, sum);
+      v = fmaf(sh.part[w][r][i], f, v);
+    }
+    // (the self part always holds the token itself, so sum > 0)
+    o[((int64_t)(seq0 + tok0 + r / s) * Hq + g * s + r % s) * D + i] = rc_from_float<TO>(v * (1.f / sum));
+  }
 }
 
 template <typename T, typename TO>
 cudaError_t launch(const recache_ctx* ctx, const AttnRowsArgs& a, cudaStream_t st) {
-  const int d = ctx->desc.head_dim, Hq = ctx->desc.n_q_heads, G = ctx->desc.n_kv_heads;
-  const int64_t rows = (int64_t)a.total * Hq;
-  if (rows == 0) return cudaSuccess;
-  const unsigned blocks = (unsigned)((rows + WARPS - 1) / WARPS);
+  const int d = ctx->desc.head_dim, Hq = ctx->desc.n_q_heads, G = ctx->desc.n_kv_heads, TQ = ROWS / (Hq / G);
+  if (a.total == 0 || a.n_seq == 0) return cudaSuccess;
+  const dim3 grid((unsigned)(a.total / TQ + a.n_seq), (unsigned)G);
   const float scale = (float)(1.0 / sqrt((double)d));
   RcLaunchScope scope(ctx, a.route_cu ? RC_K_PREFILL_ATTN : RC_K_ENCODE_ATTN, st);
-#define RC_ARGS (const T*)a.q, (TO*)a.o, a.cu, a.n_seq, a.total, a.pos0, a.slot, (const T*)a.k_self, \
-    (const T*)a.v_self, a.self_rows, (const T*)a.k_route, (const T*)a.v_route, a.route_cu, a.prefix_len, a.hist, a.route_rows, Hq, G, \
-    ctx->cos_tab, ctx->sin_tab, ctx->desc.max_pos, scale, ctx->status
-  if (d == 64) attn_rows_kernel<T, TO, 64><<<blocks, WARPS * 32, 0, st>>>(RC_ARGS);
-  else         attn_rows_kernel<T, TO, 128><<<blocks, WARPS * 32, 0, st>>>(RC_ARGS);
-#undef RC_ARGS
-  return cudaGetLastError();
+  auto go = [&](auto kernel, size_t smem) {
+    return rc_launch_overlapped(kernel, grid, WARPS * 32, smem, st, (const T*)a.q, (TO*)a.o, a.cu, a.n_seq, a.total, a.pos0, a.slot, (const T*)a.k_self,
+                                (const T*)a.v_self, a.self_rows, (const T*)a.k_route, (const T*)a.v_route, a.route_cu, a.prefix_len, a.hist,
+                                a.route_rows, Hq, G, (const float*)ctx->cos_tab, (const float*)ctx->sin_tab, ctx->desc.max_pos, scale, ctx->status);
+  };
+  return d == 64 ? go(attn_rows_kernel<T, TO, 64>, sizeof(Smem<64>)) : go(attn_rows_kernel<T, TO, 128>, sizeof(Smem<128>));
 }
 
 }  // namespace

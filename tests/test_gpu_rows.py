@@ -1,0 +1,36 @@
+"""The exact-arithmetic attention at the edges of its blocks: sequences one token around a block of
+query rows and around the key tiles of a full round of warps, every number of heads per group."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2608_19662_b200 import workloads as wl
+
+from pipeline import gpu_compact, gpu_encode, gpu_prefill, make_ctx, max_abs, oracle_encode, oracle_prefill, oracle_rows
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("hq,g,d,dtype,tol", [
+    (2, 2, 64, "f32", 1e-5), (4, 2, 64, "f32", 1e-5), (6, 2, 64, "f32", 1e-5), (5, 1, 64, "f32", 1e-5), (8, 1, 64, "f32", 1e-5),
+    (2, 2, 128, "f32", 1e-5), (3, 1, 128, "f32", 1e-5), (7, 1, 128, "f32", 1e-5), (8, 1, 128, "f32", 1e-5),
+    (4, 2, 64, "bf16", 1e-2), (3, 3, 128, "bf16", 1e-2),
+])
+def test_block_edges(hq, g, d, dtype, tol):
+    sh = wl.Shape(hq, g, d, 1e4, dtype)
+    rng = np.random.default_rng([hq, g, d])
+    lens = [1, 15, 16, 17, 0, 31, 33, 255, 257, 290]
+    pool = wl.pack_resources(sh, hq * 100 + d, lens, [rng.integers(0, 2, n).astype(np.uint8) for n in lens])
+    rc = make_ctx(sh, max_pos=1024)
+    o, kc, vc = gpu_encode(rc, pool)
+    ref, kc_ref, vc_ref = oracle_encode(pool)
+    assert max_abs(o, ref) < tol
+    lists = [[9, 1], [], [3, 4, 7, 8]]
+    vis = [rng.integers(0, 2, (g, len(x))).astype(np.uint8) for x in lists]
+    req = wl.make_requests(sh, 7, pool, lists, vis, [17, 40, 3])
+    rows = oracle_rows(pool, req)
+    out = gpu_compact(rc, pool, req, kc, vc)
+    p, _, _ = gpu_prefill(rc, req, out["k_out"], out["v_out"], out["route_cu"])
+    p_ref, _ = oracle_prefill(req, rows, kc_ref, vc_ref)
+    assert max_abs(p, p_ref) < tol
+    assert rc.poll_status() == 0
