@@ -1,4 +1,6 @@
-"""Thin ctypes binding over librecache.so: argument marshalling only.
+"""Thin binding over librecache.so: argument marshalling only, in _native.so for
+the calls of the hot path (checks, output and workspace tensors, the C call) and
+by ctypes for the rest.
 
 Every step of the hot path runs in the library's CUDA kernels; torch provides
 device memory and the current stream.  There is no CPU fallback: loading fails
@@ -15,6 +17,7 @@ import torch
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "librecache.so")
+NATIVE_PATH = os.path.join(HERE, "_native.so")
 
 F32, BF16 = 0, 1
 PACKED, PAGED = 0, 1
@@ -67,7 +70,13 @@ SIGNATURES = {
                                                 _P, _I32, _P]),
 }
 
+# what _native calls, in its order
+NATIVE_CALLS = ["encode_workspace_bytes", "compact_workspace_bytes", "prefill_workspace_bytes", "decode_workspace_bytes", "encode_resources",
+                "compact_routes", "attend_prefill", "attend_prefill_gather", "attend_prefill_history", "attend_decode",
+                "attend_decode_gather"]
+
 _lib = None
+_native = None
 
 
 def load_library() -> C.CDLL:
@@ -80,7 +89,12 @@ def load_library() -> C.CDLL:
         for name, (res, args) in SIGNATURES.items():
             fn = getattr(lib, name)
             fn.restype, fn.argtypes = res, args
-        _lib = lib
+        global _native
+        if not os.path.exists(NATIVE_PATH):
+            raise RuntimeError(f"{NATIVE_PATH} is missing: build it with `python -m paper_2608_19662_b200.build`")
+        from . import _native as native
+        native.bind(*(C.cast(getattr(lib, "recache_" + name), _P).value for name in NATIVE_CALLS))
+        _lib, _native = lib, native
     return _lib
 
 
@@ -133,12 +147,13 @@ class ReCache:
         if st != 0:
             raise ReCacheError(f"recache_create failed: {STATUS_NAMES.get(st, st)}")
         self.h = h
+        self._hv = h.value      # the handle as _native takes it
         self._ws = None
 
     def close(self):
         if getattr(self, "h", None):
             self.lib.recache_destroy(self.h)
-            self.h = None
+            self.h = self._hv = None
 
     def __del__(self):
         try:
@@ -209,17 +224,8 @@ class ReCache:
     def encode_resources(self, q, k, v, cu_seqlens, max_len, dst_slot, k_cache, v_cache, out=None,
                          out_dtype=None, workspace=None):
         """recache_encode_resources: q [T,Hq,d], k/v [T,G,d], caches [G,pool,d]. Returns o [T,Hq,d]."""
-        n_res = cu_seqlens.numel() - 1
-        total = q.shape[0]
-        od, oc = self._out_code(out_dtype)
-        if out is None:
-            out = torch.empty(q.shape, dtype=od, device=q.device)
-        ws = workspace if workspace is not None else self.workspace(self.encode_workspace_bytes(n_res, total, max_len))
-        st = self.lib.recache_encode_resources(self.h, _ptr(q), _ptr(k), _ptr(v), _ptr(cu_seqlens), n_res, total,
-                                               int(max_len), _ptr(dst_slot), _ptr(k_cache), _ptr(v_cache),
-                                               k_cache.shape[1], _ptr(out), oc, _ptr(ws), ws.numel(), _stream())
-        self._check(st, "recache_encode_resources")
-        return out
+        return _native.encode(self, self._hv, self.dtype_code, q, k, v, cu_seqlens, max_len, dst_slot, k_cache, v_cache, out, out_dtype,
+                              workspace)
 
     def encode_resources_prefixed(self, q, k, v, cu_seqlens, max_len, dst_slot, k_cache, v_cache, k_prefix=None,
                                   v_prefix=None, pos_offset=None, out=None, out_dtype=None, workspace=None):
@@ -243,113 +249,41 @@ class ReCache:
         """recache_compact_routes.  All outputs are caller-allocated tensors:
         route_cu [B*G+1], route_idx [capacity], k_out/v_out packed [capacity,d] or page pools
         [n_pages,page_tokens,d]; paged mode also needs page_table [B*G,max_pages] and free_pages."""
-        n_req = res_off.numel() - 1
-        total_listed = res_slot.numel()
-        ws = workspace if workspace is not None else self.workspace(self.compact_workspace_bytes(n_req, total_listed))
-        paged = mode == PAGED
-        st = self.lib.recache_compact_routes(
-            self.h, _ptr(k_cache), _ptr(v_cache), k_cache.shape[1], _ptr(keep), _ptr(res_off), _ptr(res_slot),
-            _ptr(res_len), n_req, total_listed, _ptr(vis), mode, _ptr(route_cu), _ptr(route_len), _ptr(route_idx),
-            route_idx.numel() if (paged or k_out is None) else min(route_idx.numel(), k_out.shape[0]), _ptr(k_out),
-            _ptr(v_out),
-            _ptr(page_table),
-            page_table.shape[1] if paged else 0, _ptr(free_pages), free_pages.numel() if paged else 0,
-            k_out.shape[0] if paged else 0, _ptr(ws), ws.numel(), _stream())
-        self._check(st, "recache_compact_routes")
+        _native.compact(self, self._hv, self.dtype_code, k_cache, v_cache, keep, res_off, res_slot, res_len, vis, mode, route_cu, route_idx,
+                        k_out, v_out, route_len, page_table, free_pages, workspace)
 
     def attend_prefill(self, q, k_conv, v_conv, cu_q, q_pos0, max_q, k_route, v_route, route_cu, k_conv_out=None,
                        v_conv_out=None, out=None, out_dtype=None, workspace=None):
         """recache_attend_prefill.  Returns (o [Tq,Hq,d], k_conv_out [G,Tq,d], v_conv_out [G,Tq,d])."""
-        n_req = cu_q.numel() - 1
-        total_q = q.shape[0]
-        g, d = k_conv.shape[1], k_conv.shape[2]
-        od, oc = self._out_code(out_dtype)
-        if out is None:
-            out = torch.empty(q.shape, dtype=od, device=q.device)
-        if k_conv_out is None:
-            k_conv_out = torch.empty((g, total_q, d), dtype=k_conv.dtype, device=q.device)
-        if v_conv_out is None:
-            v_conv_out = torch.empty((g, total_q, d), dtype=k_conv.dtype, device=q.device)
-        ws = workspace if workspace is not None else self.workspace(self.prefill_workspace_bytes(n_req, total_q, max_q))
-        st = self.lib.recache_attend_prefill(self.h, _ptr(q), _ptr(k_conv), _ptr(v_conv), _ptr(cu_q), _ptr(q_pos0),
-                                             n_req, total_q, int(max_q), _ptr(k_route), _ptr(v_route), _ptr(route_cu),
-                                             k_route.shape[0], _ptr(k_conv_out), _ptr(v_conv_out), _ptr(out), oc,
-                                             _ptr(ws), ws.numel(), _stream())
-        self._check(st, "recache_attend_prefill")
-        return out, k_conv_out, v_conv_out
+        return _native.prefill(self, self._hv, self.dtype_code, q, k_conv, v_conv, cu_q, q_pos0, max_q, k_route, v_route, route_cu, k_conv_out,
+                               v_conv_out, out, out_dtype, workspace, None)
 
     def attend_prefill_gather(self, q, k_conv, v_conv, cu_q, q_pos0, max_q, k_cache, v_cache, route_idx, route_cu,
                               k_conv_out=None, v_conv_out=None, out=None, out_dtype=None, workspace=None):
         """recache_attend_prefill_gather: the route rows are read from the resource cache [G,pool,d]
         through route_idx (index-only compaction).  Returns (o, k_conv_out, v_conv_out)."""
-        n_req = cu_q.numel() - 1
-        total_q = q.shape[0]
-        g, d = k_conv.shape[1], k_conv.shape[2]
-        od, oc = self._out_code(out_dtype)
-        if out is None:
-            out = torch.empty(q.shape, dtype=od, device=q.device)
-        if k_conv_out is None:
-            k_conv_out = torch.empty((g, total_q, d), dtype=k_conv.dtype, device=q.device)
-        if v_conv_out is None:
-            v_conv_out = torch.empty((g, total_q, d), dtype=k_conv.dtype, device=q.device)
-        ws = workspace if workspace is not None else self.workspace(self.prefill_workspace_bytes(n_req, total_q, max_q))
-        st = self.lib.recache_attend_prefill_gather(
-            self.h, _ptr(q), _ptr(k_conv), _ptr(v_conv), _ptr(cu_q), _ptr(q_pos0), n_req, total_q, int(max_q),
-            _ptr(k_cache), _ptr(v_cache), k_cache.shape[1], _ptr(route_idx), _ptr(route_cu), route_idx.numel(),
-            _ptr(k_conv_out), _ptr(v_conv_out), _ptr(out), oc, _ptr(ws), ws.numel(), _stream())
-        self._check(st, "recache_attend_prefill_gather")
-        return out, k_conv_out, v_conv_out
+        return _native.prefill(self, self._hv, self.dtype_code, q, k_conv, v_conv, cu_q, q_pos0, max_q, k_cache, v_cache, route_cu, k_conv_out,
+                               v_conv_out, out, out_dtype, workspace, route_idx)
 
     def attend_prefill_history(self, q, k_conv, v_conv, cu_q, q_pos0, max_q, k_route, v_route, route_cu,
                                k_conv_cache, v_conv_cache, conv_slot, hist_len, out=None, out_dtype=None, workspace=None):
         """recache_attend_prefill_history: a later turn over caches [G,rows,d] that already hold hist_len[b]
         rows per request from conv_slot[b]; appends the new rotated keys / values there.  Returns o."""
-        n_req = cu_q.numel() - 1
-        total_q = q.shape[0]
-        od, oc = self._out_code(out_dtype)
-        if out is None:
-            out = torch.empty(q.shape, dtype=od, device=q.device)
-        ws = workspace if workspace is not None else self.workspace(self.prefill_workspace_bytes(n_req, total_q, max_q))
-        st = self.lib.recache_attend_prefill_history(
-            self.h, _ptr(q), _ptr(k_conv), _ptr(v_conv), _ptr(cu_q), _ptr(q_pos0), n_req, total_q, int(max_q),
-            _ptr(k_route), _ptr(v_route), _ptr(route_cu), k_route.shape[0], _ptr(k_conv_cache), _ptr(v_conv_cache),
-            k_conv_cache.shape[1], _ptr(conv_slot), _ptr(hist_len), _ptr(out), oc, _ptr(ws), ws.numel(), _stream())
-        self._check(st, "recache_attend_prefill_history")
-        return out
+        return _native.prefill_history(self, self._hv, self.dtype_code, q, k_conv, v_conv, cu_q, q_pos0, max_q, k_route, v_route, route_cu,
+                                       k_conv_cache, v_conv_cache, conv_slot, hist_len, out, out_dtype, workspace)
 
     def attend_decode(self, q, q_pos, k_pages, v_pages, res_page_table, res_len, hist_page_table, hist_len,
                       k_new=None, v_new=None, out=None, out_dtype=None, workspace=None):
         """recache_attend_decode.  q [B,Hq,d]; tables [B*G,max_pages]. Returns o [B,Hq,d]."""
-        batch = q.shape[0]
-        od, oc = self._out_code(out_dtype)
-        if out is None:
-            out = torch.empty(q.shape, dtype=od, device=q.device)
-        mr, mh = res_page_table.shape[1], hist_page_table.shape[1]
-        ws = workspace if workspace is not None else self.workspace(self.decode_workspace_bytes(batch, mr, mh))
-        st = self.lib.recache_attend_decode(self.h, _ptr(q), _ptr(q_pos), batch, _ptr(k_new), _ptr(v_new),
-                                            _ptr(k_pages), _ptr(v_pages), k_pages.shape[0], _ptr(res_page_table), mr,
-                                            _ptr(res_len), _ptr(hist_page_table), mh, _ptr(hist_len), _ptr(out), oc,
-                                            _ptr(ws), ws.numel(), _stream())
-        self._check(st, "recache_attend_decode")
-        return out
+        return _native.decode(self, self._hv, self.dtype_code, q, q_pos, k_pages, v_pages, res_page_table, res_len, hist_page_table, hist_len,
+                              k_new, v_new, out, out_dtype, workspace)
 
     def attend_decode_gather(self, q, q_pos, k_cache, v_cache, route_idx, route_cu, max_res_pages, k_pages, v_pages,
                              hist_page_table, hist_len, k_new=None, v_new=None, out=None, out_dtype=None, workspace=None):
         """recache_attend_decode_gather: decode whose resource rows are read from the cache through the
         compaction's index list (nothing materialised).  Returns o [B,Hq,d]."""
-        batch = q.shape[0]
-        od, oc = self._out_code(out_dtype)
-        if out is None:
-            out = torch.empty(q.shape, dtype=od, device=q.device)
-        mh = hist_page_table.shape[1]
-        ws = workspace if workspace is not None else self.workspace(self.decode_workspace_bytes(batch, max_res_pages, mh))
-        st = self.lib.recache_attend_decode_gather(
-            self.h, _ptr(q), _ptr(q_pos), batch, _ptr(k_new), _ptr(v_new), _ptr(k_cache), _ptr(v_cache), k_cache.shape[1],
-            _ptr(route_idx), _ptr(route_cu), route_idx.numel(), int(max_res_pages), _ptr(k_pages), _ptr(v_pages),
-            k_pages.shape[0],
-            _ptr(hist_page_table), mh, _ptr(hist_len), _ptr(out), oc, _ptr(ws), ws.numel(), _stream())
-        self._check(st, "recache_attend_decode_gather")
-        return out
+        return _native.decode_gather(self, self._hv, self.dtype_code, q, q_pos, k_cache, v_cache, route_idx, route_cu, max_res_pages, k_pages,
+                                     v_pages, hist_page_table, hist_len, k_new, v_new, out, out_dtype, workspace)
 
     def attend_decode_noalloc(self, q, q_pos, k_pages, v_pages, res_page_table, res_len, hist_page_table, hist_len,
                               out, k_new=None, v_new=None):

@@ -9,10 +9,14 @@
 // shared memory at the end, so nothing synchronises in between.  For the scores
 // a lane owns a key and keeps a sum per row, with the queries broadcast from shared
 // memory (four FMA to a load); for P V a lane owns d / 32 columns and the
-// probabilities are broadcast.  Bound by FMA issue and, at the few hundred rows
-// of the calls made in earnest, by the length of one warp's chain: a warp per
-// row, with each key row read once for every query row, took 69 us for 1,250
-// tokens of six resources (4 / 2 heads of 64), ROWS_NOW us now.
+// probabilities are broadcast, with the value rows loaded eight at a time ahead
+// of their use.  Bound by the length of one warp's chain of loads and sums at the
+// few hundred rows of the calls made in earnest.  A warp per query row, which
+// read every key row once per query row, took 69 us each for 1,250 tokens in six
+// resources and for the 160-token turn over them (4 / 2 heads of 64): that pass of
+// encode, compaction and turn took 155 us with it and 66 us with this kernel (80 us
+// with 16 rows to a CTA and no early value loads, 67 and 69 us with three CTAs of 80
+// registers on an SM or four warps to a CTA).
 //
 // Key set of a row (token t of sequence b at local index j, head h, group g):
 //   route part : rows route_cu[b*G+g] .. route_cu[b*G+g+1]-1 of k_route/v_route,

@@ -878,8 +878,8 @@ cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope,
       !map_rows(&tvs, a.v_self, self_total))
     return cudaErrorInvalidValue;
   const bool has_route = (a.route_cu != nullptr || a.prefix_len > 0) && a.route_rows > 0 && a.route_idx == nullptr;
-  if (!map_rows(&tkr, has_route ? a.k_route : a.k_self, has_route ? (uint64_t)a.route_rows : self_total) ||
-      !map_rows(&tvr, has_route ? a.v_route : a.v_self, has_route ? (uint64_t)a.route_rows : self_total))
+  if (!has_route) { tkr = tks; tvr = tvs; }   // unused
+  else if (!map_rows(&tkr, a.k_route, (uint64_t)a.route_rows) || !map_rows(&tvr, a.v_route, (uint64_t)a.route_rows))
     return cudaErrorInvalidValue;
 
   TcParams p;
