@@ -51,6 +51,8 @@ __global__ void __launch_bounds__(TPB) compact_count_kernel(
     const int32_t* __restrict__ res_len, int total_listed, int64_t pool_tokens,
     int32_t* __restrict__ kept, int32_t* status) {
   __shared__ int red[TPB / 32];
+  rc_grid_wait();
+  rc_grid_launch_next();
   for (int r = blockIdx.x; r < total_listed; r += gridDim.x) {
     const int64_t s0 = res_slot[r];
     const int n = res_len[r];
@@ -85,6 +87,8 @@ __global__ void __launch_bounds__(1024) compact_plan_kernel(
   __shared__ int ws[1024 / 32 + 1];
   __shared__ int wlen_sh[32];
   __shared__ int carry_rows, carry_pages;
+  rc_grid_wait();
+  rc_grid_launch_next();
   const int n_routes = n_requests * G;
   const bool warp_per_route = n_routes <= 32;
   if (threadIdx.x == 0) { carry_rows = 0; carry_pages = 0; }
@@ -186,6 +190,8 @@ __global__ void __launch_bounds__(TPB) compact_gather_kernel(
   __shared__ int ws[TPB / 32 + 1];
   __shared__ int32_t src_tok[SUPER];   // token offset (inside the resource) of the pass's n-th kept token
   __shared__ int32_t dst_row[SUPER];   // destination row (packed row, or page * page_tokens + slot); -1 = skip
+  rc_grid_wait();
+  rc_grid_launch_next();
   const int r = blockIdx.x, g = blockIdx.y;
   if (!vis[(int64_t)g * total_listed + r]) return;
   const int64_t s0 = res_slot[r];
@@ -290,29 +296,30 @@ cudaError_t rc_launch_compact(const recache_ctx* ctx, const CompactArgs& a, cuda
   const int n_routes = a.n_requests * G;
   const int row_bytes = d * (ctx->desc.dtype == RECACHE_BF16 ? 2 : 4);
   Ws w = carve(a.workspace, n_routes, a.total_listed, G);
+  cudaError_t e = cudaSuccess;
   if (a.total_listed > 0) {
     const int blocks = a.total_listed < 4096 ? a.total_listed : 4096;
     RcLaunchScope scope(ctx, RC_K_COMPACT_COUNT, st);
-    compact_count_kernel<<<blocks, TPB, 0, st>>>(a.keep, a.res_slot, a.res_len, a.total_listed,
-                                                 a.pool_tokens, w.kept, ctx->status);
+    e = rc_launch_overlapped(compact_count_kernel, blocks, TPB, 0, st, a.keep, a.res_slot, a.res_len, a.total_listed, a.pool_tokens, w.kept,
+                             ctx->status);
+    if (e != cudaSuccess) return e;
   }
   {
     RcLaunchScope scope(ctx, RC_K_COMPACT_PLAN, st);
-    compact_plan_kernel<<<1, 1024, 0, st>>>(w.kept, a.res_off, a.n_requests, a.total_listed, a.vis, G, a.mode,
-                                            ctx->desc.page_tokens, a.route_cu, a.route_len, w.res_route_off,
-                                            w.page_cu, a.row_capacity, a.page_table, a.max_pages_per_route,
-                                            a.free_pages, a.n_free_pages, a.n_pool_pages, ctx->status);
+    e = rc_launch_overlapped(compact_plan_kernel, 1, 1024, 0, st, (const int32_t*)w.kept, a.res_off, a.n_requests, a.total_listed, a.vis, G, a.mode,
+                             ctx->desc.page_tokens, a.route_cu, a.route_len, w.res_route_off, w.page_cu, a.row_capacity, a.page_table,
+                             a.max_pages_per_route, a.free_pages, a.n_free_pages, a.n_pool_pages, ctx->status);
+    if (e != cudaSuccess) return e;
   }
   if (a.total_listed > 0) {
     const int64_t pairs = (int64_t)a.total_listed * G;
     const unsigned z = (unsigned)(pairs >= 2048 ? 1 : (2048 + pairs - 1) / pairs > 8 ? 8 : (2048 + pairs - 1) / pairs);
     dim3 grid((unsigned)a.total_listed, (unsigned)G, z);
     RcLaunchScope scope(ctx, RC_K_COMPACT_GATHER, st);
-    compact_gather_kernel<<<grid, TPB, 0, st>>>(
-        (const uint8_t*)a.k_cache, (const uint8_t*)a.v_cache, a.pool_tokens, a.keep, a.res_off, a.res_slot,
-        a.res_len, a.n_requests, a.total_listed, a.vis, G, a.mode, ctx->desc.page_tokens, a.route_cu,
-        w.res_route_off, w.page_cu, a.route_idx, a.row_capacity, (uint8_t*)a.k_out, (uint8_t*)a.v_out,
-        a.free_pages, a.n_free_pages, a.n_pool_pages, row_bytes);
+    e = rc_launch_overlapped(compact_gather_kernel, grid, TPB, 0, st, (const uint8_t*)a.k_cache, (const uint8_t*)a.v_cache, a.pool_tokens, a.keep,
+                             a.res_off, a.res_slot, a.res_len, a.n_requests, a.total_listed, a.vis, G, a.mode, ctx->desc.page_tokens,
+                             (const int32_t*)a.route_cu, (const int32_t*)w.res_route_off, (const int32_t*)w.page_cu, a.route_idx, a.row_capacity,
+                             (uint8_t*)a.k_out, (uint8_t*)a.v_out, a.free_pages, a.n_free_pages, a.n_pool_pages, row_bytes);
   }
-  return cudaGetLastError();
+  return e;
 }
