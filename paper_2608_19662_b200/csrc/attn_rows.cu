@@ -7,16 +7,16 @@
 // in tiles of 32 (tile t belongs to warp t % 8) and each runs an online softmax
 // of its own over all of them; the partial (max, sum, O) are merged through
 // shared memory at the end, so nothing synchronises in between.  For the scores
-// a lane owns a key and keeps a sum per row, with the queries broadcast from shared
-// memory (four FMA to a load); for P V a lane owns d / 32 columns and the
+// four lanes share a key's row, so that a warp's 16-byte loads touch 8 lines, not
+// 32 (with a key to a lane the loads' tag lookups alone took 512 cycles a tile),
+// and a query load from shared memory serves 16 FMA; for P V a lane owns d / 32 columns and the
 // probabilities are broadcast, with the value rows loaded eight at a time ahead
-// of their use.  Bound by the length of one warp's chain of loads and sums at the
-// few hundred rows of the calls made in earnest.  A warp per query row, which
-// read every key row once per query row, took 69 us each for 1,250 tokens in six
-// resources and for the 160-token turn over them (4 / 2 heads of 64): that pass of
-// encode, compaction and turn took 155 us with it and 66 us with this kernel (80 us
-// with 16 rows to a CTA and no early value loads, 67 and 69 us with three CTAs of 80
-// registers on an SM or four warps to a CTA).
+// of their use.  At the few hundred rows of the calls made in earnest half the time
+// is a block's start (a chain of dependent loads) and half FMA issue.  A warp per
+// query row, which read every key row once per query row, took 69 us each for 1,250
+// tokens in six resources and for the 160-token turn over them (4 / 2 heads of 64);
+// this kernel takes 24 and 11 us, and the pass of encode, compaction and turn 53 us
+// instead of 155 (four warps to a CTA: 55 us; 16 rows to a CTA: 80 us).
 //
 // Key set of a row (token t of sequence b at local index j, head h, group g):
 //   route part : rows route_cu[b*G+g] .. route_cu[b*G+g+1]-1 of k_route/v_route,
@@ -86,20 +86,26 @@ __global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
 
   // Block index -> (sequence, block of it).  Sequence b's blocks start at cu[b] / TQ + b, which leaves
   // every sequence at least the ceil(len / TQ) it needs.
+  // (32 boundaries are probed at a time: the block's start is a chain of dependent loads and little else)
   const int x = blockIdx.x;
-  int lo = 0, hi = n_seq;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (cu[mid] / TQ + mid <= x) lo = mid; else hi = mid;
+  int b = 0;
+  for (int width = n_seq; width > 1;) {
+    const int step = (width + 31) >> 5, at = b + lane * step;
+    const bool le = lane * step < width && (lane == 0 || cu[at] / TQ + at <= x);
+    const int last = 31 - __clz(__ballot_sync(0xffffffffu, le));      // (the boundaries ascend)
+    b += last * step;
+    width = min(step, width - last * step);
   }
-  const int b = lo, seq0 = cu[b], L = cu[b + 1] - seq0;
-  if (x == 0 && g == 0 && threadIdx.x == 0 && cu[n_seq] < total) rc_set_status(status, RECACHE_DEV_BAD_SEQLENS);
+  const int seq0 = cu[b], L = cu[b + 1] - seq0, n_cu = cu[n_seq];
+  const int slot_b = slot ? slot[b] : 0, hist_b = hist ? hist[b] : 0, pos_b = pos0 ? pos0[b] : 0;
+  const int route0 = route_cu ? route_cu[b * G + g] : g * prefix_len, route1 = route_cu ? route_cu[b * G + g + 1] : route0 + prefix_len;
+  if (x == 0 && g == 0 && threadIdx.x == 0 && n_cu < total) rc_set_status(status, RECACHE_DEV_BAD_SEQLENS);
   const int tok0 = (x - (seq0 / TQ + b)) * TQ;           // first token of the block, local
   if (seq0 < 0 || L < 0 || seq0 + L > total) { if (threadIdx.x == 0) rc_set_status(status, RECACHE_DEV_BAD_SEQLENS); return; }
   if (tok0 < 0 || tok0 >= L) return;
-  const int64_t base = slot ? (int64_t)slot[b] : (int64_t)seq0;
-  const int H = hist ? hist[b] : 0;      // earlier-turn rows at the start of the self part, all visible
-  const int p0 = pos0 ? pos0[b] : 0;
+  const int64_t base = slot ? (int64_t)slot_b : (int64_t)seq0;
+  const int H = hist_b;                  // earlier-turn rows at the start of the self part, all visible
+  const int p0 = pos_b;
   // tokens that can be computed: inside the sequence, the rotary table and the cache
   int n_tok = min(TQ, L - tok0);
   if (base < 0 || H < 0 || base + H + tok0 + n_tok > self_rows) {
@@ -145,8 +151,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
     if (seg == 0) {
       if (!route_cu && prefix_len <= 0) continue;
       // the route's packed rows, or (encoding behind a shared prefix) the group's prefix rows
-      const int r0 = route_cu ? route_cu[b * G + g] : g * prefix_len;
-      const int r1 = route_cu ? route_cu[b * G + g + 1] : r0 + prefix_len;
+      const int r0 = route0, r1 = route1;
       // a range outside the route tensors (e.g. after a compaction that overflowed its capacity)
       // is reported and read as an empty route
       if (r0 < 0 || r1 < r0 || (int64_t)r1 > route_rows) {
@@ -161,22 +166,46 @@ __global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
     }
     for (int k0 = 0; k0 < n; k0 += KT, ++t) {
       if (t % WARPS != warp) continue;
-      const int kk = k0 + lane, cnt = min(KT, n - k0);
-      // ---- scores of key kk with every row ----
-      float sc[ROWS];
+      const int cnt = min(KT, n - k0);
+      // ---- scores: four lanes share eight keys' rows, each a quarter of their 16-byte chunks ----
+      const int part = lane & 3, key8 = lane >> 2;
+      float sc[4][ROWS];                                 // [keys 8 kg + key8][row], this lane's chunks only
 #pragma unroll
-      for (int r = 0; r < ROWS; ++r) sc[r] = 0.f;
-      const T* krow = kb + (int64_t)min(kk, n - 1) * D;
-#pragma unroll 4
-      for (int i = 0; i < D; i += 8) {
-        float kv[8];
-        load_f<T, 8>(krow + i, kv);
+      for (int kg = 0; kg < 4; ++kg)
 #pragma unroll
-        for (int r = 0; r < ROWS; ++r) {
-          const float4 a = *reinterpret_cast<const float4*>(&sh.q[r][i]), c = *reinterpret_cast<const float4*>(&sh.q[r][i + 4]);
-          sc[r] = fmaf(kv[0], a.x, sc[r]); sc[r] = fmaf(kv[1], a.y, sc[r]); sc[r] = fmaf(kv[2], a.z, sc[r]); sc[r] = fmaf(kv[3], a.w, sc[r]);
-          sc[r] = fmaf(kv[4], c.x, sc[r]); sc[r] = fmaf(kv[5], c.y, sc[r]); sc[r] = fmaf(kv[6], c.z, sc[r]); sc[r] = fmaf(kv[7], c.w, sc[r]);
-        }
+        for (int r = 0; r < ROWS; ++r) sc[kg][r] = 0.f;
+      constexpr int EPC = 16 / (int)sizeof(T);
+      const T* kp[4];
+#pragma unroll
+      for (int kg = 0; kg < 4; ++kg) kp[kg] = kb + (int64_t)min(k0 + 8 * kg + key8, n - 1) * D + part * EPC;
+#pragma unroll 2
+      for (int i = 0; i < D; i += 4 * EPC) {
+        float kv[4][EPC];
+#pragma unroll
+        for (int kg = 0; kg < 4; ++kg) load_f<T, EPC>(kp[kg] + i, kv[kg]);
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+          for (int e = 0; e < EPC; e += 4) {
+            const float4 a = *reinterpret_cast<const float4*>(&sh.q[r][i + part * EPC + e]);
+#pragma unroll
+            for (int kg = 0; kg < 4; ++kg) {
+              sc[kg][r] = fmaf(kv[kg][e], a.x, sc[kg][r]); sc[kg][r] = fmaf(kv[kg][e + 1], a.y, sc[kg][r]);
+              sc[kg][r] = fmaf(kv[kg][e + 2], a.z, sc[kg][r]); sc[kg][r] = fmaf(kv[kg][e + 3], a.w, sc[kg][r]);
+            }
+          }
+      }
+      // the four lanes' sums, scattered: lane `part` keeps the keys of kg = part
+      const int mine = 8 * part + key8, kk = k0 + mine;
+      const bool b0 = part & 1, b1 = part & 2;
+      float v1[ROWS];
+#pragma unroll
+      for (int r = 0; r < ROWS; ++r) {
+        float u[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          u[h] = (b0 ? sc[2 * h + 1][r] : sc[2 * h][r]) + __shfl_xor_sync(0xffffffffu, b0 ? sc[2 * h][r] : sc[2 * h + 1][r], 1);
+        v1[r] = (b1 ? u[1] : u[0]) + __shfl_xor_sync(0xffffffffu, b1 ? u[0] : u[1], 2);
       }
       // the first value rows are on their way while the softmax runs
       const T* vp = vb + (int64_t)k0 * D + CPL * lane;
@@ -192,7 +221,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
       for (int r = 0; r < ROWS; ++r) {
         const int lim = seg == 0 ? n : H + tok0 + tok + 1;
         if (++head == s) { head = 0; ++tok; }
-        const float v = kk < lim && kk < n ? sc[r] * scale : -INFINITY;
+        const float v = kk < lim && kk < n ? v1[r] * scale : -INFINITY;
         float mx = v;
 #pragma unroll
         for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
@@ -206,8 +235,10 @@ __global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
           m[r] = m_new;
         }
         l[r] += pr;
-        ps[lane][r] = pr;
+        v1[r] = pr;
       }
+#pragma unroll
+      for (int r = 0; r < ROWS; r += 4) *reinterpret_cast<float4*>(&ps[mine][r]) = make_float4(v1[r], v1[r + 1], v1[r + 2], v1[r + 3]);
       __syncwarp();
       // ---- O += P V ----
 #pragma unroll
@@ -249,19 +280,23 @@ __global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
 #pragma unroll
     for (int c = 0; c < CPL; ++c) sh.part[warp][r][CPL * lane + c] = acc[r][c];
   __syncthreads();
-  for (int e = threadIdx.x; e < n_rows * D; e += WARPS * 32) {
-    const int r = e / D, i = e % D;
-    float M = -INFINITY, sum = 0.f, v = 0.f;
+  for (int r = warp; r < n_rows; r += WARPS) {
+    float mw = lane < WARPS ? sh.m[lane][r] : -INFINITY, M = mw;
 #pragma unroll
-    for (int w = 0; w < WARPS; ++w) M = fmaxf(M, sh.m[w][r]);
+    for (int off = 16; off; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
+    const float f = mw == -INFINITY ? 0.f : expf(mw - M);
+    float sum = lane < WARPS ? sh.l[lane][r] * f : 0.f;
 #pragma unroll
-    for (int w = 0; w < WARPS; ++w) {
-      const float f = sh.m[w][r] == -INFINITY ? 0.f : expf(sh.m[w][r] - M);
-      sum = fmaf(sh.l[w][r], f, sum);
-      v = fmaf(sh.part[w][r][i], f, v);
+    for (int off = 16; off; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+    const float inv = 1.f / sum;                         // (the self part always holds the token itself, so sum > 0)
+    TO* orow = o + ((int64_t)(seq0 + tok0 + r / s) * Hq + g * s + r % s) * D;
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) {
+      float v = 0.f;
+#pragma unroll
+      for (int w = 0; w < WARPS; ++w) v = fmaf(sh.part[w][r][lane + 32 * c], __shfl_sync(0xffffffffu, f, w), v);
+      orow[lane + 32 * c] = rc_from_float<TO>(v * inv);
     }
-    // (the self part always holds the token itself, so sum > 0)
-    o[((int64_t)(seq0 + tok0 + r / s) * Hq + g * s + r % s) * D + i] = rc_from_float<TO>(v * (1.f / sum));
   }
 }
 
