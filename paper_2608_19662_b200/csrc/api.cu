@@ -120,7 +120,7 @@ recache_status recache_selftest_wait_timeout(recache_ctx* ctx, int32_t* report, 
 
 static const char* kKernelNames[RC_K_COUNT] = {
     "rope_store", "tile_plan", "encode_attn", "prefill_attn", "compact_count", "compact_plan",
-    "compact_gather", "decode_append", "decode_attn", "decode_merge"};
+    "compact_gather", "decode_append", "decode_attn", "decode_merge", "prefill_merge"};
 
 int32_t recache_kernel_count(void) { return RC_K_COUNT; }
 const char* recache_kernel_name(int32_t id) { return (id >= 0 && id < RC_K_COUNT) ? kKernelNames[id] : ""; }

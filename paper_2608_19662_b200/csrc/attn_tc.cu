@@ -44,7 +44,7 @@ constexpr int NSTAGE = 2;
 constexpr int BOX_BYTES = 16384;   // [128 rows][64 bf16], 128-byte swizzle
 constexpr int TILE_BYTES = 32768;  // two boxes: head_dim halves
 constexpr int NTHREADS = 512;
-constexpr int REGS_SOFTMAX = 224, REGS_AUX = 32, REGS_EPI = 32;   // 256*224 + 128*(32 + 32) = 65536
+constexpr int REGS_SOFTMAX = 216, REGS_AUX = 40, REGS_EPI = 40;   // 256*216 + 128*(40 + 40) = 65536
 
 constexpr int SM_Q = 0;                              // 2 query tiles
 constexpr int SM_K = SM_Q + 2 * TILE_BYTES;          // NSTAGE key tiles
@@ -72,6 +72,7 @@ struct TcParams : RcPlan {
   // gather mode: route row n of group g is row route_idx[n] of gather_k / gather_v ([G][pool_tokens][128] bf16)
   const uint8_t* gather_k; const uint8_t* gather_v; const int32_t* route_idx; int64_t pool_tokens;
   void* out;
+  float* part_o; float2* part_ml;   // split launch: O [slot][tile][128 rows][128], (maximum in log2 units, sum) [slot][tile][128 rows]
   const float* cos_tab; const float* sin_tab; int max_pos;
   float scale_log2;
 };
@@ -230,7 +231,7 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
 
 using Item = RcItem;
 enum { IT_NTILES = 0, IT_G, IT_SEQ0, IT_L, IT_TOK0, IT_KVEND, IT_POS0, IT_RA0, IT_LENA, IT_NA, IT_BVALID, IT_BASE_LO,
-       IT_BASE_HI, IT_H, IT_WORDS = 16 };
+       IT_BASE_HI, IT_H, IT_PART, IT_WORDS = 16 };
 
 // ---------------------------------------------------------------- kernel --
 // Persistent: a scheduler warp draws work indices from a global counter (the
@@ -245,7 +246,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
                                                               const __grid_constant__ CUtensorMap tm_vs,
                                                               const __grid_constant__ CUtensorMap tm_kr,
                                                               const __grid_constant__ CUtensorMap tm_vr,
-                                                              const TcParams p) {
+                                                              const __grid_constant__ TcParams p) {
   extern __shared__ uint8_t smem_raw[];
   const int s = p.s, TQ = 128 / s;
 
@@ -299,7 +300,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
     const int* r = const_cast<const int*>(item_ring) + sl * IT_WORDS;   // (ordered by the barrier wait above and the arrive below)
     it.n_tiles = r[IT_NTILES]; it.g = r[IT_G]; it.seq0 = r[IT_SEQ0]; it.L = r[IT_L]; it.tok0 = r[IT_TOK0];
     it.kv_end = r[IT_KVEND]; it.pos0 = r[IT_POS0]; it.rA0 = r[IT_RA0]; it.lenA = r[IT_LENA]; it.nA = r[IT_NA];
-    it.b_valid = r[IT_BVALID]; it.H = r[IT_H];
+    it.b_valid = r[IT_BVALID]; it.H = r[IT_H]; it.part = r[IT_PART];
     it.base = (int64_t)(((uint64_t)(uint32_t)r[IT_BASE_HI] << 32) | (uint32_t)r[IT_BASE_LO]);
     if (*abort_flag) it.n_tiles = -1;
     if (release) mbar_arrive(bar(B_IEMPTY + sl));
@@ -391,7 +392,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
           uint32_t orr[16];
           TMEM_LD16(t_o + 16 * ch, orr);
           tmem_wait_ld();
-          if (row_valid) {
+          if (it.part >= 0) {
+            float* prow = p.part_o + ((int64_t)(it.part * 2 + x) * 128 + row) * D + 16 * ch;
+            st_global_v8(prow, orr[0], orr[1], orr[2], orr[3], orr[4], orr[5], orr[6], orr[7]);
+            st_global_v8(prow + 8, orr[8], orr[9], orr[10], orr[11], orr[12], orr[13], orr[14], orr[15]);
+          } else if (row_valid) {
             if constexpr (sizeof(TO) == 4) {
 #pragma unroll
               for (int c = 0; c < 16; c += 8)
@@ -426,11 +431,27 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
     if (lane == 0) {
       const int total = p.header[0] * p.G;   // (a CTA without work publishes "no more work" at once)
       bool first = true;
+      const int n_split = p.start ? p.header[3] : 0;
+      int2 cur = make_int2(0, 0), end = make_int2(0, 0);
+      if ((int)blockIdx.x < n_split) { cur = p.start[blockIdx.x]; end = p.start[blockIdx.x + 1]; }
       for (uint32_t n = 0;; ++n) {
         const int sl = n & 1u;
         mbar_wait(bar(B_IEMPTY + sl), ((n >> 1) & 1u) ^ 1u, abort_flag, p.status);
         Item it;
-        for (;;) {   // CTA c starts with index c; every later index comes from the shared counter
+        it.part = -1;
+        for (; n_split > 0;) {   // the CTA's range of the K/V tiles, one item after the other
+          if (cur.x > end.x || (cur.x == end.x && cur.y >= end.y) || *abort_flag) { it.n_tiles = -1; break; }
+          const int w = cur.x, t0 = cur.y;
+          cur = make_int2(w + 1, 0);
+          if (!rc_load_item(p, w, it)) continue;
+          const int t1 = w == end.x ? min(end.y, it.n_tiles) : it.n_tiles;
+          if (t0 > 0 || t1 < it.n_tiles) it.part = 2 * (int)blockIdx.x + (t0 > 0 ? 0 : 1);
+          else it.part = -1;
+          // (counted from the part's first tile, everything below is the same as for a whole item)
+          it.n_tiles = t1 - t0; it.nA -= t0; it.rA0 += t0 * TILE_N; it.lenA -= t0 * TILE_N;
+          break;
+        }
+        for (; n_split == 0;) {   // CTA c starts with index c; every later index comes from the shared counter
           const int w = first ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(p.header + 1, 1);
           first = false;
           if (w >= total || *abort_flag) { it.n_tiles = -1; break; }
@@ -441,7 +462,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
         if (it.n_tiles > 0) {
           r[IT_G] = it.g; r[IT_SEQ0] = it.seq0; r[IT_L] = it.L; r[IT_TOK0] = it.tok0; r[IT_KVEND] = it.kv_end;
           r[IT_POS0] = it.pos0; r[IT_RA0] = it.rA0; r[IT_LENA] = it.lenA; r[IT_NA] = it.nA; r[IT_BVALID] = it.b_valid;
-          r[IT_H] = it.H;
+          r[IT_H] = it.H; r[IT_PART] = it.part;
           r[IT_BASE_LO] = (int)(uint32_t)(it.base & 0xffffffffll); r[IT_BASE_HI] = (int)(uint32_t)((uint64_t)it.base >> 32);
         }
         mbar_arrive(bar(B_IFULL + sl));
@@ -778,7 +799,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
       // ---- hand the finished tile to the epilogue warps (they wait for its last P V themselves) ----
       if (active) {
         if (done_n > 0) mbar_wait(bar(B_ODRAIN + x), (done_n - 1u) & 1u, abort_flag, p.status);   // 1 / l of the item before was read
-        reinterpret_cast<float*>(sm_gen + SM_INVL)[x * 128 + row] = 1.f / l_sum;
+        reinterpret_cast<float*>(sm_gen + SM_INVL)[x * 128 + row] = it.part < 0 ? 1.f / l_sum : 1.f;
+        if (it.part >= 0) p.part_ml[(it.part * 2 + x) * 128 + row] = make_float2(m_ref * c2, l_sum);
         mbar_arrive(bar(B_LREADY + x));
         ++done_n;
       }
@@ -796,6 +818,58 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
   if (warp == 9) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+  }
+}
+
+// Merges the parts of the items that a split launch cut: block (c - 1, q) looks at cut c and, if it is
+// the first one inside its item, combines rows 64 q .. + 63 of the item's 256, a warp eight of them with
+// the first two parts' loads all in flight, a lane four columns.  The parts are in slot 2a + 1 of the CTA
+// a before the cut and slots 2j of those after it.  Bound by what an SM can read from L2: a whole item
+// (256-512 KB) to a block took 16 us where this takes 8; merging inside the attention launch, by the
+// last CTA of an item to end, 37 us.
+constexpr int MERGE_THREADS = 256, MERGE_BATCH = 8, MERGE_SPLIT = 4;
+static_assert(MERGE_SPLIT * MERGE_BATCH * MERGE_THREADS / 32 == 256, "rows of a tile pair");
+template <typename TO>
+__global__ void __launch_bounds__(MERGE_THREADS) attn_merge_kernel(const __grid_constant__ TcParams p) {
+  rc_grid_wait();
+  rc_grid_launch_next();
+  const int c = blockIdx.x + 1;
+  const int n = p.header[3];
+  const int4 m = p.merge[c];                             // (c < grid: there, if not written, in any case)
+  if (c >= n || m.x == 0) return;
+  const int last = c + m.x - 2, rows = m.z, lane = threadIdx.x & 31;
+  const int r0 = (256 / MERGE_SPLIT) * blockIdx.y + MERGE_BATCH * (threadIdx.x >> 5);
+  if (r0 < rows) {
+    float2 ml[2][MERGE_BATCH];
+    float4 v[2][MERGE_BATCH];
+    auto load = [&](int h, int j) {
+      const int64_t at = (int64_t)(j == c - 1 ? 2 * j + 1 : 2 * j) * 256 + r0;
+#pragma unroll
+      for (int k = 0; k < MERGE_BATCH; ++k) {
+        ml[h][k] = p.part_ml[at + k];
+        v[h][k] = *(reinterpret_cast<const float4*>(p.part_o + (at + k) * D) + lane);
+      }
+    };
+    auto add = [&]() {                                   // part 1 into part 0
+#pragma unroll
+      for (int k = 0; k < MERGE_BATCH; ++k) {
+        const float m = fmaxf(ml[0][k].x, ml[1][k].x), f0 = ex2(ml[0][k].x - m), f1 = ex2(ml[1][k].x - m);
+        ml[0][k] = make_float2(m, ml[0][k].y * f0 + ml[1][k].y * f1);
+        v[0][k].x = v[0][k].x * f0 + v[1][k].x * f1; v[0][k].y = v[0][k].y * f0 + v[1][k].y * f1;
+        v[0][k].z = v[0][k].z * f0 + v[1][k].z * f1; v[0][k].w = v[0][k].w * f0 + v[1][k].w * f1;
+      }
+    };
+    load(0, c - 1);
+    for (int j = c; j <= last; ++j) { load(1, j); add(); }
+#pragma unroll
+    for (int k = 0; k < MERGE_BATCH; ++k) {
+      const int r = r0 + k;                              // row of the pair: 128 rows are TQ tokens of s heads
+      if (r >= rows) break;
+      const float inv = 1.f / ml[0][k].y;
+      TO* o = reinterpret_cast<TO*>(p.out) + ((int64_t)(m.y + r / p.s) * p.Hq + m.w * p.s + r % p.s) * D + 4 * lane;
+      if constexpr (sizeof(TO) == 4) *reinterpret_cast<float4*>(o) = make_float4(v[0][k].x * inv, v[0][k].y * inv, v[0][k].z * inv, v[0][k].w * inv);
+      else *reinterpret_cast<uint2*>(o) = make_uint2(pack2(v[0][k].x * inv, v[0][k].y * inv), pack2(v[0][k].z * inv, v[0][k].w * inv));
+    }
   }
 }
 
@@ -860,8 +934,21 @@ static int tc_levels(const recache_ctx* ctx, int max_len) {
   return (max_len + t - 1) / t + 1;
 }
 
-int64_t rc_tc_workspace_bytes(const recache_ctx* ctx, int n_seq, int total, int max_len) {
-  return 256 + align256(tc_max_items(ctx, n_seq, total) * 8) + align256(2 * RC_SORT_MAX * 4);
+// A prefill of at most four rounds of CTAs may be split (see rc_plan_split); what that takes of the
+// workspace: cuts, unit prefix, and two partial results per CTA.
+static int tc_ctas(const recache_ctx* ctx) { return ctx->sm_count > 0 ? ctx->sm_count : 148; }
+static bool tc_may_split(const recache_ctx* ctx, int64_t max_items) {
+  const int64_t n = max_items * ctx->desc.n_kv_heads;
+  return n <= 4 * tc_ctas(ctx) && n <= RC_SORT_MAX;
+}
+constexpr int64_t PART_ROWS = 2 * 2 * 128;   // per CTA: two slots of two tiles
+
+int64_t rc_tc_workspace_bytes(const recache_ctx* ctx, int n_seq, int total, int max_len, bool prefill) {
+  const int64_t max_items = tc_max_items(ctx, n_seq, total), n = tc_ctas(ctx);
+  int64_t bytes = 256 + align256(max_items * 8) + align256(2 * RC_SORT_MAX * 4);
+  if (prefill && tc_may_split(ctx, max_items))
+    bytes += align256((n + 1) * 8) + align256((n + 1) * 16) + align256(RC_SORT_MAX * 4) + align256(n * PART_ROWS * 8) + n * PART_ROWS * D * 4;
+  return bytes;
 }
 
 cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope, const TcAttnArgs& a, cudaStream_t st) {
@@ -884,6 +971,18 @@ cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope,
 
   TcParams p;
   p.header = (int32_t*)ws; p.items = (int2*)(ws + 256); p.order = (int32_t*)(ws + 256 + align256(max_items * 8));
+  const bool may_split = a.route_cu != nullptr && tc_may_split(ctx, max_items) && tc_ctas(ctx) > 1;
+  const int sms = tc_ctas(ctx);
+  const unsigned grid = (unsigned)(may_split || max_items * G > sms ? sms : max_items * G);
+  p.start = nullptr; p.merge = nullptr; p.unit_cu = nullptr; p.part_o = nullptr; p.part_ml = nullptr; p.n_cta = (int)grid;
+  if (may_split) {
+    uint8_t* at = ws + 256 + align256(max_items * 8) + align256(2 * RC_SORT_MAX * 4);
+    p.start = (int2*)at; at += align256((int64_t)(sms + 1) * 8);
+    p.merge = (int4*)at; at += align256((int64_t)(sms + 1) * 16);
+    p.unit_cu = (int32_t*)at; at += align256(RC_SORT_MAX * 4);
+    p.part_ml = (float2*)at; at += align256(sms * PART_ROWS * 8);
+    p.part_o = (float*)at;
+  }
   p.cu = a.cu; p.pos0 = a.pos0; p.slot = a.slot; p.route_cu = a.route_cu; p.hist = a.hist;
   p.n_seq = a.n_seq; p.G = G; p.Hq = Hq; p.s = s; p.self_rows = a.self_rows; p.route_rows = a.route_rows;
   p.prefix_len = a.route_cu ? 0 : a.prefix_len;
@@ -895,17 +994,22 @@ cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope,
   const bool gather = a.route_idx != nullptr;
   p.gather_k = (const uint8_t*)a.k_cache; p.gather_v = (const uint8_t*)a.v_cache; p.route_idx = a.route_idx;
   p.pool_tokens = a.pool_tokens;
-  const cudaError_t e = rc_launch_rope_store(ctx, rope, &p, st);   // builds the work list on the side
+  cudaError_t e = rc_launch_rope_store(ctx, rope, &p, st);   // builds the work list on the side
   if (e != cudaSuccess) return e;
-  const int sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
-  const unsigned grid = (unsigned)(max_items * G < sms ? max_items * G : sms);
-  RcLaunchScope scope(ctx, a.route_cu ? RC_K_PREFILL_ATTN : RC_K_ENCODE_ATTN, st);
-  auto launch = [&](auto kernel) { return rc_launch_overlapped(kernel, grid, NTHREADS, SM_ALLOC, st, tq, tks, tvs, tkr, tvr, p); };
   const bool f32 = a.out_dtype == RECACHE_F32, rot = s >= 4;   // 2 * 128 / s <= 64 positions fit the staging area
-  if (gather) {
-    if (f32) return rot ? launch(attn_tc_kernel<float, true, true>) : launch(attn_tc_kernel<float, false, true>);
-    return rot ? launch(attn_tc_kernel<__nv_bfloat16, true, true>) : launch(attn_tc_kernel<__nv_bfloat16, false, true>);
+  {
+    RcLaunchScope scope(ctx, a.route_cu ? RC_K_PREFILL_ATTN : RC_K_ENCODE_ATTN, st);
+    auto launch = [&](auto kernel) { return rc_launch_overlapped(kernel, grid, NTHREADS, SM_ALLOC, st, tq, tks, tvs, tkr, tvr, p); };
+    if (gather) {
+      if (f32) e = rot ? launch(attn_tc_kernel<float, true, true>) : launch(attn_tc_kernel<float, false, true>);
+      else e = rot ? launch(attn_tc_kernel<__nv_bfloat16, true, true>) : launch(attn_tc_kernel<__nv_bfloat16, false, true>);
+    } else {
+      if (f32) e = rot ? launch(attn_tc_kernel<float, true, false>) : launch(attn_tc_kernel<float, false, false>);
+      else e = rot ? launch(attn_tc_kernel<__nv_bfloat16, true, false>) : launch(attn_tc_kernel<__nv_bfloat16, false, false>);
+    }
   }
-  if (f32) return rot ? launch(attn_tc_kernel<float, true, false>) : launch(attn_tc_kernel<float, false, false>);
-  return rot ? launch(attn_tc_kernel<__nv_bfloat16, true, false>) : launch(attn_tc_kernel<__nv_bfloat16, false, false>);
+  if (e != cudaSuccess || !may_split) return e;
+  RcLaunchScope scope(ctx, RC_K_PREFILL_MERGE, st);
+  return f32 ? rc_launch_overlapped(attn_merge_kernel<float>, dim3(grid - 1, MERGE_SPLIT), MERGE_THREADS, 0, st, p)
+             : rc_launch_overlapped(attn_merge_kernel<__nv_bfloat16>, dim3(grid - 1, MERGE_SPLIT), MERGE_THREADS, 0, st, p);
 }

@@ -13,7 +13,7 @@
 enum RcKernel {
   RC_K_ROPE_STORE = 0, RC_K_TILE_PLAN, RC_K_ENCODE_ATTN, RC_K_PREFILL_ATTN,
   RC_K_COMPACT_COUNT, RC_K_COMPACT_PLAN, RC_K_COMPACT_GATHER,
-  RC_K_DECODE_APPEND, RC_K_DECODE_ATTN, RC_K_DECODE_MERGE, RC_K_COUNT
+  RC_K_DECODE_APPEND, RC_K_DECODE_ATTN, RC_K_DECODE_MERGE, RC_K_PREFILL_MERGE, RC_K_COUNT
 };
 
 struct RcTimedLaunch { int id; cudaEvent_t start, stop; };
@@ -63,7 +63,6 @@ __device__ __forceinline__ void rc_grid_launch_next() { asm volatile("griddepcon
 
 template <typename... P, typename... A>
 inline cudaError_t rc_launch(bool overlapped, void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A&&... args) {
-  // (the opt-in to more than 48 KB of shared memory is per kernel and device: a few hundred nanoseconds)
   if (smem > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -266,7 +265,7 @@ struct TcAttnArgs {
   const void* k_cache = nullptr; const void* v_cache = nullptr; int64_t pool_tokens = 0; const int32_t* route_idx = nullptr;
 };
 bool rc_tc_supported(const recache_ctx* ctx);
-int64_t rc_tc_workspace_bytes(const recache_ctx* ctx, int n_seq, int total, int max_len);
+int64_t rc_tc_workspace_bytes(const recache_ctx* ctx, int n_seq, int total, int max_len, bool prefill);
 cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope, const TcAttnArgs& a, cudaStream_t st);
 
 // ---- self-test of the bounded barrier wait (report: 2 ints on the device) ----

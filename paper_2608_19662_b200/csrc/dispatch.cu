@@ -6,10 +6,10 @@
 #include "common.cuh"
 
 int64_t rc_encode_workspace_bytes(const recache_ctx* ctx, int n_res, int total, int max_len) {
-  return rc_tc_supported(ctx) ? rc_tc_workspace_bytes(ctx, n_res, total, max_len) : 0;
+  return rc_tc_supported(ctx) ? rc_tc_workspace_bytes(ctx, n_res, total, max_len, false) : 0;
 }
 int64_t rc_prefill_workspace_bytes(const recache_ctx* ctx, int n_req, int total_q, int max_q) {
-  return rc_tc_supported(ctx) ? rc_tc_workspace_bytes(ctx, n_req, total_q, max_q) : 0;
+  return rc_tc_supported(ctx) ? rc_tc_workspace_bytes(ctx, n_req, total_q, max_q, true) : 0;
 }
 int64_t rc_decode_workspace_bytes(const recache_ctx* ctx, int batch, int max_res_pages, int max_hist_pages) {
   return rc_decode_split_supported(ctx) ? rc_decode_split_workspace_bytes(ctx, batch, max_res_pages, max_hist_pages) : 0;

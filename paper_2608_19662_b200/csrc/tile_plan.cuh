@@ -7,11 +7,17 @@
 
 constexpr int RC_TILE_N = 128;       // keys of a K/V tile
 constexpr int RC_SORT_MAX = 4096;    // work items up to which the plan sorts a prefill by weight (encode: a quarter)
+constexpr int RC_ITEM_UNITS = 2;     // what beginning an item costs, in K/V tiles
 constexpr int RC_PLAN_BINS = 1024;   // weights (K/V tiles, tile pairs) are told apart up to this
 
 struct RcPlan {
-  int2* items; int32_t* header;   // header[0] = number of items, header[1] = work counter, header[2] = order[] is valid
-  int32_t* order;                 // work indices, heaviest first (launches of at most RC_SORT_MAX work items); bins behind them
+  int2* items; int32_t* header;   // header[0] = number of items, header[1] = work counter, header[2] = order[] is valid, header[3] = CTAs of a split launch
+  int32_t* order;                 // work indices, heaviest first (launches of at most RC_SORT_MAX work items); K/V tiles of each behind them
+  // Split launch (null: not possible): CTA c takes the K/V tiles from start[c] = (work index, tile) up to start[c + 1].
+  // merge[c]: what the merge does at cut c: parts of the item it is the first cut of (0: nothing to do), first token of the
+  // item's rows, rows (tokens x heads), group.
+  int2* start; int4* merge; int32_t* unit_cu;
+  int n_cta;                      // CTAs of the attention launch
   const int32_t* cu; const int32_t* pos0; const int32_t* slot; const int32_t* route_cu; const int32_t* hist;
   int n_seq, G, Hq, s;
   int prefix_len;   // > 0: every sequence sees rows g*prefix_len .. of the "route" tensors (shared prefix)
@@ -27,6 +33,7 @@ struct RcItem {
   int g, seq0, L, tok0, kv_end, pos0, rA0, lenA, nA, b_valid;
   int H;            // rows that precede the sequence's own tokens in the self part (earlier turns), all visible
   int64_t base;
+  int part;         // slot of this CTA's part of a split item, -1: the whole item
 };
 
 // Work index w -> item; false when the caller's index arrays are inconsistent
@@ -59,7 +66,7 @@ __device__ __forceinline__ bool rc_load_item(const RcPlan& p, int w, RcItem& it)
   return ok;
 }
 
-struct RcPlanSmem { int hist[RC_PLAN_BINS + 1]; int warp_sum[33]; };
+struct RcPlanSmem { int hist[RC_PLAN_BINS + 1]; int warp_sum[33]; int most; };
 
 // Exclusive block scan of one int per thread; *total gets the sum (same pattern of calls in every thread).
 __device__ __forceinline__ int rc_plan_scan(int v, RcPlanSmem& sh, int* total) {
@@ -87,6 +94,65 @@ __device__ __forceinline__ void rc_plan_scan_bins(RcPlanSmem& sh) {
   int at = rc_plan_scan(sum, sh, &total);
   for (int i = i0; i < i1; ++i) { const int c = sh.hist[i]; sh.hist[i] = at; at += c; }
   __syncthreads();
+}
+
+// A prefill whose items do not fill the CTAs evenly: their K/V tiles, laid end to end, are cut into
+// n equal ranges, so that an item may be shared by several CTAs (their partial results are merged
+// afterwards).  An item counts RC_ITEM_UNITS more than its tiles, and a cut is moved to the item's
+// edge where it would leave a part of fewer than two tiles, or a part whose first tile some row of
+// the pair does not see.  Taken only where the longest CTA gets shorter by more than the second
+// beginning (two units) and the merge (three: 5-8 us) cost: 8 conversations with 300-2048 rows of history
+// (88 items of 8-24 tiles) take 50 us instead of 57; one request of 2048 tokens over a long tool set (256
+// items of 58-73 tiles, else two rounds of 148 CTAs) 281 instead of 291.  Encoding is never split: a
+// resource's result must not depend on what is encoded beside it.  False: not worth it.
+__device__ __forceinline__ bool rc_plan_split(const RcPlan& p, RcPlanSmem& sh, int n_work) {
+  const int tid = threadIdx.x, n_thr = blockDim.x;
+  const int32_t* tiles = p.order + RC_SORT_MAX;
+  const int per = (n_work + n_thr - 1) / n_thr;
+  const int w0 = min(n_work, tid * per), w1 = min(n_work, w0 + per);
+  int units = 0, items = 0, total_units, n_items;
+  for (int w = w0; w < w1; ++w)
+    if (tiles[w] > 0) { units += tiles[w] + RC_ITEM_UNITS; ++items; }
+  rc_plan_scan(items, sh, &n_items);
+  int at = rc_plan_scan(units, sh, &total_units);
+  if (n_items == 0) return false;
+  const int n = min(p.n_cta, max(1, (total_units - RC_ITEM_UNITS * n_items) / 4));
+  const float split = (float)total_units / n + RC_ITEM_UNITS + 3;
+  const float whole = fmaxf((float)(sh.most + RC_ITEM_UNITS), (float)total_units / n_items * ((n_items + p.n_cta - 1) / p.n_cta));
+  if (split > 0.95f * whole) return false;
+  for (int w = w0; w < w1; ++w) { p.unit_cu[w] = at; if (tiles[w] > 0) at += tiles[w] + RC_ITEM_UNITS; }
+  __syncthreads();
+  for (int c = tid; c <= n; c += n_thr) {
+    int2 cut = make_int2(n_work, 0);
+    if (c < n) {
+      const int x = (int)((int64_t)total_units * c / n);
+      int lo = 0, hi = n_work;                       // the last item that starts at or before x (an empty one starts where the next does)
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (p.unit_cu[mid] <= x) lo = mid; else hi = mid;
+      }
+      cut = make_int2(lo, x - p.unit_cu[lo] - RC_ITEM_UNITS);
+      RcItem it;
+      rc_load_item(p, lo, it);
+      if (cut.y < 2) cut.y = 0;
+      else if (it.n_tiles - cut.y < 2 || cut.y > it.nA + (it.H + it.tok0) / RC_TILE_N) cut = make_int2(lo + 1, 0);
+    }
+    p.start[c] = cut;
+  }
+  __syncthreads();
+  for (int c = tid; c < n; c += n_thr) {
+    int4 m = make_int4(0, 0, 0, 0);
+    const int2 cut = p.start[c];
+    if (c > 0 && cut.y > 0 && (p.start[c - 1].x != cut.x || p.start[c - 1].y == 0)) {
+      RcItem it;
+      rc_load_item(p, cut.x, it);
+      m = make_int4(2, it.seq0 + it.tok0, min(256, (it.L - it.tok0) * p.s), it.g);
+      for (int j = c + 1; p.start[j].x == cut.x && p.start[j].y > 0; ++j) ++m.x;
+    }
+    p.merge[c] = m;
+  }
+  if (tid == 0) p.header[3] = n;
+  return true;
 }
 
 // Items = (sequence, tile-pair index): sequence by sequence, the longest sequences
@@ -119,7 +185,7 @@ __device__ __forceinline__ void rc_build_plan(const RcPlan& p, RcPlanSmem& sh) {
   // (an encode launch shares K/V between the items of a sequence only: beyond a thousand items the
   // sequence-major order, which keeps a sequence's K/V in L2, is worth more than the balance)
   const bool sorted = n_work <= (p.route_cu ? RC_SORT_MAX : RC_SORT_MAX / 4);
-  if (tid == 0) { p.header[0] = n_items; p.header[1] = 0; p.header[2] = sorted ? 1 : 0; }
+  if (tid == 0) { p.header[0] = n_items; p.header[1] = 0; p.header[2] = sorted ? 1 : 0; p.header[3] = 0; }
   if (!sorted) {
     // counting sort of the sequences by their number of tile pairs, longest first: hist[bin] = items of
     // that bin, then the first item index of the bin
@@ -140,15 +206,18 @@ __device__ __forceinline__ void rc_build_plan(const RcPlan& p, RcPlanSmem& sh) {
   if (!sorted) return;
   // Few work items (a prefill of a handful of requests): one CTA gets one or two of them, so their
   // order decides the tail.  Sort them by weight (K/V tiles), heaviest first, with a counting sort.
+  if (tid == 0) sh.most = 0;
   __syncthreads();
+  int32_t* tiles = p.order + RC_SORT_MAX;
   for (int w = tid; w < n_work; w += n_thr) {
     RcItem it;
-    const bool ok = rc_load_item(p, w, it);
-    const int bin = RC_PLAN_BINS - (ok ? min(it.n_tiles, RC_PLAN_BINS) : 0);
-    p.order[RC_SORT_MAX + w] = bin;
-    atomicAdd(&sh.hist[bin], 1);
+    const int n = rc_load_item(p, w, it) ? it.n_tiles : 0;
+    tiles[w] = n;
+    atomicAdd(&sh.hist[RC_PLAN_BINS - min(n, RC_PLAN_BINS)], 1);
+    if (p.start) atomicMax(&sh.most, n);
   }
   __syncthreads();
+  if (p.start && rc_plan_split(p, sh, n_work)) return;
   rc_plan_scan_bins(sh);
-  for (int w = tid; w < n_work; w += n_thr) p.order[atomicAdd(&sh.hist[p.order[RC_SORT_MAX + w]], 1)] = w;
+  for (int w = tid; w < n_work; w += n_thr) p.order[atomicAdd(&sh.hist[RC_PLAN_BINS - min(tiles[w], RC_PLAN_BINS)], 1)] = w;
 }

@@ -1,0 +1,54 @@
+"""Prefill launches whose items are cut across CTAs: few long items, items that end at a cut, parts that
+begin in the route, the history or the causal range, and launches on both sides of the decision."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import recache_oracle as orc
+from paper_2608_19662_b200 import workloads as wl
+
+from pipeline import dev, f64, make_ctx, max_abs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("hq,g,lens,hist,route,out", [
+    (8, 2, [5], [3000], [(0, 0)], torch.float32),                    # two items over all CTAs, no route
+    (4, 1, [70, 1], [1900, 640], [(2500, 2500), (129, 129)], torch.bfloat16),   # parts inside the route
+    (8, 1, [33, 40], [1281, 0], [(0, 700), (4000, 4000)], torch.float32),       # eight heads; an item of route tiles only
+    (16, 8, [250, 17, 129], [300, 2048, 1000], [(500, 900)] * 3, torch.float32),   # two heads: pairs of 128 tokens
+    (8, 2, [130, 64, 65, 3], [127, 128, 129, 0], [(0, 300)] * 4, torch.float32),   # short: below the decision
+    (32, 8, [1100], [0], [(1500, 2600)], torch.bfloat16),            # more items than CTAs, two rounds
+])
+def test_split_items_match_oracle(hq, g, lens, hist, route, out):
+    sh = wl.Shape(hq, g, 128, 1e6, "bf16")
+    rng = np.random.default_rng([hq, g, len(lens)])
+    B, d = len(lens), 128
+    lens, hist = np.asarray(lens), np.asarray(hist)
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    n_route = np.concatenate([rng.integers(a, b + 1, g) for a, b in route])
+    r_cu = np.concatenate([[0], np.cumsum(n_route)]).astype(np.int32)
+    room = (hist + lens + 63) // 64 * 64
+    slot = np.concatenate([[0], np.cumsum(room)])
+    rows = int(slot[-1])
+    N = lambda i, *s: wl.normal(1000 + i, s, sh.torch_dtype)
+    q, k, v = N(0, int(cu[-1]), hq, d), N(1, int(cu[-1]), g, d), N(2, int(cu[-1]), g, d)
+    kr, vr, kc, vc = N(3, int(r_cu[-1]) + 1, d), N(4, int(r_cu[-1]) + 1, d), N(5, g, rows, d), N(6, g, rows, d)
+    pos0 = (hist + 100).astype(np.int32)
+    rc = make_ctx(sh, max_pos=8192)
+    d_kc, d_vc = dev(kc), dev(vc)
+    args = (dev(q), dev(k), dev(v), dev(cu), dev(pos0), int(lens.max()), dev(kr), dev(vr), dev(r_cu))
+    tail = (dev(slot[:-1].astype(np.int32)), dev(hist.astype(np.int32)))
+    o = rc.attend_prefill_history(*args, d_kc, d_vc, *tail, out_dtype=out)
+    again = rc.attend_prefill_history(*args, d_kc, d_vc, *tail, out_dtype=out)
+    assert torch.equal(o, again)                                     # the cuts and the merge have a fixed order
+    # oracle: route rows by a list of indices into a pool that holds exactly them
+    pool_k, pool_v = np.zeros((g, int(r_cu[-1]) + 1, d)), np.zeros((g, int(r_cu[-1]) + 1, d))
+    pool_k[:], pool_v[:] = f64(kr)[None], f64(vr)[None]
+    lists = [[np.arange(r_cu[b * g + kg], r_cu[b * g + kg + 1]) for kg in range(g)] for b in range(B)]
+    hk = [f64(kc)[:, slot[b]:slot[b] + hist[b]] for b in range(B)]
+    hv = [f64(vc)[:, slot[b]:slot[b] + hist[b]] for b in range(B)]
+    ref, _ = orc.attend_prefill(f64(q), f64(k), f64(v), cu, pos0, lists, pool_k, pool_v, sh.rope_theta, storage=sh.dtype, hist_k=hk, hist_v=hv)
+    tol = 1e-2 + (2.0 ** -8 * np.abs(ref) if out == torch.bfloat16 else 0)   # bf16 results: half an ulp on top
+    assert (np.abs(f64(o) - ref) <= tol).all()
+    assert rc.poll_status() == 0
