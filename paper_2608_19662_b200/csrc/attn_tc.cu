@@ -44,7 +44,10 @@ constexpr int NSTAGE = 2;
 constexpr int BOX_BYTES = 16384;   // [128 rows][64 bf16], 128-byte swizzle
 constexpr int TILE_BYTES = 32768;  // two boxes: head_dim halves
 constexpr int NTHREADS = 512;
-constexpr int REGS_SOFTMAX = 216, REGS_AUX = 40, REGS_EPI = 40;   // 256*216 + 128*(40 + 40) = 65536
+// Registers per thread of the softmax warps and of the other eight; 256 * (softmax + aux) = 65536.  The
+// prefill's scheduler and epilogue, which know about split items, spill in 32; the encode pays 1 % for 40.
+template <bool PREFILL> constexpr int REGS_SOFTMAX = PREFILL ? 216 : 224;
+template <bool PREFILL> constexpr int REGS_AUX = PREFILL ? 40 : 32;
 
 constexpr int SM_Q = 0;                              // 2 query tiles
 constexpr int SM_K = SM_Q + 2 * TILE_BYTES;          // NSTAGE key tiles
@@ -240,7 +243,7 @@ enum { IT_NTILES = 0, IT_G, IT_SEQ0, IT_L, IT_TOK0, IT_KVEND, IT_POS0, IT_RA0, I
 // items through a two-slot ring in shared memory.
 // The next item's Q load, Q rotation and first K/V tiles overlap the current
 // item's last tiles and its epilogue.  Barrier phases run on across items.
-template <typename TO, bool ROT_SMEM, bool GATHER>
+template <typename TO, bool ROT_SMEM, bool GATHER, bool PREFILL>
 __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
                                                               const __grid_constant__ CUtensorMap tm_ks,
                                                               const __grid_constant__ CUtensorMap tm_vs,
@@ -300,14 +303,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
     const int* r = const_cast<const int*>(item_ring) + sl * IT_WORDS;   // (ordered by the barrier wait above and the arrive below)
     it.n_tiles = r[IT_NTILES]; it.g = r[IT_G]; it.seq0 = r[IT_SEQ0]; it.L = r[IT_L]; it.tok0 = r[IT_TOK0];
     it.kv_end = r[IT_KVEND]; it.pos0 = r[IT_POS0]; it.rA0 = r[IT_RA0]; it.lenA = r[IT_LENA]; it.nA = r[IT_NA];
-    it.b_valid = r[IT_BVALID]; it.H = r[IT_H]; it.part = r[IT_PART];
+    it.b_valid = r[IT_BVALID]; it.H = r[IT_H]; it.part = PREFILL ? r[IT_PART] : -1;
     it.base = (int64_t)(((uint64_t)(uint32_t)r[IT_BASE_HI] << 32) | (uint32_t)r[IT_BASE_LO]);
     if (*abort_flag) it.n_tiles = -1;
     if (release) mbar_arrive(bar(B_IEMPTY + sl));
   };
 
   if (warp >= 12) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_EPI));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_AUX<PREFILL>));
     // ===================== epilogue warps =====================
     // O of a finished query tile leaves tensor memory here, so that the softmax warps can go
     // straight to the next item's Q.  Warp 12 + q reads lanes 32 q .. 32 q + 31.
@@ -425,13 +428,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
       it = nx;
     }
   } else if (warp >= 8) {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_AUX));
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_AUX<PREFILL>));
   if (warp == 10) {
     // ===================== scheduler =====================
     if (lane == 0) {
       const int total = p.header[0] * p.G;   // (a CTA without work publishes "no more work" at once)
       bool first = true;
-      const int n_split = p.start ? p.header[3] : 0;
+      const int n_split = PREFILL && p.start ? p.header[3] : 0;
       int2 cur = make_int2(0, 0), end = make_int2(0, 0);
       if ((int)blockIdx.x < n_split) { cur = p.start[blockIdx.x]; end = p.start[blockIdx.x + 1]; }
       for (uint32_t n = 0;; ++n) {
@@ -643,7 +646,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
     }
   }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX<PREFILL>));
     // ===================== softmax warpgroups =====================
     const int x = warp >> 2;                       // tile A or B
     const int row = threadIdx.x & 127;             // row of the tile = TMEM lane
@@ -941,6 +944,16 @@ static bool tc_may_split(const recache_ctx* ctx, int64_t max_items) {
   const int64_t n = max_items * ctx->desc.n_kv_heads;
   return n <= 4 * tc_ctas(ctx) && n <= RC_SORT_MAX;
 }
+// Whether a launch is made splittable: the merge launch behind it costs 2 us even when the device decides
+// against splitting.  The host knows bounds only (capacities, of which a third is kept as a rule), so it asks
+// for so many tiles of capacity per item that the real ones can be worth cutting: a turn of one request (16
+// tiles of capacity, 5 kept) takes 36 us without the merge launch and 38 with it, 8 zero-copy turns
+// (40 and 12, two rounds of CTAs) 85 and 88.  A conversation cache holds about what it has room for.
+static bool tc_worth_splitting(const recache_ctx* ctx, const TcAttnArgs& a, int64_t max_items) {
+  const int64_t rows = a.route_rows / ((int64_t)a.n_seq * ctx->desc.n_kv_heads) + (a.hist ? a.self_rows / a.n_seq : a.max_len);
+  const int64_t tiles = a.hist ? 8 : max_items * ctx->desc.n_kv_heads <= tc_ctas(ctx) ? 32 : 64;
+  return rows >= tiles * TILE_N;
+}
 constexpr int64_t PART_ROWS = 2 * 2 * 128;   // per CTA: two slots of two tiles
 
 int64_t rc_tc_workspace_bytes(const recache_ctx* ctx, int n_seq, int total, int max_len, bool prefill) {
@@ -971,7 +984,7 @@ cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope,
 
   TcParams p;
   p.header = (int32_t*)ws; p.items = (int2*)(ws + 256); p.order = (int32_t*)(ws + 256 + align256(max_items * 8));
-  const bool may_split = a.route_cu != nullptr && tc_may_split(ctx, max_items) && tc_ctas(ctx) > 1;
+  const bool may_split = a.route_cu != nullptr && tc_may_split(ctx, max_items) && tc_ctas(ctx) > 1 && tc_worth_splitting(ctx, a, max_items);
   const int sms = tc_ctas(ctx);
   const unsigned grid = (unsigned)(may_split || max_items * G > sms ? sms : max_items * G);
   p.start = nullptr; p.merge = nullptr; p.unit_cu = nullptr; p.part_o = nullptr; p.part_ml = nullptr; p.n_cta = (int)grid;
@@ -1000,13 +1013,13 @@ cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope,
   {
     RcLaunchScope scope(ctx, a.route_cu ? RC_K_PREFILL_ATTN : RC_K_ENCODE_ATTN, st);
     auto launch = [&](auto kernel) { return rc_launch_overlapped(kernel, grid, NTHREADS, SM_ALLOC, st, tq, tks, tvs, tkr, tvr, p); };
-    if (gather) {
-      if (f32) e = rot ? launch(attn_tc_kernel<float, true, true>) : launch(attn_tc_kernel<float, false, true>);
-      else e = rot ? launch(attn_tc_kernel<__nv_bfloat16, true, true>) : launch(attn_tc_kernel<__nv_bfloat16, false, true>);
-    } else {
-      if (f32) e = rot ? launch(attn_tc_kernel<float, true, false>) : launch(attn_tc_kernel<float, false, false>);
-      else e = rot ? launch(attn_tc_kernel<__nv_bfloat16, true, false>) : launch(attn_tc_kernel<__nv_bfloat16, false, false>);
-    }
+    auto pick = [&](auto type) {
+      using TO = decltype(type);
+      if (gather) return rot ? launch(attn_tc_kernel<TO, true, true, true>) : launch(attn_tc_kernel<TO, false, true, true>);
+      if (a.route_cu) return rot ? launch(attn_tc_kernel<TO, true, false, true>) : launch(attn_tc_kernel<TO, false, false, true>);
+      return rot ? launch(attn_tc_kernel<TO, true, false, false>) : launch(attn_tc_kernel<TO, false, false, false>);
+    };
+    e = f32 ? pick(float()) : pick(__nv_bfloat16());
   }
   if (e != cudaSuccess || !may_split) return e;
   RcLaunchScope scope(ctx, RC_K_PREFILL_MERGE, st);
