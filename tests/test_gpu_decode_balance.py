@@ -63,3 +63,38 @@ def test_ragged_pages_match_oracle_and_append(hq, groups, batch, res, hist):
     assert changed == items
     assert max_abs(d_kp, kr) < 4e-2          # 1 bf16 ulp of a key in [4, 8): 3.1e-2
     assert rc.poll_status() == 0
+
+
+@pytest.mark.parametrize("hq,groups,batch,res,hist", [
+    (32, 8, 1, (500, 900), (2000, 2000)),     # one sequence: CTAs of its own for every item
+    (8, 1, 1, (0, 0), (64 * 200, 64 * 200)),  # more pages than CTAs in one item
+    (8, 2, 1, (1, 70), (1, 1)),               # fewer pages than an item has CTAs
+    (16, 8, 4, (100, 400), (64, 3000)),       # few items of very different length
+    (16, 8, 16, (0, 900), (1, 2000)),         # gathered and paged pages mixed in a CTA's range
+])
+def test_gathered_rows_match_paged(hq, groups, batch, res, hist):
+    """The zero-copy decode over the rows of a pool equals the paged one over the same rows in pages,
+    up to the order of summation (the two deal their pages out differently)."""
+    sh = wl.Shape(hq, groups, 128, 1e6, "bf16")
+    rng = np.random.default_rng([hq, batch, res[1], 7])
+    items = batch * groups
+    res_rows = rng.integers(res[0], res[1] + 1, items).astype(np.int32)
+    hist_rows = np.repeat(rng.integers(hist[0], hist[1] + 1, batch), groups).astype(np.int32)
+    kp, vp, rt, ht = _batch(rng, sh, res_rows, hist_rows)
+    pool = max(1, int(res_rows.max()) * 3)
+    kc, vc = wl.normal(11, (groups, pool, 128), sh.torch_dtype), wl.normal(12, (groups, pool, 128), sh.torch_dtype)
+    cu = np.concatenate([[0], np.cumsum(res_rows)]).astype(np.int32)
+    idx = np.concatenate([rng.permutation(pool)[:n] for n in res_rows] + [np.zeros(1, np.int64)]).astype(np.int32)
+    for it in range(items):                   # the same rows, in the item's pages
+        for n in range(int(res_rows[it])):
+            page, r = rt[it, n // PT], n % PT
+            kp[page, r], vp[page, r] = kc[it % groups, idx[cu[it] + n]], vc[it % groups, idx[cu[it] + n]]
+    rc = make_ctx(sh, max_pos=16384)
+    q = wl.normal(900, (batch, hq, 128), sh.torch_dtype)
+    q_pos = (np.arange(batch) * 7 + 3).astype(np.int32)
+    paged = rc.attend_decode(dev(q), dev(q_pos), dev(kp), dev(vp), dev(rt), dev(res_rows), dev(ht), dev(hist_rows), out_dtype=torch.float32)
+    gathered = rc.attend_decode_gather(dev(q), dev(q_pos), dev(kc), dev(vc), dev(idx), dev(cu), rt.shape[1], dev(kp), dev(vp), dev(ht),
+                                       dev(hist_rows), out_dtype=torch.float32)
+    ref = orc.attend_decode(f64(q), q_pos, f64(kp), f64(vp), rt, res_rows, ht, hist_rows, sh.rope_theta, PT, storage=sh.dtype)
+    assert max_abs(paged, ref) < 1e-2 and max_abs(gathered, ref) < 1e-2
+    assert rc.poll_status() == 0
