@@ -15,8 +15,9 @@
 // is a block's start (a chain of dependent loads) and half FMA issue.  A warp per
 // query row, which read every key row once per query row, took 69 us each for 1,250
 // tokens in six resources and for the 160-token turn over them (4 / 2 heads of 64);
-// this kernel takes 24 and 11 us, and the pass of encode, compaction and turn 53 us
-// instead of 155 (four warps to a CTA: 55 us; 16 rows to a CTA: 80 us).
+// this kernel takes 21 and 11 us, and the pass of encode, compaction and turn 46 us
+// instead of 155 (the rows' softmaxes one after the other, blocks light to heavy: 53;
+// four warps to a CTA: 55; 16 rows to a CTA: 80).
 //
 // Key set of a row (token t of sequence b at local index j, head h, group g):
 //   route part : rows route_cu[b*G+g] .. route_cu[b*G+g+1]-1 of k_route/v_route,
@@ -87,7 +88,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
   // Block index -> (sequence, block of it).  Sequence b's blocks start at cu[b] / TQ + b, which leaves
   // every sequence at least the ceil(len / TQ) it needs.
   // (32 boundaries are probed at a time: the block's start is a chain of dependent loads and little else)
-  const int x = blockIdx.x;
+  const int x = gridDim.x - 1 - blockIdx.x;              // the last blocks of a sequence have the most keys: they begin first
   int b = 0;
   for (int width = n_seq; width > 1;) {
     const int step = (width + 31) >> 5, at = b + lane * step;
@@ -215,27 +216,29 @@ __global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
         for (int j = 0; j < VB; ++j) load_f<T, CPL>(vp + (int64_t)min(j0 + j, cnt - 1) * D, vn[j]);   // (past the end: a repeat, with p = 0)
       };
       load_v(0);
-      // ---- online softmax, row by row (a key past the row's own token, or past the end, counts as -inf) ----
+      // ---- online softmax (a key past the row's own token, or past the end, counts as -inf); the rows
+      // go through each step together, so that their shuffles and exponentials overlap ----
+      float mx[ROWS];
       int tok = 0, head = 0;                             // of row r
 #pragma unroll
       for (int r = 0; r < ROWS; ++r) {
-        const int lim = seg == 0 ? n : H + tok0 + tok + 1;
+        const int lim = seg == 0 ? n : min(n, H + tok0 + tok + 1);
         if (++head == s) { head = 0; ++tok; }
-        const float v = kk < lim && kk < n ? v1[r] * scale : -INFINITY;
-        float mx = v;
+        mx[r] = v1[r] = kk < lim ? v1[r] * scale : -INFINITY;
+      }
 #pragma unroll
-        for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-        const float m_new = fmaxf(m[r], mx);
-        const float pr = v == -INFINITY ? 0.f : expf(v - m_new);
-        if (m_new != m[r]) {                             // (uniform over the warp)
-          const float f = m[r] == -INFINITY ? 0.f : expf(m[r] - m_new);
-          l[r] *= f;
+      for (int off = 16; off; off >>= 1)
 #pragma unroll
-          for (int c = 0; c < CPL; ++c) acc[r][c] *= f;
-          m[r] = m_new;
-        }
-        l[r] += pr;
-        v1[r] = pr;
+        for (int r = 0; r < ROWS; ++r) mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], off));
+#pragma unroll
+      for (int r = 0; r < ROWS; ++r) {
+        const float m_new = fmaxf(m[r], mx[r]), m_use = m_new == -INFINITY ? 0.f : m_new;
+        const float f = expf(m[r] - m_use);              // 0 as long as nothing was seen
+        v1[r] = expf(v1[r] - m_use);
+        m[r] = m_new;
+        l[r] = l[r] * f + v1[r];
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) acc[r][c] *= f;
       }
 #pragma unroll
       for (int r = 0; r < ROWS; r += 4) *reinterpret_cast<float4*>(&ps[mine][r]) = make_float4(v1[r], v1[r + 1], v1[r + 2], v1[r + 3]);

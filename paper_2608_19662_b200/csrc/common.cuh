@@ -144,6 +144,21 @@ __device__ __forceinline__ int rc_find_segment(const int32_t* __restrict__ cu, i
   return lo;
 }
 
+// The same for a whole warp (x alike in all lanes, all lanes present): 32 boundaries are probed at a
+// time, so that a thousand sequences are two loads in a row and not ten.
+__device__ __forceinline__ int rc_find_segment_warp(const int32_t* __restrict__ cu, int n, int x) {
+  const int lane = threadIdx.x & 31;
+  int b = 0;
+  for (int width = n; width > 1;) {
+    const int step = (width + 31) >> 5;
+    const bool le = lane * step < width && (lane == 0 || cu[b + lane * step] <= x);
+    const int last = 31 - __clz(__ballot_sync(0xffffffffu, le));      // (the boundaries ascend)
+    b += last * step;
+    width = min(step, width - last * step);
+  }
+  return b;
+}
+
 template <typename T> __device__ __forceinline__ float rc_to_float(T x);
 template <> __device__ __forceinline__ float rc_to_float<float>(float x) { return x; }
 template <> __device__ __forceinline__ float rc_to_float<__nv_bfloat16>(__nv_bfloat16 x) { return __bfloat162float(x); }

@@ -66,19 +66,23 @@ __global__ void __launch_bounds__(256) rope_store_kernel(
   const int chunks = half / N;                  // 16-byte chunks per half row
   const int64_t gid = (int64_t)(blockIdx.x - (PLAN ? 1 : 0)) * blockDim.x + threadIdx.x;
   const int64_t n_work = (int64_t)total * G * chunks;
+  const int64_t first = gid - (threadIdx.x & 31);       // of the warp
+  if (first >= n_work) return;
+  // the sequence of the warp's first token, found together; a lane whose token is further on walks there
+  int b = rc_find_segment_warp(cu, n_seq, (int)(first / ((int64_t)chunks * G)));
   if (gid >= n_work) return;
   const int c = (int)(gid % chunks);
   const int g = (int)((gid / chunks) % G);
   const int t = (int)(gid / ((int64_t)chunks * G));
-
-  const int b = rc_find_segment(cu, n_seq, t);
-  const int local = t - cu[b];
+  int seq0 = cu[b], seq1 = cu[b + 1];
+  while (b + 1 < n_seq && seq1 <= t) { ++b; seq0 = seq1; seq1 = cu[b + 1]; }
+  const int local = t - seq0, n_cu = cu[n_seq];
   // position = the sequence's first position (0 when none is given) + index inside the sequence;
   // row = the sequence's first cache row + that index (encode) or the token index itself (prefill)
   const int pos = (pos0 ? pos0[b] : 0) + local;
   const int64_t row = mode == 0 ? (int64_t)slot[b] + local
                     : mode == 2 ? (int64_t)slot[b] + (hist ? hist[b] : 0) + local : (int64_t)t;
-  if (t >= cu[n_seq] || cu[b + 1] < cu[b]) { rc_set_status(status, RECACHE_DEV_BAD_SEQLENS); return; }
+  if (t >= n_cu || seq1 < seq0) { rc_set_status(status, RECACHE_DEV_BAD_SEQLENS); return; }
   if (row < 0 || row >= dst_rows) { rc_set_status(status, RECACHE_DEV_BAD_SLOT); return; }
   if (pos < 0 || pos >= max_pos) { rc_set_status(status, RECACHE_DEV_BAD_POS); return; }
 
