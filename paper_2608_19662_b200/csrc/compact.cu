@@ -313,7 +313,8 @@ cudaError_t rc_launch_compact(const recache_ctx* ctx, const CompactArgs& a, cuda
   }
   if (a.total_listed > 0) {
     const int64_t pairs = (int64_t)a.total_listed * G;
-    const unsigned z = (unsigned)(pairs >= 2048 ? 1 : (2048 + pairs - 1) / pairs > 8 ? 8 : (2048 + pairs - 1) / pairs);
+    // (an index list alone is written by the first of the z CTAs of a pair)
+    const unsigned z = (unsigned)(!a.k_out || pairs >= 2048 ? 1 : (2048 + pairs - 1) / pairs > 8 ? 8 : (2048 + pairs - 1) / pairs);
     dim3 grid((unsigned)a.total_listed, (unsigned)G, z);
     RcLaunchScope scope(ctx, RC_K_COMPACT_GATHER, st);
     e = rc_launch_overlapped(compact_gather_kernel, grid, TPB, 0, st, (const uint8_t*)a.k_cache, (const uint8_t*)a.v_cache, a.pool_tokens, a.keep,
