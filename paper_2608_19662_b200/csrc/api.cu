@@ -119,7 +119,7 @@ recache_status recache_selftest_wait_timeout(recache_ctx* ctx, int32_t* report, 
 }
 
 static const char* kKernelNames[RC_K_COUNT] = {
-    "rope_store", "tile_plan", "encode_attn", "prefill_attn", "compact_count", "compact_plan",
+    "rope_store", "encode_attn", "prefill_attn", "compact_count", "compact_plan",
     "compact_gather", "decode_append", "decode_attn", "decode_merge", "prefill_merge"};
 
 int32_t recache_kernel_count(void) { return RC_K_COUNT; }

@@ -11,7 +11,7 @@
 
 // Kernels of the library, for launch counting and optional per-kernel timing.
 enum RcKernel {
-  RC_K_ROPE_STORE = 0, RC_K_TILE_PLAN, RC_K_ENCODE_ATTN, RC_K_PREFILL_ATTN,
+  RC_K_ROPE_STORE = 0, RC_K_ENCODE_ATTN, RC_K_PREFILL_ATTN,
   RC_K_COMPACT_COUNT, RC_K_COMPACT_PLAN, RC_K_COMPACT_GATHER,
   RC_K_DECODE_APPEND, RC_K_DECODE_ATTN, RC_K_DECODE_MERGE, RC_K_PREFILL_MERGE, RC_K_COUNT
 };
