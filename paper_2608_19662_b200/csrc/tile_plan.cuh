@@ -8,6 +8,7 @@
 constexpr int RC_TILE_N = 128;       // keys of a K/V tile
 constexpr int RC_SORT_MAX = 4096;    // work items up to which the plan sorts a prefill by weight (encode: a quarter)
 constexpr int RC_ITEM_UNITS = 2;     // what beginning an item costs, in K/V tiles
+constexpr int RC_L2_BLOCKS = 768;    // 100 MB: what of the 126 MB L2 a launch's keys and values may take
 constexpr int RC_PLAN_BINS = 1024;   // weights (K/V tiles, tile pairs) are told apart up to this
 
 struct RcPlan {
@@ -66,7 +67,7 @@ __device__ __forceinline__ bool rc_load_item(const RcPlan& p, int w, RcItem& it)
   return ok;
 }
 
-struct RcPlanSmem { int hist[RC_PLAN_BINS + 1]; int warp_sum[33]; int most; };
+struct RcPlanSmem { int hist[RC_PLAN_BINS + 1]; int warp_sum[33]; int most; int blocks; };   // blocks: of 256 key and value rows (128 KB) that the launch reads
 
 // Exclusive block scan of one int per thread; *total gets the sum (same pattern of calls in every thread).
 __device__ __forceinline__ int rc_plan_scan(int v, RcPlanSmem& sh, int* total) {
@@ -101,10 +102,15 @@ __device__ __forceinline__ void rc_plan_scan_bins(RcPlanSmem& sh) {
 // afterwards).  An item counts RC_ITEM_UNITS more than its tiles, and a cut is moved to the item's
 // edge where it would leave a part of fewer than two tiles, or a part whose first tile some row of
 // the pair does not see.  Taken only where the longest CTA gets shorter by more than the second
-// beginning (two units) and the merge (three: 5-8 us) cost: 8 conversations with 300-2048 rows of history
-// (88 items of 8-24 tiles) take 50 us instead of 57; one request of 2048 tokens over a long tool set (256
-// items of 58-73 tiles, else two rounds of 148 CTAs) 281 instead of 291.  Encoding is never split: a
-// resource's result must not depend on what is encoded beside it.  False: not worth it.
+// beginning (two units) and the merge (six: 6-10 us, a unit taking 1.8) cost: 8 conversations with 300-2048
+// rows of history (88 items of 8-24 tiles) take 50 us instead of 57; one request of 2048 tokens over a long
+// tool set (256 items of 58-73 tiles, else two rounds of 148 CTAs) 281 instead of 291; 8 conversations of 250
+// tokens over 4000 rows (256 items of 36) would take 159 instead of 152.  Whole items of a sequence also walk
+// its K/V in step and read it from L2, parts do not, which costs a fifth where the keys and values of the launch
+// are more than L2 holds and three or more items share them: 2048 tokens over 14,000 / 20,000 rows a group (57 /
+// 82 MB) 404 / 572 us split and 424 / 583 whole, but over 40,000 (164 MB) 1170 and 1120, and 4 x 512 tokens over
+// 24,000 each 750 and 693.  Encoding is never split: a resource's result must not depend on what is encoded
+// beside it.  False: not worth it.
 __device__ __forceinline__ bool rc_plan_split(const RcPlan& p, RcPlanSmem& sh, int n_work) {
   const int tid = threadIdx.x, n_thr = blockDim.x;
   const int32_t* tiles = p.order + RC_SORT_MAX;
@@ -117,7 +123,8 @@ __device__ __forceinline__ bool rc_plan_split(const RcPlan& p, RcPlanSmem& sh, i
   int at = rc_plan_scan(units, sh, &total_units);
   if (n_items == 0) return false;
   const int n = min(p.n_cta, max(1, (total_units - RC_ITEM_UNITS * n_items) / 4));
-  const float split = (float)total_units / n + RC_ITEM_UNITS + 3;
+  const float pace = sh.blocks > RC_L2_BLOCKS ? 1.2f : 1.f;
+  const float split = pace * total_units / n + RC_ITEM_UNITS + 6;
   const float whole = fmaxf((float)(sh.most + RC_ITEM_UNITS), (float)total_units / n_items * ((n_items + p.n_cta - 1) / p.n_cta));
   if (split > 0.95f * whole) return false;
   for (int w = w0; w < w1; ++w) { p.unit_cu[w] = at; if (tiles[w] > 0) at += tiles[w] + RC_ITEM_UNITS; }
@@ -206,8 +213,14 @@ __device__ __forceinline__ void rc_build_plan(const RcPlan& p, RcPlanSmem& sh) {
   if (!sorted) return;
   // Few work items (a prefill of a handful of requests): one CTA gets one or two of them, so their
   // order decides the tail.  Sort them by weight (K/V tiles), heaviest first, with a counting sort.
-  if (tid == 0) sh.most = 0;
+  if (tid == 0) { sh.most = 0; sh.blocks = 0; }
   __syncthreads();
+  if (p.start && n_work > 2 * n_seq * p.G)         // (else see rc_plan_split: the size does not matter)
+#pragma unroll 1
+    for (int b = b0; b < b1; ++b) {
+      const int own = cu[b + 1] - cu[b] + (p.hist ? p.hist[b] : 0);
+      atomicAdd(&sh.blocks, (max(p.route_cu[(b + 1) * p.G] - p.route_cu[b * p.G], 0) >> 8) + ((p.G * max(own, 0)) >> 8));
+    }
   int32_t* tiles = p.order + RC_SORT_MAX;
   for (int w = tid; w < n_work; w += n_thr) {
     RcItem it;

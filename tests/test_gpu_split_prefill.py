@@ -19,6 +19,7 @@ pytestmark = pytest.mark.gpu
     (16, 8, [250, 17, 129], [300, 2048, 1000], [(500, 900)] * 3, torch.float32),   # two heads: pairs of 128 tokens
     (8, 2, [130, 64, 65, 3], [127, 128, 129, 0], [(0, 300)] * 4, torch.float32),   # short: below the decision
     (32, 8, [1100], [0], [(1500, 2600)], torch.bfloat16),            # more items than CTAs, two rounds
+    (32, 8, [1290], [0], [(1500, 2600)], torch.float32),             # a second round of CTAs that is nearly empty
 ])
 def test_split_items_match_oracle(hq, g, lens, hist, route, out):
     sh = wl.Shape(hq, g, 128, 1e6, "bf16")
