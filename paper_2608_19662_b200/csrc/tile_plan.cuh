@@ -82,6 +82,7 @@ __device__ __forceinline__ int rc_plan_scan(int v, RcPlanSmem& sh, int* total) {
   if (lane == 31) sh.warp_sum[warp] = incl;
   __syncthreads();
   int before = 0, all = 0;
+#pragma unroll 1
   for (int w = 0; w < nw; ++w) { const int x = sh.warp_sum[w]; if (w < warp) before += x; all += x; }
   *total = all;
   return before + incl - v;
@@ -91,8 +92,10 @@ __device__ __forceinline__ void rc_plan_scan_bins(RcPlanSmem& sh) {
   const int per = (RC_PLAN_BINS + 1 + blockDim.x - 1) / blockDim.x;
   const int i0 = min(RC_PLAN_BINS + 1, (int)threadIdx.x * per), i1 = min(RC_PLAN_BINS + 1, i0 + per);
   int sum = 0, total;
+#pragma unroll 1
   for (int i = i0; i < i1; ++i) sum += sh.hist[i];
   int at = rc_plan_scan(sum, sh, &total);
+#pragma unroll 1
   for (int i = i0; i < i1; ++i) { const int c = sh.hist[i]; sh.hist[i] = at; at += c; }
   __syncthreads();
 }
@@ -117,6 +120,7 @@ __device__ __forceinline__ bool rc_plan_split(const RcPlan& p, RcPlanSmem& sh, i
   const int per = (n_work + n_thr - 1) / n_thr;
   const int w0 = min(n_work, tid * per), w1 = min(n_work, w0 + per);
   int units = 0, items = 0, total_units, n_items;
+#pragma unroll 1
   for (int w = w0; w < w1; ++w)
     if (tiles[w] > 0) { units += tiles[w] + RC_ITEM_UNITS; ++items; }
   rc_plan_scan(items, sh, &n_items);
@@ -127,8 +131,10 @@ __device__ __forceinline__ bool rc_plan_split(const RcPlan& p, RcPlanSmem& sh, i
   const float split = pace * total_units / n + RC_ITEM_UNITS + 6;
   const float whole = fmaxf((float)(sh.most + RC_ITEM_UNITS), (float)total_units / n_items * ((n_items + p.n_cta - 1) / p.n_cta));
   if (split > 0.95f * whole) return false;
+#pragma unroll 1
   for (int w = w0; w < w1; ++w) { p.unit_cu[w] = at; if (tiles[w] > 0) at += tiles[w] + RC_ITEM_UNITS; }
   __syncthreads();
+#pragma unroll 1
   for (int c = tid; c <= n; c += n_thr) {
     int2 cut = make_int2(n_work, 0);
     if (c < n) {
@@ -147,6 +153,7 @@ __device__ __forceinline__ bool rc_plan_split(const RcPlan& p, RcPlanSmem& sh, i
     p.start[c] = cut;
   }
   __syncthreads();
+#pragma unroll 1
   for (int c = tid; c < n; c += n_thr) {
     int4 m = make_int4(0, 0, 0, 0);
     const int2 cut = p.start[c];
@@ -154,6 +161,7 @@ __device__ __forceinline__ bool rc_plan_split(const RcPlan& p, RcPlanSmem& sh, i
       RcItem it;
       rc_load_item(p, cut.x, it);
       m = make_int4(2, it.seq0 + it.tok0, min(256, (it.L - it.tok0) * p.s), it.g);
+#pragma unroll 1
       for (int j = c + 1; p.start[j].x == cut.x && p.start[j].y > 0; ++j) ++m.x;
     }
     p.merge[c] = m;
@@ -169,6 +177,8 @@ __device__ __forceinline__ bool rc_plan_split(const RcPlan& p, RcPlanSmem& sh, i
 // share one sequence's K/V, which then stays in L2 instead of being streamed
 // from HBM once per tile pair.  One block.  (Sequences of equal length land in an
 // order that may differ between launches; no result depends on it.)
+// (Nothing is unrolled: the block runs every loop for a step or two, out of a cold instruction cache, and
+// the unrolled code took 0.3-0.4 us more of turns of 35-50 us.)
 __device__ __forceinline__ void rc_build_plan(const RcPlan& p, RcPlanSmem& sh) {
   const int tid = threadIdx.x, n_thr = blockDim.x, n_seq = p.n_seq, tok_per_item = 2 * 128 / p.s;
   const int32_t* cu = p.cu;
@@ -180,12 +190,14 @@ __device__ __forceinline__ void rc_build_plan(const RcPlan& p, RcPlanSmem& sh) {
   const int per = (n_seq + n_thr - 1) / n_thr;
   const int b0 = min(n_seq, tid * per), b1 = min(n_seq, b0 + per);
   int sum = 0, total;
+#pragma unroll 1
   for (int b = b0; b < b1; ++b) {
     const int len = cu[b + 1] - cu[b];
     if (len < 0 || (len + tok_per_item - 1) / tok_per_item > p.n_levels)   // not monotone, or longer than the max_len given
       rc_set_status(p.status, RECACHE_DEV_BAD_SEQLENS);
     sum += n_pairs(b);
   }
+#pragma unroll 1
   for (int i = tid; i <= RC_PLAN_BINS; i += n_thr) sh.hist[i] = 0;
   int k = rc_plan_scan(sum, sh, &total);
   const int n_items = min(total, p.max_items), n_work = n_items * p.G;
@@ -196,6 +208,7 @@ __device__ __forceinline__ void rc_build_plan(const RcPlan& p, RcPlanSmem& sh) {
   if (!sorted) {
     // counting sort of the sequences by their number of tile pairs, longest first: hist[bin] = items of
     // that bin, then the first item index of the bin
+#pragma unroll 1
     for (int b = b0; b < b1; ++b) {
       const int nt = n_pairs(b);
       if (nt > 0) atomicAdd(&sh.hist[RC_PLAN_BINS - min(nt, RC_PLAN_BINS)], nt);
@@ -203,10 +216,12 @@ __device__ __forceinline__ void rc_build_plan(const RcPlan& p, RcPlanSmem& sh) {
     __syncthreads();
     rc_plan_scan_bins(sh);
   }
+#pragma unroll 1
   for (int b = b0; b < b1; ++b) {
     const int nt = n_pairs(b);
     if (nt == 0) continue;
     if (!sorted) k = atomicAdd(&sh.hist[RC_PLAN_BINS - min(nt, RC_PLAN_BINS)], nt);
+#pragma unroll 1
     for (int l = nt - 1; l >= 0; --l, ++k)
       if (k < p.max_items) p.items[k] = make_int2(b, l);
   }
@@ -222,6 +237,7 @@ __device__ __forceinline__ void rc_build_plan(const RcPlan& p, RcPlanSmem& sh) {
       atomicAdd(&sh.blocks, (max(p.route_cu[(b + 1) * p.G] - p.route_cu[b * p.G], 0) >> 8) + ((p.G * max(own, 0)) >> 8));
     }
   int32_t* tiles = p.order + RC_SORT_MAX;
+#pragma unroll 1
   for (int w = tid; w < n_work; w += n_thr) {
     RcItem it;
     const int n = rc_load_item(p, w, it) ? it.n_tiles : 0;
@@ -232,5 +248,6 @@ __device__ __forceinline__ void rc_build_plan(const RcPlan& p, RcPlanSmem& sh) {
   __syncthreads();
   if (p.start && rc_plan_split(p, sh, n_work)) return;
   rc_plan_scan_bins(sh);
+#pragma unroll 1
   for (int w = tid; w < n_work; w += n_thr) p.order[atomicAdd(&sh.hist[RC_PLAN_BINS - min(tiles[w], RC_PLAN_BINS)], 1)] = w;
 }
