@@ -199,6 +199,7 @@ __global__ void __launch_bounds__(THREADS<GATHER>, 1) decode_split_kernel(const 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == NCW && lane == 0) { prefetch_tmap(&tm_k); prefetch_tmap(&tm_v); }
+  __syncthreads();         // no warp touches a barrier or the abort flag before they are set, on either way to the roles
   rc_grid_wait();
   rc_grid_launch_next();   // (the merge waits for this grid's end; it only comes up early)
 

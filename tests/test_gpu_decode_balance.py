@@ -98,3 +98,30 @@ def test_gathered_rows_match_paged(hq, groups, batch, res, hist):
     ref = orc.attend_decode(f64(q), q_pos, f64(kp), f64(vp), rt, res_rows, ht, hist_rows, sh.rope_theta, PT, storage=sh.dtype)
     assert max_abs(paged, ref) < 1e-2 and max_abs(gathered, ref) < 1e-2
     assert rc.poll_status() == 0
+
+
+@pytest.mark.parametrize("gather", [False, True])
+def test_one_sequence_right_behind_other_kernels(gather):
+    """A step of one sequence (whose blocks go straight to their roles) gives the same bits every time, whatever
+    the kernels before it left in shared memory, where its barriers are set up."""
+    sh = wl.Shape(8, 2, 128, 1e6, "bf16")
+    rng = np.random.default_rng(31)
+    rows = lambda n, lo, hi: rng.integers(lo, hi + 1, n).astype(np.int32)
+    rc = make_ctx(sh, max_pos=4096)
+    steps = []
+    for batch in (1, 12):
+        res, hist = rows(2 * batch, 100, 900), np.repeat(rows(batch, 1, 1500), 2)
+        kp, vp, rt, ht = _batch(rng, sh, res, hist)
+        q, pos = dev(wl.normal(batch, (batch, 8, 128), sh.torch_dtype)), dev(np.arange(batch, dtype=np.int32) + 9)
+        pages, tail = (dev(kp), dev(vp)), (dev(ht), dev(hist))
+        if gather:
+            cu = np.concatenate([[0], np.cumsum(res)]).astype(np.int32)
+            cache = [dev(wl.normal(40 + i, (2, 900, 128), sh.torch_dtype)) for i in range(2)]
+            idx = dev(np.concatenate([rng.permutation(900)[:n] for n in res]).astype(np.int32))
+            steps.append(lambda a=(q, pos, *cache, idx, dev(cu), rt.shape[1], *pages, *tail): rc.attend_decode_gather(*a))
+        else:
+            steps.append(lambda a=(q, pos, *pages, dev(rt), dev(res), *tail): rc.attend_decode(*a))
+    first = steps[0]()
+    got = [(steps[1](), steps[0]())[1] for _ in range(30)]
+    assert all(torch.equal(first, x) for x in got)
+    assert rc.poll_status() == 0
