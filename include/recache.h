@@ -260,6 +260,12 @@ RECACHE_API recache_status recache_attend_prefill(recache_ctx* ctx,
  * conv_slot[b] + hist_len[b] + t.  q_pos0[b] is the position of the first NEW
  * token.  With 64-aligned slots the cache doubles as the decode history pages
  * (page id = (g * cache_rows + conv_slot[b]) / 64 + n).
+ * Where the requests of a call would leave SMs idle, their keys are divided between
+ * the SMs (bf16, head_dim 128): the order of summation, and with it the last bits of a
+ * request's result, then follow from the lengths of all requests of the call.  They
+ * never follow from the capacity of a buffer.  (recache_attend_prefill and
+ * recache_attend_prefill_gather never divide: there a request's result does not
+ * depend on the other requests either.)
  */
 RECACHE_API recache_status recache_attend_prefill_history(recache_ctx* ctx,
     const void* q, const void* k_conv, const void* v_conv,

@@ -944,15 +944,16 @@ static bool tc_may_split(const recache_ctx* ctx, int64_t max_items) {
   const int64_t n = max_items * ctx->desc.n_kv_heads;
   return n <= 4 * tc_ctas(ctx) && n <= RC_SORT_MAX;
 }
-// Whether a launch is made splittable: the merge launch behind it costs 2 us even when the device decides
-// against splitting.  The host knows bounds only (capacities, of which a third is kept as a rule), so it asks
-// for so many tiles of capacity per item that the real ones can be worth cutting: a turn of one request (16
-// tiles of capacity, 5 kept) takes 36 us without the merge launch and 38 with it, 8 zero-copy turns
-// (40 and 12, two rounds of CTAs) 85 and 88.  A conversation cache holds about what it has room for.
-static bool tc_worth_splitting(const recache_ctx* ctx, const TcAttnArgs& a, int64_t max_items) {
-  const int64_t rows = a.route_rows / ((int64_t)a.n_seq * ctx->desc.n_kv_heads) + (a.hist ? a.self_rows / a.n_seq : a.max_len);
-  const int64_t tiles = a.hist ? 8 : max_items * ctx->desc.n_kv_heads <= tc_ctas(ctx) ? 32 : 64;
-  return rows >= tiles * TILE_N;
+// Whether a launch is made splittable, which costs the merge launch behind it (2 us) even when the device
+// then decides against it.  Only a later turn is: its keys are the history's, thousands for a few new tokens.
+// A first turn's result must be the same bits whether its rows are packed or gathered, and both must be free
+// to come in buffers of any size, of which the host cannot tell how much is filled.
+// Nothing here may depend on capacities, except to leave the merge launch out where rc_plan_split cannot say yes
+// whatever they hold: with one round of CTAs it wants most + RC_ITEM_UNITS >= (4 + RC_ITEM_UNITS + 6) / 0.95.
+static bool tc_splits(const recache_ctx* ctx, const TcAttnArgs& a, int64_t max_items) {
+  if (!a.hist || !tc_may_split(ctx, max_items) || tc_ctas(ctx) < 2) return false;
+  const int64_t most = a.route_rows / TILE_N + a.self_rows / TILE_N + 2;     // tiles of an item that had every row there is
+  return max_items * ctx->desc.n_kv_heads > tc_ctas(ctx) || most >= 11;
 }
 constexpr int64_t PART_ROWS = 2 * 2 * 128;   // per CTA: two slots of two tiles
 
@@ -984,7 +985,7 @@ cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope,
 
   TcParams p;
   p.header = (int32_t*)ws; p.items = (int2*)(ws + 256); p.order = (int32_t*)(ws + 256 + align256(max_items * 8));
-  const bool may_split = a.route_cu != nullptr && tc_may_split(ctx, max_items) && tc_ctas(ctx) > 1 && tc_worth_splitting(ctx, a, max_items);
+  const bool may_split = tc_splits(ctx, a, max_items);
   const int sms = tc_ctas(ctx);
   const unsigned grid = (unsigned)(may_split || max_items * G > sms ? sms : max_items * G);
   p.start = nullptr; p.merge = nullptr; p.unit_cu = nullptr; p.part_o = nullptr; p.part_ml = nullptr; p.n_cta = (int)grid;

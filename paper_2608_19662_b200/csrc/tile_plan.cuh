@@ -14,7 +14,7 @@ constexpr int RC_PLAN_BINS = 1024;   // weights (K/V tiles, tile pairs) are told
 struct RcPlan {
   int2* items; int32_t* header;   // header[0] = number of items, header[1] = work counter, header[2] = order[] is valid, header[3] = CTAs of a split launch
   int32_t* order;                 // work indices, heaviest first (launches of at most RC_SORT_MAX work items); K/V tiles of each behind them
-  // Split launch (null: not possible): CTA c takes the K/V tiles from start[c] = (work index, tile) up to start[c + 1].
+  // Split launch (null: not wanted): CTA c takes the K/V tiles from start[c] = (work index, tile) up to start[c + 1].
   // merge[c]: what the merge does at cut c: parts of the item it is the first cut of (0: nothing to do), first token of the
   // item's rows, rows (tokens x heads), group.
   int2* start; int4* merge; int32_t* unit_cu;
@@ -100,13 +100,14 @@ __device__ __forceinline__ void rc_plan_scan_bins(RcPlanSmem& sh) {
   __syncthreads();
 }
 
-// A prefill whose items do not fill the CTAs evenly: their K/V tiles, laid end to end, are cut into
+// A later turn (RcPlan.start given) whose items do not fill the CTAs evenly: their K/V tiles, laid end to end, are cut into
 // n equal ranges, so that an item may be shared by several CTAs (their partial results are merged
 // afterwards).  An item counts RC_ITEM_UNITS more than its tiles, and a cut is moved to the item's
 // edge where it would leave a part of fewer than two tiles, or a part whose first tile some row of
 // the pair does not see.  Taken only where the longest CTA gets shorter by more than the second
 // beginning (two units) and the merge (six: 6-10 us, a unit taking 1.8) cost: 8 conversations with 300-2048
-// rows of history (88 items of 8-24 tiles) take 50 us instead of 57; one request of 2048 tokens over a long
+// rows of history (88 items of 8-24 tiles) take 50 us instead of 57; measured with route rows in the place of a
+// history: one request of 2048 tokens over a long
 // tool set (256 items of 58-73 tiles, else two rounds of 148 CTAs) 281 instead of 291; 8 conversations of 250
 // tokens over 4000 rows (256 items of 36) would take 159 instead of 152.  Whole items of a sequence also walk
 // its K/V in step and read it from L2, parts do not, which costs a fifth where the keys and values of the launch

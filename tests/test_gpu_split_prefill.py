@@ -53,3 +53,64 @@ def test_split_items_match_oracle(hq, g, lens, hist, route, out):
     tol = 1e-2 + (2.0 ** -8 * np.abs(ref) if out == torch.bfloat16 else 0)   # bf16 results: half an ulp on top
     assert (np.abs(f64(o) - ref) <= tol).all()
     assert rc.poll_status() == 0
+
+
+def _padded(t, n):
+    """`t` with n more rows of NaN behind it: a buffer of a larger capacity."""
+    return torch.cat([t, torch.full((n, *t.shape[1:]), float("nan"), dtype=t.dtype, device=t.device)])
+
+
+@pytest.mark.parametrize("hq,g,lens,route", [
+    (32, 8, [512], 3000),                 # one round of CTAs, half of them idle
+    (32, 8, [1100], 2600),                # two rounds, the second nearly empty
+    (8, 1, [33, 40], 3000),               # two requests, items few and long
+])
+def test_first_turn_does_not_depend_on_capacities(hq, g, lens, route):
+    """Packed and gathered rows, in tight buffers and in large ones, and the request alone: the same bits."""
+    sh = wl.Shape(hq, g, 128, 1e6, "bf16")
+    B, d = len(lens), 128
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    n = np.full(B * g, route)
+    r_cu = np.concatenate([[0], np.cumsum(n)]).astype(np.int32)
+    N = lambda i, *s: dev(wl.normal(500 + i, s, sh.torch_dtype))
+    q, k, v = N(0, int(cu[-1]), hq, d), N(1, int(cu[-1]), g, d), N(2, int(cu[-1]), g, d)
+    kc, vc = N(3, g, route + 50, d), N(4, g, route + 50, d)
+    rng = np.random.default_rng(route)
+    idx = [np.sort(rng.permutation(route + 50)[:route]) for _ in n]
+    kr, vr = (torch.cat([c[r % g][dev(x)] for r, x in enumerate(idx)]) for c in (kc, vc))
+    idx, pos0 = dev(np.concatenate(idx).astype(np.int32)), np.full(B, 100, np.int32)
+    rc = make_ctx(sh, max_pos=8192)
+
+    def packed(extra=0, of=slice(0, B)):
+        c, r = cu[of.start:of.stop + 1], r_cu[of.start * g:of.stop * g + 1]
+        tok, rows = slice(int(c[0]), int(c[-1])), slice(int(r[0]), int(r[-1]))
+        return rc.attend_prefill(q[tok], k[tok], v[tok], dev(c - c[0]), dev(pos0[of]), max(lens), _padded(kr[rows], extra), _padded(vr[rows], extra),
+                                 dev(r - r[0]))[0]
+
+    def gathered(extra=0):
+        more = torch.zeros(extra, dtype=torch.int32, device="cuda")
+        return rc.attend_prefill_gather(q, k, v, dev(cu), dev(pos0), max(lens), kc, vc, torch.cat([idx, more]), dev(r_cu))[0]
+
+    want = packed()
+    for got in (packed(9000 * B * g), gathered(), gathered(9000 * B * g), torch.cat([packed(0, slice(b, b + 1)) for b in range(B)])):
+        assert torch.equal(want, got)
+    assert rc.poll_status() == 0
+
+
+def test_later_turn_does_not_depend_on_capacities():
+    """One long history among short ones, in a tight cache and in one with room: the same bits."""
+    sh = wl.Shape(8, 2, 128, 1e6, "bf16")
+    hist, new = np.array([3000, 0, 0, 0], np.int32), 5
+    N = lambda i, *s: dev(wl.normal(600 + i, s, sh.torch_dtype))
+    q, k, v = N(0, 4 * new, 8, 128), N(1, 4 * new, 2, 128), N(2, 4 * new, 2, 128)
+    slot = np.concatenate([[0], np.cumsum((hist + new + 63) // 64 * 64)]).astype(np.int32)
+    kc, vc, rows = N(3, 2, int(slot[-1]), 128), N(4, 2, int(slot[-1]), 128), N(5, 1, 128)
+    cu = dev(np.arange(5, dtype=np.int32) * new)
+    rc = make_ctx(sh, max_pos=8192)
+    got = []
+    for extra in (0, 20000):
+        caches = [torch.cat([c, torch.full((2, extra, 128), float("nan"), dtype=c.dtype, device="cuda")], 1) for c in (kc, vc)]
+        got.append(rc.attend_prefill_history(q, k, v, cu, dev(hist + 9), new, _padded(rows, extra), _padded(rows, extra),
+                                             torch.zeros(9, dtype=torch.int32, device="cuda"), *caches, dev(slot[:-1]), dev(hist)))
+    assert torch.equal(*got)
+    assert rc.poll_status() == 0
