@@ -135,13 +135,19 @@ RECACHE_API const char* recache_kernel_name(int32_t id);
 RECACHE_API recache_status recache_kernel_timer(recache_ctx* ctx, int32_t enable);
 RECACHE_API recache_status recache_kernel_times(recache_ctx* ctx, float* ms_total, int64_t* launches);
 
-/* Scratch sizes in bytes for the calls below (same size arguments). */
+/* Scratch sizes in bytes for the calls below (same size arguments).  They grow with every
+ * argument: a workspace sized for the largest call serves all smaller ones.
+ * recache_prefill_workspace_bytes is what every prefill needs, a few bytes per query token;
+ * recache_prefill_history_workspace_bytes is that and 39 MB (148 SMs), with which
+ * recache_attend_prefill_history may divide its requests' keys between SMs. */
 RECACHE_API int64_t recache_encode_workspace_bytes(const recache_ctx* ctx, int32_t n_resources,
                                        int32_t total_tokens, int32_t max_len);
 RECACHE_API int64_t recache_compact_workspace_bytes(const recache_ctx* ctx, int32_t n_requests,
                                         int32_t total_listed);
 RECACHE_API int64_t recache_prefill_workspace_bytes(const recache_ctx* ctx, int32_t n_requests,
                                         int32_t total_q, int32_t max_q);
+RECACHE_API int64_t recache_prefill_history_workspace_bytes(const recache_ctx* ctx, int32_t n_requests,
+                                                int32_t total_q, int32_t max_q);
 RECACHE_API int64_t recache_decode_workspace_bytes(const recache_ctx* ctx, int32_t batch,
                                        int32_t max_res_pages, int32_t max_hist_pages);
 
@@ -261,7 +267,8 @@ RECACHE_API recache_status recache_attend_prefill(recache_ctx* ctx,
  * token.  With 64-aligned slots the cache doubles as the decode history pages
  * (page id = (g * cache_rows + conv_slot[b]) / 64 + n).
  * Where the requests of a call would leave SMs idle, their keys are divided between
- * the SMs (bf16, head_dim 128): the order of summation, and with it the last bits of a
+ * the SMs (bf16, head_dim 128; only with a workspace of
+ * recache_prefill_history_workspace_bytes(), else the call runs undivided): the order of summation, and with it the last bits of a
  * request's result, then follow from the lengths of all requests of the call.  They
  * never follow from the capacity of a buffer.  (recache_attend_prefill and
  * recache_attend_prefill_gather never divide: there a request's result does not

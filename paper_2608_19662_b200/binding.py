@@ -46,6 +46,7 @@ SIGNATURES = {
     "recache_encode_workspace_bytes": (_I64, [_P, _I32, _I32, _I32]),
     "recache_compact_workspace_bytes": (_I64, [_P, _I32, _I32]),
     "recache_prefill_workspace_bytes": (_I64, [_P, _I32, _I32, _I32]),
+    "recache_prefill_history_workspace_bytes": (_I64, [_P, _I32, _I32, _I32]),
     "recache_decode_workspace_bytes": (_I64, [_P, _I32, _I32, _I32]),
     "recache_encode_resources": (C.c_int, [_P, _P, _P, _P, _P, _I32, _I32, _I32, _P, _P, _P, _I64, _P, _I32,
                                            _P, _I64, _P]),
@@ -71,9 +72,9 @@ SIGNATURES = {
 }
 
 # what _native calls, in its order
-NATIVE_CALLS = ["encode_workspace_bytes", "compact_workspace_bytes", "prefill_workspace_bytes", "decode_workspace_bytes", "encode_resources",
-                "compact_routes", "attend_prefill", "attend_prefill_gather", "attend_prefill_history", "attend_decode",
-                "attend_decode_gather"]
+NATIVE_CALLS = ["encode_workspace_bytes", "compact_workspace_bytes", "prefill_workspace_bytes", "prefill_history_workspace_bytes",
+                "decode_workspace_bytes", "encode_resources", "compact_routes", "attend_prefill", "attend_prefill_gather",
+                "attend_prefill_history", "attend_decode", "attend_decode_gather"]
 
 _lib = None
 _native = None
@@ -217,6 +218,9 @@ class ReCache:
 
     def prefill_workspace_bytes(self, n_requests, total_q, max_q) -> int:
         return int(self.lib.recache_prefill_workspace_bytes(self.h, n_requests, total_q, max_q))
+
+    def prefill_history_workspace_bytes(self, n_requests, total_q, max_q) -> int:
+        return int(self.lib.recache_prefill_history_workspace_bytes(self.h, n_requests, total_q, max_q))
 
     def decode_workspace_bytes(self, batch, max_res_pages, max_hist_pages) -> int:
         return int(self.lib.recache_decode_workspace_bytes(self.h, batch, max_res_pages, max_hist_pages))

@@ -159,6 +159,10 @@ int64_t recache_prefill_workspace_bytes(const recache_ctx* ctx, int32_t n_reques
   if (!ctx || n_requests < 0 || total_q < 0 || max_q < 0) return -1;
   return rc_prefill_workspace_bytes(ctx, n_requests, total_q, max_q);
 }
+int64_t recache_prefill_history_workspace_bytes(const recache_ctx* ctx, int32_t n_requests, int32_t total_q, int32_t max_q) {
+  if (!ctx || n_requests < 0 || total_q < 0 || max_q < 0) return -1;
+  return rc_prefill_history_workspace_bytes(ctx, n_requests, total_q, max_q);
+}
 int64_t recache_decode_workspace_bytes(const recache_ctx* ctx, int32_t batch, int32_t max_res_pages,
                                        int32_t max_hist_pages) {
   if (!ctx || batch < 0 || max_res_pages < 0 || max_hist_pages < 0) return -1;

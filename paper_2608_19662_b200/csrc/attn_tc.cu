@@ -937,13 +937,24 @@ static int tc_levels(const recache_ctx* ctx, int max_len) {
   return (max_len + t - 1) / t + 1;
 }
 
-// A prefill of at most four rounds of CTAs may be split (see rc_plan_split); what that takes of the
-// workspace: cuts, unit prefix, and two partial results per CTA.
+// A later turn of at most four rounds of CTAs may be split (see rc_plan_split).
 static int tc_ctas(const recache_ctx* ctx) { return ctx->sm_count > 0 ? ctx->sm_count : 148; }
 static bool tc_may_split(const recache_ctx* ctx, int64_t max_items) {
   const int64_t n = max_items * ctx->desc.n_kv_heads;
   return n <= 4 * tc_ctas(ctx) && n <= RC_SORT_MAX;
 }
+
+constexpr int64_t PART_ROWS = 2 * 2 * 128;   // per CTA: two slots of two tiles
+
+int64_t rc_tc_workspace_bytes(const recache_ctx* ctx, int n_seq, int total, int max_len) {
+  return 256 + align256(tc_max_items(ctx, n_seq, total) * 8) + align256(2 * RC_SORT_MAX * 4);
+}
+// What a split takes on top, whatever the call's size: cuts, unit prefix, and two partial results per CTA.
+int64_t rc_tc_split_bytes(const recache_ctx* ctx) {
+  const int64_t n = tc_ctas(ctx);
+  return align256((n + 1) * 8) + align256((n + 1) * 16) + align256(RC_SORT_MAX * 4) + align256(n * PART_ROWS * 8) + n * PART_ROWS * D * 4;
+}
+
 // Whether a launch is made splittable, which costs the merge launch behind it (2 us) even when the device
 // then decides against it.  Only a later turn is: its keys are the history's, thousands for a few new tokens.
 // A first turn's result must be the same bits whether its rows are packed or gathered, and both must be free
@@ -952,17 +963,9 @@ static bool tc_may_split(const recache_ctx* ctx, int64_t max_items) {
 // whatever they hold: with one round of CTAs it wants most + RC_ITEM_UNITS >= (4 + RC_ITEM_UNITS + 6) / 0.95.
 static bool tc_splits(const recache_ctx* ctx, const TcAttnArgs& a, int64_t max_items) {
   if (!a.hist || !tc_may_split(ctx, max_items) || tc_ctas(ctx) < 2) return false;
+  if (a.workspace_bytes < rc_tc_workspace_bytes(ctx, a.n_seq, a.total, a.max_len) + rc_tc_split_bytes(ctx)) return false;
   const int64_t most = a.route_rows / TILE_N + a.self_rows / TILE_N + 2;     // tiles of an item that had every row there is
   return max_items * ctx->desc.n_kv_heads > tc_ctas(ctx) || most >= 11;
-}
-constexpr int64_t PART_ROWS = 2 * 2 * 128;   // per CTA: two slots of two tiles
-
-int64_t rc_tc_workspace_bytes(const recache_ctx* ctx, int n_seq, int total, int max_len, bool prefill) {
-  const int64_t max_items = tc_max_items(ctx, n_seq, total), n = tc_ctas(ctx);
-  int64_t bytes = 256 + align256(max_items * 8) + align256(2 * RC_SORT_MAX * 4);
-  if (prefill && tc_may_split(ctx, max_items))
-    bytes += align256((n + 1) * 8) + align256((n + 1) * 16) + align256(RC_SORT_MAX * 4) + align256(n * PART_ROWS * 8) + n * PART_ROWS * D * 4;
-  return bytes;
 }
 
 cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope, const TcAttnArgs& a, cudaStream_t st) {
@@ -990,7 +993,7 @@ cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope,
   const unsigned grid = (unsigned)(may_split || max_items * G > sms ? sms : max_items * G);
   p.start = nullptr; p.merge = nullptr; p.unit_cu = nullptr; p.part_o = nullptr; p.part_ml = nullptr; p.n_cta = (int)grid;
   if (may_split) {
-    uint8_t* at = ws + 256 + align256(max_items * 8) + align256(2 * RC_SORT_MAX * 4);
+    uint8_t* at = ws + rc_tc_workspace_bytes(ctx, a.n_seq, a.total, a.max_len);
     p.start = (int2*)at; at += align256((int64_t)(sms + 1) * 8);
     p.merge = (int4*)at; at += align256((int64_t)(sms + 1) * 16);
     p.unit_cu = (int32_t*)at; at += align256(RC_SORT_MAX * 4);

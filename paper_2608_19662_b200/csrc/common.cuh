@@ -258,6 +258,7 @@ struct PrefillArgs {
 };
 int64_t rc_encode_workspace_bytes(const recache_ctx* ctx, int n_res, int total, int max_len);
 int64_t rc_prefill_workspace_bytes(const recache_ctx* ctx, int n_req, int total_q, int max_q);
+int64_t rc_prefill_history_workspace_bytes(const recache_ctx* ctx, int n_req, int total_q, int max_q);
 int64_t rc_decode_workspace_bytes(const recache_ctx* ctx, int batch, int max_res_pages, int max_hist_pages);
 // (rotate-and-store of the call's keys and values, then the attention)
 cudaError_t rc_launch_encode(const recache_ctx* ctx, const RopeStoreArgs& rope, const EncodeArgs& a, cudaStream_t st);
@@ -272,7 +273,7 @@ struct TcAttnArgs {
   const int32_t* slot;                     // null: causal rows start at cu[b]
   const void* k_self; const void* v_self; int64_t self_rows;   // [G][self_rows][128]
   const void* k_route; const void* v_route; const int32_t* route_cu; int64_t route_rows;
-  void* workspace;
+  void* workspace; int64_t workspace_bytes;
   int prefix_len;   // > 0 (route_cu null): all sequences see rows g*prefix_len .. of k_route/v_route ([G*prefix_len][128])
   const int32_t* hist = nullptr;   // rows preceding each sequence's own tokens in the self part (earlier turns), all visible
   // gather mode (route_idx != null): route rows are rows route_idx[.] of group g in k_cache / v_cache
@@ -280,7 +281,8 @@ struct TcAttnArgs {
   const void* k_cache = nullptr; const void* v_cache = nullptr; int64_t pool_tokens = 0; const int32_t* route_idx = nullptr;
 };
 bool rc_tc_supported(const recache_ctx* ctx);
-int64_t rc_tc_workspace_bytes(const recache_ctx* ctx, int n_seq, int total, int max_len, bool prefill);
+int64_t rc_tc_workspace_bytes(const recache_ctx* ctx, int n_seq, int total, int max_len);
+int64_t rc_tc_split_bytes(const recache_ctx* ctx);   // on top of that, for a later turn that may be split
 cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope, const TcAttnArgs& a, cudaStream_t st);
 
 // ---- self-test of the bounded barrier wait (report: 2 ints on the device) ----

@@ -21,6 +21,7 @@ struct Lib {
   decltype(&recache_encode_workspace_bytes) encode_ws;
   decltype(&recache_compact_workspace_bytes) compact_ws;
   decltype(&recache_prefill_workspace_bytes) prefill_ws;
+  decltype(&recache_prefill_history_workspace_bytes) prefill_history_ws;
   decltype(&recache_decode_workspace_bytes) decode_ws;
   decltype(&recache_encode_resources) encode;
   decltype(&recache_compact_routes) compact;
@@ -211,7 +212,7 @@ PyObject* prefill_history(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int n_req = (int)cu.numel() - 1, total = (int)q.size(0), max_q = (int)integer(a[8]);
     const at::ScalarType ot = c.out_type(a[17]);
     const at::Tensor out = given_or_empty(a[16], q.sizes(), ot, q);
-    const at::Tensor ws = c.workspace(a[18], lib.prefill_ws(c.h, n_req, total, max_q));
+    const at::Tensor ws = c.workspace(a[18], lib.prefill_history_ws(c.h, n_req, total, max_q));
     void *k = ptr(a[4]), *v = ptr(a[5]), *vr = ptr(a[10]), *vc = ptr(a[13]);
     const int32_t *pos0 = ptr_as<int32_t>(a[7]), *route_cu = ptr_as<int32_t>(a[11]), *slot = ptr_as<int32_t>(a[14]), *hist = ptr_as<int32_t>(a[15]);
     c.check(unlocked([&] {

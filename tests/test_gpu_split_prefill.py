@@ -114,3 +114,25 @@ def test_later_turn_does_not_depend_on_capacities():
                                              torch.zeros(9, dtype=torch.int32, device="cuda"), *caches, dev(slot[:-1]), dev(hist)))
     assert torch.equal(*got)
     assert rc.poll_status() == 0
+
+
+def test_one_workspace_serves_the_largest_call_and_all_smaller_ones():
+    sh = wl.Shape(32, 8, 128, 1e6, "bf16")
+    rc = make_ctx(sh, max_pos=8192)
+    sizes = [(b, t, t) for b in (1, 3, 40, 300) for t in (1, 64, 777, 40000) if t >= b]
+    for query in (rc.prefill_workspace_bytes, rc.prefill_history_workspace_bytes, rc.encode_workspace_bytes):
+        need = {size: query(*size) for size in sizes}
+        assert all(need[a] <= need[b] for a in sizes for b in sizes if all(x <= y for x, y in zip(a, b)))
+    ws = torch.empty(rc.prefill_workspace_bytes(300, 40000, 40000), dtype=torch.uint8, device="cuda")
+    assert rc.prefill_workspace_bytes(1, 512, 512) < 1 << 16 and ws.numel() < 1 << 18      # nothing set aside for parts
+    N = lambda i, *s: dev(wl.normal(700 + i, s, sh.torch_dtype))
+    new, hist = 40, 2500
+    q, k, v, kc, vc = N(0, new, 32, 128), N(1, new, 8, 128), N(2, new, 8, 128), N(3, 8, hist + new, 128), N(4, 8, hist + new, 128)
+    rows, cu, pos, none = N(5, 1, 128), dev(np.array([0, new], np.int32)), dev(np.array([hist], np.int32)), torch.zeros(9, dtype=torch.int32, device="cuda")
+    turn = lambda **kw: rc.attend_prefill(q, k, v, cu, pos, new, rows, rows, none, **kw)[0]
+    later = lambda **kw: rc.attend_prefill_history(q, k, v, cu, pos, new, rows, rows, none, kc, vc, none[:1], pos, out_dtype=torch.float32, **kw)
+    assert torch.equal(turn(), turn(workspace=ws))
+    whole, parts = later(workspace=ws), later()
+    assert rc.poll_status() == 0
+    # two orders of summation of the same rows, probabilities in bf16: 2^-9 of each, signs at random over 2500 rows
+    assert not torch.equal(whole, parts) and (whole - parts).abs().max().item() < 2e-3
