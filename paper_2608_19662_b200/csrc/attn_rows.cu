@@ -28,6 +28,8 @@
 // The query is rotated on load at position pos0[b] + j (0 + j for encoding).
 // Blocks and tiles are aligned to the sequence, never to the batch: results do
 // not depend on what else is in the launch.
+#include <float.h>
+
 #include "common.cuh"
 
 namespace {
@@ -165,6 +167,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
       vb = v_self + ((int64_t)g * self_rows + base) * D;
       n = H + tok0 + n_tok;
     }
+    const int all_see = seg == 0 ? n : H + tok0 + 1;     // keys that every row of the block sees
     for (int k0 = 0; k0 < n; k0 += KT, ++t) {
       if (t % WARPS != warp) continue;
       const int cnt = min(KT, n - k0);
@@ -253,6 +256,30 @@ __global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
 #pragma unroll
           for (int c = 0; c < CPL; ++c) v[j][c] = vn[j][c];
         if (j0 + VB < cnt) load_v(j0 + VB);
+        if (k0 + j0 + VB > all_see) {
+          // some row does not see the last of these keys (or they are repeats past the end): its p = 0 would
+          // make NaN of an infinite value, so such values are taken out and added for the rows that see them
+          bool odd = false;
+#pragma unroll
+          for (int j = 0; j < VB; ++j)
+#pragma unroll
+            for (int c = 0; c < CPL; ++c)
+              if (k0 + j0 + j >= all_see && !(fabsf(v[j][c]) <= FLT_MAX)) { v[j][c] = 0.f; odd = true; }
+          if (odd) {
+#pragma unroll 1
+            for (int j = max(all_see - k0, j0); j < min(j0 + VB, cnt); ++j) {
+              float w[CPL];
+              load_f<T, CPL>(vp + (int64_t)j * D, w);
+#pragma unroll
+              for (int c = 0; c < CPL; ++c) {
+                if (fabsf(w[c]) <= FLT_MAX) continue;
+#pragma unroll
+                for (int r = 0; r < ROWS; ++r)
+                  if (k0 + j <= H + tok0 + r / s) acc[r][c] = fmaf(ps[j][r], w[c], acc[r][c]);
+              }
+            }
+          }
+        }
 #pragma unroll
         for (int j = 0; j < VB; ++j) {
 #pragma unroll

@@ -34,3 +34,30 @@ def test_block_edges(hq, g, d, dtype, tol):
     p_ref, _ = oracle_prefill(req, rows, kc_ref, vc_ref)
     assert max_abs(p, p_ref) < tol
     assert rc.poll_status() == 0
+
+
+@pytest.mark.parametrize("hq,g,d,dtype", [(4, 2, 64, "f32"), (8, 1, 128, "f32"), (2, 2, 64, "bf16"), (3, 3, 128, "bf16")])
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+def test_values_that_are_not_finite_reach_only_the_rows_that_see_them(hq, g, d, dtype, value):
+    sh = wl.Shape(hq, g, d, 1e4, dtype)
+    lens, at, col = [290, 45, 9], (100, 44, 2), 5           # the middle of a block, a last token, a short sequence
+    pool = wl.pack_resources(sh, 3, lens, [np.ones(n, np.uint8) for n in lens])
+    rc = make_ctx(sh, max_pos=1024)
+    clean, kc, vc = gpu_encode(rc, pool)
+    for i, j in enumerate(at):
+        pool.v[int(pool.cu_seqlens[i]) + j, :, col] = value
+    o, kc, vc = gpu_encode(rc, pool)
+    for i, j in enumerate(at):
+        own, want = (x[int(pool.cu_seqlens[i]):int(pool.cu_seqlens[i + 1])] for x in (o, clean))
+        assert torch.equal(own[:j], want[:j])                # earlier tokens: as if it were not there
+        assert not torch.isfinite(own[j:, :, col]).any() and (value != value or (own[j, :, col] == value).all())
+        own[j:, :, col] = want[j:, :, col]
+        assert torch.equal(own, want)                        # later ones: that column and no other
+    # a route whose last rows (45 of them, not a multiple of the key tile) are the one with that value, then none
+    req = wl.make_requests(sh, 7, pool, [[1], []], [np.ones((g, 1), np.uint8), np.ones((g, 0), np.uint8)], [40, 20])
+    out = gpu_compact(rc, pool, req, kc, vc)
+    p, _, _ = gpu_prefill(rc, req, out["k_out"], out["v_out"], out["route_cu"])
+    assert torch.isfinite(p[40:]).all() and not torch.isfinite(p[:40, :, col]).any()
+    assert value != value or (p[:40, :, col] == value).all()
+    p[:40, :, col] = 0
+    assert torch.isfinite(p).all() and rc.poll_status() == 0
