@@ -102,12 +102,15 @@ at::Tensor given_or_empty(PyObject* o, at::IntArrayRef sizes, at::ScalarType t, 
 }
 void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
-template <typename F> recache_status unlocked(F f) {   // other Python threads run while the launches are made
-  recache_status st;
-  Py_BEGIN_ALLOW_THREADS
-  st = f();
-  Py_END_ALLOW_THREADS
-  return st;
+// Other Python threads run while the launches are made.  (The lock is taken again also where f throws: a tensor
+// without memory does when it is asked for its address.)
+struct Unlock {
+  PyThreadState* state = PyEval_SaveThread();
+  ~Unlock() { PyEval_RestoreThread(state); }
+};
+template <typename F> recache_status unlocked(F f) {
+  const Unlock u;
+  return f();
 }
 
 // Runs a call's body; exceptions become Python ones.
