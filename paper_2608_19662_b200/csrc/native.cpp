@@ -10,6 +10,7 @@
 #include <ATen/ops/empty.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Dtype.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "recache.h"
@@ -120,8 +121,8 @@ template <typename F> PyObject* guarded(Py_ssize_t n, Py_ssize_t want, F f) {
     return f();
   } catch (const Error&) {
     return nullptr;
-  } catch (const std::exception& e) {
-    PyErr_SetString(PyExc_RuntimeError, e.what());
+  } catch (const std::exception&) {
+    torch::translate_exception_to_python(std::current_exception());   // OutOfMemoryError, IndexError ... as torch raises them
     return nullptr;
   }
 }

@@ -45,3 +45,21 @@ def test_arguments_and_errors():
     rc.close()
     with pytest.raises(Exception):
         rc.encode_resources(q, k, v, cu, 70, slot, kc, vc)
+
+
+def test_out_of_memory_is_torchs_own_error():
+    """The output's allocation fails with the error type that a program catches to free memory and try again."""
+    sh = wl.QWEN3_4B
+    rc = make_ctx(sh, max_pos=8192)
+    q = torch.zeros((8192, sh.n_q_heads, sh.head_dim), dtype=sh.torch_dtype, device="cuda")
+    k = torch.zeros((8192, sh.n_kv_heads, sh.head_dim), dtype=sh.torch_dtype, device="cuda")
+    cache, cu, slot = k.transpose(0, 1).contiguous(), dev(np.array([0, 8192], np.int32)), dev(np.zeros(1, np.int32))
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    try:
+        torch.cuda.set_per_process_memory_fraction(torch.cuda.memory_reserved() / torch.cuda.get_device_properties(0).total_memory)
+        with pytest.raises(torch.OutOfMemoryError):
+            rc.encode_resources(q, k, k, cu, 8192, slot, cache, cache)
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    assert rc.encode_resources(q, k, k, cu, 8192, slot, cache, cache.clone()).shape == q.shape and rc.poll_status() == 0
