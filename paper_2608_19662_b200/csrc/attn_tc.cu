@@ -44,10 +44,11 @@ constexpr int NSTAGE = 2;
 constexpr int BOX_BYTES = 16384;   // [128 rows][64 bf16], 128-byte swizzle
 constexpr int TILE_BYTES = 32768;  // two boxes: head_dim halves
 constexpr int NTHREADS = 512;
-// Registers per thread of the softmax warps and of the other eight; 256 * (softmax + aux) = 65536.  The
-// prefill's scheduler and epilogue, which know about split items, spill in 32; the encode pays 1 % for 40.
-template <bool PREFILL> constexpr int REGS_SOFTMAX = PREFILL ? 216 : 224;
-template <bool PREFILL> constexpr int REGS_AUX = PREFILL ? 40 : 32;
+// Registers per thread of the softmax warps and of the other eight; 256 * (softmax + aux) = 65536.  Epilogue
+// warps that gather and schedulers that know about split items spill in 32 (8 zero-copy turns: 84.0 us with 32,
+// 82.2 with 40); whole items of packed rows pay for 40 (one turn of 512 tokens: 34.8 us with 40, 34.3 with 32; an encode 1 %).
+template <bool MORE_AUX> constexpr int REGS_SOFTMAX = MORE_AUX ? 216 : 224;
+template <bool MORE_AUX> constexpr int REGS_AUX = MORE_AUX ? 40 : 32;
 
 constexpr int SM_Q = 0;                              // 2 query tiles
 constexpr int SM_K = SM_Q + 2 * TILE_BYTES;          // NSTAGE key tiles
@@ -243,7 +244,7 @@ enum { IT_NTILES = 0, IT_G, IT_SEQ0, IT_L, IT_TOK0, IT_KVEND, IT_POS0, IT_RA0, I
 // items through a two-slot ring in shared memory.
 // The next item's Q load, Q rotation and first K/V tiles overlap the current
 // item's last tiles and its epilogue.  Barrier phases run on across items.
-template <typename TO, bool ROT_SMEM, bool GATHER, bool PREFILL>
+template <typename TO, bool ROT_SMEM, bool GATHER, bool SPLIT>
 __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
                                                               const __grid_constant__ CUtensorMap tm_ks,
                                                               const __grid_constant__ CUtensorMap tm_vs,
@@ -303,14 +304,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
     const int* r = const_cast<const int*>(item_ring) + sl * IT_WORDS;   // (ordered by the barrier wait above and the arrive below)
     it.n_tiles = r[IT_NTILES]; it.g = r[IT_G]; it.seq0 = r[IT_SEQ0]; it.L = r[IT_L]; it.tok0 = r[IT_TOK0];
     it.kv_end = r[IT_KVEND]; it.pos0 = r[IT_POS0]; it.rA0 = r[IT_RA0]; it.lenA = r[IT_LENA]; it.nA = r[IT_NA];
-    it.b_valid = r[IT_BVALID]; it.H = r[IT_H]; it.part = PREFILL ? r[IT_PART] : -1;
+    it.b_valid = r[IT_BVALID]; it.H = r[IT_H]; it.part = SPLIT ? r[IT_PART] : -1;
     it.base = (int64_t)(((uint64_t)(uint32_t)r[IT_BASE_HI] << 32) | (uint32_t)r[IT_BASE_LO]);
     if (*abort_flag) it.n_tiles = -1;
     if (release) mbar_arrive(bar(B_IEMPTY + sl));
   };
 
   if (warp >= 12) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_AUX<PREFILL>));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_AUX<GATHER || SPLIT>));
     // ===================== epilogue warps =====================
     // O of a finished query tile leaves tensor memory here, so that the softmax warps can go
     // straight to the next item's Q.  Warp 12 + q reads lanes 32 q .. 32 q + 31.
@@ -428,13 +429,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
       it = nx;
     }
   } else if (warp >= 8) {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_AUX<PREFILL>));
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_AUX<GATHER || SPLIT>));
   if (warp == 10) {
     // ===================== scheduler =====================
     if (lane == 0) {
       const int total = p.header[0] * p.G;   // (a CTA without work publishes "no more work" at once)
       bool first = true;
-      const int n_split = PREFILL && p.start ? p.header[3] : 0;
+      const int n_split = SPLIT ? p.header[3] : 0;
       int2 cur = make_int2(0, 0), end = make_int2(0, 0);
       if ((int)blockIdx.x < n_split) { cur = p.start[blockIdx.x]; end = p.start[blockIdx.x + 1]; }
       for (uint32_t n = 0;; ++n) {
@@ -646,7 +647,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
     }
   }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX<PREFILL>));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX<GATHER || SPLIT>));
     // ===================== softmax warpgroups =====================
     const int x = warp >> 2;                       // tile A or B
     const int row = threadIdx.x & 127;             // row of the tile = TMEM lane
@@ -1019,8 +1020,8 @@ cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope,
     auto launch = [&](auto kernel) { return rc_launch_overlapped(kernel, grid, NTHREADS, SM_ALLOC, st, tq, tks, tvs, tkr, tvr, p); };
     auto pick = [&](auto type) {
       using TO = decltype(type);
-      if (gather) return rot ? launch(attn_tc_kernel<TO, true, true, true>) : launch(attn_tc_kernel<TO, false, true, true>);
-      if (a.route_cu) return rot ? launch(attn_tc_kernel<TO, true, false, true>) : launch(attn_tc_kernel<TO, false, false, true>);
+      if (gather) return rot ? launch(attn_tc_kernel<TO, true, true, false>) : launch(attn_tc_kernel<TO, false, true, false>);
+      if (may_split) return rot ? launch(attn_tc_kernel<TO, true, false, true>) : launch(attn_tc_kernel<TO, false, false, true>);
       return rot ? launch(attn_tc_kernel<TO, true, false, false>) : launch(attn_tc_kernel<TO, false, false, false>);
     };
     e = f32 ? pick(float()) : pick(__nv_bfloat16());
