@@ -74,11 +74,11 @@ template <int D> struct Smem {
 
 template <typename T, typename TO, int D>
 __global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
-    const T* __restrict__ q, TO* __restrict__ o, const int32_t* __restrict__ cu, int n_seq, int total,
-    const int32_t* __restrict__ pos0, const int32_t* __restrict__ slot,
-    const T* __restrict__ k_self, const T* __restrict__ v_self, int64_t self_rows,
-    const T* __restrict__ k_route, const T* __restrict__ v_route, const int32_t* __restrict__ route_cu,
-    int prefix_len, const int32_t* __restrict__ hist, int64_t route_rows, int Hq, int G, const float* __restrict__ cos_tab, const float* __restrict__ sin_tab, int max_pos,
+    const T* q, TO* __restrict__ o, const int32_t* cu, int n_seq, int total,
+    const int32_t* pos0, const int32_t* slot,
+    const T* k_self, const T* v_self, int64_t self_rows,
+    const T* k_route, const T* v_route, const int32_t* route_cu,
+    int prefix_len, const int32_t* hist, int64_t route_rows, int Hq, int G, const float* __restrict__ cos_tab, const float* __restrict__ sin_tab, int max_pos,
     float scale, int32_t* status) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   Smem<D>& sh = *reinterpret_cast<Smem<D>*>(smem_raw);

@@ -57,6 +57,9 @@ struct RcLaunchScope {
 // rc_grid_wait() then waits until it has ended and its writes are visible.  Every block of every such
 // kernel executes rc_grid_wait() before it reads or writes global memory, also one that has nothing
 // to do: the end of a kernel then implies the end of all before it.
+// No input of such a kernel is declared `const ... __restrict__`: that promises that nobody writes it while
+// the kernel runs, so that its loads may use the non-coherent path and be moved up past the wait, but the kernel
+// before may still be writing it then.  (The rotary tables, which no kernel writes, are.)
 __device__ __forceinline__ void rc_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel of the stream come up once every block has said so (or ended).
 __device__ __forceinline__ void rc_grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -135,7 +138,7 @@ __device__ __forceinline__ void rc_timeout_drain() {
 }
 
 // Largest i with cu[i] <= x, for cu[0..n] non-decreasing (n >= 1).
-__device__ __forceinline__ int rc_find_segment(const int32_t* __restrict__ cu, int n, int x) {
+__device__ __forceinline__ int rc_find_segment(const int32_t* cu, int n, int x) {
   int lo = 0, hi = n;  // answer in [lo, hi)
   while (hi - lo > 1) {
     int mid = (lo + hi) >> 1;
@@ -146,7 +149,7 @@ __device__ __forceinline__ int rc_find_segment(const int32_t* __restrict__ cu, i
 
 // The same for a whole warp (x alike in all lanes, all lanes present): 32 boundaries are probed at a
 // time, so that a thousand sequences are two loads in a row and not ten.
-__device__ __forceinline__ int rc_find_segment_warp(const int32_t* __restrict__ cu, int n, int x) {
+__device__ __forceinline__ int rc_find_segment_warp(const int32_t* cu, int n, int x) {
   const int lane = threadIdx.x & 31;
   int b = 0;
   for (int width = n; width > 1;) {

@@ -47,8 +47,8 @@ __device__ __forceinline__ int block_excl_scan(int v, int* ws, int* total) {
 }
 
 __global__ void __launch_bounds__(TPB) compact_count_kernel(
-    const uint8_t* __restrict__ keep, const int32_t* __restrict__ res_slot,
-    const int32_t* __restrict__ res_len, int total_listed, int64_t pool_tokens,
+    const uint8_t* keep, const int32_t* res_slot,
+    const int32_t* res_len, int total_listed, int64_t pool_tokens,
     int32_t* __restrict__ kept, int32_t* status) {
   __shared__ int red[TPB / 32];
   rc_grid_wait();
@@ -76,13 +76,13 @@ __global__ void __launch_bounds__(TPB) compact_count_kernel(
 }
 
 __global__ void __launch_bounds__(1024) compact_plan_kernel(
-    const int32_t* __restrict__ kept, const int32_t* __restrict__ res_off, int n_requests,
-    int total_listed, const uint8_t* __restrict__ vis, int G, int mode, int page_tokens,
+    const int32_t* kept, const int32_t* res_off, int n_requests,
+    int total_listed, const uint8_t* vis, int G, int mode, int page_tokens,
     int32_t* __restrict__ route_cu, int32_t* __restrict__ route_len_out,
     int32_t* __restrict__ res_route_off,   // [G][total_listed]
     int32_t* __restrict__ page_cu,         // [n_routes + 1]
     int64_t row_capacity, int32_t* __restrict__ page_table, int max_pages_per_route,
-    const int32_t* __restrict__ free_pages, int64_t n_free_pages, int64_t n_pool_pages,
+    const int32_t* free_pages, int64_t n_free_pages, int64_t n_pool_pages,
     int32_t* status) {
   __shared__ int ws[1024 / 32 + 1];
   __shared__ int wlen_sh[32];
@@ -102,9 +102,16 @@ __global__ void __launch_bounds__(1024) compact_plan_kernel(
       if (a < 0 || e < a || e > total_listed) {
         rc_set_status(status, RECACHE_DEV_BAD_SEQLENS);
       } else if (!warp_per_route) {
-        for (int r = a; r < e; ++r) {
-          res_route_off[(int64_t)g * total_listed + r] = len;
-          if (vis[(int64_t)g * total_listed + r]) len += kept[r];
+        const uint8_t* vg = vis + (int64_t)g * total_listed;
+        for (int r0 = a; r0 < e; r0 += 4) {            // four at a time: loads are not moved across the stores
+          int v[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) v[u] = r0 + u < e && vg[r0 + u] ? kept[r0 + u] : 0;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            if (r0 + u < e) res_route_off[(int64_t)g * total_listed + r0 + u] = len;
+            len += v[u];
+          }
         }
       }
     }
@@ -179,13 +186,13 @@ constexpr int SUPER = TPB * TOK_PER_THREAD;   // tokens scanned per pass (2048)
 // the kept tokens, their (source row, destination row) pairs go to shared memory,
 // and then all threads stream the rows with eight 16-byte pieces in flight each.
 __global__ void __launch_bounds__(TPB) compact_gather_kernel(
-    const uint8_t* __restrict__ k_cache, const uint8_t* __restrict__ v_cache, int64_t pool_tokens,
-    const uint8_t* __restrict__ keep, const int32_t* __restrict__ res_off,
-    const int32_t* __restrict__ res_slot, const int32_t* __restrict__ res_len, int n_requests,
-    int total_listed, const uint8_t* __restrict__ vis, int G, int mode, int page_tokens,
-    const int32_t* __restrict__ route_cu, const int32_t* __restrict__ res_route_off,
-    const int32_t* __restrict__ page_cu, int32_t* __restrict__ route_idx, int64_t row_capacity,
-    uint8_t* __restrict__ k_out, uint8_t* __restrict__ v_out, const int32_t* __restrict__ free_pages,
+    const uint8_t* k_cache, const uint8_t* v_cache, int64_t pool_tokens,
+    const uint8_t* keep, const int32_t* res_off,
+    const int32_t* res_slot, const int32_t* res_len, int n_requests,
+    int total_listed, const uint8_t* vis, int G, int mode, int page_tokens,
+    const int32_t* route_cu, const int32_t* res_route_off,
+    const int32_t* page_cu, int32_t* __restrict__ route_idx, int64_t row_capacity,
+    uint8_t* __restrict__ k_out, uint8_t* __restrict__ v_out, const int32_t* free_pages,
     int64_t n_free_pages, int64_t n_pool_pages, int row_bytes) {
   __shared__ int ws[TPB / 32 + 1];
   __shared__ int32_t src_tok[SUPER];   // token offset (inside the resource) of the pass's n-th kept token

@@ -50,9 +50,9 @@ template <> __device__ __forceinline__ uint4 pack16<__nv_bfloat16>(const float* 
 // than the list: it only reads the call's index arrays, so it hides behind the copies).
 template <typename T, bool PLAN>
 __global__ void __launch_bounds__(256) rope_store_kernel(
-    const T* __restrict__ k, const T* __restrict__ v, T* __restrict__ k_dst, T* __restrict__ v_dst,
-    const int32_t* __restrict__ cu, int n_seq, int total, const int32_t* __restrict__ slot,
-    const int32_t* __restrict__ pos0, const int32_t* __restrict__ hist, int64_t dst_rows, int mode, int G, int d,
+    const T* k, const T* v, T* __restrict__ k_dst, T* __restrict__ v_dst,
+    const int32_t* cu, int n_seq, int total, const int32_t* slot,
+    const int32_t* pos0, const int32_t* hist, int64_t dst_rows, int mode, int G, int d,
     const float* __restrict__ cos_tab, const float* __restrict__ sin_tab, int max_pos,
     int32_t* status, const __grid_constant__ RcPlan plan, bool overlapped) {
   rc_grid_wait();
@@ -91,6 +91,8 @@ __global__ void __launch_bounds__(256) rope_store_kernel(
   T* kd = k_dst + ((int64_t)g * dst_rows + row) * d;
   T* vd = v_dst + ((int64_t)g * dst_rows + row) * d;
 
+  // (all loads before the first store, which they would not be moved across)
+  const uint4 v0 = *reinterpret_cast<const uint4*>(vsrc + c * N), v1 = *reinterpret_cast<const uint4*>(vsrc + half + c * N);
   float lo[N], hi[N], cs[N], sn[N], olo[N], ohi[N];
   unpack16<T>(*reinterpret_cast<const uint4*>(ksrc + c * N), lo);
   unpack16<T>(*reinterpret_cast<const uint4*>(ksrc + half + c * N), hi);
@@ -109,8 +111,8 @@ __global__ void __launch_bounds__(256) rope_store_kernel(
   }
   *reinterpret_cast<uint4*>(kd + c * N) = pack16<T>(olo);
   *reinterpret_cast<uint4*>(kd + half + c * N) = pack16<T>(ohi);
-  *reinterpret_cast<uint4*>(vd + c * N) = *reinterpret_cast<const uint4*>(vsrc + c * N);
-  *reinterpret_cast<uint4*>(vd + half + c * N) = *reinterpret_cast<const uint4*>(vsrc + half + c * N);
+  *reinterpret_cast<uint4*>(vd + c * N) = v0;
+  *reinterpret_cast<uint4*>(vd + half + c * N) = v1;
 }
 
 }  // namespace

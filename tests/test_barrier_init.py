@@ -12,8 +12,8 @@ INIT = re.compile(r"\bmbar_init\(|mbarrier\.init")
 USE = re.compile(r"\b(?:rc_)?mbar_(?:wait|arrive|expect_tx)\b|\btma_load\w*\(|\bcp_async_arrive\(|\btc_commit\(")
 
 
-def _kernels(text):
-    """(name, body) of every __global__ function."""
+def kernels(text):
+    """(name, signature, body) of every __global__ function."""
     text = re.sub(r"//[^\n]*", "", text)
     for m in re.finditer(r"__global__", text):
         head = text[m.start():text.index("{", m.start())]
@@ -24,7 +24,7 @@ def _kernels(text):
             depth += (text[end] == "{") - (text[end] == "}")
             if depth == 0:
                 break
-        yield re.search(r"(\w+)\s*\(", re.sub(r"__launch_bounds__\s*\((?:[^()]|\([^()]*\))*\)|__global__|template\s*<[^>]*>", "", head)).group(1), text[at:end]
+        yield re.search(r"(\w+)\s*\(", re.sub(r"__launch_bounds__\s*\((?:[^()]|\([^()]*\))*\)|__global__|template\s*<[^>]*>", "", head)).group(1), head, text[at:end]
 
 
 def _unguarded(body):
@@ -45,7 +45,7 @@ def _unguarded(body):
 
 
 FOUND = [pytest.param(body, id=f"{os.path.basename(path)}:{name}") for path in sorted(glob.glob(os.path.join(CSRC, "*.cu")))
-         for name, body in _kernels(open(path).read()) if INIT.search(body)]
+         for name, _, body in kernels(open(path).read()) if INIT.search(body)]
 
 
 def test_the_kernels_were_found():
