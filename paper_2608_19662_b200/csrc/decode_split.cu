@@ -138,7 +138,8 @@ __device__ __forceinline__ void bar_consumers() { asm volatile("bar.sync 1, %0;"
 
 // Pages of item `it`.  An item without a readable row still counts one page, so that its (zero)
 // output is written by somebody.  (A gathered page keeps its CTA longer than one that TMA brings, but
-// both variants deal alike: the same rows give the same bits whichever way they come.)
+// both variants deal alike: with the same max_res_pages, which bounds the number of CTAs, the same rows give
+// the same bits whichever way they come.)
 struct ItemPages { int n_res, n_hist, total, res_len, hist_len, r0; };
 template <bool GATHER>
 __device__ __forceinline__ ItemPages item_pages(const DecParams& p, int it) {

@@ -1,34 +1,40 @@
-"""Compaction where its counting and page tables can go wrong: resource starts at every byte offset, lengths
-around the 16-byte loads, more resources than the cluster has warps, more routes than threads."""
+"""Compaction where its three kernels change their way: the count kernel's 4096 blocks, the plan's warp per
+route up to 32 routes, thread per route beyond and second round of its 1024 threads, the gather's passes of 2048
+tokens and its number of blocks per pair (fewer where only indices are wanted); resource starts at every byte
+offset."""
 import numpy as np
 import pytest
 import torch
 
 from oracle import recache_oracle as orc
-from paper_2608_19662_b200 import PAGED
+from paper_2608_19662_b200 import PACKED, PAGED
 from paper_2608_19662_b200 import workloads as wl
 
-from pipeline import gpu_compact, make_ctx, oracle_rows
+from pipeline import dev, gpu_compact, make_ctx, oracle_rows
 
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("lens,gap,requests", [
-    (list(range(0, 70)), 1, 3),                       # every length to 69 at every alignment
-    ([1, 15, 16, 17, 31, 33, 511, 513], 5, 1),
-    ([3] * 300, 2, 2),                                # more resources than the cluster's 256 warps
-    ([40, 7], 0, 140),                                # 1120 routes: a second chunk of the plan's 1024 threads
+@pytest.mark.parametrize("lens,gap,requests,groups", [
+    (list(range(0, 70)), 1, 3, 8),                    # every length to 69 at every alignment
+    ([1, 15, 16, 17, 31, 33, 511, 513], 5, 1, 8),     # few pairs: eight blocks copy each, one where only indices are wanted
+    ([3] * 300, 2, 2, 8),                             # lists of many 32-resource steps, with a remainder
+    ([40, 7], 0, 140, 8),                             # 1120 routes: a second round of the plan's 1024 threads
+    ([70, 3, 129], 0, 32, 1),                         # 32 routes: a warp for each
+    ([70, 3, 129], 0, 33, 1),                         # 33: a thread for each; lists of one step of four, cut short
+    ([2047, 2048, 2049, 4097], 3, 1, 2),              # around the gather's passes
+    ([1, 2] * 2100, 0, 1, 2),                         # 4200 resources for the count's 4096 blocks
 ])
-def test_counts_and_tables(lens, gap, requests):
-    sh = wl.Shape(8, 8, 64, 1e4, "bf16")
+def test_counts_and_tables(lens, gap, requests, groups):
+    sh = wl.Shape(groups, groups, 64, 1e4, "bf16")
     rng = np.random.default_rng([len(lens), requests])
     pool = wl.pack_resources(sh, 5, lens, [rng.integers(0, 2, n).astype(np.uint8) for n in lens], slot_gap=gap, bulk=True)
     pool.keep[:] = np.where(pool.keep > 0, rng.integers(1, 256, pool.keep.shape), 0)     # any nonzero byte keeps
     lists = [[int(x) for x in rng.permutation(len(lens))] for _ in range(requests)]
-    vis = [rng.integers(0, 2, (8, len(x))).astype(np.uint8) for x in lists]
+    vis = [rng.integers(0, 2, (groups, len(x))).astype(np.uint8) for x in lists]
     req = wl.make_requests(sh, 9, pool, lists, vis, [1] * requests)
-    kc = wl.normal(1, (8, pool.pool_tokens, 64), sh.torch_dtype).cuda()
-    vc = wl.normal(2, (8, pool.pool_tokens, 64), sh.torch_dtype).cuda()
+    kc = wl.normal(1, (groups, pool.pool_tokens, 64), sh.torch_dtype).cuda()
+    vc = wl.normal(2, (groups, pool.pool_tokens, 64), sh.torch_dtype).cuda()
     rc = make_ctx(sh, max_pos=4096)
     rows = oracle_rows(pool, req)
     flat = [r for per in rows for r in per]
@@ -36,6 +42,12 @@ def test_counts_and_tables(lens, gap, requests):
     out = gpu_compact(rc, pool, req, kc, vc, capacity=int(cu[-1]) + 1)
     assert np.array_equal(out["route_cu"].cpu().numpy(), cu)
     assert np.array_equal(out["route_idx"].cpu().numpy()[:cu[-1]], np.concatenate(flat))
+    for name, cache in (("k_out", kc), ("v_out", vc)):
+        rows_of = torch.cat([cache[i % groups][torch.from_numpy(np.asarray(r, np.int64)).cuda()] for i, r in enumerate(flat)])
+        assert torch.equal(out[name][:cu[-1]].view(torch.int16), rows_of.view(torch.int16))
+    only = [torch.full_like(out[name], -7) for name in ("route_cu", "route_idx")]             # the index list alone
+    rc.compact_routes(kc, vc, dev(pool.keep), dev(req.res_off), dev(req.res_slot), dev(req.res_len), dev(req.vis), PACKED, *only, None, None)
+    assert torch.equal(only[0], out["route_cu"]) and torch.equal(only[1][:cu[-1]], out["route_idx"][:cu[-1]])
     n_pages = [(len(r) + 63) // 64 for r in flat]
     free = rng.permutation(sum(n_pages) + 3).astype(np.int32)
     paged = gpu_compact(rc, pool, req, kc, vc, mode=PAGED, capacity=int(cu[-1]) + 1, n_pool_pages=len(free), free_pages=free,

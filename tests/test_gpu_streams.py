@@ -1,8 +1,8 @@
 """Two contexts driven from two streams at the same time give the same results
 as one after the other, and back-to-back calls that reuse one workspace on one
-stream stay ordered: the work list of the tensor-core attention is built on a
-second stream of the context (forked from and joined to the caller's stream by
-events), which must not be visible from outside."""
+stream stay ordered: a call's first kernel, which also builds the work list of its
+attention, comes up while the last kernel of the call before still runs and uses
+the workspace."""
 import numpy as np
 import pytest
 import torch
