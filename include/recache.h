@@ -315,6 +315,8 @@ RECACHE_API recache_status recache_attend_prefill_gather(recache_ctx* ctx,
  * If k_new/v_new ([B][G][d], pre-rotation) are given, the current token's
  * rotated key and value are first written as history row hist_len[it]-1; pass
  * NULL when the caller has appended them already.  hist_len >= 1 always.
+ * (A page belongs to one item: a row that the call appends for one item is not
+ * seen by the others of the same call.)
  *   q [B][Hq][d] pre-rotation;  out_o [B][Hq][d] of out_dtype.
  */
 RECACHE_API recache_status recache_attend_decode(recache_ctx* ctx,

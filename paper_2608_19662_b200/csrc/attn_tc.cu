@@ -8,8 +8,8 @@
 //
 //   warps 0-3    softmax of tile A    warps 4-7  softmax of tile B
 //   warp  8      TMA producer         warp  9    tcgen05.mma issuer (+ TMEM alloc)
-//   warp  10     scheduler: draws work items from a global counter and publishes
-//                them through a two-slot ring in shared memory
+//   warp  10     scheduler: draws work items from a global counter (split launch:
+//                walks the CTA's range of the K/V tiles) and publishes them through a two-slot ring in shared memory
 //   warp  11     idle (completes the third warpgroup)
 //   warps 12-15  epilogue: O of a finished tile goes from tensor memory to HBM
 //                while the softmax warps already rotate the next item's Q; in
@@ -30,8 +30,9 @@
 // causal rows of the sequence itself up to the tile pair's last token.  The
 // query rows are rotated in shared memory after the TMA load (position = pos0 +
 // token index) and rounded to bf16, so no rotated copy of Q ever touches HBM.
-// Tiles are aligned to the sequence start, never to the batch: a resource gives
-// bit-identical outputs whatever else is in the launch.
+// Tiles are aligned to the sequence start, never to the batch: a resource, and a first turn,
+// gives bit-identical outputs whatever else is in the launch.  (The items of a later turn may
+// be split, see rc_plan_split; the cuts follow from the lengths of the whole launch.)
 #include <cuda.h>
 
 #include "tile_plan.cuh"

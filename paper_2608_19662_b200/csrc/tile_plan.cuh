@@ -106,15 +106,15 @@ __device__ __forceinline__ void rc_plan_scan_bins(RcPlanSmem& sh) {
 // edge where it would leave a part of fewer than two tiles, or a part whose first tile some row of
 // the pair does not see.  Taken only where the longest CTA gets shorter by more than the second
 // beginning (two units) and the merge (six: 6-10 us, a unit taking 1.8) cost: 8 conversations with 300-2048
-// rows of history (88 items of 8-24 tiles) take 50 us instead of 57; measured with route rows in the place of a
-// history: one request of 2048 tokens over a long
-// tool set (256 items of 58-73 tiles, else two rounds of 148 CTAs) 281 instead of 291; 8 conversations of 250
-// tokens over 4000 rows (256 items of 36) would take 159 instead of 152.  Whole items of a sequence also walk
-// its K/V in step and read it from L2, parts do not, which costs a fifth where the keys and values of the launch
-// are more than L2 holds and three or more items share them: 2048 tokens over 14,000 / 20,000 rows a group (57 /
-// 82 MB) 404 / 572 us split and 424 / 583 whole, but over 40,000 (164 MB) 1170 and 1120, and 4 x 512 tokens over
-// 24,000 each 750 and 693.  Encoding is never split: a resource's result must not depend on what is encoded
-// beside it.  False: not worth it.
+// rows of history (88 items of 8-24 tiles) take 50 us instead of 57.  The other figures were taken with route
+// rows in the place of a history: one request of 2048 tokens over a long tool set (256 items of 58-73 tiles,
+// else two rounds of 148 CTAs) 281 instead of 291 us; 8 conversations of 250 tokens over 4000 rows (256 items
+// of 36) would take 159 instead of 152.  Whole items of a sequence also walk its K/V in step and read it from
+// L2, parts do not, which costs a fifth where the keys and values of the launch are more than L2 holds and
+// three or more items share them: 2048 tokens over 14,000 / 20,000 rows a group (57 / 82 MB) 404 / 572 us split
+// and 424 / 583 whole, but over 40,000 (164 MB) 1170 and 1120, and 4 x 512 tokens over 24,000 each 750 and 693.
+// Encoding and first turns are never split: a resource's result must not depend on what is encoded beside it,
+// nor a first turn's on whether its rows are packed or gathered.  False: not worth it.
 __device__ __forceinline__ bool rc_plan_split(const RcPlan& p, RcPlanSmem& sh, int n_work) {
   const int tid = threadIdx.x, n_thr = blockDim.x;
   const int32_t* tiles = p.order + RC_SORT_MAX;
