@@ -25,7 +25,7 @@
 //                transposed ldmatrix fragments of the V page.
 // The current token's key and value (k_new / v_new) are appended by the warp that consumes the
 // item's last history page: into the page in HBM, and into the copy in shared memory, which was
-// loaded before the row existed.
+// loaded before the row existed.  (With many items to a CTA by a launch of its own, see the launch.)
 // The consumer warps' partial (max, sum, O) are merged through shared memory.  An item that lies
 // inside one CTA's range is written out there; the parts of one that spans several go to the
 // workspace (at most two per CTA: one for an item that began in an earlier CTA, one for an item
@@ -682,6 +682,14 @@ cudaError_t rc_launch_decode_split(const recache_ctx* ctx, const DecodeArgs& a, 
   // One sequence: its items have the history in common, so equal shares need no look at the lengths
   // (0.8 us of a step of 7).
   if (a.batch == 1 && (unsigned)G <= grid) { p.per_item = (int)grid / G; grid = (unsigned)(p.per_item * G); }
+  // Appending holds an item's consumers up by about a microsecond, a launch that appends for all takes 4-8 us:
+  // 512 items (64 sequences of 200 rows, 8 groups) 2.0 us here and 8.0 there, 1024 items 6.8 and 4.1, 8192 items
+  // 41 and 9; so up to four items a CTA.
+  if (a.k_new && p.n_items > 4 * grid_ctas(ctx)) {
+    const cudaError_t e = rc_launch_decode_append(ctx, a, st);
+    if (e != cudaSuccess) return e;
+    p.k_new = p.v_new = nullptr;
+  }
   auto run = [&](auto type, auto gathers) {
     using TO = decltype(type);
     constexpr bool GATHER = decltype(gathers)::value;

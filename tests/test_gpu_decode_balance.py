@@ -39,6 +39,7 @@ def _batch(rng, sh, res_rows, hist_rows):
     (2, 2, 5, (1, 130), (127, 129)),     # one head per group
     (16, 8, 40, (0, 200), (1, 700)),     # ragged: 320 items, ranges that begin and end inside items
     (8, 8, 70, (0, 64), (1, 64)),        # more items than CTAs and threads, one or two pages each
+    (8, 8, 80, (0, 64), (1, 130)),       # 640 items: more than four a CTA, appended by a launch of their own
 ])
 def test_ragged_pages_match_oracle_and_append(hq, groups, batch, res, hist):
     sh = wl.Shape(hq, groups, 128, 1e6, "bf16")
@@ -62,6 +63,8 @@ def test_ragged_pages_match_oracle_and_append(hq, groups, batch, res, hist):
     changed = (d_kp.cpu().view(torch.int16) != kp.view(torch.int16)).any(-1).sum().item()
     assert changed == items
     assert max_abs(d_kp, kr) < 4e-2          # 1 bf16 ulp of a key in [4, 8): 3.1e-2
+    many = items > 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert rc.kernel_times()["decode_append"][1] == int(many)
     assert rc.poll_status() == 0
 
 
