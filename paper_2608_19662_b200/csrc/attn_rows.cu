@@ -3,11 +3,13 @@
 // does not cover.
 //
 // One CTA owns a block of up to 8 query rows (8 / s consecutive tokens of a
-// sequence x the s query heads of a group).  Its eight warps deal the keys out
-// in tiles of 32 (tile t belongs to warp t % 8) and each runs an online softmax
-// of its own over all of them; the partial (max, sum, O) are merged through
-// shared memory at the end, so nothing synchronises in between.  For the scores
-// four lanes share a key's row, so that a warp's 16-byte loads touch 8 lines, not
+// sequence x the s query heads of a group).  The keys are dealt in tiles of 32 to
+// eight parts (tile t belongs to part t % 8), each with an online softmax of its
+// own over all its tiles; the parts' (max, sum, O) are merged through shared
+// memory at the end, so nothing synchronises in between.  A warp computes a part,
+// or two warps four each: where there are blocks enough to fill the GPU many times
+// and keys for a few tiles only, eight warps mostly wait for one of them.  For the
+// scores four lanes share a key's row, so that a warp's 16-byte loads touch 8 lines, not
 // 32 (with a key to a lane the loads' tag lookups alone took 512 cycles a tile),
 // and a query load from shared memory serves 16 FMA; for P V a lane owns d / 32 columns and the
 // probabilities are broadcast, with the value rows loaded eight at a time ahead
@@ -15,9 +17,10 @@
 // is a block's start (a chain of dependent loads) and half FMA issue.  A warp per
 // query row, which read every key row once per query row, took 69 us each for 1,250
 // tokens in six resources and for the 160-token turn over them (4 / 2 heads of 64);
-// this kernel takes 21 and 11 us, and the pass of encode, compaction and turn 46 us
+// this kernel takes 20 and 11 us, and the pass of encode, compaction and turn 44 us
 // instead of 155 (the rows' softmaxes one after the other, blocks light to heavy: 53;
-// four warps to a CTA: 55; 16 rows to a CTA: 80).
+// four warps to a CTA: 55; 16 rows to a CTA: 80).  It was the faster one for hundreds of
+// sequences of up to 32 keys (1000 of 1-8 29 us there, 37 here; of 17-32 147 and 146, 32 / 8 heads of 128 1907 and 2110).
 //
 // Key set of a row (token t of sequence b at local index j, head h, group g):
 //   route part : rows route_cu[b*G+g] .. route_cu[b*G+g+1]-1 of k_route/v_route,
@@ -30,11 +33,13 @@
 // not depend on what else is in the launch.
 #include <float.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace {
 
-constexpr int WARPS = 8, ROWS = 8, KT = 32, VB = 8;    // VB: value rows loaded at a time
+constexpr int PARTS = 8, ROWS = 8, KT = 32, VB = 8;    // PARTS: key tile t belongs to part t % PARTS of its row; VB: value rows loaded at a time
 
 // N consecutive elements as floats, N * sizeof(T) a multiple of 4
 template <typename T, int N> __device__ __forceinline__ void load_f(const T* p, float* f);
@@ -65,15 +70,17 @@ template <> __device__ __forceinline__ void load_f<__nv_bfloat16, 8>(const __nv_
 
 template <int D> struct Smem {
   float q[ROWS][D];
-  union {
-    float p[WARPS][KT][ROWS];                            // probabilities, key-major
-    float part[WARPS][ROWS][D];                          // partial O
-  };
-  float m[WARPS][ROWS], l[WARPS][ROWS];
+  union Part {
+    float p[KT][ROWS];                                   // probabilities of the tile at hand, key-major
+    float o[ROWS][D];                                    // at the end: the part's O
+  } part[PARTS];
+  float m[PARTS][ROWS], l[PARTS][ROWS];
 };
 
-template <typename T, typename TO, int D>
-__global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
+// WARPS warps to a CTA, each of which takes PARTS / WARPS parts, one after the other: which warp computes a
+// part makes no difference to any result.
+template <typename T, typename TO, int D, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, 16 / WARPS) attn_rows_kernel(
     const T* q, TO* __restrict__ o, const int32_t* cu, int n_seq, int total,
     const int32_t* pos0, const int32_t* slot,
     const T* k_self, const T* v_self, int64_t self_rows,
@@ -138,38 +145,34 @@ __global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
   }
   __syncthreads();
 
-  constexpr int CPL = D / 32;   // output columns per lane: CPL * lane ..
-  float acc[ROWS][CPL], m[ROWS], l[ROWS];                // l: this lane's keys only
-#pragma unroll
-  for (int r = 0; r < ROWS; ++r) {
-    m[r] = -INFINITY; l[r] = 0.f;
-#pragma unroll
-    for (int c = 0; c < CPL; ++c) acc[r][c] = 0.f;
+  // ---- the row's keys: the route's packed rows, or (encoding behind a shared prefix) the group's prefix
+  // rows; then the sequence's own.  A range outside the route tensors (e.g. after a compaction that
+  // overflowed its capacity) is reported and read as an empty route. ----
+  int n_route = 0;
+  if (route_cu || prefix_len > 0) {
+    if (route0 >= 0 && route1 >= route0 && (int64_t)route1 <= route_rows) n_route = route1 - route0;
+    else if (threadIdx.x == 0) rc_set_status(status, RECACHE_DEV_OVERFLOW);
   }
-  float (*ps)[ROWS] = sh.p[warp];
+  const int n_self = H + tok0 + n_tok, route_tiles = (n_route + KT - 1) / KT, n_tiles = route_tiles + (n_self + KT - 1) / KT;
+  const int n_parts = min(PARTS, n_tiles);               // the others have no tile
 
-  int t = 0;                                             // key tiles so far
-  for (int seg = 0; seg < 2; ++seg) {
-    const T* kb; const T* vb; int n;
-    if (seg == 0) {
-      if (!route_cu && prefix_len <= 0) continue;
-      // the route's packed rows, or (encoding behind a shared prefix) the group's prefix rows
-      const int r0 = route0, r1 = route1;
-      // a range outside the route tensors (e.g. after a compaction that overflowed its capacity)
-      // is reported and read as an empty route
-      if (r0 < 0 || r1 < r0 || (int64_t)r1 > route_rows) {
-        if (threadIdx.x == 0) rc_set_status(status, RECACHE_DEV_OVERFLOW);
-        continue;
-      }
-      kb = k_route + (int64_t)r0 * D; vb = v_route + (int64_t)r0 * D; n = r1 - r0;
-    } else {
-      kb = k_self + ((int64_t)g * self_rows + base) * D;
-      vb = v_self + ((int64_t)g * self_rows + base) * D;
-      n = H + tok0 + n_tok;
+  constexpr int CPL = D / 32;   // output columns per lane: CPL * lane ..
+  for (int w = warp; w < n_parts; w += WARPS) {
+    float acc[ROWS][CPL], m[ROWS], l[ROWS];              // l: this lane's keys only
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+      m[r] = -INFINITY; l[r] = 0.f;
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) acc[r][c] = 0.f;
     }
-    const int all_see = seg == 0 ? n : H + tok0 + 1;     // keys that every row of the block sees
-    for (int k0 = 0; k0 < n; k0 += KT, ++t) {
-      if (t % WARPS != warp) continue;
+    float (*ps)[ROWS] = sh.part[w].p;
+    for (int t = w; t < n_tiles; t += PARTS) {
+      const bool own = t >= route_tiles;                 // a tile of the sequence's own keys
+      const int k0 = (own ? t - route_tiles : t) * KT, n = own ? n_self : n_route;
+      const int64_t row0 = own ? (int64_t)g * self_rows + base : (int64_t)route0;
+      const T* kb = (own ? k_self : k_route) + row0 * D;
+      const T* vb = (own ? v_self : v_route) + row0 * D;
+      const int all_see = own ? H + tok0 + 1 : n;        // keys that every row of the block sees
       const int cnt = min(KT, n - k0);
       // ---- scores: four lanes share eight keys' rows, each a quarter of their 16-byte chunks ----
       const int part = lane & 3, key8 = lane >> 2;
@@ -225,7 +228,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
       int tok = 0, head = 0;                             // of row r
 #pragma unroll
       for (int r = 0; r < ROWS; ++r) {
-        const int lim = seg == 0 ? n : min(n, H + tok0 + tok + 1);
+        const int lim = own ? min(n, H + tok0 + tok + 1) : n;
         if (++head == s) { head = 0; ++tok; }
         mx[r] = v1[r] = kk < lim ? v1[r] * scale : -INFINITY;
       }
@@ -268,14 +271,14 @@ __global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
           if (odd) {
 #pragma unroll 1
             for (int j = max(all_see - k0, j0); j < min(j0 + VB, cnt); ++j) {
-              float w[CPL];
-              load_f<T, CPL>(vp + (int64_t)j * D, w);
+              float u[CPL];
+              load_f<T, CPL>(vp + (int64_t)j * D, u);
 #pragma unroll
               for (int c = 0; c < CPL; ++c) {
-                if (fabsf(w[c]) <= FLT_MAX) continue;
+                if (fabsf(u[c]) <= FLT_MAX) continue;
 #pragma unroll
                 for (int r = 0; r < ROWS; ++r)
-                  if (k0 + j <= H + tok0 + r / s) acc[r][c] = fmaf(ps[j][r], w[c], acc[r][c]);
+                  if (k0 + j <= H + tok0 + r / s) acc[r][c] = fmaf(ps[j][r], u[c], acc[r][c]);
               }
             }
           }
@@ -295,27 +298,24 @@ __global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
       }
       __syncwarp();
     }
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+#pragma unroll
+      for (int off = 16; off; off >>= 1) l[r] += __shfl_xor_sync(0xffffffffu, l[r], off);
+      if (lane == 0) { sh.m[w][r] = m[r]; sh.l[w][r] = l[r]; }
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) sh.part[w].o[r][CPL * lane + c] = acc[r][c];
+    }
   }
 
-  // ---- merge the warps' partial results ----
-#pragma unroll
-  for (int r = 0; r < ROWS; ++r) {
-#pragma unroll
-    for (int off = 16; off; off >>= 1) l[r] += __shfl_xor_sync(0xffffffffu, l[r], off);
-    if (lane == 0) { sh.m[warp][r] = m[r]; sh.l[warp][r] = l[r]; }
-  }
-  __syncthreads();                                       // the probabilities make room for the partial O
-#pragma unroll
-  for (int r = 0; r < ROWS; ++r)
-#pragma unroll
-    for (int c = 0; c < CPL; ++c) sh.part[warp][r][CPL * lane + c] = acc[r][c];
+  // ---- merge the parts ----
   __syncthreads();
   for (int r = warp; r < n_rows; r += WARPS) {
-    float mw = lane < WARPS ? sh.m[lane][r] : -INFINITY, M = mw;
+    float mw = lane < n_parts ? sh.m[lane][r] : -INFINITY, M = mw;
 #pragma unroll
     for (int off = 16; off; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
     const float f = mw == -INFINITY ? 0.f : expf(mw - M);
-    float sum = lane < WARPS ? sh.l[lane][r] * f : 0.f;
+    float sum = lane < n_parts ? sh.l[lane][r] * f : 0.f;
 #pragma unroll
     for (int off = 16; off; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
     const float inv = 1.f / sum;                         // (the self part always holds the token itself, so sum > 0)
@@ -324,7 +324,10 @@ __global__ void __launch_bounds__(WARPS * 32, 2) attn_rows_kernel(
     for (int c = 0; c < CPL; ++c) {
       float v = 0.f;
 #pragma unroll
-      for (int w = 0; w < WARPS; ++w) v = fmaf(sh.part[w][r][lane + 32 * c], __shfl_sync(0xffffffffu, f, w), v);
+      for (int w = 0; w < PARTS; ++w) {
+        const float fw = __shfl_sync(0xffffffffu, f, w);
+        if (w < n_parts) v = fmaf(sh.part[w].o[r][lane + 32 * c], fw, v);
+      }
       orow[lane + 32 * c] = rc_from_float<TO>(v * inv);
     }
   }
@@ -337,12 +340,24 @@ cudaError_t launch(const recache_ctx* ctx, const AttnRowsArgs& a, cudaStream_t s
   const dim3 grid((unsigned)(a.total / TQ + a.n_seq), (unsigned)G);
   const float scale = (float)(1.0 / sqrt((double)d));
   RcLaunchScope scope(ctx, a.route_cu ? RC_K_PREFILL_ATTN : RC_K_ENCODE_ATTN, st);
-  auto go = [&](auto kernel, size_t smem) {
-    return rc_launch_overlapped(kernel, grid, WARPS * 32, smem, st, (const T*)a.q, (TO*)a.o, a.cu, a.n_seq, a.total, a.pos0, a.slot, (const T*)a.k_self,
+  auto go = [&](auto kernel, size_t smem, int warps) {
+    return rc_launch_overlapped(kernel, grid, warps * 32, smem, st, (const T*)a.q, (TO*)a.o, a.cu, a.n_seq, a.total, a.pos0, a.slot, (const T*)a.k_self,
                                 (const T*)a.v_self, a.self_rows, (const T*)a.k_route, (const T*)a.v_route, a.route_cu, a.prefix_len, a.hist,
                                 a.route_rows, Hq, G, (const float*)ctx->cos_tab, (const float*)ctx->sin_tab, ctx->desc.max_pos, scale, ctx->status);
   };
-  return d == 64 ? go(attn_rows_kernel<T, TO, 64>, sizeof(Smem<64>)) : go(attn_rows_kernel<T, TO, 128>, sizeof(Smem<128>));
+  // Two warps to a CTA (6-8 CTAs to an SM instead of 2) where the blocks fill the GPU three times over with eight and a row
+  // has few keys; what the host knows of their number are averages and capacities, which is enough for a rule
+  // that no result depends on.  Eight warps / two, us: 1000 resources of 33-64 tokens 601 / 288 (4 / 2 heads of 64, fp32)
+  // and 6851 / 4252 (32 / 8 of 128), 300 of 128-256 739 / 531 and 8646 / 8326, but 16 of 150-1200 294 / 320 and
+  // 3509 / 4057; turns of 1-8 tokens over 100 rows 107 / 87 and 945 / 1021; 236 blocks of 50 keys 14.8 / 21.5, 976 34.7 / 25.1.
+  const int64_t blocks = (int64_t)grid.x * G, keys = a.total / a.n_seq / 2 + a.prefix_len + (a.route_cu ? a.route_rows / ((int64_t)a.n_seq * G) : 0) +
+                                                     (a.hist ? a.self_rows / a.n_seq : 0);
+  const bool few = blocks >= 6 * (ctx->sm_count > 0 ? ctx->sm_count : 148) && keys <= (d == 64 ? 200 : 96);
+  auto pick = [&](auto head) {
+    constexpr int D = decltype(head)::value;
+    return few ? go(attn_rows_kernel<T, TO, D, 2>, sizeof(Smem<D>), 2) : go(attn_rows_kernel<T, TO, D, 8>, sizeof(Smem<D>), 8);
+  };
+  return d == 64 ? pick(std::integral_constant<int, 64>()) : pick(std::integral_constant<int, 128>());
 }
 
 }  // namespace

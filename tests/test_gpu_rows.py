@@ -6,7 +6,7 @@ import torch
 
 from paper_2608_19662_b200 import workloads as wl
 
-from pipeline import gpu_compact, gpu_encode, gpu_prefill, make_ctx, max_abs, oracle_encode, oracle_prefill, oracle_rows
+from pipeline import dev, gpu_compact, gpu_encode, gpu_prefill, make_ctx, max_abs, oracle_encode, oracle_prefill, oracle_rows
 
 pytestmark = pytest.mark.gpu
 
@@ -61,3 +61,25 @@ def test_values_that_are_not_finite_reach_only_the_rows_that_see_them(hq, g, d, 
     assert value != value or (p[:40, :, col] == value).all()
     p[:40, :, col] = 0
     assert torch.isfinite(p).all() and rc.poll_status() == 0
+
+
+@pytest.mark.parametrize("hq,g,d,dtype,tol", [(4, 2, 64, "f32", 1e-5), (32, 8, 128, "f32", 1e-5), (8, 8, 64, "bf16", 1e-2), (5, 1, 128, "bf16", 1e-2)])
+def test_many_short_sequences(hq, g, d, dtype, tol):
+    """A launch with blocks enough for two warps each: the oracle's results, and for a resource the same bits as
+    encoded alone, by eight warps (one of them has more key tiles than there are parts)."""
+    sh = wl.Shape(hq, g, d, 1e4, dtype)
+    rng = np.random.default_rng(hq)
+    lens = rng.integers(0, 40, 700).astype(np.int32)
+    lens[[3, 350]] = 290, 65
+    pool = wl.pack_resources(sh, 11, lens, [np.ones(int(n), np.uint8) for n in lens], bulk=True)
+    rc = make_ctx(sh, max_pos=1024)
+    o, kc, vc = gpu_encode(rc, pool)
+    ref, _, _ = oracle_encode(pool)
+    assert max_abs(o, ref) < tol
+    for i in (3, 350, 351):
+        a, b = int(pool.cu_seqlens[i]), int(pool.cu_seqlens[i + 1])
+        one = torch.zeros((g, max(b - a, 1), d), dtype=sh.torch_dtype, device="cuda")
+        alone = rc.encode_resources(dev(pool.q[a:b]), dev(pool.k[a:b]), dev(pool.v[a:b]), dev(np.array([0, b - a], np.int32)), max(b - a, 1),
+                                    dev(np.zeros(1, np.int32)), one, one.clone(), out_dtype=torch.float32)
+        assert torch.equal(alone, o[a:b])
+    assert rc.poll_status() == 0
