@@ -33,17 +33,13 @@
 // Tiles are aligned to the sequence start, never to the batch: a resource, and a first turn,
 // gives bit-identical outputs whatever else is in the launch.  (The items of a later turn may
 // be split, see rc_plan_split; the cuts follow from the lengths of the whole launch.)
-#include <cuda.h>
+#include "tc_common.cuh"
 
-#include "tile_plan.cuh"
+using namespace rc_tc;
 
 namespace {
 
-constexpr int D = 128;
-constexpr int TILE_N = RC_TILE_N;
 constexpr int NSTAGE = 2;
-constexpr int BOX_BYTES = 16384;   // [128 rows][64 bf16], 128-byte swizzle
-constexpr int TILE_BYTES = 32768;  // two boxes: head_dim halves
 constexpr int NTHREADS = 512;
 // Registers per thread of the softmax warps and of the other eight; 256 * (softmax + aux) = 65536.  Epilogue
 // warps that gather and schedulers that know about split items spill in 32 (8 zero-copy turns: 84.0 us with 32,
@@ -71,172 +67,14 @@ static_assert(B_COUNT <= 32, "barrier area");
 
 constexpr uint32_t COL_S = 0, COL_O = 256;           // + 128 * tile
 
-constexpr uint32_t WAIT_PROBES = 1u << 21;           // ~2.8 s of suspended probes: a wait this long is a bug, not load
-
-struct TcParams : RcPlan {
-  // gather mode: route row n of group g is row route_idx[n] of gather_k / gather_v ([G][pool_tokens][128] bf16)
-  const uint8_t* gather_k; const uint8_t* gather_v; const int32_t* route_idx; int64_t pool_tokens;
-  void* out;
-  float* part_o; float2* part_ml;   // split launch: O [slot][tile][128 rows][128], (maximum in log2 units, sum) [slot][tile][128 rows]
-  const float* cos_tab; const float* sin_tab; int max_pos;
-  float scale_log2;
-};
-
-// ------------------------------------------------------------------ PTX --
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
 // Bounded wait: see rc_mbar_wait (no location word here).
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status) {
   rc_mbar_wait<WAIT_PROBES, 0>(bar, parity, abort_flag, status);
 }
 
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
-  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-               ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1) : "memory");
-}
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2) {
-  asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-               ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2) : "memory");
-}
-// 16-byte asynchronous copy global -> shared; src_bytes = 0 writes zeros instead
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(reinterpret_cast<uint64_t>(src)), "r"(src_bytes) : "memory");
-}
-// one arrival on the barrier once all earlier cp.async of this thread have landed (the barrier's
-// expected count already includes it)
-__device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
-  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
-}
-// plain bulk copy global -> shared (16-byte aligned, size a multiple of 16)
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(dst), "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
-  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
-}
 
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-// D[tmem] (+)= A * B with A in shared memory (mma_ss) or tensor memory (mma_ts); the 64-bit shared
-// memory descriptors advance by adds on their address field.
-__device__ __forceinline__ void mma_ss(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
-  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-               ::"r"(d), "l"(da), "l"(db), "r"(idesc), "r"(acc) : "memory");
-}
-__device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t db, uint32_t idesc, uint32_t acc) {
-  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-               ::"r"(d), "r"(a), "l"(db), "r"(idesc), "r"(acc) : "memory");
-}
-// one lane of a fully converged warp, chosen by the hardware
-__device__ __forceinline__ bool elect_one() {
-  uint32_t e;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
-  return e != 0;
-}
-
-#define RC_R32(r, o) "=r"(r[o + 0]), "=r"(r[o + 1]), "=r"(r[o + 2]), "=r"(r[o + 3]), "=r"(r[o + 4]), "=r"(r[o + 5]), \
-    "=r"(r[o + 6]), "=r"(r[o + 7]), "=r"(r[o + 8]), "=r"(r[o + 9]), "=r"(r[o + 10]), "=r"(r[o + 11]),               \
-    "=r"(r[o + 12]), "=r"(r[o + 13]), "=r"(r[o + 14]), "=r"(r[o + 15]), "=r"(r[o + 16]), "=r"(r[o + 17]),           \
-    "=r"(r[o + 18]), "=r"(r[o + 19]), "=r"(r[o + 20]), "=r"(r[o + 21]), "=r"(r[o + 22]), "=r"(r[o + 23]),           \
-    "=r"(r[o + 24]), "=r"(r[o + 25]), "=r"(r[o + 26]), "=r"(r[o + 27]), "=r"(r[o + 28]), "=r"(r[o + 29]),           \
-    "=r"(r[o + 30]), "=r"(r[o + 31])
-#define RC_W32(r, o) "r"(r[o + 0]), "r"(r[o + 1]), "r"(r[o + 2]), "r"(r[o + 3]), "r"(r[o + 4]), "r"(r[o + 5]),       \
-    "r"(r[o + 6]), "r"(r[o + 7]), "r"(r[o + 8]), "r"(r[o + 9]), "r"(r[o + 10]), "r"(r[o + 11]), "r"(r[o + 12]),      \
-    "r"(r[o + 13]), "r"(r[o + 14]), "r"(r[o + 15]), "r"(r[o + 16]), "r"(r[o + 17]), "r"(r[o + 18]), "r"(r[o + 19]),  \
-    "r"(r[o + 20]), "r"(r[o + 21]), "r"(r[o + 22]), "r"(r[o + 23]), "r"(r[o + 24]), "r"(r[o + 25]), "r"(r[o + 26]),  \
-    "r"(r[o + 27]), "r"(r[o + 28]), "r"(r[o + 29]), "r"(r[o + 30]), "r"(r[o + 31])
-#define RC_LIST32_OUT "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}"
-#define RC_LIST32_IN "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32}"
-
-// 32 consecutive columns of this thread's lane
-#define TMEM_LD32(taddr, r, o) \
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 " RC_LIST32_OUT ", [%32];" : RC_R32(r, o) : "r"(taddr) : "memory")
-#define TMEM_ST32(taddr, r, o) \
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], " RC_LIST32_IN ";" ::"r"(taddr), RC_W32(r, o) : "memory")
-
-#define TMEM_LD16(taddr, r) \
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];" \
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), \
-                 "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]) : "r"(taddr) : "memory")
-
-// one 32-byte store (the address is 32-byte aligned)
-__device__ __forceinline__ void st_global_v8(void* ptr, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t e, uint32_t f,
-                                             uint32_t g, uint32_t h) {
-  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(ptr), "r"(a), "r"(b), "r"(c), "r"(d), "r"(e),
-               "r"(f), "r"(g), "r"(h) : "memory");
-}
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// Shared-memory matrix descriptors, 128-byte swizzle, 8-row groups 1024 bytes apart.
-//  K-major operand (rows = M or N index, 64 bf16 of K per 128-byte row): SBO = 1024.
-//  MN-major operand (rows = K index, 64 bf16 of N per row): SBO = 1024 between 8-row
-//  K groups, LBO = distance between 64-wide N chunks.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)((lbo_bytes >> 4) & 0x3FFF) << 16) |
-         ((uint64_t)((sbo_bytes >> 4) & 0x3FFF) << 32) | (1ull << 46) | (2ull << 61);
-}
-// kind::f16 instruction descriptor: fp32 accumulate, bf16 A and B, M = 128, N = 128
-constexpr uint32_t IDESC_BASE = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
-constexpr uint32_t IDESC_QK = IDESC_BASE;               // A, B K-major
-constexpr uint32_t IDESC_PV = IDESC_BASE | (1u << 16);  // B (= V) MN-major
-
-// Packed fp32 pairs (one instruction, two lanes of the FMA pipe).
-__device__ __forceinline__ void fma2(float& d0, float& d1, float a0, float a1, float b, float c) {
-  asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %4};\n\tmov.b64 rc, {%5, %5};\n\t"
-      "fma.rn.f32x2 rd, ra, rb, rc;\n\tmov.b64 {%0, %1}, rd;\n\t}"
-      : "=f"(d0), "=f"(d1) : "f"(a0), "f"(a1), "f"(b), "f"(c));
-}
-__device__ __forceinline__ void add2(float& d0, float& d1, float a0, float a1) {
-  asm("{\n\t.reg .b64 ra, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rd, {%0, %1};\n\tadd.rn.f32x2 rd, rd, ra;\n\t"
-      "mov.b64 {%0, %1}, rd;\n\t}"
-      : "+f"(d0), "+f"(d1) : "f"(a0), "f"(a1));
-}
-// d = a * b + c and d = a * b on pairs (one instruction each; same rounding as the scalar forms)
-__device__ __forceinline__ void fma2v(float& d0, float& d1, float a0, float a1, float b0, float b1, float c0, float c1) {
-  asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
-      "fma.rn.f32x2 rd, ra, rb, rc;\n\tmov.b64 {%0, %1}, rd;\n\t}"
-      : "=f"(d0), "=f"(d1) : "f"(a0), "f"(a1), "f"(b0), "f"(b1), "f"(c0), "f"(c1));
-}
-__device__ __forceinline__ void mul2v(float& d0, float& d1, float a0, float a1, float b0, float b1) {
-  asm("{\n\t.reg .b64 ra, rb, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
-      "mul.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
-      : "=f"(d0), "=f"(d1) : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
-}
-__device__ __forceinline__ float fmax3(float a, float b, float c) {
-  float d;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
-}
-__device__ __forceinline__ uint32_t pack2(float a, float b) {
-  __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<uint32_t*>(&p);
-}
-
-using Item = RcItem;
 enum { IT_NTILES = 0, IT_G, IT_SEQ0, IT_L, IT_TOK0, IT_KVEND, IT_POS0, IT_RA0, IT_LENA, IT_NA, IT_BVALID, IT_BASE_LO,
-       IT_BASE_HI, IT_H, IT_PART, IT_WORDS = 16 };
+       IT_BASE_HI, IT_H, IT_WORDS = 16 };
 
 // ---------------------------------------------------------------- kernel --
 // Persistent: a scheduler warp draws work indices from a global counter (the
@@ -245,7 +83,7 @@ enum { IT_NTILES = 0, IT_G, IT_SEQ0, IT_L, IT_TOK0, IT_KVEND, IT_POS0, IT_RA0, I
 // items through a two-slot ring in shared memory.
 // The next item's Q load, Q rotation and first K/V tiles overlap the current
 // item's last tiles and its epilogue.  Barrier phases run on across items.
-template <typename TO, bool ROT_SMEM, bool GATHER, bool SPLIT>
+template <typename TO, bool ROT_SMEM, bool GATHER>
 __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
                                                               const __grid_constant__ CUtensorMap tm_ks,
                                                               const __grid_constant__ CUtensorMap tm_vs,
@@ -305,14 +143,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
     const int* r = const_cast<const int*>(item_ring) + sl * IT_WORDS;   // (ordered by the barrier wait above and the arrive below)
     it.n_tiles = r[IT_NTILES]; it.g = r[IT_G]; it.seq0 = r[IT_SEQ0]; it.L = r[IT_L]; it.tok0 = r[IT_TOK0];
     it.kv_end = r[IT_KVEND]; it.pos0 = r[IT_POS0]; it.rA0 = r[IT_RA0]; it.lenA = r[IT_LENA]; it.nA = r[IT_NA];
-    it.b_valid = r[IT_BVALID]; it.H = r[IT_H]; it.part = SPLIT ? r[IT_PART] : -1;
+    it.b_valid = r[IT_BVALID]; it.H = r[IT_H];
     it.base = (int64_t)(((uint64_t)(uint32_t)r[IT_BASE_HI] << 32) | (uint32_t)r[IT_BASE_LO]);
     if (*abort_flag) it.n_tiles = -1;
     if (release) mbar_arrive(bar(B_IEMPTY + sl));
   };
 
   if (warp >= 12) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_AUX<GATHER || SPLIT>));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_AUX<GATHER>));
     // ===================== epilogue warps =====================
     // O of a finished query tile leaves tensor memory here, so that the softmax warps can go
     // straight to the next item's Q.  Warp 12 + q reads lanes 32 q .. 32 q + 31.
@@ -397,11 +235,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
           uint32_t orr[16];
           TMEM_LD16(t_o + 16 * ch, orr);
           tmem_wait_ld();
-          if (it.part >= 0) {
-            float* prow = p.part_o + ((int64_t)(it.part * 2 + x) * 128 + row) * D + 16 * ch;
-            st_global_v8(prow, orr[0], orr[1], orr[2], orr[3], orr[4], orr[5], orr[6], orr[7]);
-            st_global_v8(prow + 8, orr[8], orr[9], orr[10], orr[11], orr[12], orr[13], orr[14], orr[15]);
-          } else if (row_valid) {
+          if (row_valid) {
             if constexpr (sizeof(TO) == 4) {
 #pragma unroll
               for (int c = 0; c < 16; c += 8)
@@ -430,33 +264,17 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
       it = nx;
     }
   } else if (warp >= 8) {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_AUX<GATHER || SPLIT>));
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_AUX<GATHER>));
   if (warp == 10) {
     // ===================== scheduler =====================
     if (lane == 0) {
       const int total = p.header[0] * p.G;   // (a CTA without work publishes "no more work" at once)
       bool first = true;
-      const int n_split = SPLIT ? p.header[3] : 0;
-      int2 cur = make_int2(0, 0), end = make_int2(0, 0);
-      if ((int)blockIdx.x < n_split) { cur = p.start[blockIdx.x]; end = p.start[blockIdx.x + 1]; }
       for (uint32_t n = 0;; ++n) {
         const int sl = n & 1u;
         mbar_wait(bar(B_IEMPTY + sl), ((n >> 1) & 1u) ^ 1u, abort_flag, p.status);
         Item it;
-        it.part = -1;
-        for (; n_split > 0;) {   // the CTA's range of the K/V tiles, one item after the other
-          if (cur.x > end.x || (cur.x == end.x && cur.y >= end.y) || *abort_flag) { it.n_tiles = -1; break; }
-          const int w = cur.x, t0 = cur.y;
-          cur = make_int2(w + 1, 0);
-          if (!rc_load_item(p, w, it)) continue;
-          const int t1 = w == end.x ? min(end.y, it.n_tiles) : it.n_tiles;
-          if (t0 > 0 || t1 < it.n_tiles) it.part = 2 * (int)blockIdx.x + (t0 > 0 ? 0 : 1);
-          else it.part = -1;
-          // (counted from the part's first tile, everything below is the same as for a whole item)
-          it.n_tiles = t1 - t0; it.nA -= t0; it.rA0 += t0 * TILE_N; it.lenA -= t0 * TILE_N;
-          break;
-        }
-        for (; n_split == 0;) {   // CTA c starts with index c; every later index comes from the shared counter
+        for (;;) {   // CTA c starts with index c; every later index comes from the shared counter
           const int w = first ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(p.header + 1, 1);
           first = false;
           if (w >= total || *abort_flag) { it.n_tiles = -1; break; }
@@ -467,7 +285,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
         if (it.n_tiles > 0) {
           r[IT_G] = it.g; r[IT_SEQ0] = it.seq0; r[IT_L] = it.L; r[IT_TOK0] = it.tok0; r[IT_KVEND] = it.kv_end;
           r[IT_POS0] = it.pos0; r[IT_RA0] = it.rA0; r[IT_LENA] = it.lenA; r[IT_NA] = it.nA; r[IT_BVALID] = it.b_valid;
-          r[IT_H] = it.H; r[IT_PART] = it.part;
+          r[IT_H] = it.H;
           r[IT_BASE_LO] = (int)(uint32_t)(it.base & 0xffffffffll); r[IT_BASE_HI] = (int)(uint32_t)((uint64_t)it.base >> 32);
         }
         mbar_arrive(bar(B_IFULL + sl));
@@ -648,7 +466,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
     }
   }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX<GATHER || SPLIT>));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX<GATHER>));
     // ===================== softmax warpgroups =====================
     const int x = warp >> 2;                       // tile A or B
     const int row = threadIdx.x & 127;             // row of the tile = TMEM lane
@@ -656,6 +474,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
     const uint32_t t_s = tmem + lane_addr + COL_S + 128 * x;
     const uint32_t t_o = tmem + lane_addr + COL_O + 128 * x;
     const float c2 = p.scale_log2;
+    const uint64_t c2c2 = pair2(c2, c2);
     uint32_t item_n = 0, cnt = 0;                  // items seen; tiles this query tile has gone through
     uint32_t kv_n = 0, done_n = 0;                 // K/V tiles of all items so far; items this query tile took part in
 
@@ -692,25 +511,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
         for (int h = 0; h < s; ++h) {
           const int r = tok * s + h;
           uint8_t* qb = qt + r * 128 + ((c ^ (r & 7)) << 4);
-          const uint4 ulo = *reinterpret_cast<uint4*>(qb), uhi = *reinterpret_cast<uint4*>(qb + BOX_BYTES);
-          const uint32_t wlo[4] = {ulo.x, ulo.y, ulo.z, ulo.w}, whi[4] = {uhi.x, uhi.y, uhi.z, uhi.w};
-          uint32_t ol[4], oh[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float l0 = __uint_as_float(wlo[i] << 16), l1 = __uint_as_float(wlo[i] & 0xffff0000u);
-            const float h0 = __uint_as_float(whi[i] << 16), h1 = __uint_as_float(whi[i] & 0xffff0000u);
-            // lo' = lo cos - hi sin, hi' = hi cos + lo sin: the products with sin are rounded first
-            // (hi * (-sin) is exactly -(hi * sin)), as in the scalar form of the other kernels
-            float t0, t1, u0, u1, a0, a1, b0, b1;
-            mul2v(t0, t1, h0, h1, -sn[2 * i], -sn[2 * i + 1]);
-            mul2v(u0, u1, l0, l1, sn[2 * i], sn[2 * i + 1]);
-            fma2v(a0, a1, l0, l1, cs[2 * i], cs[2 * i + 1], t0, t1);
-            fma2v(b0, b1, h0, h1, cs[2 * i], cs[2 * i + 1], u0, u1);
-            ol[i] = pack2(a0, a1);
-            oh[i] = pack2(b0, b1);
-          }
-          *reinterpret_cast<uint4*>(qb) = make_uint4(ol[0], ol[1], ol[2], ol[3]);
-          *reinterpret_cast<uint4*>(qb + BOX_BYTES) = make_uint4(oh[0], oh[1], oh[2], oh[3]);
+          rotate_chunk(qb, cs, sn);
         }
       }
       fence_async_smem();
@@ -726,7 +527,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
       const int t_row = it.tok0 + x * TQ + row / s;     // token (local index)
       const int t_eff = min(t_row, it.L - 1);
       const int n_tiles = it.n_tiles, nA = it.nA, lenA = it.lenA, H = it.H;
-      float m_ref = -INFINITY, l_sum = 0.f;
+      float m_ref = -INFINITY, l_sum = 0.f, l_other = 0.f;   // sums over every second tile, swapped after each (as attn_tile.cu adds them)
       if (active) {
         for (int i = 0; i < n_tiles; ++i, ++cnt) {
           mbar_wait(bar(B_SFULL + x), cnt & 1u, abort_flag, p.status);
@@ -772,19 +573,20 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
               TMEM_ST32(t_o + 32 * ch, orr, 0);
             }
             tmem_wait_st();
-            if (need) { l_sum *= f; m_ref = m_new; }
+            if (need) { l_sum = __fmul_rn(l_sum, f); l_other = __fmul_rn(l_other, f); m_ref = m_new; }
           }
           const float neg_m = -m_ref * c2;
           uint32_t pr[64];
-          float acc[4] = {0.f, 0.f, 0.f, 0.f};
+          const uint64_t neg2 = pair2(neg_m, neg_m);
+          uint64_t acc0 = 0, acc1 = 0;
 #pragma unroll
           for (int c = 0; c < 64; c += 2) {
             float x0, x1, x2, x3;
-            fma2(x0, x1, __uint_as_float(sr[2 * c]), __uint_as_float(sr[2 * c + 1]), c2, neg_m);
-            fma2(x2, x3, __uint_as_float(sr[2 * c + 2]), __uint_as_float(sr[2 * c + 3]), c2, neg_m);
+            fma2(x0, x1, __uint_as_float(sr[2 * c]), __uint_as_float(sr[2 * c + 1]), c2c2, neg2);
+            fma2(x2, x3, __uint_as_float(sr[2 * c + 2]), __uint_as_float(sr[2 * c + 3]), c2c2, neg2);
             const float p0 = ex2(x0), p1 = ex2(x1), p2 = ex2(x2), p3 = ex2(x3);
-            add2(acc[0], acc[1], p0, p1);
-            add2(acc[2], acc[3], p2, p3);
+            add2(acc0, p0, p1);
+            add2(acc1, p2, p3);
             pr[c] = pack2(p0, p1);
             pr[c + 1] = pack2(p2, p3);
             if (c == 30) {   // first half of P goes out, and into P V, while the second is computed
@@ -794,7 +596,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
               mbar_arrive(bar(B_PHALF + x));
             }
           }
-          l_sum += (acc[0] + acc[1]) + (acc[2] + acc[3]);
+          const float l_new = __fadd_rn(l_sum, sum4(acc0, acc1));
+          l_sum = l_other; l_other = l_new;
           TMEM_ST32(t_s + 32, pr, 32);
           tmem_wait_st();
           tc_fence_before();
@@ -804,8 +607,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
       // ---- hand the finished tile to the epilogue warps (they wait for its last P V themselves) ----
       if (active) {
         if (done_n > 0) mbar_wait(bar(B_ODRAIN + x), (done_n - 1u) & 1u, abort_flag, p.status);   // 1 / l of the item before was read
-        reinterpret_cast<float*>(sm_gen + SM_INVL)[x * 128 + row] = it.part < 0 ? 1.f / l_sum : 1.f;
-        if (it.part >= 0) p.part_ml[(it.part * 2 + x) * 128 + row] = make_float2(m_ref * c2, l_sum);
+        reinterpret_cast<float*>(sm_gen + SM_INVL)[x * 128 + row] = 1.f / (l_sum + l_other);
         mbar_arrive(bar(B_LREADY + x));
         ++done_n;
       }
@@ -823,58 +625,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
   if (warp == 9) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
-  }
-}
-
-// Merges the parts of the items that a split launch cut: block (c - 1, q) looks at cut c and, if it is
-// the first one inside its item, combines rows 64 q .. + 63 of the item's 256, a warp eight of them with
-// the first two parts' loads all in flight, a lane four columns.  The parts are in slot 2a + 1 of the CTA
-// a before the cut and slots 2j of those after it.  Bound by what an SM can read from L2: a whole item
-// (256-512 KB) to a block took 16 us where this takes 8; merging inside the attention launch, by the
-// last CTA of an item to end, 37 us.
-constexpr int MERGE_THREADS = 256, MERGE_BATCH = 8, MERGE_SPLIT = 4;
-static_assert(MERGE_SPLIT * MERGE_BATCH * MERGE_THREADS / 32 == 256, "rows of a tile pair");
-template <typename TO>
-__global__ void __launch_bounds__(MERGE_THREADS) attn_merge_kernel(const __grid_constant__ TcParams p) {
-  rc_grid_wait();
-  rc_grid_launch_next();
-  const int c = blockIdx.x + 1;
-  const int n = p.header[3];
-  const int4 m = p.merge[c];                             // (c < grid: there, if not written, in any case)
-  if (c >= n || m.x == 0) return;
-  const int last = c + m.x - 2, rows = m.z, lane = threadIdx.x & 31;
-  const int r0 = (256 / MERGE_SPLIT) * blockIdx.y + MERGE_BATCH * (threadIdx.x >> 5);
-  if (r0 < rows) {
-    float2 ml[2][MERGE_BATCH];
-    float4 v[2][MERGE_BATCH];
-    auto load = [&](int h, int j) {
-      const int64_t at = (int64_t)(j == c - 1 ? 2 * j + 1 : 2 * j) * 256 + r0;
-#pragma unroll
-      for (int k = 0; k < MERGE_BATCH; ++k) {
-        ml[h][k] = p.part_ml[at + k];
-        v[h][k] = *(reinterpret_cast<const float4*>(p.part_o + (at + k) * D) + lane);
-      }
-    };
-    auto add = [&]() {                                   // part 1 into part 0
-#pragma unroll
-      for (int k = 0; k < MERGE_BATCH; ++k) {
-        const float m = fmaxf(ml[0][k].x, ml[1][k].x), f0 = ex2(ml[0][k].x - m), f1 = ex2(ml[1][k].x - m);
-        ml[0][k] = make_float2(m, ml[0][k].y * f0 + ml[1][k].y * f1);
-        v[0][k].x = v[0][k].x * f0 + v[1][k].x * f1; v[0][k].y = v[0][k].y * f0 + v[1][k].y * f1;
-        v[0][k].z = v[0][k].z * f0 + v[1][k].z * f1; v[0][k].w = v[0][k].w * f0 + v[1][k].w * f1;
-      }
-    };
-    load(0, c - 1);
-    for (int j = c; j <= last; ++j) { load(1, j); add(); }
-#pragma unroll
-    for (int k = 0; k < MERGE_BATCH; ++k) {
-      const int r = r0 + k;                              // row of the pair: 128 rows are TQ tokens of s heads
-      if (r >= rows) break;
-      const float inv = 1.f / ml[0][k].y;
-      TO* o = reinterpret_cast<TO*>(p.out) + ((int64_t)(m.y + r / p.s) * p.Hq + m.w * p.s + r % p.s) * D + 4 * lane;
-      if constexpr (sizeof(TO) == 4) *reinterpret_cast<float4*>(o) = make_float4(v[0][k].x * inv, v[0][k].y * inv, v[0][k].z * inv, v[0][k].w * inv);
-      else *reinterpret_cast<uint2*>(o) = make_uint2(pack2(v[0][k].x * inv, v[0][k].y * inv), pack2(v[0][k].z * inv, v[0][k].w * inv));
-    }
   }
 }
 
@@ -930,12 +680,12 @@ bool rc_tc_supported(const recache_ctx* ctx) {
   return ctx->desc.dtype == RECACHE_BF16 && ctx->desc.head_dim == 128 && (s == 2 || s == 4 || s == 8);
 }
 
-static int tc_tok_per_cta(const recache_ctx* ctx) { return 2 * 128 / (ctx->desc.n_q_heads / ctx->desc.n_kv_heads); }
-static int64_t tc_max_items(const recache_ctx* ctx, int n_seq, int total) {
-  return (int64_t)total / tc_tok_per_cta(ctx) + n_seq;
+static int tc_tok_per_item(const recache_ctx* ctx, int item_tiles) { return item_tiles * 128 / (ctx->desc.n_q_heads / ctx->desc.n_kv_heads); }
+static int64_t tc_max_items(const recache_ctx* ctx, int n_seq, int total, int item_tiles) {
+  return (int64_t)total / tc_tok_per_item(ctx, item_tiles) + n_seq;
 }
-static int tc_levels(const recache_ctx* ctx, int max_len) {
-  const int t = tc_tok_per_cta(ctx);
+static int tc_levels(const recache_ctx* ctx, int max_len, int item_tiles) {
+  const int t = tc_tok_per_item(ctx, item_tiles);
   return (max_len + t - 1) / t + 1;
 }
 
@@ -946,10 +696,18 @@ static bool tc_may_split(const recache_ctx* ctx, int64_t max_items) {
   return n <= 4 * tc_ctas(ctx) && n <= RC_SORT_MAX;
 }
 
-constexpr int64_t PART_ROWS = 2 * 2 * 128;   // per CTA: two slots of two tiles
+// Query tiles of a work item: one (attn_tile.cu), or a pair that shares its K/V tiles (attn_tc_kernel).  The
+// results are the same bits.
+static int tc_item_tiles(const recache_ctx* ctx, const TcAttnArgs& a) {
+  if (a.route_idx) return 2;
+  if (a.route_cu) return 1;
+  return tc_max_items(ctx, a.n_seq, a.total, 1) * ctx->desc.n_kv_heads <= 4 * tc_ctas(ctx) ? 1 : 2;
+}
+
+constexpr int64_t PART_ROWS = 2 * 128;       // per CTA: two slots
 
 int64_t rc_tc_workspace_bytes(const recache_ctx* ctx, int n_seq, int total, int max_len) {
-  return 256 + align256(tc_max_items(ctx, n_seq, total) * 8) + align256(2 * RC_SORT_MAX * 4);
+  return 256 + align256(tc_max_items(ctx, n_seq, total, 1) * 8) + align256(2 * RC_SORT_MAX * 4);
 }
 // What a split takes on top, whatever the call's size: cuts, unit prefix, and two partial results per CTA.
 int64_t rc_tc_split_bytes(const recache_ctx* ctx) {
@@ -973,19 +731,21 @@ static bool tc_splits(const recache_ctx* ctx, const TcAttnArgs& a, int64_t max_i
 cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope, const TcAttnArgs& a, cudaStream_t st) {
   const int G = ctx->desc.n_kv_heads, Hq = ctx->desc.n_q_heads, s = Hq / G;
   if (a.total == 0 || a.n_seq == 0) return cudaSuccess;
-  const int64_t max_items = tc_max_items(ctx, a.n_seq, a.total);
+  const bool gather = a.route_idx != nullptr;
+  const int item_tiles = tc_item_tiles(ctx, a);
+  const int64_t max_items = tc_max_items(ctx, a.n_seq, a.total, item_tiles);
   uint8_t* ws = (uint8_t*)a.workspace;
 
-  CUtensorMap tq, tks, tvs, tkr, tvr;
+  TcMaps m;
   const uint64_t self_total = (uint64_t)G * (uint64_t)a.self_rows;
   // TMA coordinates are 32-bit row indices
   if (self_total + TILE_N > 0x7fffffffull || (uint64_t)a.route_rows + TILE_N > 0x7fffffffull) return cudaErrorInvalidValue;
-  if (!map_q(&tq, a.q, (uint64_t)a.total, Hq, s) || !map_rows(&tks, a.k_self, self_total) ||
-      !map_rows(&tvs, a.v_self, self_total))
+  if (!map_q(&m.q, a.q, (uint64_t)a.total, Hq, s) || !map_rows(&m.ks, a.k_self, self_total) ||
+      !map_rows(&m.vs, a.v_self, self_total))
     return cudaErrorInvalidValue;
-  const bool has_route = (a.route_cu != nullptr || a.prefix_len > 0) && a.route_rows > 0 && a.route_idx == nullptr;
-  if (!has_route) { tkr = tks; tvr = tvs; }   // unused
-  else if (!map_rows(&tkr, a.k_route, (uint64_t)a.route_rows) || !map_rows(&tvr, a.v_route, (uint64_t)a.route_rows))
+  const bool has_route = (a.route_cu != nullptr || a.prefix_len > 0) && a.route_rows > 0 && !gather;
+  if (!has_route) { m.kr = m.ks; m.vr = m.vs; }   // unused
+  else if (!map_rows(&m.kr, a.k_route, (uint64_t)a.route_rows) || !map_rows(&m.vr, a.v_route, (uint64_t)a.route_rows))
     return cudaErrorInvalidValue;
 
   TcParams p;
@@ -1005,30 +765,23 @@ cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope,
   p.cu = a.cu; p.pos0 = a.pos0; p.slot = a.slot; p.route_cu = a.route_cu; p.hist = a.hist;
   p.n_seq = a.n_seq; p.G = G; p.Hq = Hq; p.s = s; p.self_rows = a.self_rows; p.route_rows = a.route_rows;
   p.prefix_len = a.route_cu ? 0 : a.prefix_len;
-  p.n_levels = tc_levels(ctx, a.max_len); p.max_items = (int)max_items;
+  p.item_tiles = item_tiles; p.n_levels = tc_levels(ctx, a.max_len, item_tiles); p.max_items = (int)max_items;
   p.status = ctx->status;
   p.out = a.o;
   p.cos_tab = ctx->cos_tab; p.sin_tab = ctx->sin_tab; p.max_pos = ctx->desc.max_pos;
   p.scale_log2 = (float)(1.4426950408889634 / sqrt((double)ctx->desc.head_dim));
-  const bool gather = a.route_idx != nullptr;
   p.gather_k = (const uint8_t*)a.k_cache; p.gather_v = (const uint8_t*)a.v_cache; p.route_idx = a.route_idx;
   p.pool_tokens = a.pool_tokens;
   cudaError_t e = rc_launch_rope_store(ctx, rope, &p, st);   // builds the work list on the side
   if (e != cudaSuccess) return e;
   const bool f32 = a.out_dtype == RECACHE_F32, rot = s >= 4;   // 2 * 128 / s <= 64 positions fit the staging area
-  {
-    RcLaunchScope scope(ctx, a.route_cu ? RC_K_PREFILL_ATTN : RC_K_ENCODE_ATTN, st);
-    auto launch = [&](auto kernel) { return rc_launch_overlapped(kernel, grid, NTHREADS, SM_ALLOC, st, tq, tks, tvs, tkr, tvr, p); };
-    auto pick = [&](auto type) {
-      using TO = decltype(type);
-      if (gather) return rot ? launch(attn_tc_kernel<TO, true, true, false>) : launch(attn_tc_kernel<TO, false, true, false>);
-      if (may_split) return rot ? launch(attn_tc_kernel<TO, true, false, true>) : launch(attn_tc_kernel<TO, false, false, true>);
-      return rot ? launch(attn_tc_kernel<TO, true, false, false>) : launch(attn_tc_kernel<TO, false, false, false>);
-    };
-    e = f32 ? pick(float()) : pick(__nv_bfloat16());
-  }
-  if (e != cudaSuccess || !may_split) return e;
-  RcLaunchScope scope(ctx, RC_K_PREFILL_MERGE, st);
-  return f32 ? rc_launch_overlapped(attn_merge_kernel<float>, dim3(grid - 1, MERGE_SPLIT), MERGE_THREADS, 0, st, p)
-             : rc_launch_overlapped(attn_merge_kernel<__nv_bfloat16>, dim3(grid - 1, MERGE_SPLIT), MERGE_THREADS, 0, st, p);
+  if (item_tiles == 1) return rc_launch_attn_tile(ctx, m, p, f32, may_split, grid, st);
+  RcLaunchScope scope(ctx, a.route_cu ? RC_K_PREFILL_ATTN : RC_K_ENCODE_ATTN, st);
+  auto launch = [&](auto kernel) { return rc_launch_overlapped(kernel, grid, NTHREADS, SM_ALLOC, st, m.q, m.ks, m.vs, m.kr, m.vr, p); };
+  auto pick = [&](auto type) {
+    using TO = decltype(type);
+    if (gather) return rot ? launch(attn_tc_kernel<TO, true, true>) : launch(attn_tc_kernel<TO, false, true>);
+    return rot ? launch(attn_tc_kernel<TO, true, false>) : launch(attn_tc_kernel<TO, false, false>);
+  };
+  return f32 ? pick(float()) : pick(__nv_bfloat16());
 }

@@ -24,7 +24,8 @@ struct RcPlan {
   int prefix_len;   // > 0: every sequence sees rows g*prefix_len .. of the "route" tensors (shared prefix)
   int64_t self_rows;
   int64_t route_rows;   // rows of the packed route tensors / entries of route_idx
-  int n_levels, max_items;   // tile pairs of the longest sequence, capacity of items[]
+  int item_tiles;            // query tiles of a work item: 1, or 2 (a pair)
+  int n_levels, max_items;   // work items of the longest sequence, capacity of items[]
   int32_t* status;
 };
 
@@ -46,10 +47,10 @@ __device__ __forceinline__ bool rc_load_item(const RcPlan& p, int w, RcItem& it)
   const int TQ = 128 / p.s;
   it.seq0 = p.cu[b];
   it.L = p.cu[b + 1] - it.seq0;
-  it.tok0 = e.y * 2 * TQ;
-  it.b_valid = it.tok0 + TQ < it.L;
+  it.tok0 = e.y * p.item_tiles * TQ;
+  it.b_valid = p.item_tiles > 1 && it.tok0 + TQ < it.L;
   it.H = p.hist ? p.hist[b] : 0;
-  it.kv_end = it.H + min(it.L, it.tok0 + 2 * TQ);   // self rows the pair can see: the history, then its causal range
+  it.kv_end = it.H + min(it.L, it.tok0 + p.item_tiles * TQ);   // self rows the item can see: the history, then its causal range
   it.base = p.slot ? (int64_t)p.slot[b] : (int64_t)it.seq0;
   it.pos0 = p.pos0 ? p.pos0[b] : 0;
   it.rA0 = 0; it.lenA = 0;
@@ -161,7 +162,7 @@ __device__ __forceinline__ bool rc_plan_split(const RcPlan& p, RcPlanSmem& sh, i
     if (c > 0 && cut.y > 0 && (p.start[c - 1].x != cut.x || p.start[c - 1].y == 0)) {
       RcItem it;
       rc_load_item(p, cut.x, it);
-      m = make_int4(2, it.seq0 + it.tok0, min(256, (it.L - it.tok0) * p.s), it.g);
+      m = make_int4(2, it.seq0 + it.tok0, min(128, (it.L - it.tok0) * p.s), it.g);
 #pragma unroll 1
       for (int j = c + 1; p.start[j].x == cut.x && p.start[j].y > 0; ++j) ++m.x;
     }
@@ -181,7 +182,7 @@ __device__ __forceinline__ bool rc_plan_split(const RcPlan& p, RcPlanSmem& sh, i
 // (Nothing is unrolled: the block runs every loop for a step or two, out of a cold instruction cache, and
 // the unrolled code took 0.3-0.4 us more of turns of 35-50 us.)
 __device__ __forceinline__ void rc_build_plan(const RcPlan& p, RcPlanSmem& sh) {
-  const int tid = threadIdx.x, n_thr = blockDim.x, n_seq = p.n_seq, tok_per_item = 2 * 128 / p.s;
+  const int tid = threadIdx.x, n_thr = blockDim.x, n_seq = p.n_seq, tok_per_item = p.item_tiles * 128 / p.s;
   const int32_t* cu = p.cu;
   auto n_pairs = [&](int b) {
     const int len = cu[b + 1] - cu[b];
