@@ -59,3 +59,8 @@ def test_counts_and_tables(lens, gap, requests, groups):
         at += n
     assert np.array_equal(paged["route_len"].cpu().numpy(), [len(r) for r in flat])
     assert rc.poll_status() == 0
+
+
+@pytest.mark.parametrize("n,requests", [(255, 2), (256, 2), (257, 2), (1, 513)])   # eight groups: 4096 pairs are 512 listed resources
+def test_offsets_around_the_gather_that_plans_for_itself(n, requests):
+    test_counts_and_tables([1 + i % 3 for i in range(n)], 1, requests, 8)
