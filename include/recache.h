@@ -138,7 +138,7 @@ RECACHE_API recache_status recache_kernel_times(recache_ctx* ctx, float* ms_tota
 /* Scratch sizes in bytes for the calls below (same size arguments).  They grow with every
  * argument: a workspace sized for the largest call serves all smaller ones.
  * recache_prefill_workspace_bytes is what every prefill needs, a few bytes per query token;
- * recache_prefill_history_workspace_bytes is that and 39 MB (148 SMs), with which
+ * recache_prefill_history_workspace_bytes is that and 20 MB (148 SMs), with which
  * recache_attend_prefill_history may divide its requests' keys between SMs. */
 RECACHE_API int64_t recache_encode_workspace_bytes(const recache_ctx* ctx, int32_t n_resources,
                                        int32_t total_tokens, int32_t max_len);

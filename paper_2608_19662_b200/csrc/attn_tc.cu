@@ -697,11 +697,21 @@ static bool tc_may_split(const recache_ctx* ctx, int64_t max_items) {
 }
 
 // Query tiles of a work item: one (attn_tile.cu), or a pair that shares its K/V tiles (attn_tc_kernel).  The
-// results are the same bits.
+// results are the same bits.  One is better where the launch has few items a CTA, a pair where it has many (a
+// K/V tile is then loaded, and its MMAs are issued, for two), us with one and with a pair:
+//   encode, 4 query heads a group: 1 x 500 tokens (128 items) 18.4 / 20.1, 8 x 500 (1000) 44.6 / 45.1, 12 x 500 (1500) 69.6 / 65.3;
+//     2 x 1500 (750) 59.1 / 61.5, 3 x 1500 (1125) 89.0 / 85.3
+//   first turns: 1 x 512 tokens 32.1 / 40.3, 4 x 1024 (1024 items) 97.1 / 98.9, 16 x 256 (1024) 80.3 / 86.7, 16 x 512 (2048) 157 / 152
+// Where a route has room for more than 64 K/V tiles, an item is long, and the pair's fewer loads count for more (the
+// room is all the host knows of it; only the time depends on it): 2048 tokens over 64 long tools (512 items) 300 / 290.
+// A gather's copies are bound by the rate at which a CTA issues them, so it always takes pairs; a later turn, whose items
+// may be split, never does.
 static int tc_item_tiles(const recache_ctx* ctx, const TcAttnArgs& a) {
   if (a.route_idx) return 2;
-  if (a.route_cu) return 1;
-  return tc_max_items(ctx, a.n_seq, a.total, 1) * ctx->desc.n_kv_heads <= 4 * tc_ctas(ctx) ? 1 : 2;
+  if (a.hist) return 1;
+  const int64_t G = ctx->desc.n_kv_heads;
+  const int rounds = !a.route_cu ? 6 : a.route_rows > 64 * TILE_N * G * a.n_seq ? 2 : 8;
+  return tc_max_items(ctx, a.n_seq, a.total, 1) * G <= (int64_t)rounds * tc_ctas(ctx) ? 1 : 2;
 }
 
 constexpr int64_t PART_ROWS = 2 * 128;       // per CTA: two slots

@@ -107,8 +107,8 @@ __device__ __forceinline__ void rc_plan_scan_bins(RcPlanSmem& sh) {
 // edge where it would leave a part of fewer than two tiles, or a part whose first tile some row of
 // the pair does not see.  Taken only where the longest CTA gets shorter by more than the second
 // beginning (two units) and the merge (six: 6-10 us, a unit taking 1.8) cost: 8 conversations with 300-2048
-// rows of history (88 items of 8-24 tiles) take 50 us instead of 57.  The other figures were taken with route
-// rows in the place of a history: one request of 2048 tokens over a long tool set (256 items of 58-73 tiles,
+// rows of history (88 items of 8-24 tiles) take 50 us instead of 57 (44 with one query tile to an item: all these
+// figures were taken with pairs of them).  The other figures were taken with route rows in the place of a history: one request of 2048 tokens over a long tool set (256 items of 58-73 tiles,
 // else two rounds of 148 CTAs) 281 instead of 291 us; 8 conversations of 250 tokens over 4000 rows (256 items
 // of 36) would take 159 instead of 152.  Whole items of a sequence also walk its K/V in step and read it from
 // L2, parts do not, which costs a fifth where the keys and values of the launch are more than L2 holds and
