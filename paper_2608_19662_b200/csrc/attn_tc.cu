@@ -8,8 +8,8 @@
 //
 //   warps 0-3    softmax of tile A    warps 4-7  softmax of tile B
 //   warp  8      TMA producer         warp  9    tcgen05.mma issuer (+ TMEM alloc)
-//   warp  10     scheduler: draws work items from a global counter (split launch:
-//                walks the CTA's range of the K/V tiles) and publishes them through a two-slot ring in shared memory
+//   warp  10     scheduler: draws work items from a global counter and publishes them
+//                through a two-slot ring in shared memory
 //   warp  11     idle (completes the third warpgroup)
 //   warps 12-15  epilogue: O of a finished tile goes from tensor memory to HBM
 //                while the softmax warps already rotate the next item's Q; in
@@ -30,9 +30,8 @@
 // causal rows of the sequence itself up to the tile pair's last token.  The
 // query rows are rotated in shared memory after the TMA load (position = pos0 +
 // token index) and rounded to bf16, so no rotated copy of Q ever touches HBM.
-// Tiles are aligned to the sequence start, never to the batch: a resource, and a first turn,
-// gives bit-identical outputs whatever else is in the launch.  (The items of a later turn may
-// be split, see rc_plan_split; the cuts follow from the lengths of the whole launch.)
+// Tiles are aligned to the sequence start, never to the batch: a sequence gives
+// bit-identical outputs whatever else is in the launch.
 #include "tc_common.cuh"
 
 using namespace rc_tc;
@@ -42,8 +41,8 @@ namespace {
 constexpr int NSTAGE = 2;
 constexpr int NTHREADS = 512;
 // Registers per thread of the softmax warps and of the other eight; 256 * (softmax + aux) = 65536.  Epilogue
-// warps that gather and schedulers that know about split items spill in 32 (8 zero-copy turns: 84.0 us with 32,
-// 82.2 with 40); whole items of packed rows pay for 40 (one turn of 512 tokens: 34.8 us with 40, 34.3 with 32; an encode 1 %).
+// warps that gather spill in 32 (8 zero-copy turns: 84.0 us with 32, 82.2 with 40); packed rows pay for 40 (one turn
+// of 512 tokens: 34.8 us with 40, 34.3 with 32; an encode 1 %).
 template <bool MORE_AUX> constexpr int REGS_SOFTMAX = MORE_AUX ? 216 : 224;
 template <bool MORE_AUX> constexpr int REGS_AUX = MORE_AUX ? 40 : 32;
 
@@ -689,11 +688,14 @@ static int tc_levels(const recache_ctx* ctx, int max_len, int item_tiles) {
   return (max_len + t - 1) / t + 1;
 }
 
-// A later turn of at most four rounds of CTAs may be split (see rc_plan_split).
 static int tc_ctas(const recache_ctx* ctx) { return ctx->sm_count > 0 ? ctx->sm_count : 148; }
+// A later turn of at most this many rounds of CTAs, in items of one query tile, may be split (see rc_plan_split).
+// Of 61 turns of 3-4 rounds none was more than 1 % faster split than whole by the better of the two kernels; of 426 with
+// fewer items 89 were by 5-55 %.
+constexpr int64_t SPLIT_ROUNDS = 3;
 static bool tc_may_split(const recache_ctx* ctx, int64_t max_items) {
   const int64_t n = max_items * ctx->desc.n_kv_heads;
-  return n <= 4 * tc_ctas(ctx) && n <= RC_SORT_MAX;
+  return n <= SPLIT_ROUNDS * tc_ctas(ctx) && n <= RC_SORT_MAX;
 }
 
 // Query tiles of a work item: one (attn_tile.cu), or a pair that shares its K/V tiles (attn_tc_kernel).  The
@@ -704,14 +706,23 @@ static bool tc_may_split(const recache_ctx* ctx, int64_t max_items) {
 //   first turns: 1 x 512 tokens 32.1 / 40.3, 4 x 1024 (1024 items) 97.1 / 98.9, 16 x 256 (1024) 80.3 / 86.7, 16 x 512 (2048) 157 / 152
 // Where a route has room for more than 64 K/V tiles, an item is long, and the pair's fewer loads count for more (the
 // room is all the host knows of it; only the time depends on it): 2048 tokens over 64 long tools (512 items) 300 / 290.
-// A gather's copies are bound by the rate at which a CTA issues them, so it always takes pairs; a later turn, whose items
-// may be split, never does.
+// A gather's copies are bound by the rate at which a CTA issues them, so it always takes pairs.
+// A later turn is split, if at all, in items of one tile (tc_may_split), so up to SPLIT_ROUNDS rounds of CTAs it has one;
+// so it has where no request has a second tile to pair (32 x 16 tokens over 4000 rows, 2 heads a group 128 / 151).  Beyond,
+// never split, it goes by the room for its keys, 24 K/V tiles an item, up to eight rounds, and takes pairs from there:
+//   2 heads, 16 x 256 tokens (640 items) over 300 rows 62.4 / 64.1, over 4000 229 / 195
+//   4 heads, 8 x 256 (576) over 300 53.7 / 53.1, over 4000 209 / 183; 16 x 512 (2176) over 300 217 / 205
+//   of 320 turns of random sizes those of 3-8 rounds take 0.95 of the pair's time with up to 24 tiles an item (0.79-1.04), 1.02
+//   with more (0.94-1.14), those of more rounds 1.02 (0.95-1.11)
 static int tc_item_tiles(const recache_ctx* ctx, const TcAttnArgs& a) {
   if (a.route_idx) return 2;
-  if (a.hist) return 1;
-  const int64_t G = ctx->desc.n_kv_heads;
+  const int64_t G = ctx->desc.n_kv_heads, ctas = tc_ctas(ctx), items = tc_max_items(ctx, a.n_seq, a.total, 1) * G;
+  if (a.hist) {
+    if (items <= SPLIT_ROUNDS * ctas || a.max_len <= tc_tok_per_item(ctx, 1)) return 1;
+    return items <= 8 * ctas && a.route_rows / G + a.self_rows <= (int64_t)24 * TILE_N * a.n_seq ? 1 : 2;
+  }
   const int rounds = !a.route_cu ? 6 : a.route_rows > 64 * TILE_N * G * a.n_seq ? 2 : 8;
-  return tc_max_items(ctx, a.n_seq, a.total, 1) * G <= (int64_t)rounds * tc_ctas(ctx) ? 1 : 2;
+  return items <= rounds * ctas ? 1 : 2;
 }
 
 constexpr int64_t PART_ROWS = 2 * 128;       // per CTA: two slots
@@ -760,7 +771,7 @@ cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope,
 
   TcParams p;
   p.header = (int32_t*)ws; p.items = (int2*)(ws + 256); p.order = (int32_t*)(ws + 256 + align256(max_items * 8));
-  const bool may_split = tc_splits(ctx, a, max_items);
+  const bool may_split = item_tiles == 1 && tc_splits(ctx, a, max_items);
   const int sms = tc_ctas(ctx);
   const unsigned grid = (unsigned)(may_split || max_items * G > sms ? sms : max_items * G);
   p.start = nullptr; p.merge = nullptr; p.unit_cu = nullptr; p.part_o = nullptr; p.part_ml = nullptr; p.n_cta = (int)grid;
