@@ -741,12 +741,13 @@ int64_t rc_tc_split_bytes(const recache_ctx* ctx) {
 // A first turn's result must be the same bits whether its rows are packed or gathered, and both must be free
 // to come in buffers of any size, of which the host cannot tell how much is filled.
 // Nothing here may depend on capacities, except to leave the merge launch out where rc_plan_split cannot say yes
-// whatever they hold: with one round of CTAs it wants most + RC_ITEM_UNITS >= (4 + RC_ITEM_UNITS + 6) / 0.95.
+// whatever they hold: ranges have more than four units, and whole items take, in one round, RC_ITEM_UNITS more than the
+// longest has tiles, in more half its tiles more than a range.
 static bool tc_splits(const recache_ctx* ctx, const TcAttnArgs& a, int64_t max_items) {
   if (!a.hist || !tc_may_split(ctx, max_items) || tc_ctas(ctx) < 2) return false;
   if (a.workspace_bytes < rc_tc_workspace_bytes(ctx, a.n_seq, a.total, a.max_len) + rc_tc_split_bytes(ctx)) return false;
   const int64_t most = a.route_rows / TILE_N + a.self_rows / TILE_N + 2;     // tiles of an item that had every row there is
-  return max_items * ctx->desc.n_kv_heads > tc_ctas(ctx) || most >= 11;
+  return most > 4 + RC_MERGE_UNITS;
 }
 
 cudaError_t rc_launch_attn_tc(const recache_ctx* ctx, const RopeStoreArgs& rope, const TcAttnArgs& a, cudaStream_t st) {

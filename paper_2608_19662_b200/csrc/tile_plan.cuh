@@ -7,7 +7,8 @@
 
 constexpr int RC_TILE_N = 128;       // keys of a K/V tile
 constexpr int RC_SORT_MAX = 4096;    // work items up to which the plan sorts a prefill by weight (encode: a quarter)
-constexpr int RC_ITEM_UNITS = 2;     // what beginning an item costs, in K/V tiles
+constexpr int RC_ITEM_UNITS = 2;     // what beginning an item costs, in K/V tiles of about 0.95 us
+constexpr int RC_MERGE_UNITS = 12;   // what parts and their merge cost
 constexpr int RC_L2_BLOCKS = 768;    // 100 MB: what of the 126 MB L2 a launch's keys and values may take
 constexpr int RC_PLAN_BINS = 1024;   // weights (K/V tiles, tile pairs) are told apart up to this
 
@@ -101,19 +102,18 @@ __device__ __forceinline__ void rc_plan_scan_bins(RcPlanSmem& sh) {
   __syncthreads();
 }
 
-// A later turn (RcPlan.start given) whose items do not fill the CTAs evenly: their K/V tiles, laid end to end, are cut into
-// n equal ranges, so that an item may be shared by several CTAs (their partial results are merged
+// A later turn (RcPlan.start given) whose items, of one query tile each, do not fill the CTAs evenly: their K/V tiles, laid end
+// to end, are cut into n equal ranges, so that an item may be shared by several CTAs (their partial results are merged
 // afterwards).  An item counts RC_ITEM_UNITS more than its tiles, and a cut is moved to the item's
 // edge where it would leave a part of fewer than two tiles, or a part whose first tile some row of
-// the pair does not see.  Taken only where the longest CTA gets shorter by more than the second
-// beginning (two units) and the merge (six: 6-10 us, a unit taking 1.8) cost: 8 conversations with 300-2048
-// rows of history (88 items of 8-24 tiles) take 50 us instead of 57 (44 with one query tile to an item: all these
-// figures were taken with pairs of them).  The other figures were taken with route rows in the place of a history: one request of 2048 tokens over a long tool set (256 items of 58-73 tiles,
-// else two rounds of 148 CTAs) 281 instead of 291 us; 8 conversations of 250 tokens over 4000 rows (256 items
-// of 36) would take 159 instead of 152.  Whole items of a sequence also walk its K/V in step and read it from
-// L2, parts do not, which costs a fifth where the keys and values of the launch are more than L2 holds and
-// three or more items share them: 2048 tokens over 14,000 / 20,000 rows a group (57 / 82 MB) 404 / 572 us split
-// and 424 / 583 whole, but over 40,000 (164 MB) 1170 and 1120, and 4 x 512 tokens over 24,000 each 750 and 693.
+// the item does not see.  Taken only where the longest CTA gets shorter by more than parts and merge cost.  Whole, a launch
+// of one round ends with its longest item, one of more about half of that after the mean CTA; ranges take a tenth longer where
+// the launch reads more than L2 holds, as whole items of a sequence walk its keys in step and parts do not.  Chosen and
+// measured on 426 turns of up to three rounds, in a grid and at random: the slower way is taken at a mean
+// cost of 0.1 % and of more than 3 % in 4 of them (0.9 % and 46 with six units for the merge, which pairs of tiles had).
+//   1 request of 16 tokens, 2 heads a group, over 1000 / 4000 rows (8 items of 12 / 36 tiles): 24.0 / 32.3 us split, 22.4 / 40.7 whole
+//   4 x 16 tokens over 1000 (32 items of 13) 26.4 and 23.0; 8 x 17-250 over 300-2048 (152 items of 15) 41.0 and 37.1
+//   1 x 64 tokens, 4 heads, over 12,000 (16 items of 99) 41.0 and 91.2
 // Encoding and first turns are never split: a resource's result must not depend on what is encoded beside it,
 // nor a first turn's on whether its rows are packed or gathered.  False: not worth it.
 __device__ __forceinline__ bool rc_plan_split(const RcPlan& p, RcPlanSmem& sh, int n_work) {
@@ -129,10 +129,10 @@ __device__ __forceinline__ bool rc_plan_split(const RcPlan& p, RcPlanSmem& sh, i
   int at = rc_plan_scan(units, sh, &total_units);
   if (n_items == 0) return false;
   const int n = min(p.n_cta, max(1, (total_units - RC_ITEM_UNITS * n_items) / 4));
-  const float pace = sh.blocks > RC_L2_BLOCKS ? 1.2f : 1.f;
-  const float split = pace * total_units / n + RC_ITEM_UNITS + 6;
-  const float whole = fmaxf((float)(sh.most + RC_ITEM_UNITS), (float)total_units / n_items * ((n_items + p.n_cta - 1) / p.n_cta));
-  if (split > 0.95f * whole) return false;
+  const float pace = sh.blocks > RC_L2_BLOCKS ? 1.1f : 1.f;
+  const float split = pace * total_units / n + RC_ITEM_UNITS + RC_MERGE_UNITS;
+  const float whole = fmaxf((float)(sh.most + RC_ITEM_UNITS), n_items > p.n_cta ? (float)total_units / p.n_cta + 0.5f * sh.most : 0.f);
+  if (split > whole) return false;
 #pragma unroll 1
   for (int w = w0; w < w1; ++w) { p.unit_cu[w] = at; if (tiles[w] > 0) at += tiles[w] + RC_ITEM_UNITS; }
   __syncthreads();
@@ -232,7 +232,7 @@ __device__ __forceinline__ void rc_build_plan(const RcPlan& p, RcPlanSmem& sh) {
   // order decides the tail.  Sort them by weight (K/V tiles), heaviest first, with a counting sort.
   if (tid == 0) { sh.most = 0; sh.blocks = 0; }
   __syncthreads();
-  if (p.start && n_work > 2 * n_seq * p.G)         // (else see rc_plan_split: the size does not matter)
+  if (p.start)
 #pragma unroll 1
     for (int b = b0; b < b1; ++b) {
       const int own = cu[b + 1] - cu[b] + (p.hist ? p.hist[b] : 0);

@@ -136,3 +136,30 @@ def test_one_workspace_serves_the_largest_call_and_all_smaller_ones():
     assert rc.poll_status() == 0
     # two orders of summation of the same rows, probabilities in bf16: 2^-9 of each, signs at random over 2500 rows
     assert not torch.equal(whole, parts) and (whole - parts).abs().max().item() < 2e-3
+
+
+@pytest.mark.parametrize("new,hist,split", [
+    ([16], 2032, False),          # eight items of 16 K/V tiles: the merge would take longer than what the parts save
+    ([16], 2033, True),           # of 17
+    ([16] * 4, 1500, False),
+    ([16] * 4, 2500, True),
+    ([16] * 19, 1800, False),     # a second round of 4 CTAs; the merge would take as long
+    ([1216], 2000, False),        # 152 items of 17-26 tiles, short ones last
+    ([1216], 3000, True),         # of 24-33
+])
+def test_split_only_where_it_pays(new, hist, split):
+    """With room for parts the bits are those of the undivided call exactly where the call stays undivided (8 groups, 148 SMs)."""
+    sh = wl.Shape(16, 8, 128, 1e6, "bf16")
+    rc = make_ctx(sh, max_pos=8192)
+    B, cu = len(new), np.concatenate([[0], np.cumsum(new)]).astype(np.int32)
+    room, n = (hist + max(new) + 63) // 64 * 64, sum(new)
+    N = lambda i, *s: dev(wl.normal(900 + i, s, sh.torch_dtype))
+    q, k, v, kc, vc, rows = N(0, n, 16, 128), N(1, n, 8, 128), N(2, n, 8, 128), N(3, 8, B * room, 128), N(4, 8, B * room, 128), N(5, 1, 128)
+    slot, hists = dev(np.arange(B, dtype=np.int32) * room), dev(np.full(B, hist, np.int32))
+    none = torch.zeros(8 * B + 1, dtype=torch.int32, device="cuda")
+    later = lambda ws: rc.attend_prefill_history(q, k, v, dev(cu), hists, max(new), rows, rows, none, kc, vc, slot, hists, out_dtype=torch.float32, workspace=ws)
+    whole, got = (later(torch.empty(need(B, n, max(new)), dtype=torch.uint8, device="cuda"))
+                  for need in (rc.prefill_workspace_bytes, rc.prefill_history_workspace_bytes))
+    assert torch.equal(whole, got) != split
+    assert (whole - got).abs().max().item() < 2e-3      # two orders of summation, see above
+    assert rc.poll_status() == 0
