@@ -76,9 +76,9 @@ __global__ void __launch_bounds__(TPB) compact_count_kernel(
   }
 }
 
-struct PlanSmem { int ws[1024 / 32 + 1]; int wlen[32]; int carry_rows, carry_pages; };
+struct PlanSmem { int ws[1024 / 32 + 1]; int wlen[TPB / 2]; int carry_rows, carry_pages; };
 
-// Route lengths, prefixes, offsets and pages, by one block of up to 1024 threads.
+// Route lengths, prefixes, offsets and pages, by one block: of 1024 threads, or (no offsets wanted) of TPB.
 __device__ __forceinline__ void plan_routes(
     PlanSmem& sh, const int32_t* kept, const int32_t* res_off, int n_requests,
     int total_listed, const uint8_t* vis, int G, int mode, int page_tokens,
@@ -89,7 +89,12 @@ __device__ __forceinline__ void plan_routes(
     const int32_t* free_pages, int64_t n_free_pages, int64_t n_pool_pages,
     int32_t* status) {
   const int n_routes = n_requests * G;
-  const bool warp_per_route = n_routes <= (int)(blockDim.x >> 5);
+  const bool warp_per_route = res_route_off && n_routes <= (int)(blockDim.x >> 5);
+  // Lengths alone: a route's resources are dealt to as many lanes as there are for each route, four at a time.  (A thread
+  // to each of 9-32 routes, where the block of 1024 has a warp, took 24 us for 2 requests of 256 resources in 8
+  // groups and 14 for 2 of 128, the three launches 17 and 12.)
+  int lanes = res_route_off ? 1 : 32;
+  while (lanes > 1 && n_routes * lanes > (int)blockDim.x) lanes >>= 1;
   if (threadIdx.x == 0) { sh.carry_rows = 0; sh.carry_pages = 0; }
   __syncthreads();
   for (int r0 = 0; r0 < n_routes; r0 += blockDim.x) {
@@ -100,7 +105,7 @@ __device__ __forceinline__ void plan_routes(
       const int a = res_off[b], e = res_off[b + 1];
       if (a < 0 || e < a || e > total_listed) {
         rc_set_status(status, RECACHE_DEV_BAD_SEQLENS);
-      } else if (!warp_per_route) {
+      } else if (res_route_off && !warp_per_route) {
         const uint8_t* vg = vis + (int64_t)g * total_listed;
         for (int r0 = a; r0 < e; r0 += 4) {            // four at a time: loads are not moved across the stores
           int v[4];
@@ -108,7 +113,7 @@ __device__ __forceinline__ void plan_routes(
           for (int u = 0; u < 4; ++u) v[u] = r0 + u < e && vg[r0 + u] ? kept[r0 + u] : 0;
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            if (res_route_off && r0 + u < e) res_route_off[(int64_t)g * total_listed + r0 + u] = len;
+            if (r0 + u < e) res_route_off[(int64_t)g * total_listed + r0 + u] = len;
             len += v[u];
           }
         }
@@ -133,7 +138,7 @@ __device__ __forceinline__ void plan_routes(
               const int u = __shfl_up_sync(0xffffffffu, incl, off);
               if (lane >= off) incl += u;
             }
-            if (res_route_off && r < e) res_route_off[(int64_t)g * total_listed + r] = wlen + incl - v;
+            if (r < e) res_route_off[(int64_t)g * total_listed + r] = wlen + incl - v;
             wlen += __shfl_sync(0xffffffffu, incl, 31);
           }
         }
@@ -142,6 +147,33 @@ __device__ __forceinline__ void plan_routes(
       __syncthreads();
       if (route < n_routes && threadIdx.x < 32) len = sh.wlen[threadIdx.x];
       __syncthreads();
+    }
+    if (!res_route_off) {
+      const int sub = threadIdx.x & (lanes - 1), wr = r0 + threadIdx.x / lanes;   // (more than one pass of r0: one lane each)
+      int sum = 0;
+      if (wr < n_routes) {
+        const int b = wr / G, g = wr % G;
+        const int a = res_off[b], e = res_off[b + 1];
+        if (a >= 0 && e >= a && e <= total_listed) {
+          const uint8_t* vg = vis + (int64_t)g * total_listed;
+          for (int c = a + sub; c < e; c += 4 * lanes) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const int r = c + u * lanes;
+              const int v = r < e ? kept[r] : 0;
+              if (r < e && vg[r]) sum += v;
+            }
+          }
+        }
+      }
+      for (int off = lanes >> 1; off; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+      if (lanes == 1) {
+        len = sum;
+      } else {                                         // (at most TPB / 2 routes)
+        if (sub == 0 && wr < n_routes) sh.wlen[wr] = sum;
+        __syncthreads();
+        if (route < n_routes) len = sh.wlen[route];
+      }
     }
     const int pages = (mode == RECACHE_PAGED) ? (len + page_tokens - 1) / page_tokens : 0;
     int tot_rows, tot_pages;
@@ -238,11 +270,23 @@ __global__ void __launch_bounds__(TPB) compact_gather_kernel(
     __shared__ int before[TPB / 32], inside[TPB / 32];
     const int first = res_off[0], a = res_off[b], e = res_off[b + 1];
     int rows = 0, in = 0;
-    for (int q = threadIdx.x; q < G * total_listed; q += TPB) {
-      const int gq = q / total_listed, rq = q - gq * total_listed;
-      const int v = rq >= first && rq < e && vis[q] ? kept[rq] : 0;
-      if (rq < a || gq < g) rows += v;
-      else if (gq == g && rq < r) in += v;
+    if (G * total_listed <= 2 * TPB) {                   // a thread to a pair
+      for (int q = threadIdx.x; q < G * total_listed; q += TPB) {
+        const int gq = q / total_listed, rq = q - gq * total_listed;
+        const int v = rq >= first && rq < e && vis[q] ? kept[rq] : 0;
+        if (rq < a || gq < g) rows += v;
+        else if (gq == g && rq < r) in += v;
+      }
+    } else {   // a thread to a resource: `kept` is read once, and no pair after this one (4096 pairs: 12.8 us, a thread to a pair 18.4)
+      for (int q = max(first, 0) + threadIdx.x; q < min(e, total_listed); q += TPB) {
+        const int v = kept[q], n_groups = q < a ? G : q < r ? g + 1 : g;
+#pragma unroll 8
+        for (int gq = 0; gq < n_groups; ++gq) {
+          const int seen = vis[(int64_t)gq * total_listed + q] ? v : 0;
+          if (q >= a && gq == g) in += seen;
+          else rows += seen;
+        }
+      }
     }
     rows = __reduce_add_sync(0xffffffffu, rows); in = __reduce_add_sync(0xffffffffu, in);
     if ((threadIdx.x & 31) == 0) { before[threadIdx.x >> 5] = rows; inside[threadIdx.x >> 5] = in; }
@@ -359,8 +403,10 @@ cudaError_t rc_launch_compact(const recache_ctx* ctx, const CompactArgs& a, cuda
   }
   const int64_t pairs = (int64_t)a.total_listed * G;
   // Packed rows of few pairs: the gather's CTAs each add up what lies before their rows (a pass over 5 bytes a pair out of
-  // L2) instead of waiting for a launch that does it once.  Encode,
-  // compaction and prefill of 6 resources in fp32 43.9 -> 41.6 us.
+  // L2) instead of waiting for a launch that does it once.  Indices alone, us with a plan launch and without, eight groups
+  // that see a quarter of the list: 8-64 pairs 8.4 and 5.9; 1024 (2 requests x 64 resources) 9.5 and 6.9; 4096 as 1 x 512
+  // 20.8 and 13.4, as 2 x 256 16.8 and 12.8, as 4 x 128 15.2 and 12.9.  Where they see all of it: 2048 (4 x 64) 14.5 and 13.9,
+  // 4096 as 1 x 512 28 and 26, as 4 x 128 23 and 25, as 64 x 8 24 and 28: the pass grows with the pairs times the visible ones.
   const bool with_plan = a.mode == RECACHE_PACKED && a.total_listed > 0 && a.n_requests > 0 && pairs <= PLAN_PAIRS;
   if (!with_plan) {
     RcLaunchScope scope(ctx, RC_K_COMPACT_PLAN, st);

@@ -61,6 +61,45 @@ def test_counts_and_tables(lens, gap, requests, groups):
     assert rc.poll_status() == 0
 
 
+@pytest.mark.parametrize("n,requests,groups", [
+    (9, 8, 1), (129, 9, 1), (33, 16, 1), (17, 17, 1), (65, 32, 1), (9, 33, 1), (5, 64, 1), (9, 65, 1), (3, 128, 1), (5, 129, 1), (2, 300, 1),
+    (64, 1, 8), (65, 1, 8), (100, 5, 8),
+])
+def test_lengths_where_lanes_share_routes(n, requests, groups):
+    """A gather that plans for itself deals a route's resources to 32, 16, 8, 4, 2 or 1 lanes, four at a time, and adds up pairs
+    by pair up to 512, by resource beyond."""
+    test_counts_and_tables([1 + i % 3 for i in range(n)], 1, requests, groups)
+
+
+@pytest.mark.parametrize("requests,visible", [(2, 0.25), (4, 1.0), (64, 1.0)])
+def test_time_on_both_sides_of_the_gather_that_plans_for_itself(requests, visible):
+    """4096 pairs take no more than a fifth longer without a plan launch than a few pairs more take with one, indices alone.
+    (Measured 0.75-1.15; with a thread to each pair and to each of 9-32 routes 1.4-1.8.)"""
+    sh = wl.Shape(8, 8, 64, 1e4, "bf16")
+    rc = make_ctx(sh, max_pos=4096)
+    rng = np.random.default_rng(requests)
+    calls = []
+    for each in (512 // requests, 512 // requests + 1):
+        n = each * requests
+        pool = torch.zeros((8, 8 * n, 64), dtype=sh.torch_dtype, device="cuda")
+        ints = lambda a, t=np.int32: dev(np.ascontiguousarray(a, dtype=t))
+        args = (pool, pool, ints(np.ones(8 * n), np.uint8), ints(np.arange(requests + 1) * each), ints(np.arange(n) * 8), ints(np.full(n, 8)),
+                ints(rng.random((8, n)) < visible, np.uint8), PACKED, ints(np.zeros(8 * requests + 1)), ints(np.zeros(64 * n)), None, None)
+        calls.append((args, torch.empty(rc.compact_workspace_bytes(requests, n), dtype=torch.uint8, device="cuda")))
+    best = [1e9, 1e9]
+    start, stop = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    for _ in range(8):
+        for i, (args, ws) in enumerate(calls):
+            start.record()
+            for _ in range(100):
+                rc.compact_routes(*args, workspace=ws)
+            stop.record()
+            stop.synchronize()
+            best[i] = min(best[i], start.elapsed_time(stop))
+    assert best[0] < 1.2 * best[1], best
+    assert rc.poll_status() == 0
+
+
 @pytest.mark.parametrize("n,requests", [(255, 2), (256, 2), (257, 2), (1, 513)])   # eight groups: 4096 pairs are 512 listed resources
 def test_offsets_around_the_gather_that_plans_for_itself(n, requests):
     test_counts_and_tables([1 + i % 3 for i in range(n)], 1, requests, 8)
