@@ -262,6 +262,7 @@ __global__ void __launch_bounds__(TPB) compact_gather_kernel(
   const int n = res_len[r];
   if (n <= 0 || s0 < 0 || s0 + n > pool_tokens) return;   // flagged by the count kernel
   const int b = rc_find_segment(res_off, n_requests, r);
+  if (r < res_off[b] || r >= res_off[b + 1]) return;      // a resource that no request lists (a list with room behind its last)
   const int route = b * G + g;
   int in_route;
   int64_t route_base, page_base = 0;

@@ -103,3 +103,34 @@ def test_time_on_both_sides_of_the_gather_that_plans_for_itself(requests, visibl
 @pytest.mark.parametrize("n,requests", [(255, 2), (256, 2), (257, 2), (1, 513)])   # eight groups: 4096 pairs are 512 listed resources
 def test_offsets_around_the_gather_that_plans_for_itself(n, requests):
     test_counts_and_tables([1 + i % 3 for i in range(n)], 1, requests, 8)
+
+
+@pytest.mark.parametrize("mode", [PACKED, PAGED])
+@pytest.mark.parametrize("requests", [2, 200])            # three resources of each: 48 pairs, and more than a gather plans for
+def test_resources_that_no_request_lists_leave_no_trace(mode, requests):
+    """Lists with room before the first request and behind the last, filled with visible resources: the outputs are those of the
+    requests' own lists."""
+    groups, d = 8, 64
+    sh = wl.Shape(groups, groups, d, 1e4, "bf16")
+    rc = make_ctx(sh, max_pos=4096)
+    rng = np.random.default_rng(requests)
+    lens, spare = rng.integers(1, 40, 3 * requests).astype(np.int32), 5
+    slot = np.concatenate([[0], np.cumsum(lens)])[:-1].astype(np.int32)
+    pool = int(lens.sum())
+    k, v = (wl.normal(i, (groups, pool, d), sh.torch_dtype).cuda() for i in (1, 2))
+    keep, vis = rng.integers(0, 2, pool).astype(np.uint8), rng.integers(0, 2, (groups, 3 * requests)).astype(np.uint8)
+    n_pages = requests * groups * 2 + 1                    # a route has at most 117 rows: two pages of 64
+    got = []
+    for room in (0, spare):
+        wide = lambda a: np.concatenate([a[:room], a, a[-room:]]) if room else a
+        ones = np.ones((groups, room), np.uint8)
+        cu, idx, length = (torch.full((n,), -7, dtype=torch.int32, device="cuda") for n in (requests * groups + 1, groups * pool, requests * groups))
+        rows = (groups * pool, d) if mode == PACKED else (n_pages, 64, d)
+        k_out, v_out = (torch.full(rows, -7, dtype=sh.torch_dtype, device="cuda") for _ in range(2))
+        table = torch.full((requests * groups, 2), -7, dtype=torch.int32, device="cuda")
+        pages = dict(page_table=table, free_pages=dev(np.arange(n_pages, dtype=np.int32))) if mode == PAGED else {}
+        rc.compact_routes(k, v, dev(keep), dev((np.arange(requests + 1) * 3 + room).astype(np.int32)), dev(wide(slot)), dev(wide(lens)),
+                          dev(np.concatenate([ones, vis, ones], 1)), mode, cu, idx, k_out, v_out, route_len=length,
+                          workspace=torch.zeros(rc.compact_workspace_bytes(requests, 3 * requests + 2 * room), dtype=torch.uint8, device="cuda"), **pages)
+        got.append((cu, idx, length, k_out, v_out, table))
+    assert all(torch.equal(a, b) for a, b in zip(*got)) and rc.poll_status() == 0
