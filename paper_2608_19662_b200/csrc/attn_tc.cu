@@ -706,6 +706,9 @@ static bool tc_may_split(const recache_ctx* ctx, int64_t max_items) {
 //   first turns: 1 x 512 tokens 32.1 / 40.3, 4 x 1024 (1024 items) 97.1 / 98.9, 16 x 256 (1024) 80.3 / 86.7, 16 x 512 (2048) 157 / 152
 // Where a route has room for more than 64 K/V tiles, an item is long, and the pair's fewer loads count for more (the
 // room is all the host knows of it; only the time depends on it): 2048 tokens over 64 long tools (512 items) 300 / 290.
+// Behind a shared prefix an encode's items are as long as the prefix, which is known here:
+//   500 rows, 6 x 1000 tokens, 2 heads a group (792 items) 75.9 / 75.8; 2000 rows, 1 x 1500, 4 heads (376) 77.9 / 92.2,
+//   4 x 500 (528) 89.3 / 81.4; 8000 rows, 1 x 500 (128) 71.3 / 118, 2 x 500 (264) 145 / 124, 4 x 500, 2 heads (280) 150 / 127
 // A gather's copies are bound by the rate at which a CTA issues them, so it always takes pairs.
 // A later turn is split, if at all, in items of one tile (tc_may_split), so up to SPLIT_ROUNDS rounds of CTAs it has one;
 // so it has where no request has a second tile to pair (32 x 16 tokens over 4000 rows, 2 heads a group 128 / 151).  Beyond,
@@ -721,7 +724,9 @@ static int tc_item_tiles(const recache_ctx* ctx, const TcAttnArgs& a) {
     if (items <= SPLIT_ROUNDS * ctas || a.max_len <= tc_tok_per_item(ctx, 1)) return 1;
     return items <= 8 * ctas && a.route_rows / G + a.self_rows <= (int64_t)24 * TILE_N * a.n_seq ? 1 : 2;
   }
-  const int rounds = !a.route_cu ? 6 : a.route_rows > 64 * TILE_N * G * a.n_seq ? 2 : 8;
+  int rounds;
+  if (a.route_cu) rounds = a.route_rows > 64 * TILE_N * G * a.n_seq ? 2 : 8;
+  else rounds = a.prefix_len <= 8 * TILE_N ? 6 : a.prefix_len <= 32 * TILE_N ? 3 : 1;
   return items <= rounds * ctas ? 1 : 2;
 }
 

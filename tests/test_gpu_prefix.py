@@ -3,6 +3,7 @@
 import numpy as np
 import pytest
 import torch
+from torch.profiler import ProfilerActivity, profile
 
 from oracle import recache_oracle as orc
 from paper_2608_19662_b200 import workloads as wl
@@ -55,4 +56,34 @@ def test_prefixed_and_block_encode(shape, tol, lens, P):
     b = rc.encode_resources_prefixed(dev(pool.q), dev(pool.k), dev(pool.v), dev(pool.cu_seqlens), pool.max_len,
                                      dev(pool.dst_slot), kc2, vc2)
     assert torch.equal(a, b) and torch.equal(kc1, kc2)
+    assert rc.poll_status() == 0
+
+
+# 148 SMs, eight groups: up to 8 K/V tiles of prefix 888 work items of 128 rows are encoded one by one, up to 32 tiles 444, beyond 148
+@pytest.mark.parametrize("hq,prefix,most", [(16, 150, 888), (32, 1024, 888), (64, 1025, 444), (16, 4096, 444), (32, 4097, 148), (64, 6000, 148)])
+def test_kernel_and_bits_on_both_sides(hq, prefix, most):
+    """A resource encoded with as many others as fit under the limit, and with one more: by the kernel with a tile to an item and by the
+    one with pairs, to the same bits.  Queries times eight: rows rescale their sums several times on the way."""
+    g, d = 8, 128
+    sh = wl.Shape(hq, g, d, 1e6, "bf16")
+    rc = make_ctx(sh, max_pos=16384)
+    N = lambda i, *s: dev(wl.normal(60 + i, s, sh.torch_dtype))
+    kp, vp = N(3, g, prefix, d), N(4, g, prefix, d)
+    tile = 128 // (hq // g)
+    first, fit = 2 * tile + 5, (most // g - 2) * tile      # two resources: items = tokens / tile + 2, for each group
+    all_q, all_k, all_v = ((N(i, fit + tile, h, d).float() * f).to(sh.torch_dtype) for i, h, f in ((0, hq, 8), (1, g, 1), (2, g, 1)))
+    got = []
+    for n in (fit, fit + tile):
+        cu, q, k, v = dev(np.array([0, first, n], np.int32)), all_q[:n], all_k[:n], all_v[:n]
+        kc, vc = (torch.zeros((g, n, d), dtype=sh.torch_dtype, device="cuda") for _ in range(2))
+        run = lambda: rc.encode_resources_prefixed(q, k, v, cu, n, cu[:2], kc, vc, k_prefix=kp, v_prefix=vp,
+                                                   pos_offset=torch.full((2,), prefix, dtype=torch.int32, device="cuda"))
+        run()
+        torch.cuda.synchronize()
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            o = run()
+            torch.cuda.synchronize()
+        got.append((" ".join(e.name for e in prof.events()), o[:first]))
+    assert "attn_tile_kernel" in got[0][0] and "attn_tc_kernel" in got[1][0]
+    assert torch.equal(got[0][1], got[1][1]) and torch.isfinite(got[0][1]).all()
     assert rc.poll_status() == 0
