@@ -683,9 +683,11 @@ static int tc_tok_per_item(const recache_ctx* ctx, int item_tiles) { return item
 static int64_t tc_max_items(const recache_ctx* ctx, int n_seq, int total, int item_tiles) {
   return (int64_t)total / tc_tok_per_item(ctx, item_tiles) + n_seq;
 }
+// Work items of a sequence up to which its length is taken for what max_len says: whole pairs of tiles in both kernels, so that
+// a call is not refused by one of them that the other takes.
 static int tc_levels(const recache_ctx* ctx, int max_len, int item_tiles) {
-  const int t = tc_tok_per_item(ctx, item_tiles);
-  return (max_len + t - 1) / t + 1;
+  const int t = tc_tok_per_item(ctx, 2);
+  return ((max_len + t - 1) / t + 1) * (2 / item_tiles);
 }
 
 static int tc_ctas(const recache_ctx* ctx) { return ctx->sm_count > 0 ? ctx->sm_count : 148; }

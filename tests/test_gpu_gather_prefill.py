@@ -98,3 +98,22 @@ def test_gather_prefill_unsupported_context():
     with pytest.raises(RuntimeError):
         rc.attend_prefill_gather(dev(req.q), dev(req.k_conv), dev(req.v_conv), dev(req.cu_q), dev(req.q_pos0), req.max_q,
                                  kc, vc, r_idx, r_cu)
+
+
+@pytest.mark.parametrize("tokens,status", [(96, 0), (97, 0), (128, 0), (129, 1)])
+def test_both_prefills_take_the_same_lengths(tokens, status):
+    """A request longer than max_q says is taken up to the end of the next pair of query tiles, by packed and gathered
+    rows alike (one tile to an item here, and a pair), and reported beyond (bad lengths)."""
+    sh = wl.QWEN3_4B                                     # tiles of 32 tokens
+    g, d = sh.n_kv_heads, sh.head_dim
+    rc = make_ctx(sh, max_pos=256)
+    N = lambda i, *s: dev(wl.normal(40 + i, s, sh.torch_dtype))
+    q, k, v, rows = N(0, tokens, sh.n_q_heads, d), N(1, tokens, g, d), N(2, tokens, g, d), N(3, g, 1, d)
+    cu, none = dev(np.array([0, tokens], np.int32)), torch.zeros(g + 1, dtype=torch.int32, device="cuda")
+    packed = lambda max_q: rc.attend_prefill(q, k, v, cu, none[:1], max_q, rows[0], rows[0], none)[0]
+    want = packed(tokens)
+    assert rc.poll_status() == 0
+    for call in (packed, lambda max_q: rc.attend_prefill_gather(q, k, v, cu, none[:1], max_q, rows, rows, none, none)[0]):
+        got = call(64)
+        assert rc.poll_status() == status
+        assert status or torch.equal(got, want)
