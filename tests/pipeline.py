@@ -158,3 +158,14 @@ def sample_rows(rng, cu, n_heads, n_samples, extra_tokens=()):
     while len(rows) < n_samples:
         rows.append((int(rng.integers(0, total)), int(rng.integers(0, n_heads))))
     return rows
+
+
+def kernels_of(run):
+    """(result of run(), names of the kernels that it launched), after a first run."""
+    from torch.profiler import ProfilerActivity, profile
+    run()
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA], acc_events=True) as prof:
+        result = run()
+        torch.cuda.synchronize()
+    return result, " ".join(e.name for e in prof.events())

@@ -4,11 +4,10 @@ whichever it is, as the choice may follow from the room of a cache."""
 import numpy as np
 import pytest
 import torch
-from torch.profiler import ProfilerActivity, profile
 
 from paper_2608_19662_b200 import workloads as wl
 
-from pipeline import dev, make_ctx
+from pipeline import dev, kernels_of, make_ctx
 
 pytestmark = pytest.mark.gpu
 
@@ -22,7 +21,7 @@ def _turn(hq, batch, new, hist, room):
     rc = make_ctx(sh, max_pos=8192)
     N = lambda i, *s: dev(wl.normal(800 + i, s, sh.torch_dtype))
     n = batch * new
-    q, k, v = N(0, n, hq, d), N(1, n, g, d), N(2, n, g, d)
+    q, k, v = (N(0, n, hq, d).float() * 8).to(sh.torch_dtype), N(1, n, g, d), N(2, n, g, d)     # (a spread that makes rows rescale their sums)
     kc, vc = (torch.full((g, batch * room, d), float("nan"), dtype=sh.torch_dtype, device="cuda") for _ in range(2))
     for i, c in ((3, kc), (4, vc)):
         c.view(g, batch, room, d)[:, :, :hist] = N(i, g, batch, hist, d)
@@ -31,12 +30,7 @@ def _turn(hq, batch, new, hist, room):
     none = torch.zeros(batch * g + 1, dtype=torch.int32, device="cuda")
     rows = N(5, 1, d)
     run = lambda: rc.attend_prefill_history(q, k, v, step * new, hist_len, new, rows, rows, none, kc, vc, step[:-1] * room, hist_len)
-    run()
-    torch.cuda.synchronize()
-    with profile(activities=[ProfilerActivity.CUDA]) as prof:
-        o = run()
-        torch.cuda.synchronize()
-    names = " ".join(e.name for e in prof.events())
+    o, names = kernels_of(run)
     assert ("attn_tile_kernel" in names) != ("attn_tc_kernel" in names)
     assert rc.poll_status() == 0
     return o, "tile" if "attn_tile_kernel" in names else "pair"

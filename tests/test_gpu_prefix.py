@@ -3,12 +3,11 @@
 import numpy as np
 import pytest
 import torch
-from torch.profiler import ProfilerActivity, profile
 
 from oracle import recache_oracle as orc
 from paper_2608_19662_b200 import workloads as wl
 
-from pipeline import dev, f64, make_ctx, max_abs
+from pipeline import dev, f64, kernels_of, make_ctx, max_abs
 from test_gpu_parity import assert_rotated_close
 
 pytestmark = pytest.mark.gpu
@@ -78,12 +77,8 @@ def test_kernel_and_bits_on_both_sides(hq, prefix, most):
         kc, vc = (torch.zeros((g, n, d), dtype=sh.torch_dtype, device="cuda") for _ in range(2))
         run = lambda: rc.encode_resources_prefixed(q, k, v, cu, n, cu[:2], kc, vc, k_prefix=kp, v_prefix=vp,
                                                    pos_offset=torch.full((2,), prefix, dtype=torch.int32, device="cuda"))
-        run()
-        torch.cuda.synchronize()
-        with profile(activities=[ProfilerActivity.CUDA]) as prof:
-            o = run()
-            torch.cuda.synchronize()
-        got.append((" ".join(e.name for e in prof.events()), o[:first]))
-    assert "attn_tile_kernel" in got[0][0] and "attn_tc_kernel" in got[1][0]
-    assert torch.equal(got[0][1], got[1][1]) and torch.isfinite(got[0][1]).all()
+        o, names = kernels_of(run)
+        got.append((o[:first], names))
+    assert "attn_tile_kernel" in got[0][1] and "attn_tc_kernel" in got[1][1]
+    assert torch.equal(got[0][0], got[1][0]) and torch.isfinite(got[0][0]).all()
     assert rc.poll_status() == 0

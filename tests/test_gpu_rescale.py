@@ -12,7 +12,7 @@ import torch
 
 from paper_2608_19662_b200 import workloads as wl
 
-from pipeline import (f64, gpu_compact, gpu_encode, gpu_prefill, make_ctx, max_abs, oracle_encode, oracle_prefill,
+from pipeline import (dev, f64, gpu_compact, gpu_encode, gpu_prefill, kernels_of, make_ctx, max_abs, oracle_encode, oracle_prefill,
                       oracle_rows)
 
 pytestmark = pytest.mark.gpu
@@ -62,4 +62,36 @@ def test_wide_score_spread_takes_the_rescale_path():
     assert torch.isfinite(o_pre).all()
     assert max_abs(o_pre, ref_pre) < TOL
     assert float(np.median(np.abs(f64(o_pre) - ref_pre).max(axis=(1, 2)))) < 1e-2
+    assert rc.poll_status() == 0
+
+
+@pytest.mark.parametrize("hq", [16, 32, 64])
+def test_one_tile_and_pairs_rescale_to_the_same_bits(hq):
+    """The same spread in both tensor-core kernels, which carry a row's reference and its sums differently: resources encoded
+    alone and beside so many others that pairs of tiles are taken, and requests over packed and over gathered rows."""
+    sh = wl.Shape(hq, 8, 128, 1e6, "bf16")
+    rng = np.random.default_rng(hq)
+    lens = [700, 260, 64, 129]
+    more = lens + [1000] * 2 + [16 * 64 * 111 // hq] * 7         # 888 work items are tokens * hq / 128 / 8, for each of 8 groups
+    masks = wl.keep_mask_spans(rng, more)
+    rc = make_ctx(sh, max_pos=16384)
+    few, many = (wl.pack_resources(sh, 77, l, masks[:len(l)]) for l in (lens, more))
+    for pool in (few, many):
+        pool.q = _scaled(pool.q)
+    n = sum(lens)
+    assert torch.equal(few.q, many.q[:n])
+    (a, kc, vc), names_a = kernels_of(lambda: gpu_encode(rc, few))
+    (b, _, _), names_b = kernels_of(lambda: gpu_encode(rc, many))
+    assert "attn_tile_kernel" in names_a and "attn_tc_kernel" in names_b
+    assert torch.equal(a, b[:n]) and torch.isfinite(a).all()
+
+    lists = [[0, 1, 2, 3], [1, 0]]
+    req = wl.make_requests(sh, 99, few, lists, [wl.routes_random(rng, 8, len(l), 0.6) for l in lists], [200, 333])
+    req.q = _scaled(req.q)
+    rows = gpu_compact(rc, few, req, kc, vc)
+    (a, _, _), names_a = kernels_of(lambda: gpu_prefill(rc, req, rows["k_out"], rows["v_out"], rows["route_cu"]))
+    (b, _, _), names_b = kernels_of(lambda: rc.attend_prefill_gather(dev(req.q), dev(req.k_conv), dev(req.v_conv), dev(req.cu_q), dev(req.q_pos0), req.max_q, kc, vc,
+                                                                     rows["route_idx"], rows["route_cu"], out_dtype=torch.float32))
+    assert "attn_tile_kernel" in names_a and "attn_tc_kernel" in names_b
+    assert torch.equal(a, b) and torch.isfinite(a).all()
     assert rc.poll_status() == 0
