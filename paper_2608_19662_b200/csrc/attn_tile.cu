@@ -70,16 +70,8 @@ static_assert(SM_ALLOC <= 227 * 1024, "shared memory of a CTA");
 
 constexpr uint32_t COL_O = 0, COL_S = 128;           // + 128 * buffer
 
-// Bounded wait, see rc_mbar_wait: gives up after WAIT_PROBES probes, or when another thread of the CTA has (a word of
-// shared memory says so).  Written for size, as it stands some forty times in the kernel, whose roles together share 32 KB of
-// instruction cache: the status word is set once, where a kernel that gave up ends.
-__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, uint32_t gave_up) {
-  asm volatile("{\n\t.reg .pred p;\n\t.reg .u32 n, a;\n\tmov.u32 n, 0;\n"
-               "again:\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%0], %1;\n\t@p bra done;\n\t"
-               "ld.volatile.shared.u32 a, [%2];\n\tadd.u32 n, n, 1;\n\tsetp.ne.u32 p, a, 0;\n\t@p bra done;\n\t"
-               "setp.lt.u32 p, n, %3;\n\t@p bra again;\n\tst.volatile.shared.u32 [%2], 1;\n"
-               "done:\n\t}" ::"r"(bar), "r"(parity), "r"(gave_up), "n"(WAIT_PROBES) : "memory");
-}
+// Bounded wait: see rc_mbar_wait_small.
+__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, uint32_t gave_up) { rc_mbar_wait_small<WAIT_PROBES>(bar, parity, gave_up); }
 
 // ---------------------------------------------------------------- kernel --
 // Barriers, n counting the CTA's K/V tiles and j its items, all of them on through the launch; a phase of each is awaited before the

@@ -128,6 +128,17 @@ __device__ __forceinline__ void rc_mbar_wait(uint32_t bar, uint32_t parity, vola
     }
   }
 }
+// The same written for size, for a kernel in which it stands some forty times and whose roles together share 32 KB of instruction
+// cache: gives up after PROBES probes, or when another thread of the CTA has (the word at gave_up in shared memory
+// says so).  The status word is set once, where a kernel that gave up ends.
+template <uint32_t PROBES>
+__device__ __forceinline__ void rc_mbar_wait_small(uint32_t bar, uint32_t parity, uint32_t gave_up) {
+  asm volatile("{\n\t.reg .pred p;\n\t.reg .u32 n, a;\n\tmov.u32 n, 0;\n"
+               "again:\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%0], %1;\n\t@p bra done;\n\t"
+               "ld.volatile.shared.u32 a, [%2];\n\tadd.u32 n, n, 1;\n\tsetp.ne.u32 p, a, 0;\n\t@p bra done;\n\t"
+               "setp.lt.u32 p, n, %3;\n\t@p bra again;\n\tst.volatile.shared.u32 [%2], 1;\n"
+               "done:\n\t}" ::"r"(bar), "r"(parity), "r"(gave_up), "n"(PROBES) : "memory");
+}
 // After a wait ran out the roles fall through their loops with loads, copies and MMAs possibly
 // still in flight.  Let them land (none depends on another CTA; ~100 us is far more than any of
 // them takes) before shared and tensor memory go away under them.
