@@ -240,7 +240,9 @@ RECACHE_API recache_status recache_compact_routes(recache_ctx* ctx,
  * causal self-attention of the conversation.
  *   q [total_q][Hq][d], k_conv/v_conv [total_q][G][d] pre-rotation;
  *   cu_q [B+1], q_pos0 [B];  max_q >= every request's length;
- *   k_route/v_route packed [route_rows][d] with route_cu [B*G+1] (from compaction)
+ *   k_route/v_route packed [route_rows][d] with route_cu [B*G+1] (from compaction).  Their lengths
+ *       are on the device: the call is laid out for routes as long as route_rows allows, and with room
+ *       for more than 8192 rows a route a call of some hundred query tiles takes up to a tenth longer
  * Outputs
  *   k_conv_out/v_conv_out [G][total_q][d]: rotated conversation keys / values,
  *       head-major (the rows a later decode step keeps as history); required
@@ -268,9 +270,11 @@ RECACHE_API recache_status recache_attend_prefill(recache_ctx* ctx,
  * (page id = (g * cache_rows + conv_slot[b]) / 64 + n).
  * Where the requests of a call would leave SMs idle, their keys are divided between
  * the SMs (bf16, head_dim 128; only with a workspace of
- * recache_prefill_history_workspace_bytes(), else the call runs undivided): the order of summation, and with it the last bits of a
- * request's result, then follow from the lengths of all requests of the call.  They
- * never follow from the capacity of a buffer.  (recache_attend_prefill and
+ * recache_prefill_history_workspace_bytes(), else the call runs undivided): the order of
+ * summation, and with it the last bits of a request's result, then follow from the lengths of
+ * all requests of the call.  They never follow from the capacity of a buffer; the time of a larger
+ * call does (route_rows, cache_rows: room for more than 3072 rows a request is taken for long
+ * requests, which costs short ones some per cent).  (recache_attend_prefill and
  * recache_attend_prefill_gather never divide: there a request's result does not
  * depend on the other requests either.)
  */

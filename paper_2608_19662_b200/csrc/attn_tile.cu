@@ -1,6 +1,7 @@
-// Tensor-core attention with ONE query tile to a work item (bf16, head_dim 128, Hq/G in {2,4,8}): later turns, and encodes
-// and packed prefills of few items a CTA.  (attn_tc.cu takes a pair; rule and figures at tc_item_tiles there.  The launch
-// alone, with a pair and with one: encoding one tool 21.1 and 16.9 us, one request's turn 25.0 and 19.1, later turns 39 and 33.)
+// Tensor-core attention with ONE query tile to a work item (bf16, head_dim 128, Hq/G in {2,4,8}): encodes, packed
+// prefills and later turns of few items a CTA.  (attn_tc.cu takes a pair; rule and figures at tc_item_tiles there.  Between
+// two events, which add the launch's start to it, with a pair and with one: encoding one tool 21.1 and 16.9 us, one request's
+// turn 25.0 and 19.1, later turns 39 and 33.)
 //
 // Persistent kernel, one CTA per SM; a work item = (sequence, KV group, query tile).
 // A query tile is 128 rows = (128 / s) consecutive tokens x the s query heads of the group, so every K/V

@@ -421,10 +421,12 @@ cudaError_t rc_launch_compact(const recache_ctx* ctx, const CompactArgs& a, cuda
     const unsigned z = (unsigned)(!a.k_out || pairs >= 2048 ? 1 : (2048 + pairs - 1) / pairs > 8 ? 8 : (2048 + pairs - 1) / pairs);
     dim3 grid((unsigned)a.total_listed + (with_plan ? 1 : 0), (unsigned)G, z);
     RcLaunchScope scope(ctx, RC_K_COMPACT_GATHER, st);
-    e = rc_launch_overlapped(with_plan ? compact_gather_kernel<true> : compact_gather_kernel<false>, grid, TPB, 0, st, (const uint8_t*)a.k_cache, (const uint8_t*)a.v_cache, a.pool_tokens, a.keep,
-                             a.res_off, a.res_slot, a.res_len, a.n_requests, a.total_listed, a.vis, G, a.mode, ctx->desc.page_tokens,
-                             (const int32_t*)w.kept, a.route_cu, a.route_len, (const int32_t*)w.res_route_off, w.page_cu, a.route_idx, a.row_capacity,
-                             (uint8_t*)a.k_out, (uint8_t*)a.v_out, a.free_pages, a.n_free_pages, a.n_pool_pages, row_bytes, ctx->status);
+    e = rc_launch_overlapped(with_plan ? compact_gather_kernel<true> : compact_gather_kernel<false>, grid, TPB, 0, st,
+                             (const uint8_t*)a.k_cache, (const uint8_t*)a.v_cache, a.pool_tokens, a.keep, a.res_off, a.res_slot,
+                             a.res_len, a.n_requests, a.total_listed, a.vis, G, a.mode, ctx->desc.page_tokens,
+                             (const int32_t*)w.kept, a.route_cu, a.route_len, (const int32_t*)w.res_route_off, w.page_cu,
+                             a.route_idx, a.row_capacity, (uint8_t*)a.k_out, (uint8_t*)a.v_out, a.free_pages, a.n_free_pages,
+                             a.n_pool_pages, row_bytes, ctx->status);
   }
   return e;
 }

@@ -214,4 +214,5 @@ using Item = RcItem;
 }  // namespace rc_tc
 
 // The attention with one query tile to a work item, and the merge of the parts of a split launch (attn_tile.cu).
-cudaError_t rc_launch_attn_tile(const recache_ctx* ctx, const rc_tc::TcMaps& m, const rc_tc::TcParams& p, bool f32, bool split, unsigned grid, cudaStream_t st);
+cudaError_t rc_launch_attn_tile(const recache_ctx* ctx, const rc_tc::TcMaps& m, const rc_tc::TcParams& p, bool f32, bool split,
+                                unsigned grid, cudaStream_t st);

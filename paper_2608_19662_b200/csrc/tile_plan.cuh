@@ -10,10 +10,11 @@ constexpr int RC_SORT_MAX = 4096;    // work items up to which the plan sorts a 
 constexpr int RC_ITEM_UNITS = 2;     // what beginning an item costs, in K/V tiles of about 0.95 us
 constexpr int RC_MERGE_UNITS = 12;   // what parts and their merge cost
 constexpr int RC_L2_BLOCKS = 768;    // 100 MB: what of the 126 MB L2 a launch's keys and values may take
-constexpr int RC_PLAN_BINS = 1024;   // weights (K/V tiles, tile pairs) are told apart up to this
+constexpr int RC_PLAN_BINS = 1024;   // weights (K/V tiles, items) are told apart up to this
 
 struct RcPlan {
-  int2* items; int32_t* header;   // header[0] = number of items, header[1] = work counter, header[2] = order[] is valid, header[3] = CTAs of a split launch
+  int2* items;
+  int32_t* header;                // number of items, work counter, whether order[] is valid, CTAs of a split launch
   int32_t* order;                 // work indices, heaviest first (launches of at most RC_SORT_MAX work items); K/V tiles of each behind them
   // Split launch (null: not wanted): CTA c takes the K/V tiles from start[c] = (work index, tile) up to start[c + 1].
   // merge[c]: what the merge does at cut c: parts of the item it is the first cut of (0: nothing to do), first token of the
@@ -69,7 +70,12 @@ __device__ __forceinline__ bool rc_load_item(const RcPlan& p, int w, RcItem& it)
   return ok;
 }
 
-struct RcPlanSmem { int hist[RC_PLAN_BINS + 1]; int warp_sum[33]; int most; int blocks; };   // blocks: of 256 key and value rows (128 KB) that the launch reads
+struct RcPlanSmem {
+  int hist[RC_PLAN_BINS + 1];
+  int warp_sum[33];
+  int most;         // K/V tiles of the longest item
+  int blocks;       // of 256 key and value rows (128 KB) that the launch reads
+};
 
 // Exclusive block scan of one int per thread; *total gets the sum (same pattern of calls in every thread).
 __device__ __forceinline__ int rc_plan_scan(int v, RcPlanSmem& sh, int* total) {
@@ -172,19 +178,19 @@ __device__ __forceinline__ bool rc_plan_split(const RcPlan& p, RcPlanSmem& sh, i
   return true;
 }
 
-// Items = (sequence, tile-pair index): sequence by sequence, the longest sequences
-// first, and inside a sequence the last (heaviest) tile pair first, so that the
+// Items = (sequence, index of one or two query tiles, as item_tiles says): sequence by sequence, the longest sequences
+// first, and inside a sequence the last (heaviest) first, so that the
 // launch ends on the light items of short sequences.  With the KV group as the
 // fastest index of the flattened work list, the CTAs that run at the same time
 // share one sequence's K/V, which then stays in L2 instead of being streamed
-// from HBM once per tile pair.  One block.  (Sequences of equal length land in an
+// from HBM once per item.  One block.  (Sequences of equal length land in an
 // order that may differ between launches; no result depends on it.)
 // (Nothing is unrolled: the block runs every loop for a step or two, out of a cold instruction cache, and
 // the unrolled code took 0.3-0.4 us more of turns of 35-50 us.)
 __device__ __forceinline__ void rc_build_plan(const RcPlan& p, RcPlanSmem& sh) {
   const int tid = threadIdx.x, n_thr = blockDim.x, n_seq = p.n_seq, tok_per_item = p.item_tiles * 128 / p.s;
   const int32_t* cu = p.cu;
-  auto n_pairs = [&](int b) {
+  auto n_items_of = [&](int b) {
     const int len = cu[b + 1] - cu[b];
     return min(len > 0 ? (len + tok_per_item - 1) / tok_per_item : 0, p.n_levels);
   };
@@ -197,7 +203,7 @@ __device__ __forceinline__ void rc_build_plan(const RcPlan& p, RcPlanSmem& sh) {
     const int len = cu[b + 1] - cu[b];
     if (len < 0 || (len + tok_per_item - 1) / tok_per_item > p.n_levels)   // not monotone, or longer than the max_len given
       rc_set_status(p.status, RECACHE_DEV_BAD_SEQLENS);
-    sum += n_pairs(b);
+    sum += n_items_of(b);
   }
 #pragma unroll 1
   for (int i = tid; i <= RC_PLAN_BINS; i += n_thr) sh.hist[i] = 0;
@@ -208,11 +214,11 @@ __device__ __forceinline__ void rc_build_plan(const RcPlan& p, RcPlanSmem& sh) {
   const bool sorted = n_work <= (p.route_cu ? RC_SORT_MAX : RC_SORT_MAX / 4);
   if (tid == 0) { p.header[0] = n_items; p.header[1] = 0; p.header[2] = sorted ? 1 : 0; p.header[3] = 0; }
   if (!sorted) {
-    // counting sort of the sequences by their number of tile pairs, longest first: hist[bin] = items of
+    // counting sort of the sequences by their number of items, longest first: hist[bin] = items of
     // that bin, then the first item index of the bin
 #pragma unroll 1
     for (int b = b0; b < b1; ++b) {
-      const int nt = n_pairs(b);
+      const int nt = n_items_of(b);
       if (nt > 0) atomicAdd(&sh.hist[RC_PLAN_BINS - min(nt, RC_PLAN_BINS)], nt);
     }
     __syncthreads();
@@ -220,7 +226,7 @@ __device__ __forceinline__ void rc_build_plan(const RcPlan& p, RcPlanSmem& sh) {
   }
 #pragma unroll 1
   for (int b = b0; b < b1; ++b) {
-    const int nt = n_pairs(b);
+    const int nt = n_items_of(b);
     if (nt == 0) continue;
     if (!sorted) k = atomicAdd(&sh.hist[RC_PLAN_BINS - min(nt, RC_PLAN_BINS)], nt);
 #pragma unroll 1
