@@ -692,8 +692,8 @@ static int tc_levels(const recache_ctx* ctx, int max_len, int item_tiles) {
 
 static int tc_ctas(const recache_ctx* ctx) { return ctx->sm_count > 0 ? ctx->sm_count : 148; }
 // A later turn of at most this many rounds of CTAs, in items of one query tile, may be split (see rc_plan_split).
-// Of 61 turns of 3-4 rounds none was more than 1 % faster split than whole by the better of the two kernels; of 426 with
-// fewer items 89 were by 5-55 %.
+// Of 61 turns of 3-4 rounds none was more than 1 % faster split than whole by the better of the two kernels; of 391 with
+// fewer items 100 are 5-58 % faster split than whole.
 constexpr int64_t SPLIT_ROUNDS = 3;
 static bool tc_may_split(const recache_ctx* ctx, int64_t max_items) {
   const int64_t n = max_items * ctx->desc.n_kv_heads;
@@ -713,12 +713,12 @@ static bool tc_may_split(const recache_ctx* ctx, int64_t max_items) {
 //   4 x 500 (528) 89.3 / 81.4; 8000 rows, 1 x 500 (128) 71.3 / 118, 2 x 500 (264) 145 / 124, 4 x 500, 2 heads (280) 150 / 127
 // A gather's copies are bound by the rate at which a CTA issues them, so it always takes pairs.
 // A later turn is split, if at all, in items of one tile (tc_may_split), so up to SPLIT_ROUNDS rounds of CTAs it has one;
-// so it has where no request has a second tile to pair (32 x 16 tokens over 4000 rows, 2 heads a group 128 / 151).  Beyond,
+// so it has where no request has a second tile to pair (32 x 16 tokens over 4000 rows, 2 heads a group 118 / 141).  Beyond,
 // never split, it goes by the room for its keys, 24 K/V tiles an item, up to eight rounds, and takes pairs from there:
-//   2 heads, 16 x 256 tokens (640 items) over 300 rows 62.4 / 64.1, over 4000 229 / 195
-//   4 heads, 8 x 256 (576) over 300 53.7 / 53.1, over 4000 209 / 183; 16 x 512 (2176) over 300 217 / 205
-//   of 320 turns of random sizes those of 3-8 rounds take 0.95 of the pair's time with up to 24 tiles an item (0.79-1.04), 1.02
-//   with more (0.94-1.14), those of more rounds 1.02 (0.95-1.11)
+//   2 heads, 16 x 256 tokens (640 items) over 300 rows 62.3 / 62.2, over 4000 219 / 189
+//   4 heads, 8 x 256 (576) over 300 56.8 / 54.6, over 4000 201 / 179; 16 x 512 (2176) over 300 212 / 196
+//   187 turns in a grid and at random: those of 3-8 rounds take 0.98 of the pair's time with up to 24 tiles an item
+//   (0.79-1.07), 1.05 with more (0.96-1.16), those of more rounds 1.04 (0.94-1.15)
 static int tc_item_tiles(const recache_ctx* ctx, const TcAttnArgs& a) {
   if (a.route_idx) return 2;
   const int64_t G = ctx->desc.n_kv_heads, ctas = tc_ctas(ctx), items = tc_max_items(ctx, a.n_seq, a.total, 1) * G;
@@ -749,7 +749,7 @@ int64_t rc_tc_split_bytes(const recache_ctx* ctx) {
 // to come in buffers of any size, of which the host cannot tell how much is filled.
 // Nothing here may depend on capacities, except to leave the merge launch out where rc_plan_split cannot say yes
 // whatever they hold: ranges have more than four units, and whole items take, in one round, RC_ITEM_UNITS more than the
-// longest has tiles, in more half its tiles more than a range.
+// longest has tiles, in more 0.6 of its tiles more than a range.
 static bool tc_splits(const recache_ctx* ctx, const TcAttnArgs& a, int64_t max_items) {
   if (!a.hist || !tc_may_split(ctx, max_items) || tc_ctas(ctx) < 2) return false;
   if (a.workspace_bytes < rc_tc_workspace_bytes(ctx, a.n_seq, a.total, a.max_len) + rc_tc_split_bytes(ctx)) return false;

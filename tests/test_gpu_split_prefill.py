@@ -139,12 +139,12 @@ def test_one_workspace_serves_the_largest_call_and_all_smaller_ones():
 
 
 @pytest.mark.parametrize("new,hist,split", [
-    ([16], 2032, False),          # eight items of 16 K/V tiles: the merge would take longer than what the parts save
-    ([16], 2033, True),           # of 17
+    ([16], 1904, False),          # eight items of 15 K/V tiles: the merge would take longer than what the parts save
+    ([16], 1905, True),           # of 16
     ([16] * 4, 1500, False),
     ([16] * 4, 2500, True),
     ([16] * 19, 1800, False),     # a second round of 4 CTAs; the merge would take as long
-    ([1216], 2000, False),        # 152 items of 17-26 tiles, short ones last
+    ([1216], 1000, False),        # 152 items of 9-18 tiles, short ones last
     ([1216], 3000, True),         # of 24-33
 ])
 def test_split_only_where_it_pays(new, hist, split):
