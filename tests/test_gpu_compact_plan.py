@@ -73,7 +73,7 @@ def test_lengths_where_lanes_share_routes(n, requests, groups):
 
 @pytest.mark.parametrize("requests,visible", [(2, 0.25), (4, 1.0), (64, 1.0)])
 def test_time_on_both_sides_of_the_gather_that_plans_for_itself(requests, visible):
-    """4096 pairs take no more than a fifth longer without a plan launch than a few pairs more take with one, indices alone.
+    """4096 pairs take less than 1.3 times without a plan launch what a few pairs more take with one, indices alone.
     (Measured 0.75-1.15; with a thread to each pair and to each of 9-32 routes 1.4-1.8.)"""
     sh = wl.Shape(8, 8, 64, 1e4, "bf16")
     rc = make_ctx(sh, max_pos=4096)
@@ -96,7 +96,7 @@ def test_time_on_both_sides_of_the_gather_that_plans_for_itself(requests, visibl
             stop.record()
             stop.synchronize()
             best[i] = min(best[i], start.elapsed_time(stop))
-    assert best[0] < 1.2 * best[1], best
+    assert best[0] < 1.3 * best[1], best
     assert rc.poll_status() == 0
 
 
