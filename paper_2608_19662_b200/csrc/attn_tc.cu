@@ -749,7 +749,7 @@ int64_t rc_tc_split_bytes(const recache_ctx* ctx) {
 // to come in buffers of any size, of which the host cannot tell how much is filled.
 // Nothing here may depend on capacities, except to leave the merge launch out where rc_plan_split cannot say yes
 // whatever they hold: ranges have more than four units, and whole items take, in one round, RC_ITEM_UNITS more than the
-// longest has tiles, in more 0.6 of its tiles more than a range.
+// longest has tiles, in more at most 0.8 of its tiles more than a range.
 static bool tc_splits(const recache_ctx* ctx, const TcAttnArgs& a, int64_t max_items) {
   if (!a.hist || !tc_may_split(ctx, max_items) || tc_ctas(ctx) < 2) return false;
   if (a.workspace_bytes < rc_tc_workspace_bytes(ctx, a.n_seq, a.total, a.max_len) + rc_tc_split_bytes(ctx)) return false;

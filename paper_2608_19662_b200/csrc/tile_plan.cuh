@@ -8,7 +8,7 @@
 constexpr int RC_TILE_N = 128;       // keys of a K/V tile
 constexpr int RC_SORT_MAX = 4096;    // work items up to which the plan sorts a prefill by weight (encode: a quarter)
 constexpr int RC_ITEM_UNITS = 2;     // what beginning an item costs, in K/V tiles of about 0.95 us
-constexpr int RC_MERGE_UNITS = 10;   // what parts and their merge cost
+constexpr int RC_MERGE_UNITS = 11;   // what parts and their merge cost
 constexpr int RC_L2_BLOCKS = 768;    // 100 MB: what of the 126 MB L2 a launch's keys and values may take
 constexpr int RC_PLAN_BINS = 1024;   // weights (K/V tiles, items) are told apart up to this
 
@@ -113,10 +113,11 @@ __device__ __forceinline__ void rc_plan_scan_bins(RcPlanSmem& sh) {
 // afterwards).  An item counts RC_ITEM_UNITS more than its tiles, and a cut is moved to the item's
 // edge where it would leave a part of fewer than two tiles, or a part whose first tile some row of
 // the item does not see.  Taken only where the longest CTA gets shorter by more than parts and merge cost.  Whole, a launch
-// of one round ends with its longest item, one of more 0.6 of that after the mean CTA; ranges take a fifth longer where
+// of one round ends with its longest item, one of more 0.8 of that after the mean CTA or, of items much alike, a little
+// after as many mean items as there are rounds; ranges take a fifth longer where
 // the launch reads more than L2 holds, as whole items of a sequence walk its keys in step and parts do not.  Chosen and
-// measured on 391 turns of up to three rounds, in a grid and at random, on inputs that are not in L2: the slower way is taken
-// at a mean cost of 0.1 % and of more than 3 % in 4 of them (0.7 % and 38 with six units for the merge, which pairs of tiles had).
+// measured on 602 turns of up to three rounds, in a grid and at random, on inputs that are not in L2: the slower way is taken
+// at a mean cost of 0.1 % and of more than 3 % in 9 of them (0.8 % and 67 with six units for the merge, which pairs of tiles had).
 //   1 request of 16 tokens, 2 heads a group, over 1000 / 4000 rows (8 items of 12 / 36 tiles): 24.8 / 32.7 us split, 23.4 / 44.3 whole
 //   4 x 16 tokens over 1000 (32 items of 13) 27.1 and 24.1; 8 x 17-250 over 300-2048 (152 items of 15) 42.9 and 41.7
 //   1 x 64 tokens, 4 heads, over 12,000 (16 items of 99) 42.8 and 100.8; 16 x 64 over 4000 (256 items of 37) 127 and 109
@@ -137,8 +138,10 @@ __device__ __forceinline__ bool rc_plan_split(const RcPlan& p, RcPlanSmem& sh, i
   const int n = min(p.n_cta, max(1, (total_units - RC_ITEM_UNITS * n_items) / 4));
   const float pace = sh.blocks > RC_L2_BLOCKS ? 1.2f : 1.f;
   const float split = pace * total_units / n + RC_ITEM_UNITS + RC_MERGE_UNITS;
-  const float whole = fmaxf((float)(sh.most + RC_ITEM_UNITS), n_items > p.n_cta ? (float)total_units / p.n_cta + 0.6f * sh.most : 0.f);
-  if (split > 0.95f * whole) return false;
+  float whole = 0.f;
+  if (n_items > p.n_cta)
+    whole = fminf((float)total_units / p.n_cta + 0.8f * sh.most, 1.05f * total_units / n_items * ((n_items + p.n_cta - 1) / p.n_cta));
+  if (split > fmaxf((float)(sh.most + RC_ITEM_UNITS), whole)) return false;
 #pragma unroll 1
   for (int w = w0; w < w1; ++w) { p.unit_cu[w] = at; if (tiles[w] > 0) at += tiles[w] + RC_ITEM_UNITS; }
   __syncthreads();

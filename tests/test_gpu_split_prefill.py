@@ -144,7 +144,7 @@ def test_one_workspace_serves_the_largest_call_and_all_smaller_ones():
     ([16] * 4, 1500, False),
     ([16] * 4, 2500, True),
     ([16] * 19, 1800, False),     # a second round of 4 CTAs; the merge would take as long
-    ([1216], 1000, False),        # 152 items of 9-18 tiles, short ones last
+    ([1216], 700, False),         # 152 items of 6-15 tiles, short ones last
     ([1216], 3000, True),         # of 24-33
 ])
 def test_split_only_where_it_pays(new, hist, split):
